@@ -178,6 +178,80 @@ __device__ __forceinline__ void bitcos_decode_row(const uint4 bm, const uint32_t
     }
 }
 
+// Inclusive scan over the lanes of a warp (the shuffle's own in-range predicate guards each addition).
+__device__ __forceinline__ uint32_t warp_scan_add(uint32_t v) {
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1)
+        asm volatile(
+            "{\n\t.reg .b32 o;\n\t.reg .pred p;\n\t"
+            "shfl.sync.up.b32 o|p, %0, %1, 0, 0xFFFFFFFF;\n\t"
+            "@p add.u32 %0, %0, o;\n\t}"
+            : "+r"(v)
+            : "r"(d));
+    return v;
+}
+// c + (low half of a) * (byte 0 of b) + (high half of a) * (byte 1 of b)
+__device__ __forceinline__ uint32_t dp2a_lo(uint32_t a, uint32_t b, uint32_t c) {
+    uint32_t d;
+    asm("dp2a.lo.u32.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+    return d;
+}
+
+// ---------------------------------------------------------------------------------------------
+// Decoder A in tensor-core fragment order (four tokens and more): a lane decodes presence word
+// t = lane % 4 of the four rows g + 8 i (g = lane / 4), which is exactly what the A operand of
+// mma.m16n8k32 wants of it when the 128 products of a group are taken in the order
+// "nibble 2 kb of every word, nibble 2 kb + 1 of every word": w[8 i + 2 kb] and w[8 i + 2 kb + 1] are the
+// fragment registers of row g + 8 i for k-block kb.  No transposition through shared memory.
+//   tile       the tile's 128 presence words (row major) in shared memory
+//   sg         the tile's piece of the sign vector; first = bit position of the tile's first sign bit in it
+// The words of the tile in order are index 32 i + lane, so a word's first sign bit is found by four warp
+// scans of the population counts, two to a register (a tile has at most 4096 non-zeros).
+// Every word keeps its sign window fixed and a running position: dp4a(e, e, pos) adds a nibble's
+// population count in the instruction that computes it, and one rotate brings the next four sign bits to
+// bits 12..15 (even nibbles; from a copy turned by four, to bits 8..11 for odd ones).
+// ---------------------------------------------------------------------------------------------
+__device__ __forceinline__ void bitcos_decode_fragments(const uint8_t *tile, const uint8_t *sg, uint32_t first, const uint8_t *lut,
+                                                        uint32_t lane4, int (&w)[32]) {
+    uint32_t P[4], c[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) P[i] = lds32(tile, 128u * i + lane4);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) c[i] = __popc(P[i]);
+    const uint32_t c01 = c[0] + (c[1] << 16), c23 = c[2] + (c[3] << 16);
+    const uint32_t s01 = warp_scan_add(c01), s23 = warp_scan_add(c23);
+    const uint32_t t01 = __shfl_sync(0xFFFFFFFFu, s01, 31), t23 = __shfl_sync(0xFFFFFFFFu, s23, 31);
+    // positions of the first sign bit of this lane's four words
+    const uint32_t b1 = dp2a_lo(t01, 0x0001u, first), b2 = dp2a_lo(t01, 0x0101u, first), b3 = dp2a_lo(t23, 0x0001u, b2);
+    const uint32_t at[4] = {dp2a_lo(s01 - c01, 0x0001u, first), dp2a_lo(s01 - c01, 0x0100u, b1), dp2a_lo(s23 - c23, 0x0001u, b2),
+                            dp2a_lo(s23 - c23, 0x0100u, b3)};
+    uint32_t A[4], B[4];
+    int pos[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const uint32_t o = (at[i] >> 3) & ~3u;
+        A[i] = __funnelshift_r(lds32(sg, o), lds32(sg, o + 4u), at[i]);
+        B[i] = __funnelshift_r(A[i], A[i], 4);
+        pos[i] = 20;                                  // a right rotation by 20 puts bit 0 on bit 12
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            // address bits 0..6 = lane * 4, bits 8..15 = presence byte k (bits 16.. are 0)
+            const uint32_t R = __byte_perm(P[i], lane4, 0x6504 | (k << 4));
+            uint32_t t = __funnelshift_r(A[i], A[i], pos[i]);
+            int e = static_cast<int>(lds32(lut, bit_select(t, R, 0xF000u)));
+            w[8 * i + 2 * k] = e;
+            pos[i] = __dp4a(e, e, pos[i]);
+            t = __funnelshift_r(B[i], B[i], pos[i]);
+            e = static_cast<int>(lds32(lut + 128, bit_select(t, R, 0x0F00u)));
+            w[8 * i + 2 * k + 1] = e;
+            if (k < 3) pos[i] = __dp4a(e, e, pos[i]);
+        }
+    }
+}
+
 // int32 accumulator of a decoded row against one token's group activations xg[0..7] (shared memory).
 __device__ __forceinline__ int row_contract(const int (&w)[32], const int4 *xg) {
     int a0 = 0, a1 = 0, a2 = 0, a3 = 0;

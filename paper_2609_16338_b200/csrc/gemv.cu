@@ -16,8 +16,9 @@
 // and an arrival counter), so results do not depend on scheduling.
 //
 // Contraction.  One or two tokens: dp4a against activations kept in shared memory.  Four tokens
-// and more: the decoded rows pass through a small shared-memory buffer to ldmatrix and
-// mma.m16n8k32 (int8 in, int32 out), so that the decode is paid once per call whatever the batch.
+// and more: mma.m16n8k32 (int8 in, int32 out), so that the decode is paid once per call whatever the
+// batch; BITCOS tiles are decoded in fragment order (bitcos_decode_fragments), the rows of the two
+// baseline formats pass through a small shared-memory buffer to ldmatrix.
 //
 // BITCOS decode (paper Section II-D, Eq. 4, adapted): the GPU has no bit-deposit
 // instruction, so four weights at a time are rebuilt from a (presence nibble, next four
@@ -1275,6 +1276,11 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
     bool tl_first = true;
     constexpr int RS = red_slots(NB);
     constexpr bool kMma = NB >= kMmaMinBatch;          // contraction on the tensor cores
+    // BITCOS tiles are decoded straight into the tensor cores' fragment order; the other formats (and the
+    // 16-bit variant) pass through the transposition buffer, whose 16 128-bit stores and ldmatrix of a tile
+    // keep the shared-memory pipe busy for about 70 clocks.  25600x5120: 22.0 -> 18.2 us at four tokens,
+    // 24.4 -> 20.4 at eight, 33.9 -> 31.9 at sixteen.
+    constexpr bool kFrag = kMma && FMT == kBitcos && !kBlend;
     constexpr int NH = NB > 8 ? 2 : 1;                 // 8-token halves of the batch
     constexpr int NV = kMma ? NH * 8 : NB;             // partial sums a lane hands to the epilogue warp
     const uint32_t lane4 = static_cast<uint32_t>(lane) * 4u;
@@ -1292,7 +1298,7 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
             xfrag[h] = nullptr;
             if (kMma && n < pr.nb(pb))
                 xfrag[h] = kBlend ? pb.x + static_cast<int64_t>(n) * pb.K * 2 + 64 * (lane & 3)
-                                  : pb.x + static_cast<int64_t>(pr.xrow(pb) ? __ldg(pr.xrow(pb) + n) : n) * pb.K + 16 * (lane & 3);
+                                  : pb.x + static_cast<int64_t>(pr.xrow(pb) ? __ldg(pr.xrow(pb) + n) : n) * pb.K + (kFrag ? 32 : 16) * (lane & 3);
         }
     };
     // (blended weights: of token lane / 4 this lane holds bytes 64 c .. 64 c + 63 of the group's 256,
@@ -1323,7 +1329,7 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
             if (xfrag[h]) {
                 const int4 *px = reinterpret_cast<const int4 *>(xfrag[h] + static_cast<int64_t>(g) * kGroup);
                 u0 = __ldg(px);
-                u1 = __ldg(px + 4);
+                u1 = __ldg(px + (kFrag ? 1 : 4));
             }
             bf[h][0] = u0.x; bf[h][1] = u0.y; bf[h][2] = u0.z; bf[h][3] = u0.w;
             bf[h][4] = u1.x; bf[h][5] = u1.y; bf[h][6] = u1.z; bf[h][7] = u1.w;
@@ -1422,7 +1428,10 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
             const uint8_t *xs = kXQ ? reinterpret_cast<const uint8_t *>(q_scr)
                                     : ((!Segs::kSingle && pl.x_in_stage) ? stage + off_x : xs_base) + static_cast<uint32_t>(g) * kGroup;
             int w[32];
-            if (FMT == kBitcos) {
+            if constexpr (kFrag) {
+                const uint32_t toff = *reinterpret_cast<const uint32_t *>(stage + off_toff + ((d.x >> 8) << 2));
+                bitcos_decode_fragments(stage + static_cast<uint32_t>(tile) * 512u, stage + off_sign, toff - d.w, lut, lane4, w);
+            } else if (FMT == kBitcos) {
                 const uint4 bm = *reinterpret_cast<const uint4 *>(stage + off_bm);
                 const int c = __popc(bm.x) + __popc(bm.y) + __popc(bm.z) + __popc(bm.w);
                 int incl = c;
@@ -1503,6 +1512,17 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
                     for (int mh = 0; mh < 2; ++mh)
 #pragma unroll
                         for (int r = 0; r < 4; ++r) acc[h][mh][r] = 0;
+                if constexpr (kFrag) {
+#pragma unroll
+                    for (int kb = 0; kb < 4; ++kb)
+#pragma unroll
+                        for (int mh = 0; mh < 2; ++mh) {
+                            const uint32_t a[4] = {static_cast<uint32_t>(w[16 * mh + 2 * kb]), static_cast<uint32_t>(w[16 * mh + 8 + 2 * kb]),
+                                                   static_cast<uint32_t>(w[16 * mh + 2 * kb + 1]), static_cast<uint32_t>(w[16 * mh + 9 + 2 * kb])};
+#pragma unroll
+                            for (int h = 0; h < NH; ++h) mma_s8(acc[h][mh], a, bf[h][2 * kb], bf[h][2 * kb + 1]);
+                        }
+                } else {
 #pragma unroll
                 for (int kb = 0; kb < 4; ++kb) {
                     // 32 weights of every row through the buffer: one k-block of the contraction
@@ -1519,10 +1539,14 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
                         for (int h = 0; h < NH; ++h) mma_s8(acc[h][mh], a, bf[h][2 * kb], bf[h][2 * kb + 1]);
                     }
                 }
+                }
                 // accumulator r of (h, mh): row 16 mh + lane / 4 + 8 (r / 2), token 8 h + 2 (lane % 4) + (r & 1)
                 float scq[4];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) scq[j] = __shfl_sync(0xFFFFFFFFu, sc, (lane >> 2) + 8 * j);
+                for (int j = 0; j < 4; ++j)
+                    scq[j] = kFrag ? bf16_to_float(*reinterpret_cast<const uint16_t *>(stage + L.payload_cap + L.sign_cap +
+                                                                                        static_cast<uint32_t>(tile * kRows + 8 * j + (lane >> 2)) * 2u))
+                                   : __shfl_sync(0xFFFFFFFFu, sc, (lane >> 2) + 8 * j);
 #pragma unroll
                 for (int h = 0; h < NH; ++h)
 #pragma unroll

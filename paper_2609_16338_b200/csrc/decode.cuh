@@ -211,46 +211,45 @@ __device__ __forceinline__ uint32_t dp2a_lo(uint32_t a, uint32_t b, uint32_t c) 
 // population count in the instruction that computes it, and one rotate brings the next four sign bits to
 // bits 12..15 (even nibbles; from a copy turned by four, to bits 8..11 for odd ones).
 // ---------------------------------------------------------------------------------------------
-__device__ __forceinline__ void bitcos_decode_fragments(const uint8_t *tile, const uint8_t *sg, uint32_t first, const uint8_t *lut,
-                                                        uint32_t lane4, int (&w)[32]) {
-    uint32_t P[4], c[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) P[i] = lds32(tile, 128u * i + lane4);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) c[i] = __popc(P[i]);
-    const uint32_t c01 = c[0] + (c[1] << 16), c23 = c[2] + (c[3] << 16);
-    const uint32_t s01 = warp_scan_add(c01), s23 = warp_scan_add(c23);
-    const uint32_t t01 = __shfl_sync(0xFFFFFFFFu, s01, 31), t23 = __shfl_sync(0xFFFFFFFFu, s23, 31);
-    // positions of the first sign bit of this lane's four words
-    const uint32_t b1 = dp2a_lo(t01, 0x0001u, first), b2 = dp2a_lo(t01, 0x0101u, first), b3 = dp2a_lo(t23, 0x0001u, b2);
-    const uint32_t at[4] = {dp2a_lo(s01 - c01, 0x0001u, first), dp2a_lo(s01 - c01, 0x0100u, b1), dp2a_lo(s23 - c23, 0x0001u, b2),
-                            dp2a_lo(s23 - c23, 0x0100u, b3)};
-    uint32_t A[4], B[4];
+struct FragmentRows {
+    uint32_t P[4], A[4], B[4];
     int pos[4];
+    __device__ __forceinline__ void open(const uint8_t *tile, const uint8_t *sg, uint32_t first, uint32_t lane4) {
+        uint32_t c[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const uint32_t o = (at[i] >> 3) & ~3u;
-        A[i] = __funnelshift_r(lds32(sg, o), lds32(sg, o + 4u), at[i]);
-        B[i] = __funnelshift_r(A[i], A[i], 4);
-        pos[i] = 20;                                  // a right rotation by 20 puts bit 0 on bit 12
+        for (int i = 0; i < 4; ++i) P[i] = lds32(tile, 128u * i + lane4);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) c[i] = __popc(P[i]);
+        const uint32_t c01 = c[0] + (c[1] << 16), c23 = c[2] + (c[3] << 16);
+        const uint32_t s01 = warp_scan_add(c01), s23 = warp_scan_add(c23);
+        const uint32_t t01 = __shfl_sync(0xFFFFFFFFu, s01, 31), t23 = __shfl_sync(0xFFFFFFFFu, s23, 31);
+        // positions of the first sign bit of this lane's four words
+        const uint32_t b1 = dp2a_lo(t01, 0x0001u, first), b2 = dp2a_lo(t01, 0x0101u, first), b3 = dp2a_lo(t23, 0x0001u, b2);
+        const uint32_t at[4] = {dp2a_lo(s01 - c01, 0x0001u, first), dp2a_lo(s01 - c01, 0x0100u, b1), dp2a_lo(s23 - c23, 0x0001u, b2),
+                                dp2a_lo(s23 - c23, 0x0100u, b3)};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint32_t o = (at[i] >> 3) & ~3u;
+            A[i] = __funnelshift_r(lds32(sg, o), lds32(sg, o + 4u), at[i]);
+            B[i] = __funnelshift_r(A[i], A[i], 4);
+            pos[i] = 20;                              // a right rotation by 20 puts bit 0 on bit 12
+        }
     }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
+    // fragment registers of byte k (nibbles 2 k and 2 k + 1) of the four rows: e[2 i], e[2 i + 1]
+    __device__ __forceinline__ void step(int k, const uint8_t *lut, uint32_t lane4, int (&e)[8]) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             // address bits 0..6 = lane * 4, bits 8..15 = presence byte k (bits 16.. are 0)
             const uint32_t R = __byte_perm(P[i], lane4, 0x6504 | (k << 4));
             uint32_t t = __funnelshift_r(A[i], A[i], pos[i]);
-            int e = static_cast<int>(lds32(lut, bit_select(t, R, 0xF000u)));
-            w[8 * i + 2 * k] = e;
-            pos[i] = __dp4a(e, e, pos[i]);
+            e[2 * i] = static_cast<int>(lds32(lut, bit_select(t, R, 0xF000u)));
+            pos[i] = __dp4a(e[2 * i], e[2 * i], pos[i]);
             t = __funnelshift_r(B[i], B[i], pos[i]);
-            e = static_cast<int>(lds32(lut + 128, bit_select(t, R, 0x0F00u)));
-            w[8 * i + 2 * k + 1] = e;
-            if (k < 3) pos[i] = __dp4a(e, e, pos[i]);
+            e[2 * i + 1] = static_cast<int>(lds32(lut + 128, bit_select(t, R, 0x0F00u)));
+            if (k < 3) pos[i] = __dp4a(e[2 * i + 1], e[2 * i + 1], pos[i]);
         }
     }
-}
+};
 
 // int32 accumulator of a decoded row against one token's group activations xg[0..7] (shared memory).
 __device__ __forceinline__ int row_contract(const int (&w)[32], const int4 *xg) {

@@ -74,7 +74,7 @@ struct Plan {
     int CS;          // column blocks per row
     int RBC;         // row blocks per item (1 unless CS == 1)
     int NW;          // decoder warps per thread block = ceil(CG * RBC / tpw)
-    int tpw;         // tiles of an item per decoder warp: 1, or 2 on large matrices (one or two tokens)
+    int tpw;         // tiles of an item per decoder warp: 1, or 2 on large matrices
     int64_t items;   // ceil(RB / RBC) * CS
     int cyclic;      // 1: blocks take whole row-block chunks round robin; 0: contiguous balanced ranges
     int stages;      // depth of the shared-memory ring (2 .. kMaxStages), set at launch
@@ -250,6 +250,21 @@ Plan make_plan(int64_t M, int64_t K, int max_warps_per_block, int tpw = 1) {
     return p;
 }
 
+// Pairs of tiles (BITCOS, two tokens and more): a warp takes two neighbouring groups of one row block and adds their
+// sums in registers, so with whole rows per item a row block takes ceil(G / 2) warps.
+Plan make_pair_plan(int64_t M, int64_t K, int max_warps) {
+    Plan p = make_plan(M, K, max_warps, 2);
+    if (p.CS == 1) {
+        const int wr = (p.CG + 1) / 2;
+        const int64_t RB = padded_rows(M) / kRows;
+        p.RBC = max_warps / wr;
+        if (p.RBC > RB) p.RBC = static_cast<int>(RB);
+        p.NW = p.RBC * wr;
+        p.items = (RB + p.RBC - 1) / p.RBC;
+    }
+    return p;
+}
+
 // workspace: [0, 256) header (word 0 = status), arrival counters, partial sums
 constexpr size_t kHeaderBytes = 256;
 size_t counters_bytes(int64_t RB) { return static_cast<size_t>((RB * 4 + 255) / 256 * 256); }
@@ -271,7 +286,7 @@ struct SmemLayout {
     uint32_t x;          // activations, [nb][K], if x_bytes != 0
     uint32_t x_bytes;    // 0: the activations do not fit and are read from global memory
     uint32_t red;        // 2 x [NW][NB][32] floats
-    uint32_t scr;        // tensor-core path: NW transposition buffers of kScrBytes
+    uint32_t scr;        // tensor-core path of the baselines and the 16-bit variant: NW transposition buffers of kScrBytes
     uint32_t bar;        // mbarriers, then per-stage sign base words
     uint32_t total;
 };
@@ -292,7 +307,18 @@ __host__ __device__ constexpr int red_swizzle(int row) {
 // decoders may run ahead of it).
 __host__ __device__ constexpr int red_slots(int nbmax) { return nbmax <= 1 ? 8 : nbmax <= 2 ? 4 : 2; }
 
-__host__ __device__ inline SmemLayout smem_layout(int fmt, const Plan &pl, int G, int nbmax, int64_t K) {
+// Bytes from one token's activations to the next in shared memory (the 16 bytes on top keep two tokens'
+// fragment loads off each other's banks).
+__host__ __device__ constexpr int64_t x_stride(int64_t K) { return K + 16; }
+
+// Which products decode their tiles in the tensor cores' fragment order (run_segments): BITCOS from two tokens on.
+// (clocks per tile and multiprocessor, 18944 -> 56832 x 5120, rows -> fragments: 107 -> 121 with one token, which
+// therefore keeps rows and dp4a; 148 -> 121 with two, 170 -> 133 with four, 186 -> 157 with eight, 268 -> 253 with
+// sixteen; with two tiles per warp 115, 127, 137 and 206.)
+__host__ __device__ constexpr bool fragment_order(int fmt, int nb) { return fmt == kBitcos && nb >= 2; }
+
+// scr: the tensor-core path passes its rows through transposition buffers
+__host__ __device__ inline SmemLayout smem_layout(int fmt, const Plan &pl, int G, int nbmax, int64_t K, bool scr) {
     SmemLayout L{};
     uint32_t off = 0;
     L.lut = off;
@@ -314,14 +340,14 @@ __host__ __device__ inline SmemLayout smem_layout(int fmt, const Plan &pl, int G
     }
     L.scale_cap = tiles * 64;
     L.off_cap = align_up(L.off_cap, 16);
-    L.x_cap = pl.x_in_stage ? static_cast<uint32_t>(nbmax * K) : 0u;
+    L.x_cap = pl.x_in_stage ? static_cast<uint32_t>(nbmax * x_stride(K)) : 0u;
     L.stage = off;
     L.stage_bytes = align_up(L.payload_cap + L.sign_cap + L.scale_cap + L.off_cap + L.x_cap, 128);
     off += L.stage_bytes * static_cast<uint32_t>(pl.stages);
     L.x = off;
     // (the tensor-core path takes its activation fragments straight from global memory)
     L.x_bytes = (nbmax < kMmaMinBatch && !pl.x_in_stage && static_cast<int64_t>(nbmax) * K <= kXResidentBytes)
-                    ? static_cast<uint32_t>(nbmax * K) : 0u;
+                    ? static_cast<uint32_t>(nbmax * x_stride(K)) : 0u;
     // (at least 128 bytes per decoder warp and token: the products that take 16-bit activations
     // quantise each warp's group into its own slice of this area)
     uint32_t x_area = L.x_bytes;
@@ -330,7 +356,7 @@ __host__ __device__ inline SmemLayout smem_layout(int fmt, const Plan &pl, int G
     L.red = off;
     off += static_cast<uint32_t>(red_slots(nbmax) / pl.tpw) * tiles * static_cast<uint32_t>(nbmax) * kRows * 4;
     L.scr = off;
-    off += (nbmax >= kMmaMinBatch) ? static_cast<uint32_t>(pl.NW) * kScrBytes : 0u;
+    off += scr ? static_cast<uint32_t>(pl.NW) * kScrBytes : 0u;
     L.bar = off;
     off += 512;          // mbarriers, then (16-byte aligned) one 16-byte item descriptor per stage
     L.total = off;
@@ -642,7 +668,7 @@ __device__ __forceinline__ void issue_item(const Problem &pb, const View &pr, co
         // find them next to the weights and need no block-wide staging step per group
         if (pl.x_in_stage)
             for (int b = 0; b < pr.nb(pb) && b < 2; ++b)
-                bulk_copy(d_scales + L.scale_cap + L.off_cap + static_cast<uint32_t>(b) * static_cast<uint32_t>(pb.K),
+                bulk_copy(d_scales + L.scale_cap + L.off_cap + static_cast<uint32_t>(b) * static_cast<uint32_t>(x_stride(pb.K)),
                           pb.x + static_cast<int64_t>(xrows[b]) * pb.K, static_cast<uint32_t>(pb.K), bar);
     };
     if (FMT == kBitcos) {
@@ -796,7 +822,8 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
     const Plan *plp = &pl_in;
 #define pb (*pbp)
 #define pl (*plp)
-    const SmemLayout L = smem_layout(FMT, pl, segs.shape().G, NB, segs.shape().K);
+    constexpr bool kFrag = fragment_order(FMT, NB) && !Segs::kBlend;
+    const SmemLayout L = smem_layout(FMT, pl, segs.shape().G, NB, segs.shape().K, NB >= kMmaMinBatch && !kFrag);
     typename Segs::View pr{};
     Walk wk{};
     const uint8_t *lut = smem + L.lut;
@@ -804,7 +831,8 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
     // per stage: {tiles | (first tile & 3) << 8, first group, first row block, first sign bit held}
     uint32_t *sign_base = reinterpret_cast<uint32_t *>(smem + L.bar + 384);
     const uint32_t bar0 = smem_addr(smem + L.bar);
-    static_assert(TPW == 1 || (TPW == 2 && NB < kMmaMinBatch), "two tiles per warp: one or two tokens only");
+    static_assert(TPW == 1 || (TPW == 2 && (kFrag || NB < kMmaMinBatch)), "two tiles per warp: fragment order, or one or two tokens");
+    constexpr bool kPairs = kFrag && TPW == 2;                 // one partial sum per warp, not per tile
     // one activation scale per token and group (applied by the decoder warps, tile by tile)
     // instead of one per token (applied by the epilogue warp to the finished sums)
     constexpr bool kXQ = Segs::kQuantize;                      // (one or two tokens only)
@@ -812,9 +840,9 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
     static_assert(!kBlend || (NB == 8 && FMT == kBitcos && TPW == 1), "blended weights: the eight-token BITCOS kernel");
     constexpr bool kXG = Segs::kGroupScales || kXQ || kBlend;   // no token scale in the epilogue
     static_assert(!kXQ || NB < kMmaMinBatch, "16-bit activations: one or two tokens only");
-    const uint32_t red_slot = static_cast<uint32_t>(pl.NW * TPW) * NB * kRows;     // floats per partial-sum slot
-    // partial-sum slots in use: red_slots(NB), half as many (of twice the size) with two tiles per warp
-    constexpr int rs_log2 = (red_slots(NB) == 8 ? 3 : red_slots(NB) == 4 ? 2 : 1) - (TPW - 1);
+    const uint32_t red_slot = static_cast<uint32_t>(kPairs ? pl.NW : pl.NW * TPW) * NB * kRows;     // floats per partial-sum slot
+    // partial-sum slots in use: red_slots(NB), half as many (of twice the size) where a warp leaves two tiles' sums
+    constexpr int rs_log2 = (red_slots(NB) == 8 ? 3 : red_slots(NB) == 4 ? 2 : 1) - (kPairs ? 0 : TPW - 1);
     constexpr int rs_mask = (1 << rs_log2) - 1;
 
     // Programmatic dependent launch: the next kernel in the stream may be scheduled as soon as
@@ -1050,7 +1078,7 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
         for (int b = 0; b < NB; ++b) {
             if (b < pr.nb(pb)) {
                 const int4 *src = reinterpret_cast<const int4 *>(pb.x + static_cast<int64_t>(xr[b]) * pb.K);
-                for (int q = tid; q < per_tok; q += nthr) xs[b * per_tok + q] = __ldg(src + q);
+                for (int q = tid; q < per_tok; q += nthr) xs[b * (per_tok + 1) + q] = __ldg(src + q);
             }
         }
     }
@@ -1067,7 +1095,7 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
 #pragma unroll
                 for (int b = 0; b < NB; ++b)
                     if (b < pr.nb(pb))
-                        bulk_copy(smem_addr(smem + L.x) + static_cast<uint32_t>(b) * static_cast<uint32_t>(pb.K),
+                        bulk_copy(smem_addr(smem + L.x) + static_cast<uint32_t>(b) * static_cast<uint32_t>(x_stride(pb.K)),
                                   pb.x + static_cast<int64_t>(xr[b]) * pb.K, static_cast<uint32_t>(pb.K), bar0 + 8u * kBarX);
             }
         };
@@ -1106,7 +1134,7 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
         // (up to 40 partial sums when a warp decodes two tiles per item: two trees of 20)
         auto sum_groups = [&](const float *base, int n) {
             float t = sum_groups20(base, n);
-            if (TPW == 2 && n > kMaxWarps) t += sum_groups20(base + kMaxWarps * NB * kRows, n - kMaxWarps);
+            if (TPW == 2 && !kPairs && n > kMaxWarps) t += sum_groups20(base + kMaxWarps * NB * kRows, n - kMaxWarps);
             return t;
         };
         // tensor-core layout: the same for four tokens at a time, n <= 20 float4 spaced one warp's
@@ -1191,11 +1219,11 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
                 // whole row blocks: one output per row.  The sums are formed first, the slot is
                 // handed back, and only then are the outputs stored, so that the release of the
                 // slot never waits for a global store.
-                const int nrb = r.nt / pb.G;
+                const int nrb = r.nt / pb.G, parts = kPairs ? (pb.G + 1) / 2 : pb.G;
                 for (int i = 0; i < nrb; ++i) {
                     const int64_t m = static_cast<int64_t>(r.rb0 + i) * kRows + lane;
                     float t_b[NB];
-                    sums(rs, i * pb.G, pb.G, t_b);
+                    sums(rs, i * parts, parts, t_b);
                     if (i == nrb - 1) {
                         __syncwarp();
                         if (lane == 0) mbar_arrive(bar0 + 8u * (kBarRedEmpty + slot));
@@ -1209,7 +1237,7 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
             // one column block of row block rb0: add it to the running sum
             const bool starts = (r.cs == 0) || (k == 0);
             float t_b[NB];
-            sums(rs, 0, r.nt, t_b);
+            sums(rs, 0, kPairs ? (r.nt + 1) / 2 : r.nt, t_b);
 #pragma unroll
             for (int b = 0; b < NB; ++b) run[b] = starts ? t_b[b] : run[b] + t_b[b];
             __syncwarp();
@@ -1256,6 +1284,298 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
         return;
     }
 
+    // ------------------------------------------------------------------ decoder warps, fragment order
+    // (tiles decoded straight into the A operands of the tensor cores, FragmentRows: no transposition through
+    // shared memory, and two tokens come out of the products that one would need)
+    if constexpr (kFrag) {
+        constexpr int NC = NB < 8 ? NB : 8;              // tokens in the n dimension of one product
+        constexpr int NH = NB > 8 ? 2 : 1;               // 8-token halves of the batch
+        // The eight columns of a product hold the tokens over and over (column n: token n % NC), so with fewer than
+        // eight tokens every lane has all of a tile's sums of its rows somewhere in its quad, and the quad
+        // shares out the rows: of rows g + 8 s (g = lane / 4), lane t takes slots s0 .. s0 + NS - 1, and of the
+        // tokens n0 and n0 + 1.
+        constexpr int NS = NC == 8 ? 4 : NC == 4 ? 2 : 1;
+        const int g8 = lane >> 2, t4 = lane & 3;
+        const int s0 = NC == 8 ? 0 : NC == 4 ? 2 * (t4 >> 1) : t4;
+        const int n0 = NC == 8 ? 2 * t4 : NC == 4 ? 2 * (t4 & 1) : 0;
+        const uint32_t lane4 = static_cast<uint32_t>(lane) * 4u;
+        // CS == 1: tile t of an item always is row block t / G of the chunk, group t % G
+        // (a phased launch works these out again for every job)
+        int rbl = 0, g_first = 0;
+        auto place = [&]() {
+            const int wr = (pb.G + TPW - 1) / TPW;       // warps per row block when items are whole rows
+            rbl = pl.CS == 1 ? warp / wr : 0;
+            g_first = (warp - rbl * wr) * TPW;
+        };
+        place();
+        int tile0 = rbl * pb.G + g_first;
+        uint32_t x_parity = 0;      // phase parity of the activations' barrier: one phase per segment of a phased launch
+        if (!mbar_wait(bar0 + 8u * kBarLut, 0)) {
+            if (lane == 0 && pr.status(pb)) *pr.status(pb) = 1u;
+            return;
+        }
+        if (warp == 0 && lane == 0) BITCOS_TL(3, clock64());
+        bool tl_first = true;
+        // B operand: of token g8 % NC (+ 8) this lane holds the 32 activations of presence word t4 of the group
+        const int8_t *xfrag[NH];
+        auto token_fragments = [&]() {
+#pragma unroll
+            for (int h = 0; h < NH; ++h) {
+                const int n = 8 * h + g8 % NC;
+                xfrag[h] = nullptr;
+                if (NB >= kMmaMinBatch && n < pr.nb(pb))
+                    xfrag[h] = pb.x + static_cast<int64_t>(pr.xrow(pb) ? __ldg(pr.xrow(pb) + n) : n) * pb.K + 32 * t4;
+            }
+        };
+        uint32_t bf[NH][8];
+        float xg[NH][2];            // group scales of the tokens whose sums this lane keeps
+        auto load_x = [&](int grp, const uint8_t *xs) {
+            if constexpr (NB < kMmaMinBatch) {
+                const uint4 *px = reinterpret_cast<const uint4 *>(xs + 32 * t4 + (g8 & 1) * (kXQ ? kGroup : static_cast<int>(x_stride(pb.K))));
+                const uint4 u0 = px[0], u1 = px[1];
+                bf[0][0] = u0.x; bf[0][1] = u0.y; bf[0][2] = u0.z; bf[0][3] = u0.w;
+                bf[0][4] = u1.x; bf[0][5] = u1.y; bf[0][6] = u1.z; bf[0][7] = u1.w;
+            } else {
+#pragma unroll
+                for (int h = 0; h < NH; ++h) {
+                    int4 u0 = make_int4(0, 0, 0, 0), u1 = make_int4(0, 0, 0, 0);
+                    if (xfrag[h]) {
+                        const int4 *px = reinterpret_cast<const int4 *>(xfrag[h] + static_cast<int64_t>(grp) * kGroup);
+                        u0 = __ldg(px);
+                        u1 = __ldg(px + 1);
+                    }
+                    bf[h][0] = u0.x; bf[h][1] = u0.y; bf[h][2] = u0.z; bf[h][3] = u0.w;
+                    bf[h][4] = u1.x; bf[h][5] = u1.y; bf[h][6] = u1.z; bf[h][7] = u1.w;
+                }
+            }
+            if constexpr (kXG && !kXQ) {
+                // (after the dependency wait: the scales come from the kernel before this one)
+#pragma unroll
+                for (int h = 0; h < NH; ++h)
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) {
+                        const int b = 8 * h + n0 + r;
+                        xg[h][r] = (b < pr.nb(pb)) ? __ldg(pb.x_scale + static_cast<int64_t>(b) * pb.G + grp) : 0.f;
+                    }
+            }
+        };
+        // 16-bit activations: the group this warp has quantised last, its scales, and its buffer
+        // ([token][128] int8 inside the activation area)
+        int q_g = -1;
+        float q_scale[2] = {};
+        uint32_t *q_scr = reinterpret_cast<uint32_t *>(smem + L.x) + static_cast<uint32_t>(warp) * (NB * kRows);
+        uint2 qv[2];
+        auto fetch_group = [&](int grp) {
+#pragma unroll
+            for (int b = 0; b < 2; ++b)
+                if (b < pr.nb(pb))
+                    qv[b] = __ldg(reinterpret_cast<const uint2 *>(reinterpret_cast<const uint16_t *>(pb.x) + static_cast<int64_t>(b) * pb.K +
+                                                                  static_cast<int64_t>(grp) * kGroup) + lane);
+        };
+        auto quantize_group = [&](int grp) {
+            // this warp quantises the group its tile multiplies (four values per lane, largest magnitude by
+            // shuffles) into its own 128 bytes per token
+            __syncwarp();                     // the previous tile's fragments have been read
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                if (b < pr.nb(pb)) {
+                    const uint2 v = qv[b];
+                    float a = fmaxf(fmaxf(fabsf(bf16_lo(v.x)), fabsf(bf16_hi(v.x))), fmaxf(fabsf(bf16_lo(v.y)), fabsf(bf16_hi(v.y))));
+#pragma unroll
+                    for (int dd = 16; dd; dd >>= 1) a = fmaxf(a, __shfl_xor_sync(0xFFFFFFFFu, a, dd));
+                    a = fmaxf(a, kAmaxFloor);
+                    const float inv = __fdiv_rn(127.0f, a);
+                    q_scale[b] = __fdiv_rn(a, 127.0f);
+                    q_scr[b * kRows + lane] = quant_pair(v.x, inv) | (quant_pair(v.y, inv) << 16);
+                }
+            }
+            __syncwarp();
+            q_g = grp;
+        };
+        // byte offsets inside a stage that depend on nothing but the layout
+        const uint32_t off_sign = L.payload_cap, off_scales = L.payload_cap + L.sign_cap;
+        const uint32_t off_x = off_scales + L.scale_cap + L.off_cap;                     // activations inside a stage
+        // where this lane leaves its partial sums inside a slot
+        float *rd0 = red + (NB >= kMmaMinBatch ? static_cast<uint32_t>(warp * kRows + g8) * NB : static_cast<uint32_t>(warp * NB * kRows + g8 + 8 * s0));
+        const uint8_t *stage = smem + L.stage;
+        uint32_t full_bar = bar0 + 8u * static_cast<uint32_t>(kBarFull), phase = 0;
+        int s = 0;
+        int kk = 0;                 // items decoded so far, over all segments
+        bool x_ready = false, x_held = false;
+        bool more_segments = false;
+        do {
+        if (!kLate) {
+            token_fragments();
+            x_ready = true;
+            x_held = false;
+        }
+        for (const int kk_end = kk + wk.count; kk < kk_end; ++kk) {
+            if (!mbar_wait(full_bar, phase)) {
+                if (lane == 0 && pr.status(pb)) *pr.status(pb) = 1u;
+                return;
+            }
+            if (tl_first && warp == 0 && lane == 0) BITCOS_TL(4, clock64());
+            if (tl_first && warp == 0 && lane == 0) BITCOS_TLP(src, 1);
+            const uint4 d = reinterpret_cast<const uint4 *>(sign_base)[s];
+            const int nt = static_cast<int>(d.x & 0xFFu);
+            float ysum[NH][NS][2];
+#pragma unroll
+            for (int h = 0; h < NH; ++h)
+#pragma unroll
+                for (int j = 0; j < NS; ++j) ysum[h][j][0] = ysum[h][j][1] = 0.f;
+#pragma unroll 1
+            for (int ti = 0; ti < TPW; ++ti) {
+                const int tile = tile0 + ti;
+                if (tile >= nt || (TPW == 2 && pl.CS == 1 && g_first + ti >= pb.G)) break;
+                // group: the item's first (0 when items are whole rows) + the tile's place in its row block
+                const int grp = static_cast<int>(d.y) + g_first + ti;
+                const uint8_t *xs = kXQ ? reinterpret_cast<const uint8_t *>(q_scr)
+                                        : ((!Segs::kSingle && pl.x_in_stage) ? stage + off_x : smem + L.x) + static_cast<uint32_t>(grp) * kGroup;
+                // from global memory: ahead of the decode, which hides the latency (not before the dependency is
+                // resolved); a warp whose group never changes keeps its fragments
+                if (NB >= kMmaMinBatch && x_ready && !(TPW == 1 && pl.CS == 1 && x_held)) {
+                    load_x(grp, xs);
+                    x_held = true;
+                }
+                if (kXQ && x_ready && grp != q_g) fetch_group(grp);
+                const uint32_t toff = *reinterpret_cast<const uint32_t *>(stage + off_scales + L.scale_cap + 4u * static_cast<uint32_t>(tile) + ((d.x >> 8) << 2));
+                FragmentRows rows;
+                rows.open(stage + 512u * static_cast<uint32_t>(tile), stage + off_sign, toff - d.w, lane4);
+                // One tile per warp: everything is decoded before the first product (launches of a few items, where a
+                // block's first decode runs while it waits for its dependency).  Two tiles: product by product.
+                constexpr bool kFused = TPW == 2;
+                int e[kFused ? 1 : 4][8];
+                if (!kFused) {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) rows.step(k, lut, lane4, e[kFused ? 0 : k]);
+                }
+                if (!x_ready) {
+                    // first contraction of this warp: the previous kernel must be complete before the activations
+                    // are read (the decode above did not need them)
+                    if (tl_first && warp == 0 && lane == 0) BITCOS_TL(5, clock64());
+                    if (tl_first && warp == 0 && lane == 0) BITCOS_TLP(src, 2);
+                    asm volatile("griddepcontrol.wait;" ::: "memory");
+                    if (kEarly && !kXQ && !mbar_wait(bar0 + 8u * kBarX, x_parity)) {
+                        if (lane == 0 && pr.status(pb)) *pr.status(pb) = 1u;
+                        return;
+                    }
+                    x_ready = true;
+                    if (tl_first && warp == 0 && lane == 0) BITCOS_TL(6, clock64());
+                    if (tl_first && warp == 0 && lane == 0) BITCOS_TLP(src, 3);
+                    token_fragments();
+                    if (NB >= kMmaMinBatch) {
+                        load_x(grp, xs);
+                        x_held = true;
+                    }
+                    if (kXQ) fetch_group(grp);
+                }
+                if (kXQ && grp != q_g) quantize_group(grp);
+                if (NB < kMmaMinBatch) load_x(grp, xs);
+                int acc[NH][2][4];
+#pragma unroll
+                for (int h = 0; h < NH; ++h)
+#pragma unroll
+                    for (int mh = 0; mh < 2; ++mh)
+#pragma unroll
+                        for (int r = 0; r < 4; ++r) acc[h][mh][r] = 0;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    int(&ek)[8] = e[kFused ? 0 : k];
+                    if (kFused) rows.step(k, lut, lane4, ek);
+#pragma unroll
+                    for (int mh = 0; mh < 2; ++mh) {
+                        const uint32_t a[4] = {static_cast<uint32_t>(ek[4 * mh]), static_cast<uint32_t>(ek[4 * mh + 2]),
+                                               static_cast<uint32_t>(ek[4 * mh + 1]), static_cast<uint32_t>(ek[4 * mh + 3])};
+#pragma unroll
+                        for (int h = 0; h < NH; ++h) mma_s8(acc[h][mh], a, bf[h][2 * k], bf[h][2 * k + 1]);
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < NS; ++j) {
+                    const float sc = bf16_to_float(*reinterpret_cast<const uint16_t *>(stage + off_scales + 2u * static_cast<uint32_t>(tile * kRows + g8 + 8 * (s0 + j))));
+#pragma unroll
+                    for (int h = 0; h < NH; ++h)
+#pragma unroll
+                        for (int r = 0; r < 2; ++r) {
+                            // row slot s of a token pair's accumulators: acc[h][s / 2][2 * (s % 2) + column]
+                            int v;
+                            if (NC == 8) v = acc[h][j >> 1][2 * (j & 1) + r];
+                            else if (NC == 4) v = (t4 & 2) ? acc[h][1][2 * j + r] : acc[h][0][2 * j + r];
+                            else {
+                                const int lo = (t4 & 1) ? acc[h][0][2 + r] : acc[h][0][r], hi = (t4 & 1) ? acc[h][1][2 + r] : acc[h][1][r];
+                                v = (t4 & 2) ? hi : lo;
+                            }
+                            float y = sc * static_cast<float>(v);
+                            if (kXQ) y *= q_scale[r];
+                            else if (kXG) y *= xg[h][r];
+                            ysum[h][j][r] += y;
+                            if (Segs::kDebug && pb.acc_debug) {
+                                const int b = 8 * h + n0 + r;
+                                const int64_t m = (static_cast<int64_t>(d.z) + rbl) * kRows + g8 + 8 * (s0 + j);
+                                if (b < pr.nb(pb) && m < pb.M) pb.acc_debug[((pr.out_row0(pb) + b) * pb.M + m) * pb.G + grp] = v;
+                            }
+                        }
+                }
+            }
+            // partial sums for the epilogue warp (several slots, so decoders may run ahead of it); the stage goes
+            // back to the producer when the epilogue warp has seen them
+            const int slot = kk & rs_mask;
+            if ((kk >> rs_log2) > 0) {
+                if (!mbar_wait(bar0 + 8u * (kBarRedEmpty + slot), static_cast<uint32_t>(((kk >> rs_log2) - 1) & 1))) {
+                    if (lane == 0 && pr.status(pb)) *pr.status(pb) = 1u;
+                    return;
+                }
+            }
+            float *rd = rd0 + slot * red_slot;
+            if (NB >= kMmaMinBatch) {
+#pragma unroll
+                for (int h = 0; h < NH; ++h)
+#pragma unroll
+                    for (int j = 0; j < NS; ++j)
+                        *reinterpret_cast<float2 *>(rd + 8 * (s0 + j) * NB + ((8 * h + n0) ^ red_swizzle<NB>(g8 + 8 * (s0 + j)))) =
+                            make_float2(ysum[h][j][0], ysum[h][j][1]);
+            } else {
+                rd[0] = ysum[0][0][0];
+                rd[kRows] = ysum[0][0][1];
+            }
+            __syncwarp();
+            mbar_arrive_lane0(bar0 + 8u * (kBarRedFull + slot), lane);
+            if (tl_first && warp == 0 && lane == 0) BITCOS_TL(7, clock64());
+            tl_first = false;
+            stage += L.stage_bytes;
+            full_bar += 8u;
+            if (++s == pl.stages) {
+                s = 0;
+                stage = smem + L.stage;
+                full_bar = bar0 + 8u * static_cast<uint32_t>(kBarFull);
+                phase ^= 1u;
+            }
+        }
+        if (warp == 0 && lane == 0) BITCOS_TL(10, clock64());
+        if (warp == 0 && lane == 0) BITCOS_TLP(src, 4);
+        if constexpr (Segs::kHetero) {
+            // Every decoder warp passes every phase of the activations' barrier, a warp without a tile in
+            // this segment included: a warp that skipped one could not tell the phase before from the
+            // phase after by its parity.
+            if (!x_ready && !mbar_wait(bar0 + 8u * kBarX, x_parity)) {
+                if (lane == 0 && pr.status(pb)) *pr.status(pb) = 1u;
+                return;
+            }
+            more_segments = next_segment();
+            tl_first = true;
+            if (more_segments) {
+                x_ready = false;
+                x_parity ^= 1u;
+                place();
+                tile0 = rbl * pb.G + g_first;
+            }
+        } else {
+            more_segments = next_segment();
+        }
+        } while (more_segments);
+        return;
+    }
+
     // ------------------------------------------------------------------ decoder warps
     // CS == 1: tile t of an item always is row block t / G of the chunk, group t % G; this warp
     // decodes tile `warp` and, with two tiles per warp, tile `warp + NW`
@@ -1276,11 +1596,6 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
     bool tl_first = true;
     constexpr int RS = red_slots(NB);
     constexpr bool kMma = NB >= kMmaMinBatch;          // contraction on the tensor cores
-    // BITCOS tiles are decoded straight into the tensor cores' fragment order; the other formats (and the
-    // 16-bit variant) pass through the transposition buffer, whose 16 128-bit stores and ldmatrix of a tile
-    // keep the shared-memory pipe busy for about 70 clocks.  25600x5120: 22.0 -> 18.2 us at four tokens,
-    // 24.4 -> 20.4 at eight, 33.9 -> 31.9 at sixteen.
-    constexpr bool kFrag = kMma && FMT == kBitcos && !kBlend;
     constexpr int NH = NB > 8 ? 2 : 1;                 // 8-token halves of the batch
     constexpr int NV = kMma ? NH * 8 : NB;             // partial sums a lane hands to the epilogue warp
     const uint32_t lane4 = static_cast<uint32_t>(lane) * 4u;
@@ -1298,7 +1613,7 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
             xfrag[h] = nullptr;
             if (kMma && n < pr.nb(pb))
                 xfrag[h] = kBlend ? pb.x + static_cast<int64_t>(n) * pb.K * 2 + 64 * (lane & 3)
-                                  : pb.x + static_cast<int64_t>(pr.xrow(pb) ? __ldg(pr.xrow(pb) + n) : n) * pb.K + (kFrag ? 32 : 16) * (lane & 3);
+                                  : pb.x + static_cast<int64_t>(pr.xrow(pb) ? __ldg(pr.xrow(pb) + n) : n) * pb.K + 16 * (lane & 3);
         }
     };
     // (blended weights: of token lane / 4 this lane holds bytes 64 c .. 64 c + 63 of the group's 256,
@@ -1329,7 +1644,7 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
             if (xfrag[h]) {
                 const int4 *px = reinterpret_cast<const int4 *>(xfrag[h] + static_cast<int64_t>(g) * kGroup);
                 u0 = __ldg(px);
-                u1 = __ldg(px + (kFrag ? 1 : 4));
+                u1 = __ldg(px + 4);
             }
             bf[h][0] = u0.x; bf[h][1] = u0.y; bf[h][2] = u0.z; bf[h][3] = u0.w;
             bf[h][4] = u1.x; bf[h][5] = u1.y; bf[h][6] = u1.z; bf[h][7] = u1.w;
@@ -1428,10 +1743,7 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
             const uint8_t *xs = kXQ ? reinterpret_cast<const uint8_t *>(q_scr)
                                     : ((!Segs::kSingle && pl.x_in_stage) ? stage + off_x : xs_base) + static_cast<uint32_t>(g) * kGroup;
             int w[32];
-            if constexpr (kFrag) {
-                const uint32_t toff = *reinterpret_cast<const uint32_t *>(stage + off_toff + ((d.x >> 8) << 2));
-                bitcos_decode_fragments(stage + static_cast<uint32_t>(tile) * 512u, stage + off_sign, toff - d.w, lut, lane4, w);
-            } else if (FMT == kBitcos) {
+            if (FMT == kBitcos) {
                 const uint4 bm = *reinterpret_cast<const uint4 *>(stage + off_bm);
                 const int c = __popc(bm.x) + __popc(bm.y) + __popc(bm.z) + __popc(bm.w);
                 int incl = c;
@@ -1512,17 +1824,6 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
                     for (int mh = 0; mh < 2; ++mh)
 #pragma unroll
                         for (int r = 0; r < 4; ++r) acc[h][mh][r] = 0;
-                if constexpr (kFrag) {
-#pragma unroll
-                    for (int kb = 0; kb < 4; ++kb)
-#pragma unroll
-                        for (int mh = 0; mh < 2; ++mh) {
-                            const uint32_t a[4] = {static_cast<uint32_t>(w[16 * mh + 2 * kb]), static_cast<uint32_t>(w[16 * mh + 8 + 2 * kb]),
-                                                   static_cast<uint32_t>(w[16 * mh + 2 * kb + 1]), static_cast<uint32_t>(w[16 * mh + 9 + 2 * kb])};
-#pragma unroll
-                            for (int h = 0; h < NH; ++h) mma_s8(acc[h][mh], a, bf[h][2 * kb], bf[h][2 * kb + 1]);
-                        }
-                } else {
 #pragma unroll
                 for (int kb = 0; kb < 4; ++kb) {
                     // 32 weights of every row through the buffer: one k-block of the contraction
@@ -1539,14 +1840,10 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
                         for (int h = 0; h < NH; ++h) mma_s8(acc[h][mh], a, bf[h][2 * kb], bf[h][2 * kb + 1]);
                     }
                 }
-                }
                 // accumulator r of (h, mh): row 16 mh + lane / 4 + 8 (r / 2), token 8 h + 2 (lane % 4) + (r & 1)
                 float scq[4];
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    scq[j] = kFrag ? bf16_to_float(*reinterpret_cast<const uint16_t *>(stage + L.payload_cap + L.sign_cap +
-                                                                                        static_cast<uint32_t>(tile * kRows + 8 * j + (lane >> 2)) * 2u))
-                                   : __shfl_sync(0xFFFFFFFFu, sc, (lane >> 2) + 8 * j);
+                for (int j = 0; j < 4; ++j) scq[j] = __shfl_sync(0xFFFFFFFFu, sc, (lane >> 2) + 8 * j);
 #pragma unroll
                 for (int h = 0; h < NH; ++h)
 #pragma unroll
@@ -1617,7 +1914,7 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
             for (int b = 0; b < NB; ++b) {
                 if (kMma) break;
                 if (NB == 1 || b < pr.nb(pb)) {       // a call has at least one token
-                    const int a = contract<FMT>(w, reinterpret_cast<const int4 *>(xs + static_cast<uint32_t>(b) * (kXQ ? static_cast<uint32_t>(kGroup) : static_cast<uint32_t>(pb.K))), lane);
+                    const int a = contract<FMT>(w, reinterpret_cast<const int4 *>(xs + static_cast<uint32_t>(b) * (kXQ ? static_cast<uint32_t>(kGroup) : static_cast<uint32_t>(x_stride(pb.K)))), lane);
                     ysum[b] = sc * static_cast<float>(a);
                     if (kXG) ysum[b] *= xgs[NB < kMmaMinBatch ? b : 0];
                     if (Segs::kDebug && pb.acc_debug) {
@@ -1712,11 +2009,13 @@ __device__ __forceinline__ void run_problem(const Problem &pr, const Plan &pl, u
     run_segments<FMT, NB, TPW>(one, pl, smem, block, fo, fo_index, pf, first_sent);
 }
 
-template <int FMT, int NB, int TPW = 1, bool XG = false, bool XQ = false, bool BL = false>
+// (DEBUG: the instantiation that also dumps the int32 accumulators.  The dump's addresses cost registers on the tile
+// loop whether it is asked for or not, so calls without it run a kernel that has no such code.)
+template <int FMT, int NB, int TPW = 1, bool XG = false, bool XQ = false, bool BL = false, bool DEBUG = false>
 __global__ void __launch_bounds__(max_block_threads(NB), 1) gemv_kernel(const Problem pr, const Plan pl,
                                                                         const __grid_constant__ FirstOff fo) {
     extern __shared__ __align__(128) uint8_t smem[];
-    run_problem<FMT, NB, !BL, TPW, XG, XQ, BL>(pr, pl, smem,
+    run_problem<FMT, NB, DEBUG, TPW, XG, XQ, BL>(pr, pl, smem,
                          block_walk(fo, static_cast<int>(blockIdx.x), pl, static_cast<int>(blockIdx.x), static_cast<int>(gridDim.x)),
                          static_cast<int>(blockIdx.x), &fo, static_cast<int>(blockIdx.x));
 }
@@ -1941,7 +2240,7 @@ __device__ __forceinline__ bool grouped_problem(Problem &pr, const Problem &base
 }
 
 // The pieces of the groups that fall into one thread block's range of the flat item list.
-template <int NB>
+template <int NB, bool DEBUG>
 struct GroupedSegs {
     const Problem *base;
     const GroupedArgs *ga;
@@ -1951,7 +2250,7 @@ struct GroupedSegs {
     static constexpr bool kSingle = false;
     static constexpr bool kHetero = false;
     static constexpr bool kListsLate = true;   // the routing lists are read only after the previous kernel has completed
-    static constexpr bool kDebug = true;
+    static constexpr bool kDebug = DEBUG;
     static constexpr bool kGroupScales = false;
     static constexpr bool kQuantize = false;
     static constexpr bool kBlend = false;
@@ -1992,7 +2291,7 @@ struct GroupedSegs {
 // that crosses from one group to the next keeps its pipeline running (the producer is already
 // copying the next group's weights while the last tiles of this one are decoded).  Otherwise:
 // blockIdx.y = group, and the blocks of a row of the grid share that group's items.
-template <int FMT, int NB>
+template <int FMT, int NB, bool DEBUG>
 __global__ void __launch_bounds__(max_block_threads(NB), 1) gemv_grouped_kernel(const __grid_constant__ Problem base, const Plan pl,
                                                                                 const __grid_constant__ GroupedArgs ga) {
     extern __shared__ __align__(128) uint8_t smem[];
@@ -2009,14 +2308,14 @@ __global__ void __launch_bounds__(max_block_threads(NB), 1) gemv_grouped_kernel(
         if (static_cast<int>(blockIdx.y) >= n_groups) return;
         Problem pr;
         if (!grouped_problem<NB>(pr, base, ga, static_cast<int>(blockIdx.y))) return;
-        run_problem<FMT, NB>(pr, pl, smem, make_walk(pl, static_cast<int>(blockIdx.x), static_cast<int>(gridDim.x)),
+        run_problem<FMT, NB, DEBUG>(pr, pl, smem, make_walk(pl, static_cast<int>(blockIdx.x), static_cast<int>(gridDim.x)),
                                  static_cast<int>(blockIdx.x));
         return;
     }
     const int64_t ipg = pl.items, total = ipg * n_groups;
     const int64_t nblk = gridDim.x, b = blockIdx.x;
     const int64_t q = total / nblk, rem = total - q * nblk;
-    GroupedSegs<NB> segs;
+    GroupedSegs<NB, DEBUG> segs;
     segs.base = &base;
     segs.ga = &ga;
     segs.ipg = ipg;
@@ -2229,11 +2528,11 @@ int prepare_kernel(int *sms_out, int *smem_budget_out) {
 
 // Ring depth: as many stages as fit next to the tables, activations and partial sums (the loaded
 // DRAM latency of this part needs on the order of 100 KB in flight per multiprocessor).
-inline int choose_stages(int fmt, const Plan &pl, int G, int nb, int64_t K, int smem_budget) {
+inline int choose_stages(int fmt, const Plan &pl, int G, int nb, int64_t K, int smem_budget, bool scr) {
     Plan p = pl;
     for (int st = kMaxStages; st > 2; --st) {
         p.stages = st;
-        if (static_cast<int>(smem_layout(fmt, p, G, nb, K).total) <= smem_budget) return st;
+        if (static_cast<int>(smem_layout(fmt, p, G, nb, K, scr).total) <= smem_budget) return st;
     }
     return 2;
 }
@@ -2336,36 +2635,59 @@ void fill_first_off(FirstOff &fo, int base, const uint32_t *off_host, const Prob
 // every block still gets several items: from eight of the one-tile items per multiprocessor on.  (Between
 // three and eight the gain depends on the shape and the format: 8192x5120 -3 % at one token but +6 % at
 // two, 4096x12288 +3 %, 2-bit +3 %; so those keep one tile per warp.)
-inline bool wants_two_tiles(const Plan &pl, int nb_template, int sms) {
-    return nb_template < kMmaMinBatch && pl.items >= 8 * static_cast<int64_t>(sms);
+// In fragment order a warp's two tiles also share one set of partial sums (added in registers: half the stores, and
+// half the additions of the epilogue warp) and the decode runs product by product, so the line lies lower, from 64
+// tiles per multiprocessor on.  Below it, 2x6912x2560 in one launch (58 tiles): layer pass 17.2 -> 17.9 us at two
+// tokens, 20.2 -> 22.2 at eight; above it, 8192x5120 (69 tiles): 6.80 -> 6.77, 8.41 -> 7.93, 12.0 -> 11.4 at sixteen;
+// 25600x5120 (216): 15.8 -> 15.5, 19.8 -> 18.1, 31.1 -> 27.1.
+inline bool wants_two_tiles(int fmt, int64_t items, int64_t tiles, int nb_template, int sms) {
+    if (fragment_order(fmt, nb_template)) return tiles >= 64 * static_cast<int64_t>(sms);
+    return nb_template < kMmaMinBatch && items >= 8 * static_cast<int64_t>(sms);
+}
+inline int64_t tile_count(int64_t M, int64_t K) { return padded_rows(M) / kRows * (K / kGroup); }
+// The plan of such a product.
+inline Plan two_tile_plan(int fmt, int64_t M, int64_t K, int nb_template) {
+    return fragment_order(fmt, nb_template) ? make_pair_plan(M, K, decoder_warps(nb_template)) : make_plan(M, K, decoder_warps(nb_template), 2);
 }
 
 template <int FMT, int NB, bool XG = false, bool XQ = false, bool BL = false>
 int launch(const Problem &pr, const Plan &pl_in, cudaStream_t stream, const uint32_t *off_host = nullptr) {
     // the one- and two-token instantiations keep the activations in shared memory (nb_bucket sees to it)
     if (NB < kMmaMinBatch && static_cast<int64_t>(NB) * pr.K > kXResidentBytes) return BITCOS_ERR_SHAPE;
+    constexpr bool kTwo = !BL && (NB < kMmaMinBatch || fragment_order(FMT, NB));      // a two-tile instantiation exists
+    constexpr bool kScr = NB >= kMmaMinBatch && (BL || !fragment_order(FMT, NB));
     int sms = 0, budget = 0;
     int rc = prepare_kernel<gemv_kernel<FMT, NB, 1, XG, XQ, BL>>(&sms, &budget);
     if (rc) return rc;
-    const bool two = wants_two_tiles(pl_in, NB, sms);
-    if constexpr (NB < kMmaMinBatch) {
+    const bool two = kTwo && !pr.acc_debug && wants_two_tiles(FMT, pl_in.items, tile_count(pr.M, pr.K), NB, sms);
+    if constexpr (kTwo) {
         if (two) {
             rc = prepare_kernel<gemv_kernel<FMT, NB, 2, XG, XQ>>(&sms, &budget);
             if (rc) return rc;
         }
     }
-    const Plan pl = two ? make_plan(pr.M, pr.K, decoder_warps(pr.nb), 2) : pl_in;
+    if constexpr (!BL) {
+        if (pr.acc_debug) {
+            rc = prepare_kernel<gemv_kernel<FMT, NB, 1, XG, XQ, false, true>>(&sms, &budget);
+            if (rc) return rc;
+        }
+    }
+    const Plan pl = two ? two_tile_plan(FMT, pr.M, pr.K, NB) : pl_in;
     int grid = 1;
     Plan plw = pl;
     choose_walk(plw, small_launch_cap(pl.items, sms), &grid);
-    plw.stages = choose_stages(FMT, pl, pr.G, NB, pr.K, budget);
-    const SmemLayout L = smem_layout(FMT, plw, pr.G, NB, pr.K);
+    plw.stages = choose_stages(FMT, pl, pr.G, NB, pr.K, budget, kScr);
+    const SmemLayout L = smem_layout(FMT, plw, pr.G, NB, pr.K, kScr);
     FirstOff fo;
     fo.valid = (FMT == kBitcos && off_host) ? 1 : 0;
     fo.walks = 1;
     fill_first_off(fo, 0, off_host, pr, plw, grid);
-    if constexpr (NB < kMmaMinBatch) {
+    if constexpr (kTwo) {
         if (two) return launch_pdl(gemv_kernel<FMT, NB, 2, XG, XQ>, dim3(grid), (pl.NW + 2) * 32, L.total, stream, pr, plw, fo);
+    }
+    if constexpr (!BL) {
+        if (pr.acc_debug)
+            return launch_pdl(gemv_kernel<FMT, NB, 1, XG, XQ, false, true>, dim3(grid), (pl.NW + 2) * 32, L.total, stream, pr, plw, fo);
     }
     return launch_pdl(gemv_kernel<FMT, NB, 1, XG, XQ, BL>, dim3(grid), (pl.NW + 2) * 32, L.total, stream, pr, plw, fo);
 }
@@ -2407,13 +2729,13 @@ inline int plan_multi(MultiArgs &ma, int nb_template, int sms, bool *two_out, in
     int64_t total_items = 0;
     for (int j = 0; j < ma.n; ++j) total_items += ma.pl[j].items;
     // enough items altogether: every problem with two tiles per decoder warp
-    Plan all{};
-    all.items = total_items;
-    const bool two = wants_two_tiles(all, nb_template, sms);
+    int64_t tiles = 0;
+    for (int j = 0; j < ma.n; ++j) tiles += tile_count(ma.pr[j].M, ma.pr[j].K);
+    const bool two = wants_two_tiles(kBitcos, total_items, tiles, nb_template, sms);
     if (two) {
         total_items = 0;
         for (int j = 0; j < ma.n; ++j) {
-            ma.pl[j] = make_plan(ma.pr[j].M, ma.pr[j].K, decoder_warps(nb_template), 2);
+            ma.pl[j] = two_tile_plan(kBitcos, ma.pr[j].M, ma.pr[j].K, nb_template);
             total_items += ma.pl[j].items;
         }
     }
@@ -2529,11 +2851,9 @@ int launch_multi(MultiArgs &ma, cudaStream_t stream, const uint32_t *const *off_
     bool two = false;
     int grids[kMaxJobs];
     const int total = plan_multi(ma, NB, sms, &two, grids);
-    if constexpr (NB < kMmaMinBatch) {
-        if (two) {
-            rc = prepare_kernel<gemv_multi_kernel<NB, 2, XQ, XG>>(&sms, &budget);
-            if (rc) return rc;
-        }
+    if (two) {
+        rc = prepare_kernel<gemv_multi_kernel<NB, 2, XQ, XG>>(&sms, &budget);
+        if (rc) return rc;
     }
     int nw = 0;
     uint32_t smem = 0;
@@ -2542,8 +2862,8 @@ int launch_multi(MultiArgs &ma, cudaStream_t stream, const uint32_t *const *off_
     fo.walks = 1;
     for (int j = 0; j < ma.n; ++j) fo.valid = (fo.valid && off_host[j]) ? 1 : 0;
     for (int j = 0; j < ma.n; ++j) {
-        ma.pl[j].stages = choose_stages(kBitcos, ma.pl[j], ma.pr[j].G, NB, ma.pr[j].K, budget);
-        const SmemLayout L = smem_layout(kBitcos, ma.pl[j], ma.pr[j].G, NB, ma.pr[j].K);
+        ma.pl[j].stages = choose_stages(kBitcos, ma.pl[j], ma.pr[j].G, NB, ma.pr[j].K, budget, false);
+        const SmemLayout L = smem_layout(kBitcos, ma.pl[j], ma.pr[j].G, NB, ma.pr[j].K, false);
         if (L.total > smem) smem = L.total;
         if (ma.pl[j].NW > nw) nw = ma.pl[j].NW;
     }
@@ -2593,7 +2913,7 @@ int launch_multi(MultiArgs &ma, cudaStream_t stream, const uint32_t *const *off_
             }
             fc.c[b] = FirstCopies{};
             if (fo.count[b] <= 0) continue;
-            const SmemLayout L = smem_layout(kBitcos, ma.pl[j], ma.pr[j].G, NB, ma.pr[j].K);
+            const SmemLayout L = smem_layout(kBitcos, ma.pl[j], ma.pr[j].G, NB, ma.pr[j].K, false);
             fill_first_copies(fc.c[b], ma.pr[j], ma.pl[j], L, fo.first[b], fo.lo[b], fo.hi[b]);
         }
     }
@@ -2603,9 +2923,7 @@ int launch_multi(MultiArgs &ma, cudaStream_t stream, const uint32_t *const *off_
         }
     }
     const NoFirstCopies none{0};
-    if constexpr (NB < kMmaMinBatch) {
-        if (two) return launch_pdl(gemv_multi_kernel<NB, 2, XQ, XG>, dim3(total), (nw + 2) * 32, smem, stream, ma, fo, none);
-    }
+    if (two) return launch_pdl(gemv_multi_kernel<NB, 2, XQ, XG>, dim3(total), (nw + 2) * 32, smem, stream, ma, fo, none);
     return launch_pdl(gemv_multi_kernel<NB, 1, XQ, XG>, dim3(total), (nw + 2) * 32, smem, stream, ma, fo, none);
 }
 
@@ -2630,12 +2948,15 @@ int launch_nb(const Problem &pr, const Plan &pl, cudaStream_t stream, const uint
 template <int FMT, int NB>
 int launch_grouped(const Problem &pr, const Plan &pl, const GroupedArgs &ga, int n_groups, cudaStream_t stream) {
     if (NB < kMmaMinBatch && static_cast<int64_t>(NB) * pr.K > kXResidentBytes) return BITCOS_ERR_SHAPE;
+    constexpr bool kScr = NB >= kMmaMinBatch && !fragment_order(FMT, NB);
     int sms = 0, budget = 0;
-    int rc = prepare_kernel<gemv_grouped_kernel<FMT, NB>>(&sms, &budget);
+    int rc = pr.acc_debug ? prepare_kernel<gemv_grouped_kernel<FMT, NB, true>>(&sms, &budget)
+                          : prepare_kernel<gemv_grouped_kernel<FMT, NB, false>>(&sms, &budget);
     if (rc) return rc;
+    const auto kernel = pr.acc_debug ? gemv_grouped_kernel<FMT, NB, true> : gemv_grouped_kernel<FMT, NB, false>;
     Plan plw = pl;
-    plw.stages = choose_stages(FMT, pl, pr.G, NB, pr.K, budget);
-    const SmemLayout L = smem_layout(FMT, plw, pr.G, NB, pr.K);
+    plw.stages = choose_stages(FMT, pl, pr.G, NB, pr.K, budget, kScr);
+    const SmemLayout L = smem_layout(FMT, plw, pr.G, NB, pr.K, kScr);
     GroupedArgs gaw = ga;
     gaw.n_groups = n_groups;
     if (pl.CS == 1) {
@@ -2645,9 +2966,9 @@ int launch_grouped(const Problem &pr, const Plan &pl, const GroupedArgs &ga, int
         gaw.flat = 1;
         plw.cyclic = 0;
         plw.x_in_stage = NB < kMmaMinBatch ? 1 : 0;
-        plw.stages = choose_stages(FMT, plw, pr.G, NB, pr.K, budget);
-        const SmemLayout Lf = smem_layout(FMT, plw, pr.G, NB, pr.K);
-        return launch_pdl(gemv_grouped_kernel<FMT, NB>, dim3(static_cast<unsigned>(total < sms ? total : sms)), (pl.NW + 2) * 32,
+        plw.stages = choose_stages(FMT, plw, pr.G, NB, pr.K, budget, kScr);
+        const SmemLayout Lf = smem_layout(FMT, plw, pr.G, NB, pr.K, kScr);
+        return launch_pdl(kernel, dim3(static_cast<unsigned>(total < sms ? total : sms)), (pl.NW + 2) * 32,
                           Lf.total, stream, pr, plw, gaw);
     }
     // the machine is shared by all groups: spread its multiprocessors over them
@@ -2656,7 +2977,7 @@ int launch_grouped(const Problem &pr, const Plan &pl, const GroupedArgs &ga, int
     int gx = 1;
     choose_walk(plw, per_group, &gx);
     gaw.flat = 0;
-    return launch_pdl(gemv_grouped_kernel<FMT, NB>, dim3(gx, n_groups), (pl.NW + 2) * 32, L.total, stream, pr, plw, gaw);
+    return launch_pdl(kernel, dim3(gx, n_groups), (pl.NW + 2) * 32, L.total, stream, pr, plw, gaw);
 }
 
 // Validates the arguments every product shares; fills nothing.
@@ -3072,7 +3393,7 @@ int launch_phased(PhasedArgs &pa, int n_jobs, const int *job_phase, cudaStream_t
         if (pa.pr[j].K > kmax) kmax = pa.pr[j].K;
         if (pa.pr[j].G > gmax) gmax = pa.pr[j].G;
     }
-    layout.stages = choose_stages(kBitcos, layout, gmax, NB, kmax, budget);
+    layout.stages = choose_stages(kBitcos, layout, gmax, NB, kmax, budget, false);
     pa.layout = layout;
     pa.shape = Problem{};
     pa.shape.K = kmax;
@@ -3110,7 +3431,7 @@ int launch_phased(PhasedArgs &pa, int n_jobs, const int *job_phase, cudaStream_t
         }
         if (next > grid) grid = next;
     }
-    const SmemLayout L = smem_layout(kBitcos, layout, gmax, NB, kmax);
+    const SmemLayout L = smem_layout(kBitcos, layout, gmax, NB, kmax, false);
     if (static_cast<int>(L.total) > budget) return BITCOS_ERR_SHAPE;
     return launch_pdl(gemv_phased_kernel<NB>, dim3(static_cast<unsigned>(grid)), (layout.NW + 2) * 32, L.total, stream, pa);
 }

@@ -1,0 +1,71 @@
+"""BITCOS from two tokens on: tiles decoded in tensor-core fragment order, one or two per warp.
+
+Two tiles per warp are taken from 64 tiles per multiprocessor on.  The shapes lie on both sides of that line and where
+the pairing can go wrong: an odd number of groups (the last warp of a row block has one tile), a single group, rows cut
+into column blocks of odd width, a ragged last row block.  Against the oracle, within the task's 1e-5 of sum|terms|.
+"""
+import numpy as np
+import pytest
+
+import datagen
+import oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+REL = 1e-5
+
+
+@pytest.fixture(scope="module")
+def bc():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2609_16338_b200 as m
+    from paper_2609_16338_b200 import build
+    build.build()
+    m.load_library()
+    return m
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def check(y, y_ref, mag, what):
+    yv = y.cpu().numpy().astype(np.float64)
+    assert (np.abs(yv - y_ref) <= REL * mag).all(), what
+    assert (yv[mag == 0] == 0).all(), what
+
+
+@pytest.mark.parametrize("groups,above", [(1, True), (5, True), (5, False), (20, True), (39, True), (41, True), (57, True)])
+def test_products_around_the_two_tile_line(bc, groups, above):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    blocks = -(-64 * sms // groups) - (0 if above else 1)          # row blocks: the line is 64 tiles per multiprocessor
+    M, K = 32 * blocks - 5, 128 * groups
+    W, S = datagen.trits(groups, M, K, 0.4219), datagen.scales(groups, M, K)
+    Wd, ws = bc.bitcos_pack(W, S).to_device(), bc.make_workspace(M, K)
+    for B in (2, 3, 8, 13):
+        x, xs = datagen.activations(groups + B, B, K)
+        _, y_ref, mag = oracle.gemv_dense(W, S, x, xs)
+        y, _ = bc.bitcos_gemv(Wd, dev(x), dev(xs), workspace=ws)
+        check(y, y_ref, mag, (groups, B))
+        y2 = torch.full_like(y, float("nan"))
+        bc.bitcos_gemv_multi([(Wd, dev(x), dev(xs), y2, ws)])
+        assert torch.equal(y, y2)
+        # one scale per token and group: equal scales give the per-token product
+        xg = np.repeat(xs[:, None], groups, axis=1)
+        yg, _ = bc.bitcos_gemv_group_scales(Wd, dev(x), dev(xg), workspace=ws)
+        check(yg, y_ref, mag, (groups, B, "group scales"))
+    assert bc.workspace_status(ws) == 0
+
+
+def test_bf16_activations_with_two_tiles_per_warp(bc):
+    """Two tokens quantised inside the launch: the two tiles of a warp are two different groups."""
+    M, K = 32 * 500 - 9, 128 * 21
+    W, S = datagen.trits(3, M, K, 0.4219), datagen.scales(3, M, K)
+    Wd, ws = bc.bitcos_pack(W, S).to_device(), bc.make_workspace(M, K)
+    xb = dev(datagen.activations_bf16(5, 2, K).view(np.int16)).view(torch.bfloat16)
+    xq, xg = bc.bitcos_quantize_activations(xb)
+    want, _ = bc.bitcos_gemv_group_scales(Wd, xq, xg, workspace=ws)
+    got, _ = bc.bitcos_gemv_bf16(Wd, xb, workspace=ws)
+    assert torch.equal(got, want)

@@ -2741,14 +2741,17 @@ inline int plan_multi(MultiArgs &ma, int nb_template, int sms, bool *two_out, in
     }
     *two_out = two;
     sms = small_launch_cap(total_items, sms);
+    int64_t cap[kMaxJobs], sum = 0;
+    for (int j = 0; j < ma.n; ++j) {
+        cap[j] = ma.pl[j].items;
+        if (total_items > sms) cap[j] = std::max<int64_t>(1, ma.pl[j].items * sms / total_items);
+        sum += cap[j];
+    }
+    // (the blocks that the smallest jobs were rounded up to come from the largest: no launch is wider than the machine)
+    for (; sum > std::max(sms, ma.n); --sum) --*std::max_element(cap, cap + ma.n);
     int next = 0;
     for (int j = 0; j < ma.n; ++j) {
-        int64_t cap = ma.pl[j].items;
-        if (total_items > sms) {
-            cap = ma.pl[j].items * sms / total_items;
-            if (cap < 1) cap = 1;
-        }
-        choose_walk(ma.pl[j], static_cast<int>(cap), &grids[j]);
+        choose_walk(ma.pl[j], static_cast<int>(cap[j]), &grids[j]);
         next += grids[j];
     }
     return next;

@@ -198,11 +198,11 @@ __device__ __forceinline__ uint32_t dp2a_lo(uint32_t a, uint32_t b, uint32_t c) 
 }
 
 // ---------------------------------------------------------------------------------------------
-// Decoder A in tensor-core fragment order (four tokens and more): a lane decodes presence word
+// Decoder A in tensor-core fragment order (two tokens and more): a lane decodes presence word
 // t = lane % 4 of the four rows g + 8 i (g = lane / 4), which is exactly what the A operand of
 // mma.m16n8k32 wants of it when the 128 products of a group are taken in the order
-// "nibble 2 kb of every word, nibble 2 kb + 1 of every word": w[8 i + 2 kb] and w[8 i + 2 kb + 1] are the
-// fragment registers of row g + 8 i for k-block kb.  No transposition through shared memory.
+// "nibble 2 kb of every word, nibble 2 kb + 1 of every word": step(kb) gives the fragment registers of all
+// four rows for k-block kb.  No transposition through shared memory.
 //   tile       the tile's 128 presence words (row major) in shared memory
 //   sg         the tile's piece of the sign vector; first = bit position of the tile's first sign bit in it
 // The words of the tile in order are index 32 i + lane, so a word's first sign bit is found by four warp

@@ -21,7 +21,6 @@ from __future__ import annotations
 import argparse
 import ctypes as C
 import os
-import subprocess
 
 import numpy as np
 
@@ -37,11 +36,8 @@ NAMES = ["q+k+v", "o", "gate+up", "down"]
 def build_debug_library() -> str:
     from . import build
     path = os.path.join(build.HERE, "libbitcos_timeline.so")
-    newest = max(os.path.getmtime(f) for f in build.SOURCES + build.HEADERS)
-    if not os.path.exists(path) or os.path.getmtime(path) < newest:
-        cmd = build.nvcc_command(("-DBITCOS_TIMELINE",))
-        cmd[cmd.index("-o") + 1] = path
-        subprocess.check_call(cmd)
+    if build.stale(path):
+        build.compile_library(path, ("-DBITCOS_TIMELINE",))
     return path
 
 

@@ -1,7 +1,8 @@
-"""ctypes binding of libbitcos.so: same names as the C ABI, argument marshalling only.
+"""Binding of libbitcos.so: same names as the C ABI, argument marshalling only.
 
 Host packers take and return numpy arrays.  Device entry points take torch CUDA tensors
-(used here only as owners of device memory) and enqueue on torch's current stream.
+(used here only as owners of device memory) and enqueue on torch's current stream.  The launching
+calls go through csrc/calls.c, everything else through ctypes.
 """
 from __future__ import annotations
 
@@ -53,6 +54,7 @@ class _Weights(C.Structure):
 
 
 _lib = None
+_calls = None           # csrc/calls.c, bound to the library
 
 
 def library_path() -> str:
@@ -122,8 +124,28 @@ def load_library():
     L.bitcos_count_nnz_device.argtypes = [vp, i64, i64, C.POINTER(u64), vp, vp]
     L.bitcos_pack_device.argtypes = [vp, vp, i64, i64, vp, vp, sz, vp, vp, vp, C.POINTER(u64), vp, vp]
     L.bitcos_gemv_group_scales.argtypes = [C.POINTER(_Weights), vp, vp, C.c_int, vp, vp, vp, sz, vp]
+    _bind_calls(L)
     _lib = L
     return L
+
+
+def _bind_calls(L):
+    global _calls
+    try:
+        from . import _calls as calls
+    except ImportError as e:
+        raise BitcosError(-1, "load_library", f"_calls.so is missing: run `python -m paper_2609_16338_b200.build` ({e})")
+    for name in dir(calls):
+        if name in EXPORTED_SYMBOLS:
+            calls.bind(name, C.cast(getattr(L, name), C.c_void_p).value)
+    _calls = calls
+
+
+def _native():
+    """The bound calls (loads the library on the first use)."""
+    if _calls is None:
+        load_library()
+    return _calls
 
 
 def _check(status: int, what: str):
@@ -348,9 +370,19 @@ def bitcos_gemv_workspace_bytes(M: int, K: int) -> int:
     return int(load_library().bitcos_gemv_workspace_bytes(M, K))
 
 
-def _stream():
-    import torch
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+_raw_stream = None
+
+
+def _stream() -> int:
+    """The handle of torch's current stream on the current device (torch.cuda.current_stream() would build a Stream
+    object around the same handle: 3.5 us instead of 0.2)."""
+    global _raw_stream
+    if _raw_stream is None:
+        import torch
+        torch.cuda.init()
+        _raw_stream = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+    stream, device = _raw_stream
+    return stream(device())
 
 
 def make_workspace(M: int, K: int, device="cuda", copies: int = 1):
@@ -372,6 +404,8 @@ def workspace_status(workspace) -> int:
 
 
 def _outputs(M, K, batch, y, acc_debug, device):
+    if y is not None and (acc_debug is None or acc_debug is False):
+        return y, None
     import torch
     if y is None:
         y = torch.empty((batch, M), dtype=torch.float32, device=device)
@@ -385,87 +419,98 @@ def _outputs(M, K, batch, y, acc_debug, device):
 
 def bitcos_gemv(W: DeviceBitcos, x, x_scale, y=None, acc_debug=None, workspace=None):
     """y[b][m] = x_scale[b] * sum_g scale[m][g] * sum_{k in g} W[m][k] x[b][k]; returns (y, acc or None)."""
-    batch = x.shape[0]
+    batch = x.size(0)
     if workspace is None:
         workspace = make_workspace(W.M, W.K, x.device)
     y, acc = _outputs(W.M, W.K, batch, y, acc_debug, x.device)
-    _check(load_library().bitcos_gemv(C.byref(W.desc), x.data_ptr(), x_scale.data_ptr(), batch, y.data_ptr(),
-                                      acc.data_ptr() if acc is not None else None, workspace.data_ptr(),
-                                      workspace.numel(), _stream()), "bitcos_gemv")
+    status = (_calls or _native()).bitcos_gemv(C.addressof(W.desc), x.data_ptr(), x_scale.data_ptr(), batch, y.data_ptr(),
+                                               0 if acc is None else acc.data_ptr(), workspace.data_ptr(),
+                                               workspace.numel(), _stream())
+    if status:
+        _check(status, "bitcos_gemv")
     return y, acc
 
 
 def bitcos_gemv_group_scales(W: DeviceBitcos, x, x_group_scale, y=None, acc_debug=None, workspace=None):
     """bitcos_gemv with one activation scale per token and group of 128: x_group_scale float32 [batch, K / 128]."""
-    batch = x.shape[0]
-    if tuple(x_group_scale.shape) != (batch, W.K // 128):
+    batch = x.size(0)
+    if x_group_scale.shape != (batch, W.K // 128):
         raise ValueError("x_group_scale must be [batch, K / 128]")
     if workspace is None:
         workspace = make_workspace(W.M, W.K, x.device)
     y, acc = _outputs(W.M, W.K, batch, y, acc_debug, x.device)
-    _check(load_library().bitcos_gemv_group_scales(C.byref(W.desc), x.data_ptr(), x_group_scale.data_ptr(), batch,
-                                                   y.data_ptr(), acc.data_ptr() if acc is not None else None,
-                                                   workspace.data_ptr(), workspace.numel(), _stream()),
-           "bitcos_gemv_group_scales")
+    status = (_calls or _native()).bitcos_gemv_group_scales(
+        C.addressof(W.desc), x.data_ptr(), x_group_scale.data_ptr(), batch, y.data_ptr(), 0 if acc is None else acc.data_ptr(),
+        workspace.data_ptr(), workspace.numel(), _stream())
+    if status:
+        _check(status, "bitcos_gemv_group_scales")
     return y, acc
+
+
+def _check_bf16(x_bf16):
+    import torch
+    if x_bf16.dtype != torch.bfloat16 or x_bf16.dim() != 2 or not x_bf16.is_contiguous():
+        raise ValueError("x_bf16 must be a contiguous bfloat16 [batch, K] tensor")
 
 
 def bitcos_gemv_bf16(W: DeviceBitcos, x_bf16, y=None, acc_debug=None, workspace=None):
     """The product from bfloat16 activations [batch, K] (batch 1 or 2), quantised per group of 128 inside the launch."""
-    import torch
-    if x_bf16.dtype != torch.bfloat16 or x_bf16.dim() != 2 or not x_bf16.is_contiguous():
-        raise ValueError("x_bf16 must be a contiguous bfloat16 [batch, K] tensor")
-    batch = x_bf16.shape[0]
+    _check_bf16(x_bf16)
+    batch = x_bf16.size(0)
     if workspace is None:
         workspace = make_workspace(W.M, W.K, x_bf16.device)
     y, acc = _outputs(W.M, W.K, batch, y, acc_debug, x_bf16.device)
-    _check(load_library().bitcos_gemv_bf16(C.byref(W.desc), x_bf16.data_ptr(), batch, y.data_ptr(),
-                                           acc.data_ptr() if acc is not None else None, workspace.data_ptr(),
-                                           workspace.numel(), _stream()), "bitcos_gemv_bf16")
+    status = (_calls or _native()).bitcos_gemv_bf16(C.addressof(W.desc), x_bf16.data_ptr(), batch, y.data_ptr(),
+                                                    0 if acc is None else acc.data_ptr(), workspace.data_ptr(),
+                                                    workspace.numel(), _stream())
+    if status:
+        _check(status, "bitcos_gemv_bf16")
     return y, acc
 
 
 def bitcos_gemv_blend_bf16(W: DeviceBitcos, x_bf16, y=None, workspace=None):
     """The 16-bit variant: weights rebuilt as +-s times unquantised bfloat16 activations [batch, K], batch 1..8."""
-    import torch
-    if x_bf16.dtype != torch.bfloat16 or x_bf16.dim() != 2 or not x_bf16.is_contiguous():
-        raise ValueError("x_bf16 must be a contiguous bfloat16 [batch, K] tensor")
-    batch = x_bf16.shape[0]
+    _check_bf16(x_bf16)
+    batch = x_bf16.size(0)
     if workspace is None:
         workspace = make_workspace(W.M, W.K, x_bf16.device)
     y, _ = _outputs(W.M, W.K, batch, y, None, x_bf16.device)
-    _check(load_library().bitcos_gemv_blend_bf16(C.byref(W.desc), x_bf16.data_ptr(), batch, y.data_ptr(),
-                                                 workspace.data_ptr(), workspace.numel(), _stream()),
-           "bitcos_gemv_blend_bf16")
+    status = (_calls or _native()).bitcos_gemv_blend_bf16(C.addressof(W.desc), x_bf16.data_ptr(), batch, y.data_ptr(),
+                                                          workspace.data_ptr(), workspace.numel(), _stream())
+    if status:
+        _check(status, "bitcos_gemv_blend_bf16")
     return y
 
 
 def bitcos_quantize_activations(x_bf16, group: int = 128, xq=None, x_scale=None):
     """bf16 activations [batch, K] on the device -> (int8 codes [batch, K], float32 scales
     [batch, K / 128] for group = 128, [batch] for group = 0)."""
-    import torch
-    if x_bf16.dtype != torch.bfloat16 or x_bf16.dim() != 2 or not x_bf16.is_contiguous():
-        raise ValueError("x_bf16 must be a contiguous bfloat16 [batch, K] tensor")
+    _check_bf16(x_bf16)
     batch, K = x_bf16.shape
+    if xq is None or x_scale is None:
+        import torch
     if xq is None:
         xq = torch.empty((batch, K), dtype=torch.int8, device=x_bf16.device)
     if x_scale is None:
         shape = (batch,) if group == 0 else (batch, K // 128)
         x_scale = torch.empty(shape, dtype=torch.float32, device=x_bf16.device)
-    _check(load_library().bitcos_quantize_activations(x_bf16.data_ptr(), batch, K, group, xq.data_ptr(),
-                                                      x_scale.data_ptr(), _stream()), "bitcos_quantize_activations")
+    status = (_calls or _native()).bitcos_quantize_activations(x_bf16.data_ptr(), batch, K, group, xq.data_ptr(),
+                                                               x_scale.data_ptr(), _stream())
+    if status:
+        _check(status, "bitcos_quantize_activations")
     return xq, x_scale
 
 
 def _plain_gemv(name, W: DevicePlain, x, x_scale, y, acc_debug, workspace):
-    batch = x.shape[0]
+    batch = x.size(0)
     if workspace is None:
         workspace = make_workspace(W.M, W.K, x.device)
     y, acc = _outputs(W.M, W.K, batch, y, acc_debug, x.device)
-    _check(getattr(load_library(), name)(W.words.data_ptr(), W.scales.data_ptr(), W.M, W.K, x.data_ptr(),
-                                         x_scale.data_ptr(), batch, y.data_ptr(),
-                                         acc.data_ptr() if acc is not None else None, workspace.data_ptr(),
-                                         workspace.numel(), _stream()), name)
+    status = getattr(_calls or _native(), name)(W.words.data_ptr(), W.scales.data_ptr(), W.M, W.K, x.data_ptr(),
+                                                x_scale.data_ptr(), batch, y.data_ptr(), 0 if acc is None else acc.data_ptr(),
+                                                workspace.data_ptr(), workspace.numel(), _stream())
+    if status:
+        _check(status, name)
     return y, acc
 
 
@@ -505,20 +550,16 @@ def group_pairs(pair_expert, pair_xrow):
 
 
 def _grouped(name, E: DeviceExperts, group_expert, group_begin, pair_xrow, max_group_size, x, x_scale, y, acc_debug, workspace):
-    import torch
     n_groups, n_pairs = group_expert.numel(), pair_xrow.numel()
     if workspace is None:
         workspace = make_workspace(E.M, E.K, x.device, copies=n_groups)
-    if y is None:
-        y = torch.empty((n_pairs, E.M), dtype=torch.float32, device=x.device)
-    acc = None
-    if acc_debug is True:
-        acc = torch.empty((n_pairs, E.M, E.K // GROUP), dtype=torch.int32, device=x.device)
-    _check(getattr(load_library(), name)(E.table.data_ptr(), len(E.experts), E.M, E.K, group_expert.data_ptr(),
-                                         group_begin.data_ptr(), n_groups, pair_xrow.data_ptr(), n_pairs,
-                                         max_group_size, x.data_ptr(), x.shape[0], x_scale.data_ptr(), y.data_ptr(),
-                                         acc.data_ptr() if acc is not None else None, workspace.data_ptr(),
-                                         workspace.numel(), _stream()), name)
+    y, acc = _outputs(E.M, E.K, n_pairs, y, True if acc_debug is True else None, x.device)
+    status = getattr(_calls or _native(), name)(
+        E.table.data_ptr(), len(E.experts), E.M, E.K, group_expert.data_ptr(), group_begin.data_ptr(), n_groups,
+        pair_xrow.data_ptr(), n_pairs, max_group_size, x.data_ptr(), x.size(0), x_scale.data_ptr(), y.data_ptr(),
+        0 if acc is None else acc.data_ptr(), workspace.data_ptr(), workspace.numel(), _stream())
+    if status:
+        _check(status, name)
     return y, acc
 
 
@@ -540,29 +581,27 @@ def bitcos_group_pairs_device(pair_expert, pair_xrow, n_experts: int):
     xr = torch.zeros(P, dtype=torch.int32, device=dev)
     order = torch.full((P,), -1, dtype=torch.int32, device=dev)
     ng = torch.zeros(1, dtype=torch.int32, device=dev)
-    _check(load_library().bitcos_group_pairs_device(pair_expert.data_ptr(), pair_xrow.data_ptr(), P, n_experts, ge.data_ptr(),
-                                                    gb.data_ptr(), xr.data_ptr(), order.data_ptr(), ng.data_ptr(), _stream()),
-           "bitcos_group_pairs_device")
+    status = (_calls or _native()).bitcos_group_pairs_device(
+        pair_expert.data_ptr(), pair_xrow.data_ptr(), P, n_experts, ge.data_ptr(), gb.data_ptr(), xr.data_ptr(),
+        order.data_ptr(), ng.data_ptr(), _stream())
+    if status:
+        _check(status, "bitcos_group_pairs_device")
     return ge, gb, xr, order, ng
 
 
 def bitcos_gemv_grouped_lists(E: DeviceExperts, group_expert, group_begin, n_groups_dev, pair_xrow, max_group_size, x, x_scale,
                               y=None, acc_debug=None, workspace=None):
     """bitcos_gemv_grouped with the number of groups left on the device (see bitcos_group_pairs_device)."""
-    import torch
     max_groups, n_pairs = group_expert.numel(), pair_xrow.numel()
     if workspace is None:
         workspace = make_workspace(E.M, E.K, x.device, copies=max_groups)
-    if y is None:
-        y = torch.empty((n_pairs, E.M), dtype=torch.float32, device=x.device)
-    acc = None
-    if acc_debug is True:
-        acc = torch.empty((n_pairs, E.M, E.K // GROUP), dtype=torch.int32, device=x.device)
-    _check(load_library().bitcos_gemv_grouped_lists(E.table.data_ptr(), len(E.experts), E.M, E.K, group_expert.data_ptr(),
-                                                    group_begin.data_ptr(), n_groups_dev.data_ptr(), max_groups,
-                                                    pair_xrow.data_ptr(), n_pairs, max_group_size, x.data_ptr(), x.shape[0],
-                                                    x_scale.data_ptr(), y.data_ptr(), acc.data_ptr() if acc is not None else None,
-                                                    workspace.data_ptr(), workspace.numel(), _stream()), "bitcos_gemv_grouped_lists")
+    y, acc = _outputs(E.M, E.K, n_pairs, y, True if acc_debug is True else None, x.device)
+    status = (_calls or _native()).bitcos_gemv_grouped_lists(
+        E.table.data_ptr(), len(E.experts), E.M, E.K, group_expert.data_ptr(), group_begin.data_ptr(), n_groups_dev.data_ptr(),
+        max_groups, pair_xrow.data_ptr(), n_pairs, max_group_size, x.data_ptr(), x.size(0), x_scale.data_ptr(), y.data_ptr(),
+        0 if acc is None else acc.data_ptr(), workspace.data_ptr(), workspace.numel(), _stream())
+    if status:
+        _check(status, "bitcos_gemv_grouped_lists")
     return y, acc
 
 
@@ -586,6 +625,7 @@ class MultiJobs:
         self.batch = jobs[0][1].shape[0]
         self.arr = (_Job * len(jobs))(*[_Job(C.addressof(W.desc), x.data_ptr(), xs.data_ptr() if xs is not None else None,
                                              y.data_ptr(), ws.data_ptr(), ws.numel()) for (W, x, xs, y, ws) in jobs])
+        self.n, self.address = len(jobs), C.addressof(self.arr)
 
 
 class NextWeights:
@@ -595,6 +635,7 @@ class NextWeights:
     def __init__(self, weights):
         self.keep = list(weights)
         self.arr = (C.c_void_p * len(self.keep))(*[C.addressof(W.desc) for W in self.keep])
+        self.n, self.address = len(self.keep), C.addressof(self.arr)
 
 
 def bitcos_gemv_multi_plan(shapes, batch=1, multiprocessors=148, busy_multiprocessors=0):
@@ -623,13 +664,15 @@ def bitcos_gemv_multi(jobs, next=None, prev=None):
     will read, which this launch asks to be brought into L2; `prev` = the matrices of the launch directly before
     this one in the stream, from which the launch works out how many of its blocks will start late."""
     mj = jobs if isinstance(jobs, MultiJobs) else MultiJobs(jobs)
+    calls = _calls or _native()
     if next is None and prev is None:
-        _check(load_library().bitcos_gemv_multi(mj.arr, len(mj.arr), mj.batch, _stream()), "bitcos_gemv_multi")
+        status = calls.bitcos_gemv_multi(mj.address, mj.n, mj.batch, _stream())
     else:
         nw = next if isinstance(next, NextWeights) else NextWeights(next or [])
         pw = prev if isinstance(prev, NextWeights) else NextWeights(prev or [])
-        _check(load_library().bitcos_gemv_multi_chained(mj.arr, len(mj.arr), mj.batch, pw.arr, len(pw.keep), nw.arr,
-                                                        len(nw.keep), _stream()), "bitcos_gemv_multi_chained")
+        status = calls.bitcos_gemv_multi_chained(mj.address, mj.n, mj.batch, pw.address, pw.n, nw.address, nw.n, _stream())
+    if status:
+        _check(status, "bitcos_gemv_multi" if next is None and prev is None else "bitcos_gemv_multi_chained")
     return [j[3] for j in mj.keep]
 
 
@@ -697,10 +740,11 @@ class HostPhases:
         self.phases = (C.c_int * len(weights))(*[int(p) for p in phases])
 
     def run(self):
-        _check(load_library().bitcos_gemv_phases_host(self.arr, self.phases, len(self.arr), self.batch,
-                                                      self.in_host.data_ptr(), self.in_dev.data_ptr(), self.in_bytes,
-                                                      self.out_host.data_ptr(), self.out_dev.data_ptr(), self.out_bytes,
-                                                      _stream()), "bitcos_gemv_phases_host")
+        status = (_calls or _native()).bitcos_gemv_phases_host(
+            C.addressof(self.arr), C.addressof(self.phases), len(self.arr), self.batch, self.in_host.data_ptr(),
+            self.in_dev.data_ptr(), self.in_bytes, self.out_host.data_ptr(), self.out_dev.data_ptr(), self.out_bytes, _stream())
+        if status:
+            _check(status, "bitcos_gemv_phases_host")
         return self.y
 
 
@@ -708,8 +752,9 @@ def bitcos_gemv_multi_group_scales(jobs):
     """bitcos_gemv_multi with one activation scale per token and group: jobs = MultiJobs or a list of
     (W, x, x_group_scale [batch, K / 128], y, workspace) tuples."""
     mj = jobs if isinstance(jobs, MultiJobs) else MultiJobs(jobs)
-    _check(load_library().bitcos_gemv_multi_group_scales(mj.arr, len(mj.arr), mj.batch, _stream()),
-           "bitcos_gemv_multi_group_scales")
+    status = (_calls or _native()).bitcos_gemv_multi_group_scales(mj.address, mj.n, mj.batch, _stream())
+    if status:
+        _check(status, "bitcos_gemv_multi_group_scales")
     return [j[3] for j in mj.keep]
 
 
@@ -717,7 +762,9 @@ def bitcos_gemv_multi_bf16(jobs):
     """bitcos_gemv_multi with bfloat16 activations quantised inside the launch: jobs = MultiJobs or a list of
     (W, x_bf16, None, y, workspace) tuples, batch 1 or 2."""
     mj = jobs if isinstance(jobs, MultiJobs) else MultiJobs(jobs)
-    _check(load_library().bitcos_gemv_multi_bf16(mj.arr, len(mj.arr), mj.batch, _stream()), "bitcos_gemv_multi_bf16")
+    status = (_calls or _native()).bitcos_gemv_multi_bf16(mj.address, mj.n, mj.batch, _stream())
+    if status:
+        _check(status, "bitcos_gemv_multi_bf16")
     return [j[3] for j in mj.keep]
 
 

@@ -1,9 +1,10 @@
-"""Builds libbitcos.so (CUDA kernels for sm_100a + host packers) in-tree with nvcc."""
+"""Builds libbitcos.so (CUDA kernels for sm_100a + host packers, nvcc) and the binding's _calls.so (gcc) in-tree."""
 from __future__ import annotations
 
 import os
 import shutil
 import subprocess
+import sysconfig
 import tempfile
 from concurrent.futures import ThreadPoolExecutor
 
@@ -11,6 +12,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libbitcos.so")
+CALLS = os.path.join(HERE, "_calls.so")                # the Python binding's entry (csrc/calls.c)
+CALLS_SOURCE = os.path.join(CSRC, "calls.c")
 INST = os.path.join(CSRC, "gemv_inst.cu")
 INST_PARTS = 11             # the parts of gemv_inst.cuh, each compiled by a process of its own
 SOURCES = [os.path.join(CSRC, "gemv.cu"), os.path.join(CSRC, "probe.cu"), os.path.join(CSRC, "pack_device.cu"),
@@ -48,6 +51,9 @@ def stale(lib=LIB, sources=None) -> bool:
 def build(force: bool = False, verbose: bool = False) -> str:
     if force or stale():
         compile_library(LIB, ("-Xptxas", "-v") if verbose else ())
+    if force or stale(CALLS, [CALLS_SOURCE]):
+        subprocess.check_call(["gcc", "-O2", "-fPIC", "-shared", "-Wall", "-I" + sysconfig.get_paths()["include"], "-o", CALLS,
+                               CALLS_SOURCE])
     return LIB
 
 

@@ -517,7 +517,8 @@ int bitcos_gemv_grouped(const bitcos_weights *experts, int n_experts, int64_t M,
  * BITCOS_GROUP_EXPERTS_MAX).  Outputs (device): group_expert [min(n_pairs, n_experts)], group_begin
  * [min(n_pairs, n_experts) + 1], pair_xrow_sorted [n_pairs], order [n_pairs] (sorted pair i is input
  * pair order[i]: output row i of the grouped product belongs to it), n_groups [1].  Experts ascending,
- * input order kept inside a group.  A pair with an expert id out of range is left out.
+ * input order kept inside a group.  A pair with an expert id out of range is left out; what the groups leave of
+ * the lists is filled with 0, of order with -1.
  *
  * bitcos_gemv_grouped_lists: bitcos_gemv_grouped with the NUMBER of groups read from device memory
  * (n_groups_device, as bitcos_group_pairs_device wrote it; values above max_groups are clipped).

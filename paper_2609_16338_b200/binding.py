@@ -576,11 +576,9 @@ def bitcos_group_pairs_device(pair_expert, pair_xrow, n_experts: int):
     P = pair_expert.numel()
     cap = min(P, n_experts)
     dev = pair_expert.device
-    ge = torch.zeros(cap, dtype=torch.int32, device=dev)
-    gb = torch.zeros(cap + 1, dtype=torch.int32, device=dev)
-    xr = torch.zeros(P, dtype=torch.int32, device=dev)
-    order = torch.full((P,), -1, dtype=torch.int32, device=dev)
-    ng = torch.zeros(1, dtype=torch.int32, device=dev)
+    # (one allocation; the call writes all of every list)
+    lists = torch.empty(2 * cap + 2 * P + 2, dtype=torch.int32, device=dev)
+    ge, gb, xr, order, ng = lists.split((cap, cap + 1, P, P, 1))
     status = (_calls or _native()).bitcos_group_pairs_device(
         pair_expert.data_ptr(), pair_xrow.data_ptr(), P, n_experts, ge.data_ptr(), gb.data_ptr(), xr.data_ptr(),
         order.data_ptr(), ng.data_ptr(), _stream())

@@ -121,47 +121,92 @@ __global__ void __launch_bounds__(32, 1) wait_probe_kernel(unsigned int *status,
 // that a decode loop whose router runs on the GPU never has to bring the pairs to the host: count
 // the pairs of every expert, give every expert that has any a group (experts ascending), place
 // every pair behind the pairs of the same expert that precede it in the input.  A pair whose expert
-// id is out of range is dropped (it gets no group and order -1 is never written for it; its output
-// row is simply not produced).
+// id is out of range is dropped: it gets no group.  What the groups leave of the output lists is
+// filled (0, order -1), so that the caller need not.
+// Latency is all there is to it (a few KB), so every step is one round of the block: the experts are
+// scanned by all threads, four to a thread at most, and one warp finds the stable places 32 pairs at a
+// time (match_any: the earlier lanes with the same expert), without reading global memory.
+// 64 pairs, 128 experts: 8.6 -> 2.2 us against one thread that walks the experts, every pair counting the pairs
+// before it, and the caller's five fill kernels.
 // ---------------------------------------------------------------------------------------------
 constexpr int kGroupPairsThreads = 256;
+constexpr int kExpertsPerThread = BITCOS_GROUP_EXPERTS_MAX / kGroupPairsThreads;
 __global__ void __launch_bounds__(kGroupPairsThreads) group_pairs_kernel(const int32_t *__restrict__ pair_expert,
                                                                          const int32_t *__restrict__ pair_xrow, int n_pairs, int n_experts,
-                                                                         int32_t *group_expert, int32_t *group_begin,
-                                                                         int32_t *pair_xrow_sorted, int32_t *order, int32_t *n_groups) {
+                                                                         int32_t *__restrict__ group_expert, int32_t *__restrict__ group_begin,
+                                                                         int32_t *__restrict__ pair_xrow_sorted, int32_t *__restrict__ order,
+                                                                         int32_t *__restrict__ n_groups) {
+    __shared__ int count[BITCOS_GROUP_EXPERTS_MAX];      // pairs per expert, then the expert's next free position
+    __shared__ int16_t place[BITCOS_GROUP_PAIRS_MAX];    // a pair's expert (-1: out of range), then its position
+    __shared__ uint32_t warp_sum[kGroupPairsThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int e = tid; e < BITCOS_GROUP_EXPERTS_MAX; e += kGroupPairsThreads) count[e] = 0;
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    __shared__ int count[BITCOS_GROUP_EXPERTS_MAX];      // pairs per expert, then the expert's first position
-    for (int e = threadIdx.x; e < n_experts; e += kGroupPairsThreads) count[e] = 0;
     __syncthreads();
-    for (int i = threadIdx.x; i < n_pairs; i += kGroupPairsThreads) {
-        const int e = pair_expert[i];
-        if (e >= 0 && e < n_experts) atomicAdd(&count[e], 1);
+    for (int i = tid; i < n_pairs; i += kGroupPairsThreads) {
+        const int e = __ldg(pair_expert + i);
+        const bool in = e >= 0 && e < n_experts;
+        place[i] = static_cast<int16_t>(in ? e : -1);
+        if (in) atomicAdd(&count[e], 1);
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int pos = 0, g = 0;
-        for (int e = 0; e < n_experts; ++e) {
-            const int c = count[e];
-            count[e] = pos;
-            if (c) {
-                group_expert[g] = e;
-                group_begin[g] = pos;
-                ++g;
-            }
-            pos += c;
+    // pairs (low half: at most 4096) and groups (high half: at most 1024) in front of every expert
+    int c[kExpertsPerThread];
+    uint32_t mine = 0;
+#pragma unroll
+    for (int j = 0; j < kExpertsPerThread; ++j) {
+        c[j] = count[tid * kExpertsPerThread + j];
+        mine += static_cast<uint32_t>(c[j]) + (c[j] ? 0x10000u : 0u);
+    }
+    const uint32_t upto = warp_scan_add(mine);
+    if (lane == 31) warp_sum[warp] = upto;
+    __syncthreads();
+    uint32_t before = upto - mine, total = 0;
+#pragma unroll
+    for (int w = 0; w < kGroupPairsThreads / 32; ++w) {
+        if (w < warp) before += warp_sum[w];
+        total += warp_sum[w];
+    }
+#pragma unroll
+    for (int j = 0; j < kExpertsPerThread; ++j) {
+        const int pos = static_cast<int>(before & 0xFFFFu), g = static_cast<int>(before >> 16);
+        count[tid * kExpertsPerThread + j] = pos;
+        if (c[j]) {
+            group_expert[g] = tid * kExpertsPerThread + j;
+            group_begin[g] = pos;
         }
-        group_begin[g] = pos;
-        *n_groups = g;
+        before += static_cast<uint32_t>(c[j]) + (c[j] ? 0x10000u : 0u);
+    }
+    const int kept = static_cast<int>(total & 0xFFFFu), groups = static_cast<int>(total >> 16);
+    const int cap = n_pairs < n_experts ? n_pairs : n_experts;
+    for (int g = groups + tid; g <= cap; g += kGroupPairsThreads) {
+        group_begin[g] = g == groups ? kept : 0;
+        if (g < cap) group_expert[g] = 0;
+    }
+    for (int i = kept + tid; i < n_pairs; i += kGroupPairsThreads) {
+        pair_xrow_sorted[i] = 0;
+        order[i] = -1;
+    }
+    if (tid == 0) *n_groups = groups;
+    __syncthreads();
+    if (warp == 0) {
+        for (int base = 0; base < n_pairs; base += 32) {
+            const int i = base + lane;
+            const int e = i < n_pairs ? place[i] : -1;
+            const uint32_t same = __match_any_sync(0xFFFFFFFFu, e);
+            const int at = e >= 0 ? count[e] + __popc(same & ((1u << lane) - 1u)) : -1;      // input order inside a group
+            __syncwarp();
+            if (e >= 0 && lane == __ffs(same) - 1) count[e] += __popc(same);
+            if (i < n_pairs) place[i] = static_cast<int16_t>(at);
+            __syncwarp();
+        }
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < n_pairs; i += kGroupPairsThreads) {
-        const int e = pair_expert[i];
-        if (e < 0 || e >= n_experts) continue;
-        int rank = 0;
-        for (int j = 0; j < i; ++j) rank += (pair_expert[j] == e) ? 1 : 0;      // stable: input order inside a group
-        const int at = count[e] + rank;
-        pair_xrow_sorted[at] = pair_xrow[i];
+    for (int i = tid; i < n_pairs; i += kGroupPairsThreads) {
+        const int at = place[i];
+        if (at < 0) continue;
+        pair_xrow_sorted[at] = __ldg(pair_xrow + i);
         order[at] = i;
     }
 }

@@ -1110,63 +1110,88 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
         float run[NB];          // running sum of the current row block over this block's items
 #pragma unroll
         for (int b = 0; b < NB; ++b) run[b] = 0.f;
-        // per-token activation scales: kept in registers for up to two tokens, fetched where they
-        // are used (a cached load per output block) for more
-        float xsc[NB < kMmaMinBatch ? NB : 1] = {};
-        auto xscale = [&](int b) {
-            return kXG ? 1.f : NB < kMmaMinBatch ? xsc[NB < kMmaMinBatch ? b : 0] : __ldg(pb.x_scale + xr[b]);
-        };
+        // per-token activation scales, fetched once per segment (sixteen: a cached load per output block)
+        constexpr bool kHoldScales = !kXG && NB <= 8;
+        float xsc[kHoldScales ? NB : 1] = {};
+        auto xscale = [&](int b) { return kXG ? 1.f : kHoldScales ? xsc[kHoldScales ? b : 0] : __ldg(pb.x_scale + xr[b]); };
         Share pend[2];
         int n_pend = 0;
         ItemIter it;
         int kk = 0;             // items consumed so far, over all segments
         int es = 0;             // stage of the item the epilogue looks at next
-        constexpr int RS = red_slots(NB);
-        // sum of n <= 20 partial sums of token b, spaced NB * 32 floats apart: all loads are issued
-        // before the first addition, and the additions always follow the same tree
-        auto sum_groups20 = [&](const float *base, int n) {
-            float v[kMaxWarps];
+        // The sums of n <= 20 partial sums, in an order that depends on n alone.  This one warp serves every row block of
+        // the launch at the few issue slots the decoders leave it (one in six clocks or so), and with short rows they come
+        // fast (six tiles a row block at K = 768): what counts there is its instructions, with long rows its latency at the
+        // end of a launch.  Clocks per tile and multiprocessor at eight tokens against twenty guarded loads a sum and a
+        // scale fetched per output: K = 768 300 -> 182, K = 2048 180 -> 148, K = 2560 163 -> 145.
+        // Up to two tokens (spaced NB * 32 floats apart): a tree of pairs, all loads before the first addition.
+        auto tree = [&](auto size, const float *base, int n) {
+            constexpr int N = decltype(size)::value;
+            float v[N];
 #pragma unroll
-            for (int j = 0; j < kMaxWarps; ++j) v[j] = (j < n) ? base[j * NB * kRows] : 0.f;
+            for (int j = 0; j < N; ++j) v[j] = (j < n) ? base[j * NB * kRows] : 0.f;
 #pragma unroll
-            for (int w2 = 1; w2 < kMaxWarps; w2 *= 2)
+            for (int w2 = 1; w2 < N; w2 *= 2)
 #pragma unroll
-                for (int j = 0; j + w2 < kMaxWarps; j += 2 * w2) v[j] += v[j + w2];
+                for (int j = 0; j + w2 < N; j += 2 * w2) v[j] += v[j + w2];
             return v[0];
         };
-        // (up to 40 partial sums when a warp decodes two tiles per item: two trees of 20)
+        auto sum_groups20 = [&](const float *base, int n) {
+            if (n <= 8) return tree(std::integral_constant<int, 8>{}, base, n);
+            return tree(std::integral_constant<int, kMaxWarps>{}, base, n);
+        };
+        // (up to 40 when a warp leaves the sums of two tiles: two trees)
         auto sum_groups = [&](const float *base, int n) {
             float t = sum_groups20(base, n);
             if (TPW == 2 && !kPairs && n > kMaxWarps) t += sum_groups20(base + kMaxWarps * NB * kRows, n - kMaxWarps);
             return t;
         };
-        // tensor-core layout: the same for four tokens at a time, n <= 20 float4 spaced one warp's
-        // rows apart, in two batches of ten to bound the registers in flight
+        // Tensor-core layout: four tokens at a time, spaced one warp's rows apart; more than eight in two batches of ten,
+        // all loads of a batch before its first addition (three smaller batches cost the sixteen-token layer 3 %).
         constexpr int RF = NB;
+        auto add4 = [](float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); };
         auto sum_groups4 = [&](const float *base, int n) {
+            auto at = [&](int j) { return *reinterpret_cast<const float4 *>(base + j * kRows * RF); };
             float4 tot = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (n > 8) {
 #pragma unroll
-            for (int j0 = 0; j0 < kMaxWarps; j0 += 10) {
-                float4 v[10];
+                for (int j0 = 0; j0 < kMaxWarps; j0 += 10) {
+                    float4 v[10];
 #pragma unroll
-                for (int j = 0; j < 10; ++j)
-                    v[j] = (j0 + j < n) ? *reinterpret_cast<const float4 *>(base + (j0 + j) * kRows * RF)
-                                        : make_float4(0.f, 0.f, 0.f, 0.f);
+                    for (int j = 0; j < 10; ++j) v[j] = (j0 + j < n) ? at(j0 + j) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-                for (int w2 = 1; w2 < 10; w2 *= 2)
+                    for (int w2 = 1; w2 < 10; w2 *= 2)
 #pragma unroll
-                    for (int j = 0; j + w2 < 10; j += 2 * w2) {
-                        v[j].x += v[j + w2].x;
-                        v[j].y += v[j + w2].y;
-                        v[j].z += v[j + w2].z;
-                        v[j].w += v[j + w2].w;
-                    }
-                tot.x += v[0].x;
-                tot.y += v[0].y;
-                tot.z += v[0].z;
-                tot.w += v[0].w;
+                        for (int j = 0; j + w2 < 10; j += 2 * w2) v[j] = add4(v[j], v[j + w2]);
+                    tot = add4(tot, v[0]);
+                }
+                return tot;
+            }
+#pragma unroll 1
+            for (; n >= 4; n -= 4, base += 4 * kRows * RF) {
+                const float4 a = at(0), b = at(1), c = at(2), d = at(3);
+                tot = add4(tot, add4(add4(a, b), add4(c, d)));
+            }
+            if (n >= 1) {
+                const float4 a = at(0);
+                if (n >= 2) {
+                    const float4 b = at(1);
+                    if (n == 3) tot = add4(tot, at(2));
+                    tot = add4(tot, b);
+                }
+                tot = add4(tot, a);
             }
             return tot;
+        };
+        // one row block's outputs: row m of every token, one M apart
+        auto store_rows = [&](int64_t m, const float (&t)[NB]) {
+            if (m >= pb.M) return;
+            float *out = pb.y + pr.out_row0(pb) * pb.M + m;
+            const int64_t step = pb.M;
+            const int nb = pr.nb(pb);
+#pragma unroll
+            for (int b = 0; b < NB; ++b, out += step)
+                if (b < nb) *out = xscale(b) * t[b];
         };
         // sums over warps j0 .. j0 + n - 1 of a slot, for this lane's row and every token
         auto sums = [&](const float *rs, int j0, int n, float (&tot)[NB]) {
@@ -1202,9 +1227,9 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
         }
         n_pend = 0;
         it.init(pl, wk.first);
-        if (NB < kMmaMinBatch && !kXG) {
+        if (kHoldScales) {
 #pragma unroll
-            for (int b = 0; b < NB; ++b) xsc[NB < kMmaMinBatch ? b : 0] = __ldg(pb.x_scale + xr[b]);
+            for (int b = 0; b < NB; ++b) xsc[kHoldScales ? b : 0] = __ldg(pb.x_scale + xr[b]);
         }
         for (int k = 0; k < wk.count; ++k, ++kk, it.next(pl, wk)) {
             const int slot = kk & rs_mask;
@@ -1231,9 +1256,7 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
                         __syncwarp();
                         if (lane == 0) mbar_arrive(bar0 + 8u * (kBarRedEmpty + slot));
                     }
-#pragma unroll
-                    for (int b = 0; b < NB; ++b)
-                        if (b < pr.nb(pb) && m < pb.M) pb.y[(pr.out_row0(pb) + b) * pb.M + m] = xscale(b) * t_b[b];
+                    store_rows(m, t_b);
                 }
                 continue;
             }
@@ -1251,9 +1274,7 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
             const int64_t m = static_cast<int64_t>(r.rb0) * kRows + lane;
             if (first_cs == 0 && r.cs == pl.CS - 1) {
                 // the whole row block was ours
-#pragma unroll
-                for (int b = 0; b < NB; ++b)
-                    if (b < pr.nb(pb) && m < pb.M) pb.y[(pr.out_row0(pb) + b) * pb.M + m] = xscale(b) * run[b];
+                store_rows(m, run);
             } else {
                 // shared row block: publish our share, then count ourselves in
                 Share sh;

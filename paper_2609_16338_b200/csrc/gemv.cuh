@@ -2263,13 +2263,48 @@ __device__ __forceinline__ bool grouped_problem(Problem &pr, const Problem &base
     return true;
 }
 
+// PARTS: groups have up to 2 NB tokens, those of more than NB run as two parts of at most NB: the groups' parts in order,
+// found by a warp from the routing lists.  All lanes take part; the lists are read (and checked) again where they are used.
+template <int NB>
+__device__ __forceinline__ bool two_parts(const GroupedArgs &ga, int g) {
+    return static_cast<int64_t>(__ldg(ga.group_begin + g + 1)) - __ldg(ga.group_begin + g) > NB;
+}
+template <int NB>
+__device__ __forceinline__ int count_parts(const GroupedArgs &ga, int n_groups) {
+    int extra = 0;
+    for (int g = threadIdx.x & 31; g < n_groups; g += 32) extra += two_parts<NB>(ga, g) ? 1 : 0;
+    return n_groups + __reduce_add_sync(0xFFFFFFFFu, extra);
+}
+// group and part of the part number `part` (< count_parts)
+template <int NB>
+__device__ __forceinline__ void find_part(const GroupedArgs &ga, int n_groups, int part, int &grp, int &half) {
+    const int lane = threadIdx.x & 31;
+    for (int base = 0; base < n_groups; base += 32) {
+        const int g = base + lane;
+        const bool in = g < n_groups, two = in && two_parts<NB>(ga, g);
+        const uint32_t twos = __ballot_sync(0xFFFFFFFFu, two);
+        const int at = lane + __popc(twos & ((1u << lane) - 1u));      // this group's first part, counted from the chunk's
+        const uint32_t hit = __ballot_sync(0xFFFFFFFFu, in && at <= part && part <= at + (two ? 1 : 0));
+        if (hit) {
+            const int j = __ffs(hit) - 1;
+            grp = base + j;
+            half = part - __shfl_sync(0xFFFFFFFFu, at, j);
+            return;
+        }
+        part -= 32 + __popc(twos);
+    }
+    grp = n_groups;
+    half = 0;
+}
+
 // The pieces of the groups that fall into one thread block's range of the flat item list.
-template <int NB, bool DEBUG>
+template <int NB, bool DEBUG, bool PARTS>
 struct GroupedSegs {
     const Problem *base;
     const GroupedArgs *ga;
-    int64_t lo, hi, ipg;      // this block's range of the list; items per group
+    int64_t lo, hi, ipg;      // this block's range of the list; items per group (or part)
     int grp;                  // group of item lo
+    int half, shift;          // PARTS: which of the group's parts that is; parts beyond the first in front of it
     typedef GroupView View;
     static constexpr bool kSingle = false;
     static constexpr bool kHetero = false;
@@ -2282,7 +2317,7 @@ struct GroupedSegs {
     __device__ __forceinline__ int block_in_job(int block) const { return block; }
     __device__ __forceinline__ bool next(View &v, Walk &w) {
         while (lo < hi) {
-            const int64_t g_lo = static_cast<int64_t>(grp) * ipg;
+            const int64_t g_lo = static_cast<int64_t>(PARTS ? grp + shift + half : grp) * ipg;
             const int64_t seg_hi = hi < g_lo + ipg ? hi : g_lo + ipg;
             w.first = static_cast<int>(lo - g_lo);
             w.count = static_cast<int>(seg_hi - lo);
@@ -2290,11 +2325,20 @@ struct GroupedSegs {
             w.q = 1;
             w.rem = 0;
             lo = seg_hi;
-            const int g = grp++;
-            const GroupDesc gd = read_group(*ga, base->xrow, base->status, g, NB);
+            const int g = grp, h = PARTS ? half : 0;
+            const GroupDesc gd = read_group(*ga, base->xrow, base->status, g, PARTS ? 2 * NB : NB);
+            if (PARTS && h == 0 && static_cast<int64_t>(gd.end) - gd.begin > NB) {
+                half = 1;
+            } else {
+                ++grp;
+                if (PARTS) {
+                    shift += h;
+                    half = 0;
+                }
+            }
             if (!gd.ok || gd.empty) continue;
-            const int e = gd.e, begin = gd.begin, end = gd.end;
-            const bitcos_weights *wd = ga->experts + e;
+            const int begin = gd.begin + h * NB;
+            const bitcos_weights *wd = ga->experts + gd.e;
             v.payload_ = wd->bitmap;
             v.signs_ = wd->signs;
             v.tile_off_ = wd->tile_off;
@@ -2303,7 +2347,7 @@ struct GroupedSegs {
             v.status_ = reinterpret_cast<unsigned int *>(reinterpret_cast<uint8_t *>(base->status) +
                                                          static_cast<size_t>(g) * ga->ws_stride);
             v.begin_ = begin;
-            v.nb_ = min(end - begin, NB);
+            v.nb_ = min(gd.end - begin, NB);
             return true;
         }
         return false;
@@ -2315,7 +2359,7 @@ struct GroupedSegs {
 // that crosses from one group to the next keeps its pipeline running (the producer is already
 // copying the next group's weights while the last tiles of this one are decoded).  Otherwise:
 // blockIdx.y = group, and the blocks of a row of the grid share that group's items.
-template <int FMT, int NB, bool DEBUG>
+template <int FMT, int NB, bool DEBUG, bool PARTS>
 __global__ void __launch_bounds__(max_block_threads(NB), 1) gemv_grouped_kernel(const __grid_constant__ Problem base, const Plan pl,
                                                                                 const __grid_constant__ GroupedArgs ga) {
     extern __shared__ __align__(128) uint8_t smem[];
@@ -2336,16 +2380,27 @@ __global__ void __launch_bounds__(max_block_threads(NB), 1) gemv_grouped_kernel(
                                  static_cast<int>(blockIdx.x));
         return;
     }
-    const int64_t ipg = pl.items, total = ipg * n_groups;
+    int parts = n_groups;
+    if constexpr (PARTS) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        parts = count_parts<NB>(ga, n_groups);
+    }
+    const int64_t ipg = pl.items, total = ipg * parts;
     const int64_t nblk = gridDim.x, b = blockIdx.x;
     const int64_t q = total / nblk, rem = total - q * nblk;
-    GroupedSegs<NB, DEBUG> segs;
+    GroupedSegs<NB, DEBUG, PARTS> segs;
     segs.base = &base;
     segs.ga = &ga;
     segs.ipg = ipg;
     segs.lo = b * q + (b < rem ? b : rem);
     segs.hi = segs.lo + q + (b < rem ? 1 : 0);
     segs.grp = static_cast<int>(segs.lo / ipg);
+    segs.half = segs.shift = 0;
+    if constexpr (PARTS) {
+        const int part = segs.grp;
+        find_part<NB>(ga, n_groups, part, segs.grp, segs.half);
+        segs.shift = part - segs.half - segs.grp;
+    }
     run_segments<FMT, NB, 1>(segs, pl, smem, static_cast<int>(b));
 }
 
@@ -2814,15 +2869,18 @@ int launch_nb(const Problem &pr, const Plan &pl, cudaStream_t stream, const uint
     return launch<FMT, 16, XG>(pr, pl, stream, off_host);
 }
 
-template <int FMT, int NB>
+template <int FMT, int NB, bool PARTS = false>
 int launch_grouped(const Problem &pr, const Plan &pl, const GroupedArgs &ga, int n_groups, cudaStream_t stream) {
     if (NB < kMmaMinBatch && static_cast<int64_t>(NB) * pr.K > kXResidentBytes) return BITCOS_ERR_SHAPE;
     constexpr bool kScr = NB >= kMmaMinBatch && !fragment_order(FMT, NB);
     int sms = 0, budget = 0;
-    int rc = pr.acc_debug ? prepare_kernel<gemv_grouped_kernel<FMT, NB, true>>(&sms, &budget)
-                          : prepare_kernel<gemv_grouped_kernel<FMT, NB, false>>(&sms, &budget);
+    auto kernel = gemv_grouped_kernel<FMT, NB, false, PARTS>;
+    int rc = prepare_kernel<gemv_grouped_kernel<FMT, NB, false, PARTS>>(&sms, &budget);
+    if (pr.acc_debug) {
+        kernel = gemv_grouped_kernel<FMT, NB, true, PARTS>;
+        if (!rc) rc = prepare_kernel<gemv_grouped_kernel<FMT, NB, true, PARTS>>(&sms, &budget);
+    }
     if (rc) return rc;
-    const auto kernel = pr.acc_debug ? gemv_grouped_kernel<FMT, NB, true> : gemv_grouped_kernel<FMT, NB, false>;
     Plan plw = pl;
     plw.stages = choose_stages(FMT, pl, pr.G, NB, pr.K, budget, kScr);
     const SmemLayout L = smem_layout(FMT, plw, pr.G, NB, pr.K, kScr);

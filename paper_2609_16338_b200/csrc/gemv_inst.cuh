@@ -12,7 +12,7 @@ namespace bitcos_kernels {
 #define BITCOS_SINGLE(FMT, NB, XG, XQ, BL) \
     BITCOS_INST int launch<FMT, NB, XG, XQ, BL>(const Problem &, const Plan &, cudaStream_t, const uint32_t *);
 #define BITCOS_MULTI(NB, XQ, XG) BITCOS_INST int launch_multi<NB, XQ, XG>(MultiArgs &, cudaStream_t, const uint32_t *const *, int);
-#define BITCOS_GROUPED(FMT, NB) BITCOS_INST int launch_grouped<FMT, NB>(const Problem &, const Plan &, const GroupedArgs &, int, cudaStream_t);
+#define BITCOS_GROUPED(FMT, NB, PARTS) BITCOS_INST int launch_grouped<FMT, NB, PARTS>(const Problem &, const Plan &, const GroupedArgs &, int, cudaStream_t);
 #define BITCOS_PHASED(NB) BITCOS_INST int launch_phased<NB>(PhasedArgs &, int, const int *, cudaStream_t);
 
 #if BITCOS_IN(1)
@@ -69,25 +69,26 @@ BITCOS_SINGLE(kBit2, 8, false, false, false)
 BITCOS_SINGLE(kBit2, 16, false, false, false)
 #endif
 #if BITCOS_IN(9)
-BITCOS_GROUPED(kBitcos, 1)
-BITCOS_GROUPED(kBitcos, 2)
-BITCOS_GROUPED(kBitcos, 4)
-BITCOS_GROUPED(kBitcos, 8)
-BITCOS_GROUPED(kBitcos, 16)
+BITCOS_GROUPED(kBitcos, 1, false)
+BITCOS_GROUPED(kBitcos, 2, false)
+BITCOS_GROUPED(kBitcos, 4, false)
+BITCOS_GROUPED(kBitcos, 8, false)
+BITCOS_GROUPED(kBitcos, 8, true)
+BITCOS_GROUPED(kBitcos, 16, false)
 #endif
 #if BITCOS_IN(10)
-BITCOS_GROUPED(kTrit5, 1)
-BITCOS_GROUPED(kTrit5, 2)
-BITCOS_GROUPED(kTrit5, 4)
-BITCOS_GROUPED(kTrit5, 8)
-BITCOS_GROUPED(kTrit5, 16)
+BITCOS_GROUPED(kTrit5, 1, false)
+BITCOS_GROUPED(kTrit5, 2, false)
+BITCOS_GROUPED(kTrit5, 4, false)
+BITCOS_GROUPED(kTrit5, 8, false)
+BITCOS_GROUPED(kTrit5, 16, false)
 #endif
 #if BITCOS_IN(11)
-BITCOS_GROUPED(kBit2, 1)
-BITCOS_GROUPED(kBit2, 2)
-BITCOS_GROUPED(kBit2, 4)
-BITCOS_GROUPED(kBit2, 8)
-BITCOS_GROUPED(kBit2, 16)
+BITCOS_GROUPED(kBit2, 1, false)
+BITCOS_GROUPED(kBit2, 2, false)
+BITCOS_GROUPED(kBit2, 4, false)
+BITCOS_GROUPED(kBit2, 8, false)
+BITCOS_GROUPED(kBit2, 16, false)
 #endif
 
 #undef BITCOS_SINGLE

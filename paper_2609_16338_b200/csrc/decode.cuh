@@ -84,6 +84,23 @@ constexpr LutBig make_bitcos_lut() {
     return t;
 }
 
+// BITCOS as bf16 (the 16-bit variant): byte address = ((s << 4) | m) * 256 + lane * 8; an entry is the four weights as
+// bf16 +1 / 0 / -1, two to a word.
+constexpr LutBig make_bitcos_bf16_lut() {
+    const Lut256 base = make_nibble_lut();
+    LutBig t{};
+    for (int idx = 0; idx < kLutBytes / 4; ++idx) {
+        const uint32_t e = base.v[idx >> 6] >> ((idx & 1) ? 16 : 0);
+        uint32_t w = 0;
+        for (int i = 0; i < 2; ++i) {
+            const uint32_t b = (e >> (8 * i)) & 0xFFu;
+            w |= (b == 0 ? 0u : b == 1 ? 0x3F80u : 0xBF80u) << (16 * i);
+        }
+        t.v[idx] = w;
+    }
+    return t;
+}
+
 // Five-trit: byte address = byte value * 256 + lane * 8 (lo word, hi word).
 constexpr LutBig make_trit5_big() {
     const Lut256x2 base = make_trit5_lut();
@@ -120,6 +137,12 @@ __device__ __forceinline__ uint32_t bit_select(uint32_t a, uint32_t b, uint32_t 
 __device__ __forceinline__ uint32_t or_and(uint32_t a, uint32_t b, uint32_t c) {
     uint32_t d;
     asm("lop3.b32 %0, %1, %2, %3, 0xF8;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+    return d;
+}
+// c + sum of the products of the bytes of a and b, all unsigned
+__device__ __forceinline__ uint32_t dp4a_uu(uint32_t a, uint32_t b, uint32_t c) {
+    uint32_t d;
+    asm("dp4a.u32.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
     return d;
 }
 __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
@@ -247,6 +270,25 @@ struct FragmentRows {
             t = __funnelshift_r(B[i], B[i], pos[i]);
             e[2 * i + 1] = static_cast<int>(lds32(lut + 128, bit_select(t, R, 0x0F00u)));
             if (k < 3) pos[i] = __dp4a(e[2 * i + 1], e[2 * i + 1], pos[i]);
+        }
+    }
+    // The same as bf16 +-1 for mma.m16n8k16, nibble j = 0 .. 7 of the four rows: e[2 i] = weights 0 and 1, e[2 i + 1] =
+    // weights 2 and 3 (two words from an 8-byte entry of the bf16 table; B holds the presence words moved down by four, so
+    // that odd nibbles use the same table: open() is followed by shift_presence()).  A non-zero bf16 weight's
+    // high byte is 63 or 191, both -1 modulo 32, so 31 times its high byte counts 1 in the five bits that a rotation uses.
+    __device__ __forceinline__ void shift_presence() {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) B[i] = P[i] >> 4;
+    }
+    __device__ __forceinline__ void step_bf16(int j, const uint8_t *lut, uint32_t lane8, uint32_t (&e)[8]) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint32_t R = __byte_perm((j & 1) ? B[i] : P[i], lane8, 0x6504 | ((j >> 1) << 4));
+            const uint32_t t = __funnelshift_r(A[i], A[i], pos[i]);
+            const uint2 v = lds64(lut, bit_select(t, R, 0xF000u));
+            e[2 * i] = v.x;
+            e[2 * i + 1] = v.y;
+            if (j < 7) pos[i] = static_cast<int>(dp4a_uu(v.y, 0x1F001F00u, dp4a_uu(v.x, 0x1F001F00u, static_cast<uint32_t>(pos[i]))));
         }
     }
 };

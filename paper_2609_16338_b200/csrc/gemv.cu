@@ -733,7 +733,9 @@ int bitcos_gemv_blend_bf16(const bitcos_weights *W, const uint16_t *x_bf16, int 
     const Plan pl = make_plan(W->M, W->K, decoder_warps(8));
     Problem pr{};
     fill_problem(pr, W->bitmap, W->signs, W->tile_off, W->scales, W->M, W->K, x, nullptr, batch, y, nullptr, workspace);
-    return launch<kBitcos, 8, false, false, true>(pr, pl, static_cast<cudaStream_t>(cuda_stream), W->tile_off_host);
+    cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
+    if (batch <= 4) return launch<kBitcos, 4, false, false, true>(pr, pl, stream, W->tile_off_host);
+    return launch<kBitcos, 8, false, false, true>(pr, pl, stream, W->tile_off_host);
 }
 
 int bitcos_gemv_bf16(const bitcos_weights *W, const uint16_t *x_bf16, int batch, float *y, int32_t *acc_debug,

@@ -68,6 +68,7 @@ inline thread_local int g_last_cuda_error = 0;
 // its copy from global memory with one bulk asynchronous copy.
 __device__ __align__(128) const LutBig g_bitcos_lut = make_bitcos_lut();
 __device__ __align__(128) const LutBig g_trit5_lut = make_trit5_big();
+__device__ __align__(128) const LutBig g_bitcos_bf16_lut = make_bitcos_bf16_lut();
 
 // ---------------------------------------------------------------------------------------------
 // Launch plan and problem description.
@@ -289,7 +290,7 @@ struct SmemLayout {
     uint32_t x;          // activations, [nb][K], if x_bytes != 0
     uint32_t x_bytes;    // 0: the activations do not fit and are read from global memory
     uint32_t red;        // 2 x [NW][NB][32] floats
-    uint32_t scr;        // tensor-core path of the baselines and the 16-bit variant: NW transposition buffers of kScrBytes
+    uint32_t scr;        // tensor-core path of the baselines: NW transposition buffers of kScrBytes
     uint32_t bar;        // mbarriers, then per-stage sign base words
     uint32_t total;
 };
@@ -445,20 +446,6 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], 
     asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-// Four decoded weights (bytes 0x00, 0x01, 0xFF) -> four bf16 values 0, +s, -s (the scale blended
-// into the weight, Section II-B): the low three bits of a weight byte (0, 1, 7) pick the high and
-// the low byte of its bf16 value out of two small byte tables built from the scale.
-//   hi_a / hi_b: bytes {0, s_hi, -, -} / {-, -, -, s_hi | 0x80};  lo_a / lo_b: {0, s_lo, -, -} / {-, -, -, s_lo}
-// p01 = (w0, w1), p23 = (w2, w3) as bf16x2.
-__device__ __forceinline__ void blend4(uint32_t t, uint32_t hi_a, uint32_t hi_b, uint32_t lo_a, uint32_t lo_b, uint32_t &p01,
-                                       uint32_t &p23) {
-    uint32_t u = t & 0x07070707u;
-    u |= u >> 4;                                   // byte 0: n0 | n1 << 4, byte 2: n2 | n3 << 4
-    const uint32_t sel = prmt(u, 0u, 0x4420u);     // n0 | n1 << 4 | n2 << 8 | n3 << 12
-    const uint32_t hi = prmt(hi_a, hi_b, sel), lo = prmt(lo_a, lo_b, sel);
-    p01 = prmt(lo, hi, 0x5140u);
-    p23 = prmt(lo, hi, 0x7362u);
 }
 __device__ __forceinline__ void sts128(uint32_t addr, int a, int b, int c, int d) {
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
@@ -825,7 +812,7 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
     const Plan *plp = &pl_in;
 #define pb (*pbp)
 #define pl (*plp)
-    constexpr bool kFrag = fragment_order(FMT, NB) && !Segs::kBlend;
+    constexpr bool kFrag = fragment_order(FMT, NB);
     const SmemLayout L = smem_layout(FMT, pl, segs.shape().G, NB, segs.shape().K, NB >= kMmaMinBatch && !kFrag);
     typename Segs::View pr{};
     Walk wk{};
@@ -840,7 +827,7 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
     // instead of one per token (applied by the epilogue warp to the finished sums)
     constexpr bool kXQ = Segs::kQuantize;                      // (one or two tokens only)
     constexpr bool kBlend = Segs::kBlend;                      // (tensor-core path, up to eight tokens)
-    static_assert(!kBlend || (NB == 8 && FMT == kBitcos && TPW == 1), "blended weights: the eight-token BITCOS kernel");
+    static_assert(!kBlend || ((NB == 4 || NB == 8) && FMT == kBitcos), "16-bit weights: the four- and eight-token BITCOS kernels");
     constexpr bool kXG = Segs::kGroupScales || kXQ || kBlend;   // no token scale in the epilogue
     static_assert(!kXQ || NB < kMmaMinBatch, "16-bit activations: one or two tokens only");
     const uint32_t red_slot = static_cast<uint32_t>(kPairs ? pl.NW : pl.NW * TPW) * NB * kRows;     // floats per partial-sum slot
@@ -985,7 +972,7 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
         if constexpr (Segs::kListsLate) {
             if (lane == 0 && FMT != kBit2) {
                 mbar_expect_tx(bar0 + 8u * kBarLut, kLutBytes);
-                bulk_copy(smem_addr(smem + L.lut), FMT == kBitcos ? g_bitcos_lut.v : g_trit5_lut.v, kLutBytes,
+                bulk_copy(smem_addr(smem + L.lut), Segs::kBlend ? g_bitcos_bf16_lut.v : FMT == kBitcos ? g_bitcos_lut.v : g_trit5_lut.v, kLutBytes,
                           bar0 + 8u * kBarLut);
                 lut_issued = true;
             }
@@ -997,7 +984,7 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
         // needs no address arithmetic.
         if (lane == 0 && have && FMT != kBit2 && !lut_issued) {
             mbar_expect_tx(bar0 + 8u * kBarLut, kLutBytes);
-            bulk_copy(smem_addr(smem + L.lut), FMT == kBitcos ? g_bitcos_lut.v : g_trit5_lut.v, kLutBytes,
+            bulk_copy(smem_addr(smem + L.lut), Segs::kBlend ? g_bitcos_bf16_lut.v : FMT == kBitcos ? g_bitcos_lut.v : g_trit5_lut.v, kLutBytes,
                       bar0 + 8u * kBarLut);
         }
         if (lane == 0) BITCOS_TL(15, clock64());
@@ -1348,10 +1335,11 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
                 const int n = 8 * h + g8 % NC;
                 xfrag[h] = nullptr;
                 if (NB >= kMmaMinBatch && n < pr.nb(pb))
-                    xfrag[h] = pb.x + static_cast<int64_t>(pr.xrow(pb) ? __ldg(pr.xrow(pb) + n) : n) * pb.K + 32 * t4;
+                    xfrag[h] = kBlend ? pb.x + 2 * (static_cast<int64_t>(n) * pb.K + 32 * t4)
+                                      : pb.x + static_cast<int64_t>(pr.xrow(pb) ? __ldg(pr.xrow(pb) + n) : n) * pb.K + 32 * t4;
             }
         };
-        uint32_t bf[NH][8];
+        uint32_t bf[NH][kBlend ? 16 : 8];
         float xg[NH][2];            // group scales of the tokens whose sums this lane keeps
         auto load_x = [&](int grp, const uint8_t *xs) {
             if constexpr (NB < kMmaMinBatch) {
@@ -1359,6 +1347,13 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
                 const uint4 u0 = px[0], u1 = px[1];
                 bf[0][0] = u0.x; bf[0][1] = u0.y; bf[0][2] = u0.z; bf[0][3] = u0.w;
                 bf[0][4] = u1.x; bf[0][5] = u1.y; bf[0][6] = u1.z; bf[0][7] = u1.w;
+            } else if constexpr (kBlend) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    int4 u = make_int4(0, 0, 0, 0);
+                    if (xfrag[0]) u = __ldg(reinterpret_cast<const int4 *>(xfrag[0] + static_cast<int64_t>(grp) * (2 * kGroup)) + q);
+                    bf[0][4 * q] = u.x; bf[0][4 * q + 1] = u.y; bf[0][4 * q + 2] = u.z; bf[0][4 * q + 3] = u.w;
+                }
             } else {
 #pragma unroll
                 for (int h = 0; h < NH; ++h) {
@@ -1372,7 +1367,7 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
                     bf[h][4] = u1.x; bf[h][5] = u1.y; bf[h][6] = u1.z; bf[h][7] = u1.w;
                 }
             }
-            if constexpr (kXG && !kXQ) {
+            if constexpr (kXG && !kXQ && !kBlend) {
                 // (after the dependency wait: the scales come from the kernel before this one)
 #pragma unroll
                 for (int h = 0; h < NH; ++h)
@@ -1467,7 +1462,9 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
                 rows.open(stage + 512u * static_cast<uint32_t>(tile), stage + off_sign, toff - d.w, lane4);
                 // One tile per warp: everything is decoded before the first product (launches of a few items, where a
                 // block's first decode runs while it waits for its dependency).  Two tiles: product by product.
-                constexpr bool kFused = TPW == 2;
+                // (The 16-bit variant always: its decoded row would be 64 registers.)
+                constexpr bool kFused = TPW == 2 || kBlend;
+                if (kBlend) rows.shift_presence();
                 int e[kFused ? 1 : 4][8];
                 if (!kFused) {
 #pragma unroll
@@ -1495,13 +1492,30 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
                 }
                 if (kXQ && grp != q_g) quantize_group(grp);
                 if (NB < kMmaMinBatch) load_x(grp, xs);
-                int acc[NH][2][4];
+                // int32 sums, or fp32 ones of the 16-bit variant: weights +-1 against the activations as they are, the scale
+                // applied to the group's sum (every product is exact).  Its table holds bf16 words, so that a lookup is two
+                // fragment registers: 18944 -> 56832 x 5120 176 clocks per tile and multiprocessor at one token, 213 at four and
+                // eight; 8192x5120 at four tokens 13.8 -> 11.3 us against rebuilding +-s from int8 weights and a pass
+                // through shared memory.
+                typename std::conditional<kBlend, float, int>::type acc[NH][2][4];
 #pragma unroll
                 for (int h = 0; h < NH; ++h)
 #pragma unroll
                     for (int mh = 0; mh < 2; ++mh)
 #pragma unroll
                         for (int r = 0; r < 4; ++r) acc[h][mh][r] = 0;
+                if constexpr (kBlend) {
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        uint32_t ej[8];
+                        rows.step_bf16(j, lut, 2u * lane4, ej);
+#pragma unroll
+                        for (int mh = 0; mh < 2; ++mh) {
+                            const uint32_t a[4] = {ej[4 * mh], ej[4 * mh + 2], ej[4 * mh + 1], ej[4 * mh + 3]};
+                            mma_bf16(acc[0][mh], a, bf[0][2 * j], bf[0][2 * j + 1]);
+                        }
+                    }
+                } else {
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     int(&ek)[8] = e[kFused ? 0 : k];
@@ -1514,6 +1528,7 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
                         for (int h = 0; h < NH; ++h) mma_s8(acc[h][mh], a, bf[h][2 * k], bf[h][2 * k + 1]);
                     }
                 }
+                }
 #pragma unroll
                 for (int j = 0; j < NS; ++j) {
                     const float sc = bf16_to_float(*reinterpret_cast<const uint16_t *>(stage + off_scales + 2u * static_cast<uint32_t>(tile * kRows + g8 + 8 * (s0 + j))));
@@ -1522,18 +1537,18 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
 #pragma unroll
                         for (int r = 0; r < 2; ++r) {
                             // row slot s of a token pair's accumulators: acc[h][s / 2][2 * (s % 2) + column]
-                            int v;
+                            typename std::conditional<kBlend, float, int>::type v;
                             if (NC == 8) v = acc[h][j >> 1][2 * (j & 1) + r];
                             else if (NC == 4) v = (t4 & 2) ? acc[h][1][2 * j + r] : acc[h][0][2 * j + r];
                             else {
-                                const int lo = (t4 & 1) ? acc[h][0][2 + r] : acc[h][0][r], hi = (t4 & 1) ? acc[h][1][2 + r] : acc[h][1][r];
+                                const auto lo = (t4 & 1) ? acc[h][0][2 + r] : acc[h][0][r], hi = (t4 & 1) ? acc[h][1][2 + r] : acc[h][1][r];
                                 v = (t4 & 2) ? hi : lo;
                             }
                             float y = sc * static_cast<float>(v);
                             if (kXQ) y *= q_scale[r];
-                            else if (kXG) y *= xg[h][r];
+                            else if (kXG && !kBlend) y *= xg[h][r];
                             ysum[h][j][r] += y;
-                            if (Segs::kDebug && pb.acc_debug) {
+                            if constexpr (Segs::kDebug) if (pb.acc_debug) {
                                 const int b = 8 * h + n0 + r;
                                 const int64_t m = (static_cast<int64_t>(d.z) + rbl) * kRows + g8 + 8 * (s0 + j);
                                 if (b < pr.nb(pb) && m < pb.M) pb.acc_debug[((pr.out_row0(pb) + b) * pb.M + m) * pb.G + grp] = v;
@@ -1636,27 +1651,14 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
             const int n = 8 * h + (lane >> 2);
             xfrag[h] = nullptr;
             if (kMma && n < pr.nb(pb))
-                xfrag[h] = kBlend ? pb.x + static_cast<int64_t>(n) * pb.K * 2 + 64 * (lane & 3)
-                                  : pb.x + static_cast<int64_t>(pr.xrow(pb) ? __ldg(pr.xrow(pb) + n) : n) * pb.K + 16 * (lane & 3);
+                xfrag[h] = pb.x + static_cast<int64_t>(pr.xrow(pb) ? __ldg(pr.xrow(pb) + n) : n) * pb.K + 16 * (lane & 3);
         }
     };
-    // (blended weights: of token lane / 4 this lane holds bytes 64 c .. 64 c + 63 of the group's 256,
-    // four 16-byte loads; k-step j of the contraction uses words 2 j and 2 j + 1 of those sixteen)
-    uint32_t bf[NH][kBlend ? 16 : 8];
+    uint32_t bf[NH][8];
     float xgq[NH][2];           // group scales of the two tokens whose accumulators this lane holds
     auto load_bf = [&](int g) {
 #pragma unroll
         for (int h = 0; h < NH; ++h) {
-            if constexpr (kBlend) {
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    int4 u = make_int4(0, 0, 0, 0);
-                    if (xfrag[h]) u = __ldg(reinterpret_cast<const int4 *>(xfrag[h] + static_cast<int64_t>(g) * (2 * kGroup)) + q);
-                    bf[h][4 * q + 0] = u.x; bf[h][4 * q + 1] = u.y;
-                    bf[h][4 * q + 2] = u.z; bf[h][4 * q + 3] = u.w;
-                }
-                continue;
-            }
             if (kXG && !kXQ) {
 #pragma unroll
                 for (int r = 0; r < 2; ++r) {
@@ -1803,44 +1805,7 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
                 load_bf(g);
                 x_ready = true;
             }
-            if constexpr (kBlend) {
-                // Weights +-s as bf16 against the unquantised activations: eight k-steps of sixteen
-                // products.  K-step j takes weight word j of each of the row's four 32-weight runs
-                // (k = 32 c + 4 j .. + 3), which is the order the activation words above are held in.
-                float accf[NH][2][4];
-#pragma unroll
-                for (int h = 0; h < NH; ++h)
-#pragma unroll
-                    for (int mh = 0; mh < 2; ++mh)
-#pragma unroll
-                        for (int r = 0; r < 4; ++r) accf[h][mh][r] = 0.f;
-                const uint32_t sbits = *reinterpret_cast<const uint16_t *>(stage + off_scale);
-                const uint32_t s_hi = sbits >> 8, s_lo = sbits & 0xFFu;
-                const uint32_t hi_a = s_hi << 8, hi_b = (s_hi | 0x80u) << 24, lo_a = s_lo << 8, lo_b = s_lo << 24;
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    if (j) __syncwarp();             // everyone has read the previous block back
-                    uint32_t p01[4], p23[4];
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) blend4(static_cast<uint32_t>(w[8 * c + j]), hi_a, hi_b, lo_a, lo_b, p01[c], p23[c]);
-                    sts128(scr_st, p01[0], p01[1], p01[2], p01[3]);
-                    sts128(scr_st + 16u, p23[0], p23[1], p23[2], p23[3]);
-                    __syncwarp();
-#pragma unroll
-                    for (int mh = 0; mh < 2; ++mh) {
-                        uint32_t a[4];
-                        ldmatrix_x4(a, scr_ld + static_cast<uint32_t>(mh * 16 * kScrRowBytes));
-#pragma unroll
-                        for (int h = 0; h < NH; ++h) mma_bf16(accf[h][mh], a, bf[h][2 * j], bf[h][2 * j + 1]);
-                    }
-                }
-#pragma unroll
-                for (int h = 0; h < NH; ++h)
-#pragma unroll
-                    for (int mh = 0; mh < 2; ++mh)
-#pragma unroll
-                        for (int r = 0; r < 4; ++r) ysum[(h * 2 + mh) * 4 + r] = accf[h][mh][r];
-            } else if (kMma) {
+            if (kMma) {
                 int acc[NH][2][4];
 #pragma unroll
                 for (int h = 0; h < NH; ++h)
@@ -2575,15 +2540,15 @@ template <int FMT, int NB, bool XG = false, bool XQ = false, bool BL = false>
 int launch(const Problem &pr, const Plan &pl_in, cudaStream_t stream, const uint32_t *off_host = nullptr) {
     // the one- and two-token instantiations keep the activations in shared memory (nb_bucket sees to it)
     if (NB < kMmaMinBatch && static_cast<int64_t>(NB) * pr.K > kXResidentBytes) return BITCOS_ERR_SHAPE;
-    constexpr bool kTwo = !BL && (NB < kMmaMinBatch || fragment_order(FMT, NB));      // a two-tile instantiation exists
-    constexpr bool kScr = NB >= kMmaMinBatch && (BL || !fragment_order(FMT, NB));
+    constexpr bool kTwo = NB < kMmaMinBatch || fragment_order(FMT, NB);      // a two-tile instantiation exists
+    constexpr bool kScr = NB >= kMmaMinBatch && !fragment_order(FMT, NB);
     int sms = 0, budget = 0;
     int rc = prepare_kernel<gemv_kernel<FMT, NB, 1, XG, XQ, BL>>(&sms, &budget);
     if (rc) return rc;
     const bool two = kTwo && !pr.acc_debug && wants_two_tiles(FMT, pl_in.items, tile_count(pr.M, pr.K), NB, sms);
     if constexpr (kTwo) {
         if (two) {
-            rc = prepare_kernel<gemv_kernel<FMT, NB, 2, XG, XQ>>(&sms, &budget);
+            rc = prepare_kernel<gemv_kernel<FMT, NB, 2, XG, XQ, BL>>(&sms, &budget);
             if (rc) return rc;
         }
     }
@@ -2604,7 +2569,7 @@ int launch(const Problem &pr, const Plan &pl_in, cudaStream_t stream, const uint
     fo.walks = 1;
     fill_first_off(fo, 0, off_host, pr, plw, grid);
     if constexpr (kTwo) {
-        if (two) return launch_pdl(gemv_kernel<FMT, NB, 2, XG, XQ>, dim3(grid), (pl.NW + 2) * 32, L.total, stream, pr, plw, fo);
+        if (two) return launch_pdl(gemv_kernel<FMT, NB, 2, XG, XQ, BL>, dim3(grid), (pl.NW + 2) * 32, L.total, stream, pr, plw, fo);
     }
     if constexpr (!BL) {
         if (pr.acc_debug)

@@ -32,9 +32,10 @@ BITCOS_SINGLE(kBitcos, 4, false, false, false)
 BITCOS_SINGLE(kBitcos, 4, true, false, false)
 BITCOS_SINGLE(kBitcos, 8, false, false, false)
 BITCOS_SINGLE(kBitcos, 8, true, false, false)
-BITCOS_SINGLE(kBitcos, 8, false, false, true)
 #endif
 #if BITCOS_IN(4)
+BITCOS_SINGLE(kBitcos, 4, false, false, true)
+BITCOS_SINGLE(kBitcos, 8, false, false, true)
 BITCOS_SINGLE(kBitcos, 16, false, false, false)
 BITCOS_SINGLE(kBitcos, 16, true, false, false)
 BITCOS_MULTI(16, false, false)

@@ -69,3 +69,19 @@ def test_bf16_activations_with_two_tiles_per_warp(bc):
     want, _ = bc.bitcos_gemv_group_scales(Wd, xq, xg, workspace=ws)
     got, _ = bc.bitcos_gemv_bf16(Wd, xb, workspace=ws)
     assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("groups,blocks", [(1, 9472), (5, 1895), (41, 232), (54, 80), (3, 1)])
+def test_16_bit_variant(bc, groups, blocks):
+    """Weights +-1 in fragment order against bf16 activations, one and two tiles per warp, four and eight columns; the
+    bound is the one of the variant's own tests ((128 + 200) fp32 additions of exact products)."""
+    M, K = 32 * blocks - 3, 128 * groups
+    W, S = datagen.trits(groups + 7, M, K, 0.4711), datagen.scales(groups, M, K)
+    Wd, ws = bc.bitcos_pack(W, S).to_device(), bc.make_workspace(M, K)
+    for B in (1, 4, 5, 8):
+        bits = datagen.activations_bf16(groups + B, B, K)
+        y_ref, mag = oracle.gemv_dense_blend(W, S, datagen.bf16_bits_to_f32(bits))
+        y = bc.bitcos_gemv_blend_bf16(Wd, dev(bits.view(np.int16)).view(torch.bfloat16), workspace=ws)
+        err = np.abs(y.cpu().numpy().astype(np.float64) - y_ref)
+        assert (err <= 2e-5 * mag).all(), (groups, B)
+    assert bc.workspace_status(ws) == 0

@@ -1,11 +1,21 @@
 // Device-side BITCOS packer: dense int8 trits and row-major bf16 scales in device memory -> the
 // four packed buffers of the layout in bitcos.h (Section II-A of the paper: presence bitmap,
 // compacted sign vector in the same order; entry offsets per tile), byte for byte what the host
-// packer writes.  Three kernels: bitmap + scales + per-tile counts; an exclusive scan of the counts
-// (the entry offsets); the sign vector.  A set-up path, not the hot path: one warp per 32 x 128
-// tile, lane = row, the same decomposition as the products.
+// packer writes.  Three kernels: bitmap + scales + per-tile counts (and the sign vector zeroed); an exclusive
+// scan of the counts (the entry offsets); the sign vector.  One warp per 32 x 128 tile.
+//
+// Bound by memory: the trits (a byte each) are read twice, the second time from L2 where they fit there.
+// Eight lanes take a row's 128 bytes, 16 weights a lane, four rows a load: whole lines, where one lane per row
+// (the products' order) touched 32 rows a load at half a sector each.  Those 16-weight chunks in the order (load, lane)
+// are the tile's weights in order, so the masks go out as 16-bit stores of 64 bytes a warp, and the sign bits
+// of a chunk lie where a scan of the chunk counts puts them.
+//
+// 8192x5120 (42 MB of trits), a whole call through the binding: 156 -> 89 us.  The kernels take 35 of them (13 + 6 + 19
+// before they overlapped, from L2 at the second reading), the rest is one wait for the stream and the caller's
+// allocations; two waits, two fills, the offsets copied out and a copy of the sign vector by the copy engine went.
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstddef>
 #include <cstdint>
 
@@ -35,116 +45,163 @@ inline int check_cuda(cudaError_t e) {
 inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 inline int64_t padded_rows(int64_t M) { return (M + kRows - 1) / kRows * kRows; }
 
-// Presence and negative masks of the four bytes of a word (bit i <-> byte i), and whether all
-// four are in {-1, 0, +1}.
-__device__ __forceinline__ uint32_t byte_tops(uint32_t m) {
-    // bits 7, 15, 23, 31 -> bits 0..3 (the four partial products land on distinct bits: no carries)
-    return ((m & 0x80808080u) * 0x00204081u) >> 28;
-}
-__device__ __forceinline__ void masks4(uint32_t w, uint32_t &pres, uint32_t &neg, bool &ok) {
-    const uint32_t zero = __vcmpeq4(w, 0u), one = __vcmpeq4(w, 0x01010101u), minus = __vcmpeq4(w, 0xFFFFFFFFu);
-    pres |= byte_tops(~zero);
-    neg |= byte_tops(minus);
-    ok = ok && ((zero | one | minus) == 0xFFFFFFFFu);
-}
-
-// The 128 weights of (row m, group g) as four presence words and four negative words (bit i of
-// word j <-> k = 128 g + 32 j + i); rows beyond M read as zero.
-__device__ __forceinline__ bool load_row_masks(const int8_t *__restrict__ trits, int64_t M, int64_t K, int64_t m, int g,
-                                               uint32_t (&pres)[4], uint32_t (&neg)[4]) {
-    bool ok = true;
+// 16 consecutive weights (a 16-byte load) -> presence and negative masks of 16 bits; `bad` collects what is not in
+// {-1, 0, +1} (any bit of it).  A trit's bit 0 says present, its bit 7 negative; a negative one must be 0xFF, any
+// other 0 or 1.  The multiplications gather one bit per byte (distinct bits, no carries).
+__device__ __forceinline__ void masks16(const uint4 &v, uint32_t &pres, uint32_t &neg, uint32_t &bad) {
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    uint32_t p = 0u, n = 0u;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) pres[j] = neg[j] = 0u;
-    if (m >= M) return true;
-    const uint4 *src = reinterpret_cast<const uint4 *>(trits + m * K + static_cast<int64_t>(g) * kGroup);
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {                     // 16 weights per load
-        const uint4 v = __ldg(src + q);
-        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-        uint32_t p = 0u, n = 0u;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            uint32_t pp = 0u, nn = 0u;
-            masks4(w[i], pp, nn, ok);
-            p |= pp << (4 * i);
-            n |= nn << (4 * i);
-        }
-        pres[q >> 1] |= p << (16 * (q & 1));
-        neg[q >> 1] |= n << (16 * (q & 1));
+    for (int i = 0; i < 4; ++i) {
+        const uint32_t top = w[i] & 0x80808080u, all = (top >> 7) * 0xFFu;
+        bad |= (w[i] ^ all) & (0xFEFEFEFEu | all);
+        p = (p >> 4) | (((w[i] & 0x01010101u) * 0x10204080u) & 0xF0000000u);
+        n = (n >> 4) | ((top * 0x00204081u) & 0xF0000000u);
     }
-    return ok;
+    pres = p >> 16;
+    neg = n >> 16;
 }
 
-// Kernel 1: bitmap, scales in tile order, number of non-zero weights per tile (into tile_off).
+// Chunk i of this lane in the tile (row block rb, group g): weights 16 (lane % 8) .. + 15 of row 4 i + lane / 8; rows
+// beyond M read as zero.
+__device__ __forceinline__ uint4 load_chunk(const int8_t *__restrict__ trits, int64_t M, int64_t K, int64_t rb, int g, int i, int lane) {
+    const int64_t m = rb * kRows + 4 * i + (lane >> 3);
+    if (m >= M) return make_uint4(0u, 0u, 0u, 0u);
+    return __ldg(reinterpret_cast<const uint4 *>(trits + m * K + static_cast<int64_t>(g) * kGroup) + (lane & 7));
+}
+
+// Kernel 1: bitmap, scales in tile order, number of non-zero weights per tile (into tile_off, with two bits above it for
+// what is wrong with the tile); and zeros over the sign vector, into which kernel 3 ORs the words that two tiles share.
+constexpr uint32_t kBadTrit = 0x80000000u, kBadScale = 0x40000000u, kCountMask = 0x3FFFFFFFu;
+// (A block per eight tiles, no loop: with a grid of eight blocks per multiprocessor most warps had one tile and a few two.)
 __global__ void __launch_bounds__(kPackWarps * 32) pack_bitmap_kernel(const int8_t *__restrict__ trits,
                                                                       const uint16_t *__restrict__ scales, int64_t M, int64_t K,
-                                                                      uint32_t *__restrict__ bitmap,
+                                                                      uint16_t *__restrict__ bitmap,
                                                                       uint16_t *__restrict__ scales_tiled,
                                                                       uint32_t *__restrict__ tile_off, int64_t n_tiles,
-                                                                      unsigned int *__restrict__ flags) {
+                                                                      uint4 *__restrict__ signs, int64_t sign_quads) {
     const int lane = threadIdx.x & 31;
     const int G = static_cast<int>(K / kGroup);
-    for (int64_t t = static_cast<int64_t>(blockIdx.x) * kPackWarps + (threadIdx.x >> 5); t < n_tiles;
-         t += static_cast<int64_t>(gridDim.x) * kPackWarps) {
+    uint32_t bad = 0u;
+    const int64_t t = static_cast<int64_t>(blockIdx.x) * kPackWarps + (threadIdx.x >> 5);
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (t < n_tiles) {
         const int64_t rb = t / G;
         const int g = static_cast<int>(t - rb * G);
+        uint4 v[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = load_chunk(trits, M, K, rb, g, i, lane);
         const int64_t m = rb * kRows + lane;
-        uint32_t pres[4], neg[4];
-        const bool ok = load_row_masks(trits, M, K, m, g, pres, neg);
-        if (!ok) atomicOr(flags + kFlagTrit, 1u);
-        reinterpret_cast<uint4 *>(bitmap)[t * kRows + lane] = make_uint4(pres[0], pres[1], pres[2], pres[3]);
         uint16_t s = 0;
-        if (m < M) {
-            s = scales[m * G + g];
-            if ((s & 0x8000u) || (s & 0x7F80u) == 0x7F80u) atomicOr(flags + kFlagScale, 1u);
+        if (m < M) s = __ldg(scales + m * G + g);
+        uint32_t c = 0u;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            uint32_t pres, neg;
+            masks16(v[i], pres, neg, bad);
+            bitmap[t * 256 + 32 * i + lane] = static_cast<uint16_t>(pres);
+            c += __popc(pres);
         }
         scales_tiled[t * kRows + lane] = s;
-        unsigned int c = __popc(pres[0]) + __popc(pres[1]) + __popc(pres[2]) + __popc(pres[3]);
-#pragma unroll
-        for (int d = 16; d; d >>= 1) c += __shfl_xor_sync(0xFFFFFFFFu, c, d);
+        c = __reduce_add_sync(0xFFFFFFFFu, c);
+        if (__any_sync(0xFFFFFFFFu, bad != 0u)) c |= kBadTrit;
+        if (__any_sync(0xFFFFFFFFu, (s & 0x8000u) || (s & 0x7F80u) == 0x7F80u)) c |= kBadScale;
         if (lane == 0) tile_off[t] = c;
     }
+    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < sign_quads; i += static_cast<int64_t>(gridDim.x) * blockDim.x)
+        signs[i] = make_uint4(0u, 0u, 0u, 0u);
 }
 
-// Kernel 2: exclusive scan of the per-tile counts in place, one thread block walking the array in
-// chunks; tile_off[n_tiles] and the 64-bit total receive the sum.
+// Kernel 2: exclusive scan of the per-tile counts in place, one thread block walking the array 8192 tiles at a time
+// (eight to a thread); tile_off[n_tiles] and the 64-bit total receive the sum, the words after it up to n_words zero.
+// The offsets also go straight to the host's copy where that is mapped (off_host, may be NULL): 41 KB that cross the bus
+// while kernel 3 runs, where a copy after it took 11 us.
 constexpr int kScanThreads = 1024;
-__global__ void __launch_bounds__(kScanThreads) scan_counts_kernel(uint32_t *__restrict__ tile_off, int64_t n_tiles,
-                                                                   unsigned int *__restrict__ flags) {
-    __shared__ unsigned long long warp_sum[kScanThreads / 32];
-    __shared__ unsigned long long carry_s;
+constexpr int kScanQuads = 2;       // 16-byte loads per thread
+__global__ void __launch_bounds__(kScanThreads) scan_counts_kernel(uint32_t *__restrict__ tile_off, uint32_t *__restrict__ off_host,
+                                                                   int64_t n_tiles, int64_t n_words,
+                                                                   unsigned int *__restrict__ flags, volatile unsigned int *report) {
+    __shared__ uint32_t warp_sum[kScanThreads / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (threadIdx.x == 0) carry_s = 0ull;
-    __syncthreads();
-    for (int64_t base = 0; base < n_tiles; base += kScanThreads) {
-        const int64_t i = base + threadIdx.x;
-        const unsigned long long v = (i < n_tiles) ? tile_off[i] : 0ull;
-        unsigned long long inc = v;
+    unsigned long long carry = 0ull;                 // the same in every thread
+    bool over = false;
+    uint32_t seen = 0u;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    for (int64_t base = 0; base < n_tiles; base += kScanThreads * kScanQuads * 4) {
+        const int64_t i0 = base + static_cast<int64_t>(threadIdx.x) * (kScanQuads * 4);
+        uint32_t c[kScanQuads * 4];
+        uint32_t mine = 0u;
+#pragma unroll
+        for (int q = 0; q < kScanQuads; ++q) {
+            uint4 v = make_uint4(0u, 0u, 0u, 0u);
+            const int64_t i = i0 + 4 * q;
+            if (i < n_words) v = __ldcg(reinterpret_cast<const uint4 *>(tile_off + i));      // (n_words: a multiple of four)
+            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const uint32_t x = i + j < n_tiles ? w[j] : 0u;
+                seen |= x;
+                c[4 * q + j] = x & kCountMask;
+                mine += c[4 * q + j];
+            }
+        }
+        uint32_t upto = mine;                        // (a pass holds at most 8192 x 4096 non-zeros)
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
-            const unsigned long long o = __shfl_up_sync(0xFFFFFFFFu, inc, d);
-            if (lane >= d) inc += o;
+            const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, upto, d);
+            if (lane >= d) upto += o;
         }
-        if (lane == 31) warp_sum[warp] = inc;
+        if (lane == 31) warp_sum[warp] = upto;
         __syncthreads();
-        unsigned long long before = carry_s;
-        for (int w = 0; w < warp; ++w) before += warp_sum[w];
-        const unsigned long long excl = before + inc - v;
-        if (i < n_tiles) {
-            if (excl > 0xFFFFFFFFull) atomicOr(flags + kFlagOverflow, 1u);
-            tile_off[i] = static_cast<uint32_t>(excl);
+        uint32_t w_upto = warp_sum[lane];            // every warp scans the warps' sums itself
+        const uint32_t w_mine = w_upto;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, w_upto, d);
+            if (lane >= d) w_upto += o;
         }
+        const uint32_t before = __shfl_sync(0xFFFFFFFFu, w_upto - w_mine, warp), pass = __shfl_sync(0xFFFFFFFFu, w_upto, 31);
+        unsigned long long at = carry + before + (upto - mine);
+#pragma unroll
+        for (int q = 0; q < kScanQuads; ++q) {
+            const int64_t i = i0 + 4 * q;
+            uint32_t w[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                w[j] = i + j <= n_tiles ? static_cast<uint32_t>(at) : 0u;
+                over = over || (i + j <= n_tiles && at > 0xFFFFFFFFull);
+                at += c[4 * q + j];
+            }
+            if (i < n_words) {
+                *reinterpret_cast<uint4 *>(tile_off + i) = make_uint4(w[0], w[1], w[2], w[3]);
+                if (off_host) *reinterpret_cast<uint4 *>(off_host + i) = make_uint4(w[0], w[1], w[2], w[3]);
+            }
+        }
+        carry += pass;
         __syncthreads();
-        if (threadIdx.x == kScanThreads - 1) carry_s = before + inc;
-        __syncthreads();
+    }
+    const int any_over = __syncthreads_or(over || carry > 0xFFFFFFFFull);
+    const int any_trit = __syncthreads_or((seen & kBadTrit) != 0u), any_scale = __syncthreads_or((seen & kBadScale) != 0u);
+    // the sentinel, where the last pass ended exactly on it
+    for (int64_t i = n_tiles + threadIdx.x; i < n_words; i += kScanThreads) {
+        tile_off[i] = i == n_tiles ? static_cast<uint32_t>(carry) : 0u;
+        if (off_host) off_host[i] = i == n_tiles ? static_cast<uint32_t>(carry) : 0u;
     }
     if (threadIdx.x == 0) {
-        const unsigned long long total = carry_s;
-        if (total > 0xFFFFFFFFull) atomicOr(flags + kFlagOverflow, 1u);
-        tile_off[n_tiles] = static_cast<uint32_t>(total);
-        flags[kNnzLo] = static_cast<unsigned int>(total);
-        flags[kNnzLo + 1] = static_cast<unsigned int>(total >> 32);
+        flags[kFlagTrit] = any_trit ? 1u : 0u;
+        flags[kFlagScale] = any_scale ? 1u : 0u;
+        flags[kFlagOverflow] = any_over ? 1u : 0u;
+        flags[kNnzLo] = static_cast<unsigned int>(carry);
+        flags[kNnzLo + 1] = static_cast<unsigned int>(carry >> 32);
+        // what the host wants to know, straight into its memory
+        report[kFlagTrit] = any_trit ? 1u : 0u;
+        report[kFlagScale] = any_scale ? 1u : 0u;
+        report[kFlagOverflow] = any_over ? 1u : 0u;
+        report[kNnzLo] = static_cast<unsigned int>(carry);
+        report[kNnzLo + 1] = static_cast<unsigned int>(carry >> 32);
     }
+    __threadfence_system();
 }
 
 // The bits of `src` at the set positions of `mask`, packed towards bit 0 (the inverse of the
@@ -170,51 +227,76 @@ __device__ __forceinline__ uint32_t extract_bits(uint32_t src, uint32_t mask) {
     return x;
 }
 
-// Kernel 3: the sign vector.  Row r of tile t owns the bits [tile_off[t] + (non-zeros of rows
-// 0 .. r-1 of the tile), + its own non-zeros); it ORs them into the (zero-filled) vector.
+// Kernel 3: the sign vector.  Tile t owns the bits tile_off[t] .. tile_off[t + 1] - 1; its chunks' sign bits are gathered in
+// shared memory, aligned to the vector's words, and go out as whole words, the first and the last (which the tile may
+// share with its neighbours) by an atomic OR.  Two chunks are compacted at a time, in the halves of one word.  Nothing
+// is written if the counts found something wrong or the vector does not fit its buffer (the host reports it).
+constexpr int kSignWords = kRows * kGroup / 32 + 1;      // 4096 bits starting anywhere in a word
 __global__ void __launch_bounds__(kPackWarps * 32) pack_signs_kernel(const int8_t *__restrict__ trits, int64_t M, int64_t K,
                                                                      const uint32_t *__restrict__ tile_off,
-                                                                     uint32_t *__restrict__ signs, int64_t n_tiles) {
+                                                                     uint32_t *__restrict__ signs, unsigned long long max_nnz, int64_t n_tiles,
+                                                                     const unsigned int *__restrict__ flags) {
+    __shared__ uint32_t words[kPackWarps][kSignWords + 3];
     const int lane = threadIdx.x & 31;
     const int G = static_cast<int>(K / kGroup);
-    for (int64_t t = static_cast<int64_t>(blockIdx.x) * kPackWarps + (threadIdx.x >> 5); t < n_tiles;
-         t += static_cast<int64_t>(gridDim.x) * kPackWarps) {
+    uint32_t *buf = words[threadIdx.x >> 5];
+    const int64_t t = static_cast<int64_t>(blockIdx.x) * kPackWarps + (threadIdx.x >> 5);
+    if (t < n_tiles) {
         const int64_t rb = t / G;
         const int g = static_cast<int>(t - rb * G);
-        uint32_t pres[4], neg[4];
-        load_row_masks(trits, M, K, rb * kRows + lane, g, pres, neg);
-        const unsigned int c = __popc(pres[0]) + __popc(pres[1]) + __popc(pres[2]) + __popc(pres[3]);
-        unsigned int inc = c;
+        uint4 v[8];
 #pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const unsigned int o = __shfl_up_sync(0xFFFFFFFFu, inc, d);
-            if (lane >= d) inc += o;
-        }
-        // this row's sign bits, compacted: up to 128 bits in four words
-        uint32_t sb[5] = {0u, 0u, 0u, 0u, 0u};
-        int filled = 0;
+        for (int i = 0; i < 8; ++i) v[i] = load_chunk(trits, M, K, rb, g, i, lane);
+        for (uint32_t i = lane; i < kSignWords; i += 32) buf[i] = 0u;
+        // the chunks' sign bits and where they lie inside the tile
+        uint32_t both[4], cnt[4], at0[4], at1[4], at = 0u;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const uint32_t bits = extract_bits(neg[j], pres[j]);
-            const int n = __popc(pres[j]);
-            const int w = filled >> 5, sh = filled & 31;
-            if (n) {
-                sb[w] |= bits << sh;
-                if (sh && sh + n > 32) sb[w + 1] |= bits >> (32 - sh);
+        for (int i = 0; i < 4; ++i) {
+            uint32_t p0, n0, p1, n1, bad = 0u;
+            masks16(v[2 * i], p0, n0, bad);
+            masks16(v[2 * i + 1], p1, n1, bad);
+            both[i] = extract_bits(n0 | (n1 << 16), p0 | (p1 << 16));
+            cnt[i] = __popc(p0) | (__popc(p1) << 16);
+            uint32_t upto = cnt[i];                  // (at most 512 per load: both scans in one register)
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, upto, d);
+                if (lane >= d) upto += o;
             }
-            filled += n;
+            const uint32_t total = __shfl_sync(0xFFFFFFFFu, upto, 31), before = upto - cnt[i];
+            at0[i] = at + (before & 0xFFFFu);
+            at1[i] = at + (total & 0xFFFFu) + (before >> 16);
+            at += (total & 0xFFFFu) + (total >> 16);
         }
-        // shifted to the row's position in the vector
-        const uint64_t q0 = static_cast<uint64_t>(__ldg(tile_off + t)) + (inc - c);
-        const uint64_t w0 = q0 >> 5;
-        const int sh = static_cast<int>(q0 & 31u);
-        const int words = (sh + static_cast<int>(c) + 31) >> 5;
-        uint32_t prev = 0u;
-        for (int i = 0; i < words; ++i) {
-            const uint32_t cur = (i < 4) ? sb[i] : 0u;
-            const uint32_t out = sh ? ((cur << sh) | (prev >> (32 - sh))) : cur;
-            if (out) atomicOr(signs + w0 + i, out);
-            prev = cur;
+        // All of that needed the trits alone; the tile's place needs the scan.
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        // (from L2: this kernel may have been resident before those words were written)
+        if (__ldcg(flags + kFlagTrit) || __ldcg(flags + kFlagScale) || __ldcg(flags + kFlagOverflow) ||
+            (__ldcg(flags + kNnzLo) | (static_cast<unsigned long long>(__ldcg(flags + kNnzLo + 1)) << 32)) > max_nnz)
+            return;
+        const uint32_t first = __ldcg(tile_off + t);
+        const uint32_t sh0 = first & 31u, bits = sh0 + at;      // bits of the buffer in use
+        __syncwarp();
+        auto put = [&](uint32_t pos, uint32_t b, uint32_t n) {
+            if (!b) return;
+            atomicOr(buf + (pos >> 5), b << (pos & 31u));
+            if ((pos & 31u) + n > 32u) atomicOr(buf + (pos >> 5) + 1, b >> (32u - (pos & 31u)));
+        };
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint32_t c0 = cnt[i] & 0xFFFFu;    // (at most 16)
+            put(sh0 + at0[i], both[i] & ((1u << c0) - 1u), c0);
+            put(sh0 + at1[i], both[i] >> c0, cnt[i] >> 16);
+        }
+        __syncwarp();
+        uint32_t *out = signs + (first >> 5);
+        const uint32_t full = bits >> 5;             // whole words, the first one among them if sh0 == 0
+        for (uint32_t i = lane; i < (bits + 31u) >> 5; i += 32) {
+            if ((i == 0 && sh0) || i >= full) {
+                if (buf[i]) atomicOr(out + i, buf[i]);
+            } else {
+                out[i] = buf[i];
+            }
         }
     }
 }
@@ -223,22 +305,18 @@ __global__ void __launch_bounds__(kPackWarps * 32) pack_signs_kernel(const int8_
 __global__ void __launch_bounds__(256) count_nnz_kernel(const int8_t *__restrict__ trits, int64_t n16,
                                                         unsigned int *__restrict__ flags) {
     unsigned long long c = 0ull;
-    bool ok = true;
+    uint32_t bad = 0u;
     const uint4 *src = reinterpret_cast<const uint4 *>(trits);
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n16;
          i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
         const uint4 v = __ldg(src + i);
-        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            uint32_t p = 0u, n = 0u;
-            masks4(w[j], p, n, ok);
-            c += __popc(p);
-        }
+        uint32_t pres, neg;
+        masks16(v, pres, neg, bad);
+        c += __popc(pres);
     }
 #pragma unroll
     for (int d = 16; d; d >>= 1) c += __shfl_xor_sync(0xFFFFFFFFu, c, d);
-    if (!__all_sync(0xFFFFFFFFu, ok) && (threadIdx.x & 31) == 0) atomicOr(flags + kFlagTrit, 1u);
+    if (bad) atomicOr(flags + kFlagTrit, 1u);
     if ((threadIdx.x & 31) == 0 && c) atomicAdd(reinterpret_cast<unsigned long long *>(flags + kNnzLo), c);
 }
 
@@ -249,6 +327,61 @@ int grid_for(int64_t units, int per_block) {
     const int64_t want = (units + per_block - 1) / per_block;
     const int64_t cap = static_cast<int64_t>(sms) * 8;
     return static_cast<int>(want < 1 ? 1 : (want < cap ? want : cap));
+}
+
+// The host's end of scan_counts_kernel's report: 64-byte slots of one pinned page, mapped into every device, taken for the
+// time of a call (a copy of 32 bytes to pageable memory costs about 10 us more than this).  A caller that finds no
+// free slot gets none and reads the scratch words by a copy.
+constexpr int kReportSlots = 64;
+struct ReportSlot {
+    static std::atomic<uint64_t> &taken() {
+        static std::atomic<uint64_t> t{0};
+        return t;
+    }
+    static unsigned int *page() {
+        static unsigned int *p = [] {
+            void *v = nullptr;
+            if (cudaHostAlloc(&v, kReportSlots * 64, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+                cudaGetLastError();
+                v = nullptr;
+            }
+            return static_cast<unsigned int *>(v);
+        }();
+        return p;
+    }
+    int slot = -1;
+    ReportSlot() {
+        if (!page()) return;
+        uint64_t t = taken().load();
+        while (~t) {
+            const int i = __builtin_ctzll(~t);
+            if (taken().compare_exchange_weak(t, t | (1ull << i))) {
+                slot = i;
+                return;
+            }
+        }
+    }
+    ~ReportSlot() {
+        if (slot >= 0) taken().fetch_and(~(1ull << slot));
+    }
+    ReportSlot(const ReportSlot &) = delete;
+    ReportSlot &operator=(const ReportSlot &) = delete;
+    unsigned int *host() const { return slot < 0 ? nullptr : page() + slot * 16; }
+};
+
+// A launch that may start while the kernel before it is still running (what depends on it waits in the kernel).
+template <typename... KArgs, typename... Args>
+int launch_behind(void (*kernel)(KArgs...), int64_t grid, int threads, cudaStream_t stream, Args... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(static_cast<unsigned>(grid));
+    cfg.blockDim = dim3(static_cast<unsigned>(threads));
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return check_cuda(cudaLaunchKernelEx(&cfg, kernel, args...));
 }
 
 int read_flags(const void *scratch, cudaStream_t stream, unsigned int (&h)[8]) {
@@ -293,20 +426,50 @@ int bitcos_pack_device(const int8_t *trits, const uint16_t *scales_bf16, int64_t
     size_t off_bytes = 0;
     int rc = bitcos_pack_sizes(M, K, 0, nullptr, nullptr, &off_bytes, nullptr);
     if (rc) return rc;
+    // the sign bits the caller's buffer has room for (32 bytes of zero slack behind them; the whole is a multiple of 16)
+    const size_t slack = 32;
+    unsigned long long max_nnz = 0;
+    if (sign_capacity_bytes >= slack) max_nnz = static_cast<unsigned long long>((sign_capacity_bytes - slack) / 16 * 16) * 8;
     unsigned int *flags = static_cast<unsigned int *>(scratch);
-    rc = check_cuda(cudaMemsetAsync(scratch, 0, BITCOS_PACK_SCRATCH_BYTES, stream));
-    if (rc) return rc;
-    rc = check_cuda(cudaMemsetAsync(tile_off, 0, off_bytes, stream));
-    if (rc) return rc;
-    pack_bitmap_kernel<<<grid_for(n_tiles, kPackWarps), kPackWarps * 32, 0, stream>>>(trits, scales_bf16, M, K, bitmap,
-                                                                                    scales_tiled, tile_off, n_tiles, flags);
+    // the host's copy of the offsets, if the device can write there
+    uint32_t *off_mapped = nullptr;
+    if (tile_off_host) {
+        cudaPointerAttributes at{};
+        if (cudaPointerGetAttributes(&at, tile_off_host) == cudaSuccess && at.type == cudaMemoryTypeHost && at.devicePointer && aligned16(at.devicePointer))
+            off_mapped = static_cast<uint32_t *>(at.devicePointer);
+        else
+            cudaGetLastError();
+    }
+    const int64_t grid = (n_tiles + kPackWarps - 1) / kPackWarps;
+    if (grid > 0x7FFFFFFF) return BITCOS_ERR_SHAPE;
+    const ReportSlot report;
+    unsigned int *report_dev = flags;                // (no slot: the words report on themselves)
+    if (report.host()) {
+        rc = check_cuda(cudaHostGetDevicePointer(reinterpret_cast<void **>(&report_dev), report.host(), 0));
+        if (rc) return rc;
+    }
+    pack_bitmap_kernel<<<static_cast<unsigned>(grid), kPackWarps * 32, 0, stream>>>(
+        trits, scales_bf16, M, K, reinterpret_cast<uint16_t *>(bitmap), scales_tiled, tile_off, n_tiles, reinterpret_cast<uint4 *>(signs),
+        static_cast<int64_t>(sign_capacity_bytes / 16));
     rc = check_cuda(cudaGetLastError());
     if (rc) return rc;
-    scan_counts_kernel<<<1, kScanThreads, 0, stream>>>(tile_off, n_tiles, flags);
-    rc = check_cuda(cudaGetLastError());
+    rc = launch_behind(scan_counts_kernel, 1, kScanThreads, stream, tile_off, off_mapped, n_tiles, static_cast<int64_t>(off_bytes / 4), flags,
+                       static_cast<volatile unsigned int *>(report_dev));
     if (rc) return rc;
+    rc = launch_behind(pack_signs_kernel, grid, kPackWarps * 32, stream, trits, M, K, static_cast<const uint32_t *>(tile_off), signs, max_nnz,
+                       n_tiles, static_cast<const unsigned int *>(flags));
+    if (rc) return rc;
+    if (tile_off_host && !off_mapped) {
+        rc = check_cuda(cudaMemcpyAsync(tile_off_host, tile_off, off_bytes, cudaMemcpyDeviceToHost, stream));
+        if (rc) return rc;
+    }
     unsigned int h[8];
-    rc = read_flags(scratch, stream, h);
+    if (report.host()) {
+        rc = check_cuda(cudaStreamSynchronize(stream));
+        for (int i = 0; i < 8; ++i) h[i] = static_cast<const volatile unsigned int *>(report.host())[i];
+    } else {
+        rc = read_flags(scratch, stream, h);         // (waits for the stream)
+    }
     if (rc) return rc;
     if (h[kFlagTrit]) return BITCOS_ERR_TRIT;
     if (h[kFlagScale]) return BITCOS_ERR_SCALE;
@@ -316,17 +479,6 @@ int bitcos_pack_device(const int8_t *trits, const uint16_t *scales_bf16, int64_t
     rc = bitcos_pack_sizes(M, K, nnz, nullptr, &need, nullptr, nullptr);
     if (rc) return rc;
     if (sign_capacity_bytes < need) return BITCOS_ERR_CAPACITY;
-    rc = check_cuda(cudaMemsetAsync(signs, 0, sign_capacity_bytes, stream));
-    if (rc) return rc;
-    pack_signs_kernel<<<grid_for(n_tiles, kPackWarps), kPackWarps * 32, 0, stream>>>(trits, M, K, tile_off, signs, n_tiles);
-    rc = check_cuda(cudaGetLastError());
-    if (rc) return rc;
-    if (tile_off_host) {
-        rc = check_cuda(cudaMemcpyAsync(tile_off_host, tile_off, off_bytes, cudaMemcpyDeviceToHost, stream));
-        if (rc) return rc;
-    }
-    rc = check_cuda(cudaStreamSynchronize(stream));
-    if (rc) return rc;
     if (nnz_out) *nnz_out = nnz;
     return BITCOS_OK;
 }

@@ -88,3 +88,38 @@ def test_device_pack_error_codes(bc):
         bc.bitcos_pack_device(torch.zeros((4, 100), dtype=torch.int8, device="cuda"),
                               torch.zeros((4, 1), dtype=torch.int16, device="cuda"))
     assert e.value.status == 2
+
+
+@pytest.mark.parametrize("M,K,z", [(32, 128 * 8191, 0.5), (32 * 4096, 256, 0.47), (32 * 4096 - 31, 256, 0.3), (3, 128 * 8193, 0.9)])
+def test_device_pack_around_a_scan_pass(bc, M, K, z):
+    """The entry offsets are scanned 8192 tiles at a time: one tile fewer, exactly as many, one more; and sign bits of
+    a few non-zeros a tile, where several tiles share a word."""
+    W, S = datagen.trits(3300 + M, M, K, z), datagen.scales(3300 + M, M, K)
+    if z == 0.9:
+        W[:, ::3] = 0
+        W[1:] = 0
+    Wd = bc.bitcos_pack_device(torch.from_numpy(W).cuda(), torch.from_numpy(S.view(np.int16)).cuda())
+    host = bc.bitcos_pack(W, S)
+    assert Wd.nnz == host.nnz
+    assert np.array_equal(u32(Wd.bitmap), host.bitmap) and np.array_equal(u32(Wd.signs), host.signs)
+    assert np.array_equal(u32(Wd.tile_off), host.tile_off_buf) and np.array_equal(Wd.tile_off_host, host.tile_off)
+    assert np.array_equal(Wd.scales.cpu().numpy().view(np.uint16), host.scales)
+
+
+def test_device_pack_into_a_vector_that_is_too_small(bc):
+    """The C call with a sign vector one bit short, and exactly as large as needed; offsets to pageable memory."""
+    import ctypes as C
+    M, K = 96, 640
+    W, S = datagen.trits(3400, M, K, 0.4), datagen.scales(3400, M, K)
+    host = bc.bitcos_pack(W, S)
+    L = bc.load_library()
+    t, sc = torch.from_numpy(W).cuda(), torch.from_numpy(S.view(np.int16)).cuda()
+    bitmap, off = torch.empty(host.bitmap.size, dtype=torch.int32, device="cuda"), torch.empty(host.tile_off_buf.size, dtype=torch.int32, device="cuda")
+    signs, tiled = torch.empty(host.signs.size, dtype=torch.int32, device="cuda"), torch.empty(host.scales.size, dtype=torch.int16, device="cuda")
+    scratch, off_host, nnz = torch.empty(256, dtype=torch.uint8, device="cuda"), np.zeros(host.tile_off_buf.size, np.uint32), C.c_uint64(0)
+    for short, want in ((16, 6), (0, 0)):
+        rc = L.bitcos_pack_device(t.data_ptr(), sc.data_ptr(), M, K, bitmap.data_ptr(), signs.data_ptr(), host.signs.nbytes - short,
+                                  off.data_ptr(), tiled.data_ptr(), off_host.ctypes.data, C.byref(nnz), scratch.data_ptr(),
+                                  torch.cuda.current_stream().cuda_stream)
+        assert rc == want
+    assert nnz.value == host.nnz and np.array_equal(u32(signs), host.signs) and np.array_equal(off_host, host.tile_off_buf)

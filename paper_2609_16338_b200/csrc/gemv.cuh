@@ -254,12 +254,12 @@ inline Plan make_plan(int64_t M, int64_t K, int max_warps_per_block, int tpw = 1
     return p;
 }
 
-// Pairs of tiles (BITCOS, two tokens and more): a warp takes two neighbouring groups of one row block and adds their
-// sums in registers, so with whole rows per item a row block takes ceil(G / 2) warps.
-inline Plan make_pair_plan(int64_t M, int64_t K, int max_warps) {
-    Plan p = make_plan(M, K, max_warps, 2);
+// Several tiles per warp (BITCOS, two tokens and more): a warp takes tpw neighbouring groups of one row block and adds
+// their sums in registers, so with whole rows per item a row block takes ceil(G / tpw) warps.
+inline Plan make_run_plan(int64_t M, int64_t K, int max_warps, int tpw) {
+    Plan p = make_plan(M, K, max_warps, tpw);
     if (p.CS == 1) {
-        const int wr = (p.CG + 1) / 2;
+        const int wr = (p.CG + tpw - 1) / tpw;
         const int64_t RB = padded_rows(M) / kRows;
         p.RBC = max_warps / wr;
         if (p.RBC > RB) p.RBC = static_cast<int>(RB);
@@ -321,6 +321,10 @@ __host__ __device__ constexpr int64_t x_stride(int64_t K) { return K + 16; }
 // sixteen; with two tiles per warp 115, 127, 137 and 206.)
 __host__ __device__ constexpr bool fragment_order(int fmt, int nb) { return fmt == kBitcos && nb >= 2; }
 
+// Tiles per warp in large launches (wants_two_tiles): two, or three with the fourteen decoder warps of more than eight tokens, which two
+// tiles each would leave four of idle where rows have 20 or 40 groups (25600x5120 at sixteen tokens 27.1 -> 24.7 us).
+__host__ __device__ constexpr int wide_tiles(int fmt, int nb) { return fragment_order(fmt, nb) && nb > 8 ? 3 : 2; }
+
 // scr: the tensor-core path passes its rows through transposition buffers
 __host__ __device__ inline SmemLayout smem_layout(int fmt, const Plan &pl, int G, int nbmax, int64_t K, bool scr) {
     SmemLayout L{};
@@ -331,7 +335,7 @@ __host__ __device__ inline SmemLayout smem_layout(int fmt, const Plan &pl, int G
     if (fmt == kBitcos) {
         L.payload_cap = tiles * 512;
         L.sign_cap = tiles * 512 + 64;
-        L.off_cap = pl.tpw == 2 ? 192 : 128;   // the item's slice of tile_off (at most 21 or 41, + 3 + 3 words)
+        L.off_cap = pl.tpw > 1 ? 192 : 128;   // the item's slice of tile_off (at most 21 or 43, + 3 + 3 words)
     } else if (fmt == kTrit5) {
         const uint32_t WPR = (26u * static_cast<uint32_t>(G) + 3) / 4;
         // whole rows when CS == 1, else at most CG groups (+1 shared word) of one row block
@@ -358,7 +362,8 @@ __host__ __device__ inline SmemLayout smem_layout(int fmt, const Plan &pl, int G
     if (L.x_bytes && x_area < static_cast<uint32_t>(pl.NW * nbmax * kGroup)) x_area = static_cast<uint32_t>(pl.NW * nbmax * kGroup);
     off += align_up(x_area, 128);
     L.red = off;
-    off += static_cast<uint32_t>(red_slots(nbmax) / pl.tpw) * tiles * static_cast<uint32_t>(nbmax) * kRows * 4;
+    // (several tiles per warp leave one partial sum, or with rows and dp4a two in half as many slots)
+    off += static_cast<uint32_t>(red_slots(nbmax) * pl.NW * nbmax) * kRows * 4;
     L.scr = off;
     off += scr ? static_cast<uint32_t>(pl.NW) * kScrBytes : 0u;
     L.bar = off;
@@ -821,8 +826,8 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
     // per stage: {tiles | (first tile & 3) << 8, first group, first row block, first sign bit held}
     uint32_t *sign_base = reinterpret_cast<uint32_t *>(smem + L.bar + 384);
     const uint32_t bar0 = smem_addr(smem + L.bar);
-    static_assert(TPW == 1 || (TPW == 2 && (kFrag || NB < kMmaMinBatch)), "two tiles per warp: fragment order, or one or two tokens");
-    constexpr bool kPairs = kFrag && TPW == 2;                 // one partial sum per warp, not per tile
+    static_assert(TPW == 1 || kFrag || (TPW == 2 && NB < kMmaMinBatch), "several tiles per warp: fragment order, or one or two tokens");
+    constexpr bool kPairs = kFrag && TPW > 1;                  // one partial sum per warp, not per tile
     // one activation scale per token and group (applied by the decoder warps, tile by tile)
     // instead of one per token (applied by the epilogue warp to the finished sums)
     constexpr bool kXQ = Segs::kQuantize;                      // (one or two tokens only)
@@ -1234,7 +1239,7 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
                 // whole row blocks: one output per row.  The sums are formed first, the slot is
                 // handed back, and only then are the outputs stored, so that the release of the
                 // slot never waits for a global store.
-                const int nrb = r.nt / pb.G, parts = kPairs ? (pb.G + 1) / 2 : pb.G;
+                const int nrb = r.nt / pb.G, parts = kPairs ? (pb.G + TPW - 1) / TPW : pb.G;
                 for (int i = 0; i < nrb; ++i) {
                     const int64_t m = static_cast<int64_t>(r.rb0 + i) * kRows + lane;
                     float t_b[NB];
@@ -1250,7 +1255,7 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
             // one column block of row block rb0: add it to the running sum
             const bool starts = (r.cs == 0) || (k == 0);
             float t_b[NB];
-            sums(rs, 0, kPairs ? (r.nt + 1) / 2 : r.nt, t_b);
+            sums(rs, 0, kPairs ? (r.nt + TPW - 1) / TPW : r.nt, t_b);
 #pragma unroll
             for (int b = 0; b < NB; ++b) run[b] = starts ? t_b[b] : run[b] + t_b[b];
             __syncwarp();
@@ -1445,7 +1450,7 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
 #pragma unroll 1
             for (int ti = 0; ti < TPW; ++ti) {
                 const int tile = tile0 + ti;
-                if (tile >= nt || (TPW == 2 && pl.CS == 1 && g_first + ti >= pb.G)) break;
+                if (tile >= nt || (TPW > 1 && pl.CS == 1 && g_first + ti >= pb.G)) break;
                 // group: the item's first (0 when items are whole rows) + the tile's place in its row block
                 const int grp = static_cast<int>(d.y) + g_first + ti;
                 const uint8_t *xs = kXQ ? reinterpret_cast<const uint8_t *>(q_scr)
@@ -1463,7 +1468,7 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
                 // One tile per warp: everything is decoded before the first product (launches of a few items, where a
                 // block's first decode runs while it waits for its dependency).  Two tiles: product by product.
                 // (The 16-bit variant always: its decoded row would be 64 registers.)
-                constexpr bool kFused = TPW == 2 || kBlend;
+                constexpr bool kFused = TPW > 1 || kBlend;
                 if (kBlend) rows.shift_presence();
                 int e[kFused ? 1 : 4][8];
                 if (!kFused) {
@@ -2533,7 +2538,8 @@ inline bool wants_two_tiles(int fmt, int64_t items, int64_t tiles, int nb_templa
 inline int64_t tile_count(int64_t M, int64_t K) { return padded_rows(M) / kRows * (K / kGroup); }
 // The plan of such a product.
 inline Plan two_tile_plan(int fmt, int64_t M, int64_t K, int nb_template) {
-    return fragment_order(fmt, nb_template) ? make_pair_plan(M, K, decoder_warps(nb_template)) : make_plan(M, K, decoder_warps(nb_template), 2);
+    return fragment_order(fmt, nb_template) ? make_run_plan(M, K, decoder_warps(nb_template), wide_tiles(fmt, nb_template))
+                                            : make_plan(M, K, decoder_warps(nb_template), 2);
 }
 
 template <int FMT, int NB, bool XG = false, bool XQ = false, bool BL = false>
@@ -2548,7 +2554,7 @@ int launch(const Problem &pr, const Plan &pl_in, cudaStream_t stream, const uint
     const bool two = kTwo && !pr.acc_debug && wants_two_tiles(FMT, pl_in.items, tile_count(pr.M, pr.K), NB, sms);
     if constexpr (kTwo) {
         if (two) {
-            rc = prepare_kernel<gemv_kernel<FMT, NB, 2, XG, XQ, BL>>(&sms, &budget);
+            rc = prepare_kernel<gemv_kernel<FMT, NB, wide_tiles(FMT, NB), XG, XQ, BL>>(&sms, &budget);
             if (rc) return rc;
         }
     }
@@ -2569,7 +2575,7 @@ int launch(const Problem &pr, const Plan &pl_in, cudaStream_t stream, const uint
     fo.walks = 1;
     fill_first_off(fo, 0, off_host, pr, plw, grid);
     if constexpr (kTwo) {
-        if (two) return launch_pdl(gemv_kernel<FMT, NB, 2, XG, XQ, BL>, dim3(grid), (pl.NW + 2) * 32, L.total, stream, pr, plw, fo);
+        if (two) return launch_pdl(gemv_kernel<FMT, NB, wide_tiles(FMT, NB), XG, XQ, BL>, dim3(grid), (pl.NW + 2) * 32, L.total, stream, pr, plw, fo);
     }
     if constexpr (!BL) {
         if (pr.acc_debug)
@@ -2741,7 +2747,7 @@ int launch_multi(MultiArgs &ma, cudaStream_t stream, const uint32_t *const *off_
     int grids[kMaxJobs];
     const int total = plan_multi(ma, NB, sms, &two, grids);
     if (two) {
-        rc = prepare_kernel<gemv_multi_kernel<NB, 2, XQ, XG>>(&sms, &budget);
+        rc = prepare_kernel<gemv_multi_kernel<NB, wide_tiles(kBitcos, NB), XQ, XG>>(&sms, &budget);
         if (rc) return rc;
     }
     int nw = 0;
@@ -2812,7 +2818,7 @@ int launch_multi(MultiArgs &ma, cudaStream_t stream, const uint32_t *const *off_
         }
     }
     const NoFirstCopies none{0};
-    if (two) return launch_pdl(gemv_multi_kernel<NB, 2, XQ, XG>, dim3(total), (nw + 2) * 32, smem, stream, ma, fo, none);
+    if (two) return launch_pdl(gemv_multi_kernel<NB, wide_tiles(kBitcos, NB), XQ, XG>, dim3(total), (nw + 2) * 32, smem, stream, ma, fo, none);
     return launch_pdl(gemv_multi_kernel<NB, 1, XQ, XG>, dim3(total), (nw + 2) * 32, smem, stream, ma, fo, none);
 }
 

@@ -41,6 +41,7 @@
 #include <algorithm>
 #include <cstring>
 #include <mutex>
+#include <tuple>
 #include <type_traits>
 #include <utility>
 #include <vector>
@@ -2467,8 +2468,11 @@ inline void choose_walk(Plan &pl, int sms, int *grid) {
 // Launches with programmatic stream serialization, so that this kernel's prologue (barrier
 // set-up, table and first weight copies) may overlap the tail of the previous kernel in the
 // stream.  BITCOS_PDL=0 turns it off (for A/B runs).
+// (arguments of exactly the kernel's types, taken by reference: the largest are 7 KB, and every copy on the way counts
+// against launches of 2 us)
 template <typename... KArgs, typename... Args>
-int launch_pdl(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t stream, Args... args) {
+int launch_pdl(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t stream, const Args &...args) {
+    static_assert(std::is_same<std::tuple<typename std::remove_cv<KArgs>::type...>, std::tuple<Args...>>::value, "the kernel's own types");
     static const char *env = std::getenv("BITCOS_PDL");
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
@@ -2480,7 +2484,8 @@ int launch_pdl(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cu
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = (env && env[0] == '0') ? 0 : 1;
-    return check_cuda(cudaLaunchKernelEx(&cfg, kernel, args...));
+    void *pointers[] = {const_cast<void *>(static_cast<const void *>(&args))...};
+    return check_cuda(cudaLaunchKernelExC(&cfg, reinterpret_cast<const void *>(kernel), pointers));
 }
 
 // While a launch sequence is being recorded for replay (bitcos_gemv_phases_host), every value a
@@ -2501,22 +2506,30 @@ inline void fill_first_off(FirstOff &fo, int base, const uint32_t *off_host, con
         fo.walks = 0;
         return;
     }
-    for (int b = 0; b < grid; ++b) {
-        const Walk wk = make_walk(pl, b, grid);
-        fo.first[base + b] = wk.first;
-        fo.count[base + b] = wk.count;
-    }
     if (!off_host) fo.valid = 0;
-    if (!fo.valid) return;
-    for (int b = 0; b < grid; ++b) {
-        const Walk wk = make_walk(pl, b, grid);
-        fo.lo[base + b] = fo.hi[base + b] = 0;
-        if (wk.count <= 0) continue;
-        ItemIter it;
-        it.init(pl, wk.first);
-        const ItemRange r = item_range(pr, pl, it.c, it.cs);
-        fo.lo[base + b] = host_offset(off_host, r.t0);
-        fo.hi[base + b] = host_offset(off_host, r.t0 + r.nt);
+    // (make_walk for every block, with its divisions once: 148 blocks took 3 us of the caller's time)
+    const int items = static_cast<int>(pl.items), units = pl.cyclic ? items / pl.CS : items;
+    const int q = units / grid, rem = units - q * grid;
+    for (int b = 0, first = 0; b < grid; ++b) {
+        const int count = q + (b < rem ? 1 : 0);
+        fo.first[base + b] = pl.cyclic ? b * pl.CS : first;
+        fo.count[base + b] = pl.cyclic ? count * pl.CS : count;
+        if (fo.valid) {
+            fo.lo[base + b] = fo.hi[base + b] = 0;
+            if (count > 0) {
+                ItemIter it;
+                if (pl.cyclic) {
+                    it.c = b;
+                    it.cs = 0;
+                } else {
+                    it.init(pl, first);
+                }
+                const ItemRange r = item_range(pr, pl, it.c, it.cs);
+                fo.lo[base + b] = host_offset(off_host, r.t0);
+                fo.hi[base + b] = host_offset(off_host, r.t0 + r.nt);
+            }
+        }
+        first += count;
     }
 }
 

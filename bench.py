@@ -797,7 +797,7 @@ def batch_detail(bc, torch, stream, M=8192, K=5120, z=0.4711):
         x, xs = datagen.activations(seed, B, K)
         xd, xsd = torch.from_numpy(x).cuda(), torch.from_numpy(xs).cuda()
         y = torch.empty((B, M), dtype=torch.float32, device="cuda")
-        row = {"batch": B, "contraction": "dp4a" if B < 4 else "mma.m16n8k32.s8"}
+        row = {"batch": B, "contraction": {"bitcos": "dp4a" if B < 2 else "mma.m16n8k32.s8", "baselines": "dp4a" if B < 3 else "mma.m16n8k32.s8"}}
         for name, (Wd, f) in fmts.items():
             n_copies = max(2, int(np.ceil(4.2 * L2_BYTES / Wd.payload_bytes())))
             reps = [Wd] + [Wd.clone() for _ in range(n_copies - 1)]

@@ -2,7 +2,7 @@
 
 Two tiles per warp are taken from 64 tiles per multiprocessor on.  The shapes lie on both sides of that line and where
 the pairing can go wrong: an odd number of groups (the last warp of a row block has one tile), a single group, rows cut
-into column blocks of odd width, a ragged last row block.  Against the oracle, within the task's 1e-5 of sum|terms|.
+into column blocks of odd width, a ragged last row block.  Against the oracle, within 1e-5 of sum|terms|.
 """
 import numpy as np
 import pytest

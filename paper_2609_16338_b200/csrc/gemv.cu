@@ -893,8 +893,12 @@ int host_step_enqueue(const bitcos_gemv_job *jobs, const int *job_phase, int n_j
     }
     if (rc) return rc;
     // the outputs already on their way, as [begin, end) offsets of the block
-    std::vector<std::pair<size_t, size_t>> sent;
-    int forks = 0;
+    std::pair<size_t, size_t> sent[kMaxJobs];
+    int n_sent = 0, forks = 0;
+    auto output_range = [&](int j) {
+        const size_t off = static_cast<size_t>(reinterpret_cast<const uint8_t *>(jobs[j].y) - static_cast<const uint8_t *>(out_device));
+        return std::pair<size_t, size_t>(off, off + static_cast<size_t>(batch) * static_cast<size_t>(jobs[j].W->M) * sizeof(float));
+    };
     const bitcos_weights *w[kMaxJobs];
     for (int j = 0; j < n_jobs; ++j) w[j] = jobs[j].W;
     int prev_first = 0, prev_n = 0;
@@ -906,20 +910,28 @@ int host_step_enqueue(const bitcos_gemv_job *jobs, const int *job_phase, int n_j
         rc = bitcos_gemv_multi_chained(jobs + first, last - first + 1, batch, w + prev_first, prev_n, w + last + 1, next_n, stream);
         if (rc) return rc;
         if (rec && last + 1 < n_jobs && forks < BITCOS_MAX_PHASES) {
-            // this phase's outputs go out beside the phases that follow
+            // this phase's outputs go out beside the phases that follow, those that a later job writes over excepted
+            // (what the caller gets is the block after the last phase)
             CopyPieces out{static_cast<const uint8_t *>(out_device), static_cast<uint8_t *>(rec->out_mapped), 0, {}, {}};
             for (int j = first; j <= last; ++j) {
-                const size_t off = static_cast<size_t>(reinterpret_cast<const uint8_t *>(jobs[j].y) - static_cast<const uint8_t *>(out_device));
-                const size_t bytes = static_cast<size_t>(batch) * static_cast<size_t>(jobs[j].W->M) * sizeof(float);
-                out.off[out.n] = off;
-                out.bytes[out.n++] = bytes;
-                sent.emplace_back(off, off + bytes);
+                const std::pair<size_t, size_t> r = output_range(j);
+                bool final = true;
+                for (int i = last + 1; i < n_jobs; ++i) {
+                    const std::pair<size_t, size_t> later = output_range(i);
+                    final = final && (later.second <= r.first || r.second <= later.first);
+                }
+                if (!final) continue;
+                out.off[out.n] = r.first;
+                out.bytes[out.n++] = r.second - r.first;
+                sent[n_sent++] = r;
             }
-            rc = check_cuda(cudaEventRecord(rec->event[forks], stream));
-            if (!rc) rc = check_cuda(cudaStreamWaitEvent(rec->side, rec->event[forks], 0));
-            if (!rc) rc = launch_copy(out, rec->side);
-            if (rc) return rc;
-            ++forks;
+            if (out.n) {
+                rc = check_cuda(cudaEventRecord(rec->event[forks], stream));
+                if (!rc) rc = check_cuda(cudaStreamWaitEvent(rec->side, rec->event[forks], 0));
+                if (!rc) rc = launch_copy(out, rec->side);
+                if (rc) return rc;
+                ++forks;
+            }
         }
         prev_first = first;
         prev_n = last - first + 1;
@@ -927,16 +939,16 @@ int host_step_enqueue(const bitcos_gemv_job *jobs, const int *job_phase, int n_j
     }
     if (rec) {
         // everything that is not on its way yet: the last phase's outputs, and whatever else the block holds
-        std::sort(sent.begin(), sent.end());
+        std::sort(sent, sent + n_sent);
         CopyPieces out{static_cast<const uint8_t *>(out_device), static_cast<uint8_t *>(rec->out_mapped), 0, {}, {}};
         size_t at = 0;
-        for (size_t i = 0; i <= sent.size(); ++i) {
-            const size_t end = i < sent.size() ? sent[i].first : out_bytes;
+        for (int i = 0; i <= n_sent; ++i) {
+            const size_t end = i < n_sent ? sent[i].first : out_bytes;
             if (end > at) {
                 out.off[out.n] = at;
                 out.bytes[out.n++] = end - at;
             }
-            if (i < sent.size() && sent[i].second > at) at = sent[i].second;
+            if (i < n_sent && sent[i].second > at) at = sent[i].second;
         }
         rc = launch_copy(out, stream);
         if (!rc && forks) rc = check_cuda(cudaEventRecord(rec->event[BITCOS_MAX_PHASES], rec->side));

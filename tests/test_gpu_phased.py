@@ -183,6 +183,31 @@ def test_recorded_host_step_follows_weights_repacked_in_place(bc):
     check("weights repacked in place")
 
 
+def test_phases_that_write_the_same_outputs(bc):
+    """Jobs of different phases may share a range of the output block (a buffer used again): the caller gets the block
+    as the last phase left it, on the first call (direct), the second (recorded) and the replays alike."""
+    B = 1
+    shapes = [(640, 2560), (320, 1280), (100, 512), (64, 384)]
+    first_float = [0, 160, 600, 200]          # phase 1 inside phase 0, phase 2 over its end, phase 3 inside phases 0 and 1
+    Wh = [datagen.trits(4700 + i, M, K, 0.4219) for i, (M, K) in enumerate(shapes)]
+    Sh = [datagen.scales(4700 + i, M, K) for i, (M, K) in enumerate(shapes)]
+    devs = [bc.bitcos_pack(W, S).to_device() for W, S in zip(Wh, Sh)]
+    hp = bc.HostPhases([(d, bc.make_workspace(M, K)) for d, (M, K) in zip(devs, shapes)], [0, 1, 2, 3], batch=B)
+    for job, f in zip(hp.arr, first_float):
+        job.y = hp.out_dev.data_ptr() + 4 * f
+    out = hp.out_host.numpy().view(np.float32)
+    for rep in range(5):
+        y_ref, mag = np.zeros(out.size), np.zeros(out.size)
+        for i, (M, K) in enumerate(shapes):
+            x, xs = datagen.activations(4700 + 10 * rep + i, B, K)
+            hp.x[i][:] = x
+            hp.x_scale[i][:] = xs
+            _, y_ref[first_float[i]:first_float[i] + M], mag[first_float[i]:first_float[i] + M] = oracle.gemv_dense(Wh[i], Sh[i], x, xs)
+        hp.run()
+        err = np.abs(out.astype(np.float64) - y_ref)
+        assert (err <= REL * mag).all(), (rep, np.flatnonzero(err > REL * mag)[:8])
+
+
 def test_host_steps_from_two_threads(bc):
     """bitcos_gemv_phases_host from two host threads at once, each with its own matrices, blocks and stream (the
     records of seen steps are shared between threads, recording happens on one stream of the library's own)."""

@@ -468,7 +468,10 @@ int bitcos_gemv_multi_host(const bitcos_gemv_host_job *jobs, int n_jobs, int bat
  * compares them with the host arrays' current contents and falls back to enqueueing directly if
  * they differ, so matrices re-packed into the same buffers are handled; the packed arrays in device
  * memory are read when the kernels run and may change freely.  Up to 64 argument sets are kept
- * (least recently used replaced).  Pageable host blocks are never recorded.  Thread safe.
+ * (least recently used replaced).  Pageable host blocks are never recorded, and a block that is no
+ * longer pinned and mapped where it was when the step was recorded (unregistered, freed) is noticed
+ * before the replay: that call enqueues directly.  Both blocks have to stay valid until the call
+ * returns.  Thread safe.
  * ERR_CAPACITY if a job's x, x_scale or y lies outside its block.  The paper has no counterpart (it
  * measures resident activations). */
 int bitcos_gemv_phases_host(const bitcos_gemv_job *jobs, const int *job_phase, int n_jobs, int batch, const void *in_host,

@@ -4,6 +4,8 @@
 #include "gemv.cuh"
 #include "gemv_inst.cuh"
 
+#include <cuda.h>
+
 namespace {
 
 using namespace bitcos_kernels;
@@ -332,7 +334,39 @@ __global__ void __launch_bounds__(kQuantThreads) quantize_tokens_kernel(const ui
 
 namespace bitcos_detail {
 // for the library's other translation units: the error bitcos_last_cuda_error reports
-void record_cuda_error(int e) { g_last_cuda_error = e; }
+void record_cuda_error(int e) { bitcos_kernels::g_last_cuda_error = e; }
+
+// Where a kernel finds the host memory [p, p + bytes): its device address if all of it lies in one pinned allocation (or
+// one registered range) that is mapped into the device, else NULL.  Asked before every launch that is going to touch host
+// memory, because a range that was mapped at an earlier call may have been unregistered or freed since
+// (0.2 us a call: one driver call without a lock on the stream).
+void *mapped_host(const void *p, size_t bytes) {
+    typedef CUresult (*Attributes)(unsigned int, CUpointer_attribute *, void **, CUdeviceptr);
+    static const Attributes attributes = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 7000, cudaEnableDefault, &found) != cudaSuccess ||
+            found != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return reinterpret_cast<Attributes>(f);
+    }();
+    if (!attributes) return nullptr;
+    CUpointer_attribute ask[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                 CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    unsigned int type = 0, managed = 0;
+    CUdeviceptr at = 0, start = 0;
+    size_t size = 0;
+    void *answers[] = {&type, &managed, &at, &start, &size};
+    if (attributes(5, ask, answers, reinterpret_cast<CUdeviceptr>(p)) != CUDA_SUCCESS || type != CU_MEMORYTYPE_HOST || (managed & 0xFFu) || !at)
+        return nullptr;
+    // (the range is given at the address asked for, host and device addresses being the same ones, or at the mapped one)
+    const CUdeviceptr host = reinterpret_cast<CUdeviceptr>(p);
+    const CUdeviceptr in = host >= start && host - start < size ? host : at;
+    if (in < start || in - start > size || bytes > size - (in - start)) return nullptr;
+    return reinterpret_cast<void *>(at);
+}
 }  // namespace bitcos_detail
 
 extern "C" {
@@ -960,8 +994,8 @@ int host_step_enqueue(const bitcos_gemv_job *jobs, const int *job_phase, int n_j
 
 // Recorded steps.  A record is keyed by everything the enqueued work depends on, by value: the job
 // list, the descriptors behind it, the blocks and their sizes, the device; and it remembers every
-// entry offset its plans took from the host copies of tile_off, which a replay compares with what
-// is there now (packed arrays in device memory may change freely between calls: the kernels read
+// entry offset its plans took from the host copies of tile_off and where the host blocks were mapped, which a
+// replay compares with what is there now (packed arrays in device memory may change freely between calls: the kernels read
 // them when they run).  Anything that does not match is simply enqueued directly.
 struct alignas(8) HostStepKey {
     int n_jobs, batch, device, pad;
@@ -978,6 +1012,8 @@ struct HostStepRecord {
     std::vector<std::pair<const uint32_t *, uint32_t>> offsets;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
+    const void *in_mapped = nullptr;      // the host blocks as the record's copies address them
+    void *out_mapped = nullptr;
     uint64_t last_use = 0;
     int seen = 0;          // calls with this key so far
     bool failed = false;   // recording did not work for this key: never tried again
@@ -1045,28 +1081,26 @@ bool host_step_replay(const bitcos_gemv_job *jobs, const int *job_phase, int n_j
     }
     rec->last_use = ++g_host_steps_clock;
     if (rec->failed) return false;
+    const void *in_mapped = bitcos_detail::mapped_host(in_host, in_bytes);
+    void *out_mapped = bitcos_detail::mapped_host(out_host, out_bytes);
     if (rec->exec) {
-        for (const auto &o : rec->offsets)
-            if (*o.first != o.second) {        // the host copy of the entry offsets changed under the same descriptor
-                cudaGraphExecDestroy(rec->exec);
-                cudaGraphDestroy(rec->graph);
-                rec->exec = nullptr;
-                rec->graph = nullptr;
-                rec->offsets.clear();
-                rec->seen = 1;
-                return false;
-            }
+        // the host blocks where the record's copies expect them, the entry offsets as its plans took them
+        bool stale = in_mapped != rec->in_mapped || out_mapped != rec->out_mapped;
+        for (size_t i = 0; !stale && i < rec->offsets.size(); ++i) stale = *rec->offsets[i].first != rec->offsets[i].second;
+        if (stale) {
+            cudaGraphExecDestroy(rec->exec);
+            cudaGraphDestroy(rec->graph);
+            rec->exec = nullptr;
+            rec->graph = nullptr;
+            rec->offsets.clear();
+            rec->seen = 1;
+            return false;
+        }
         return cudaGraphLaunch(rec->exec, stream) == cudaSuccess;
     }
     // second sight: record the step on a stream of the library's own (nothing runs), then replay it
     ++rec->seen;
-    cudaPointerAttributes ai{}, ao{};
-    if (cudaPointerGetAttributes(&ai, in_host) != cudaSuccess || cudaPointerGetAttributes(&ao, out_host) != cudaSuccess ||
-        ai.type != cudaMemoryTypeHost || ao.type != cudaMemoryTypeHost || !ai.devicePointer || !ao.devicePointer) {
-        cudaGetLastError();
-        rec->failed = true;       // pageable host blocks: their copies are not recorded
-        return false;
-    }
+    if (!in_mapped || !out_mapped) return false;       // pageable host blocks: their copies are not recorded
     if (!g_record_stream) {
         bool ok = cudaStreamCreateWithFlags(&g_recorded_copies.side, cudaStreamNonBlocking) == cudaSuccess;
         for (cudaEvent_t &e : g_recorded_copies.event) ok = ok && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess;
@@ -1078,8 +1112,8 @@ bool host_step_replay(const bitcos_gemv_job *jobs, const int *job_phase, int n_j
             return false;
         }
     }
-    g_recorded_copies.in_mapped = ai.devicePointer;
-    g_recorded_copies.out_mapped = ao.devicePointer;
+    g_recorded_copies.in_mapped = rec->in_mapped = in_mapped;
+    g_recorded_copies.out_mapped = rec->out_mapped = out_mapped;
     if (cudaStreamBeginCapture(g_record_stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
         cudaGetLastError();
         rec->failed = true;

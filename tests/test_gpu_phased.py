@@ -208,6 +208,52 @@ def test_phases_that_write_the_same_outputs(bc):
         assert (err <= REL * mag).all(), (rep, np.flatnonzero(err > REL * mag)[:8])
 
 
+def test_host_blocks_that_are_pinned_for_some_calls_only(bc):
+    """A recorded step addresses the host blocks where they were mapped when it was recorded.  With the same addresses
+    unregistered, registered again and registered for another size, every call still returns its own product: what is not mapped as a
+    whole at the time of the call is copied, not read or written by a kernel."""
+    import mmap
+    B = 1
+    shapes = [(1600, 2560), (320, 1280)]
+    Wh = [datagen.trits(4800 + i, M, K, 0.4219) for i, (M, K) in enumerate(shapes)]
+    Sh = [datagen.scales(4800 + i, M, K) for i, (M, K) in enumerate(shapes)]
+    devs = [bc.bitcos_pack(W, S).to_device() for W, S in zip(Wh, Sh)]
+    hp = bc.HostPhases([(d, bc.make_workspace(M, K)) for d, (M, K) in zip(devs, shapes)], [0, 1], batch=B)
+    rt = torch.cuda.cudart()
+    pages = 2 * mmap.PAGESIZE
+    assert hp.in_bytes <= pages // 2 < hp.out_bytes <= pages
+    blocks = {name: np.frombuffer(mmap.mmap(-1, pages), dtype=np.uint8) for name in ("in", "out")}
+    hp.in_host, hp.out_host = (torch.from_numpy(blocks[n]) for n in ("in", "out"))
+    mapped = {}
+
+    def pin(name, size):
+        if mapped.pop(name, 0):
+            assert int(rt.cudaHostUnregister(blocks[name].ctypes.data)) == 0
+        if size:
+            assert int(rt.cudaHostRegister(blocks[name].ctypes.data, size, 0)) == 0
+            mapped[name] = size
+
+    rep = 0
+    for in_size, out_size in ((pages, pages), (0, pages), (pages, pages), (pages, 0), (pages, pages), (pages // 2, pages), (0, 0)):
+        pin("in", in_size)
+        pin("out", out_size)
+        for _ in range(3):
+            rep += 1
+            refs = []
+            for i, (M, K) in enumerate(shapes):
+                x, xs = datagen.activations(4800 + 10 * rep + i, B, K)
+                blocks["in"][hp.x_off[i]:hp.x_off[i] + B * K] = x.reshape(-1).view(np.uint8)
+                blocks["in"][hp.xs_off[i]:hp.xs_off[i] + 4 * B] = xs.view(np.uint8)
+                refs.append(oracle.gemv_dense(Wh[i], Sh[i], x, xs))
+            blocks["out"][:] = 0xFF
+            hp.run()
+            for i, (_, y_ref, mag) in enumerate(refs):
+                y = blocks["out"][hp.y_off[i]:hp.y_off[i] + 4 * B * shapes[i][0]].view(np.float32).reshape(B, -1)
+                assert (np.abs(y.astype(np.float64) - y_ref) <= REL * mag).all(), (in_size, out_size, rep, i)
+    pin("in", 0)
+    pin("out", 0)
+
+
 def test_host_steps_from_two_threads(bc):
     """bitcos_gemv_phases_host from two host threads at once, each with its own matrices, blocks and stream (the
     records of seen steps are shared between threads, recording happens on one stream of the library's own)."""

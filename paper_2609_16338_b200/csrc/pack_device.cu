@@ -23,6 +23,7 @@
 
 namespace bitcos_detail {
 void record_cuda_error(int e);      // defined next to bitcos_last_cuda_error
+void *mapped_host(const void *p, size_t bytes);
 }
 
 namespace {
@@ -40,6 +41,7 @@ constexpr int kNnzLo = 4;           // 64-bit count of non-zero weights (two wor
 inline int check_cuda(cudaError_t e) {
     if (e == cudaSuccess) return BITCOS_OK;
     bitcos_detail::record_cuda_error(static_cast<int>(e));
+    cudaGetLastError();                 // (or the next call's launch check would find this one's error)
     return BITCOS_ERR_CUDA;
 }
 inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -431,15 +433,9 @@ int bitcos_pack_device(const int8_t *trits, const uint16_t *scales_bf16, int64_t
     unsigned long long max_nnz = 0;
     if (sign_capacity_bytes >= slack) max_nnz = static_cast<unsigned long long>((sign_capacity_bytes - slack) / 16 * 16) * 8;
     unsigned int *flags = static_cast<unsigned int *>(scratch);
-    // the host's copy of the offsets, if the device can write there
-    uint32_t *off_mapped = nullptr;
-    if (tile_off_host) {
-        cudaPointerAttributes at{};
-        if (cudaPointerGetAttributes(&at, tile_off_host) == cudaSuccess && at.type == cudaMemoryTypeHost && at.devicePointer && aligned16(at.devicePointer))
-            off_mapped = static_cast<uint32_t *>(at.devicePointer);
-        else
-            cudaGetLastError();
-    }
+    // the host's copy of the offsets, if the device can write there (all of it: else it is copied)
+    uint32_t *off_mapped = tile_off_host ? static_cast<uint32_t *>(bitcos_detail::mapped_host(tile_off_host, off_bytes)) : nullptr;
+    if (!aligned16(off_mapped)) off_mapped = nullptr;
     const int64_t grid = (n_tiles + kPackWarps - 1) / kPackWarps;
     if (grid > 0x7FFFFFFF) return BITCOS_ERR_SHAPE;
     const ReportSlot report;

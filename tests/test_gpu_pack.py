@@ -123,3 +123,34 @@ def test_device_pack_into_a_vector_that_is_too_small(bc):
                                   torch.cuda.current_stream().cuda_stream)
         assert rc == want
     assert nnz.value == host.nnz and np.array_equal(u32(signs), host.signs) and np.array_equal(off_host, host.tile_off_buf)
+
+
+def test_device_pack_with_offsets_to_memory_that_is_pinned_in_part(bc):
+    """The offsets go to the host by the packer's own stores only where all of the caller's buffer is mapped; a buffer of
+    which one page is registered is left to the runtime's copy, which refuses it."""
+    import ctypes as C
+    import mmap
+    M, K = 25600, 5120
+    L = bc.load_library()
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    t = torch.randint(-1, 2, (M, K), generator=gen, device="cuda", dtype=torch.int8)
+    sc = torch.full((M, K // 128), 0.5, device="cuda").to(torch.bfloat16)
+    want = bc.bitcos_pack_device(t, sc)
+    signs, off = torch.empty(M * K // 32 + 64, dtype=torch.int32, device="cuda"), torch.empty_like(want.tile_off)
+    bitmap, tiled = torch.empty_like(want.bitmap), torch.empty_like(want.scales)
+    scratch = torch.empty(256, dtype=torch.uint8, device="cuda")
+    size = -(-4 * off.numel() // mmap.PAGESIZE) * mmap.PAGESIZE
+    host = np.frombuffer(mmap.mmap(-1, size), dtype=np.uint32)
+    rt = torch.cuda.cudart()
+    for pinned, status in ((size, 0), (mmap.PAGESIZE, 8), (0, 0)):
+        if pinned:
+            assert int(rt.cudaHostRegister(host.ctypes.data, pinned, 0)) == 0
+        host[:] = 0xFFFFFFFF
+        rc = L.bitcos_pack_device(t.data_ptr(), sc.data_ptr(), M, K, bitmap.data_ptr(), signs.data_ptr(), 4 * signs.numel(), off.data_ptr(),
+                                  tiled.data_ptr(), host.ctypes.data, None, scratch.data_ptr(), torch.cuda.current_stream().cuda_stream)
+        assert rc == status, pinned
+        if status == 0:
+            assert np.array_equal(host[:off.numel()].view(np.int32), want.tile_off.cpu().numpy()), pinned
+            assert torch.equal(off, want.tile_off) and torch.equal(bitmap, want.bitmap), pinned
+        if pinned:
+            assert int(rt.cudaHostUnregister(host.ctypes.data)) == 0

@@ -444,20 +444,25 @@ int bitcos_pack_device(const int8_t *trits, const uint16_t *scales_bf16, int64_t
         rc = check_cuda(cudaHostGetDevicePointer(reinterpret_cast<void **>(&report_dev), report.host(), 0));
         if (rc) return rc;
     }
-    pack_bitmap_kernel<<<static_cast<unsigned>(grid), kPackWarps * 32, 0, stream>>>(
-        trits, scales_bf16, M, K, reinterpret_cast<uint16_t *>(bitmap), scales_tiled, tile_off, n_tiles, reinterpret_cast<uint4 *>(signs),
-        static_cast<int64_t>(sign_capacity_bytes / 16));
-    rc = check_cuda(cudaGetLastError());
-    if (rc) return rc;
-    rc = launch_behind(scan_counts_kernel, 1, kScanThreads, stream, tile_off, off_mapped, n_tiles, static_cast<int64_t>(off_bytes / 4), flags,
-                       static_cast<volatile unsigned int *>(report_dev));
-    if (rc) return rc;
-    rc = launch_behind(pack_signs_kernel, grid, kPackWarps * 32, stream, trits, M, K, static_cast<const uint32_t *>(tile_off), signs, max_nnz,
-                       n_tiles, static_cast<const unsigned int *>(flags));
-    if (rc) return rc;
-    if (tile_off_host && !off_mapped) {
-        rc = check_cuda(cudaMemcpyAsync(tile_off_host, tile_off, off_bytes, cudaMemcpyDeviceToHost, stream));
-        if (rc) return rc;
+    auto enqueue = [&]() -> int {
+        pack_bitmap_kernel<<<static_cast<unsigned>(grid), kPackWarps * 32, 0, stream>>>(
+            trits, scales_bf16, M, K, reinterpret_cast<uint16_t *>(bitmap), scales_tiled, tile_off, n_tiles, reinterpret_cast<uint4 *>(signs),
+            static_cast<int64_t>(sign_capacity_bytes / 16));
+        int e = check_cuda(cudaGetLastError());
+        if (!e)
+            e = launch_behind(scan_counts_kernel, 1, kScanThreads, stream, tile_off, off_mapped, n_tiles, static_cast<int64_t>(off_bytes / 4),
+                              flags, static_cast<volatile unsigned int *>(report_dev));
+        if (!e)
+            e = launch_behind(pack_signs_kernel, grid, kPackWarps * 32, stream, trits, M, K, static_cast<const uint32_t *>(tile_off), signs,
+                              max_nnz, n_tiles, static_cast<const unsigned int *>(flags));
+        if (!e && tile_off_host && !off_mapped)
+            e = check_cuda(cudaMemcpyAsync(tile_off_host, tile_off, off_bytes, cudaMemcpyDeviceToHost, stream));
+        return e;
+    };
+    rc = enqueue();
+    if (rc) {
+        cudaStreamSynchronize(stream);               // what was enqueued writes the report's slot and the caller's buffers
+        return rc;
     }
     unsigned int h[8];
     if (report.host()) {

@@ -149,6 +149,8 @@ def test_device_pack_with_offsets_to_memory_that_is_pinned_in_part(bc):
         rc = L.bitcos_pack_device(t.data_ptr(), sc.data_ptr(), M, K, bitmap.data_ptr(), signs.data_ptr(), 4 * signs.numel(), off.data_ptr(),
                                   tiled.data_ptr(), host.ctypes.data, None, scratch.data_ptr(), torch.cuda.current_stream().cuda_stream)
         assert rc == status, pinned
+        # (whatever happened, nothing of the call is still running)
+        assert torch.cuda.current_stream().query(), pinned
         if status == 0:
             assert np.array_equal(host[:off.numel()].view(np.int32), want.tile_off.cpu().numpy()), pinned
             assert torch.equal(off, want.tile_off) and torch.equal(bitmap, want.bitmap), pinned

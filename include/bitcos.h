@@ -50,6 +50,9 @@
 #ifdef __cplusplus
 extern "C" {
 #endif
+#ifdef __GNUC__
+#pragma GCC visibility push(default)
+#endif
 
 #define BITCOS_GROUP 128
 #define BITCOS_TILE_ROWS 32
@@ -552,6 +555,9 @@ int bit2_gemv_grouped(const bitcos_weights *experts, int n_experts, int64_t M, i
                       int max_group_size, const int8_t *x, int n_xrows, const float *x_scale, float *y,
                       int32_t *acc_debug, void *workspace, size_t workspace_bytes, void *cuda_stream);
 
+#ifdef __GNUC__
+#pragma GCC visibility pop
+#endif
 #ifdef __cplusplus
 }
 #endif

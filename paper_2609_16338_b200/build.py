@@ -23,8 +23,10 @@ HEADERS = [INST, *(os.path.join(CSRC, h) for h in ("gemv.cuh", "gemv_inst.cuh", 
 
 
 def nvcc_flags():
+    # (only what bitcos.h declares is exported: the statics of inline functions would otherwise be one object for every copy
+    # of the library in a process, and a second copy would find the first one's kernels set up)
     return ["-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "--compress-mode=size",
-            "-I" + os.path.join(ROOT, "include"), "-Xcompiler", "-fPIC,-fopenmp,-O2"]
+            "-I" + os.path.join(ROOT, "include"), "-Xcompiler", "-fPIC,-fopenmp,-O2,-fvisibility=hidden"]
 
 
 def compile_library(out, extra=()):

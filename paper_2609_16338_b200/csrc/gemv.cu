@@ -678,7 +678,7 @@ int bitcos_gemv_phased(const bitcos_gemv_job *jobs, const int *job_phase, int n_
 
 #ifdef BITCOS_TIMELINE
 // Debug build only: device buffer of slots x 160 blocks x 16 stamps; every multi launch takes the next slot.
-void bitcos_debug_timeline(unsigned long long *buf, int slots) {
+__attribute__((visibility("default"))) void bitcos_debug_timeline(unsigned long long *buf, int slots) {
     g_tl_buf = buf;
     g_tl_slots = slots;
     g_tl_next = 0;

@@ -36,6 +36,16 @@ def test_library_exports_every_declared_symbol():
     assert sorted(bc.EXPORTED_SYMBOLS) == names
 
 
+def test_library_exports_nothing_else():
+    """Two copies of the library in one process must not share state: no kernel, no template and above all no symbol of
+    the kind that the loader makes unique in the process (the statics of inline functions) is visible outside."""
+    import subprocess
+    table = subprocess.run(["nm", "-D", "--defined-only", bc.library_path()], check=True, capture_output=True, text=True).stdout
+    symbols = [line.split()[-2:] for line in table.splitlines()]
+    assert sorted(name for kind, name in symbols if kind == "T") == declared_functions()
+    assert not [name for kind, name in symbols if kind in "uVBDR" or "bitcos_kernels" in name]
+
+
 @pytest.mark.parametrize("M,K,z", [(256, 512, 0.42), (32, 128, 0.3), (100, 384, 0.47), (1, 128, 0.5), (640, 256, 0.33)])
 def test_bitcos_pack_matches_oracle_bytes(M, K, z):
     W = datagen.trits(31, M, K, z)

@@ -2005,7 +2005,8 @@ __device__ __forceinline__ void run_problem(const Problem &pr, const Plan &pl, u
 }
 
 // (DEBUG: the instantiation that also dumps the int32 accumulators.  The dump's addresses cost registers on the tile
-// loop whether it is asked for or not, so calls without it run a kernel that has no such code.)
+// loop whether it is asked for or not, so calls without it run a kernel that has no such code; the plan, and with it the
+// order of the sums, is the same.)
 template <int FMT, int NB, int TPW = 1, bool XG = false, bool XQ = false, bool BL = false, bool DEBUG = false>
 __global__ void __launch_bounds__(max_block_threads(NB), 1) gemv_kernel(const Problem pr, const Plan pl,
                                                                         const __grid_constant__ FirstOff fo) {
@@ -2555,6 +2556,14 @@ inline Plan two_tile_plan(int fmt, int64_t M, int64_t K, int nb_template) {
                                             : make_plan(M, K, decoder_warps(nb_template), 2);
 }
 
+// A launch of one product's kernel (set up for large shared memory on its first use).
+template <auto kernel>
+int launch_single(const Problem &pr, const Plan &plw, const FirstOff &fo, int grid, uint32_t smem, cudaStream_t stream) {
+    int sms = 0, budget = 0;
+    const int rc = prepare_kernel<kernel>(&sms, &budget);
+    return rc ? rc : launch_pdl(kernel, dim3(grid), (plw.NW + 2) * 32, smem, stream, pr, plw, fo);
+}
+
 template <int FMT, int NB, bool XG = false, bool XQ = false, bool BL = false>
 int launch(const Problem &pr, const Plan &pl_in, cudaStream_t stream, const uint32_t *off_host = nullptr) {
     // the one- and two-token instantiations keep the activations in shared memory (nb_bucket sees to it)
@@ -2564,19 +2573,8 @@ int launch(const Problem &pr, const Plan &pl_in, cudaStream_t stream, const uint
     int sms = 0, budget = 0;
     int rc = prepare_kernel<gemv_kernel<FMT, NB, 1, XG, XQ, BL>>(&sms, &budget);
     if (rc) return rc;
-    const bool two = kTwo && !pr.acc_debug && wants_two_tiles(FMT, pl_in.items, tile_count(pr.M, pr.K), NB, sms);
-    if constexpr (kTwo) {
-        if (two) {
-            rc = prepare_kernel<gemv_kernel<FMT, NB, wide_tiles(FMT, NB), XG, XQ, BL>>(&sms, &budget);
-            if (rc) return rc;
-        }
-    }
-    if constexpr (!BL) {
-        if (pr.acc_debug) {
-            rc = prepare_kernel<gemv_kernel<FMT, NB, 1, XG, XQ, false, true>>(&sms, &budget);
-            if (rc) return rc;
-        }
-    }
+    // (with and without the accumulator dump: the same plan, so the same order of the sums)
+    const bool two = kTwo && wants_two_tiles(FMT, pl_in.items, tile_count(pr.M, pr.K), NB, sms);
     const Plan pl = two ? two_tile_plan(FMT, pr.M, pr.K, NB) : pl_in;
     int grid = 1;
     Plan plw = pl;
@@ -2588,11 +2586,14 @@ int launch(const Problem &pr, const Plan &pl_in, cudaStream_t stream, const uint
     fo.walks = 1;
     fill_first_off(fo, 0, off_host, pr, plw, grid);
     if constexpr (kTwo) {
-        if (two) return launch_pdl(gemv_kernel<FMT, NB, wide_tiles(FMT, NB), XG, XQ, BL>, dim3(grid), (pl.NW + 2) * 32, L.total, stream, pr, plw, fo);
+        constexpr int kWide = wide_tiles(FMT, NB);
+        if constexpr (!BL) {
+            if (two && pr.acc_debug) return launch_single<gemv_kernel<FMT, NB, kWide, XG, XQ, false, true>>(pr, plw, fo, grid, L.total, stream);
+        }
+        if (two) return launch_single<gemv_kernel<FMT, NB, kWide, XG, XQ, BL>>(pr, plw, fo, grid, L.total, stream);
     }
     if constexpr (!BL) {
-        if (pr.acc_debug)
-            return launch_pdl(gemv_kernel<FMT, NB, 1, XG, XQ, false, true>, dim3(grid), (pl.NW + 2) * 32, L.total, stream, pr, plw, fo);
+        if (pr.acc_debug) return launch_single<gemv_kernel<FMT, NB, 1, XG, XQ, false, true>>(pr, plw, fo, grid, L.total, stream);
     }
     return launch_pdl(gemv_kernel<FMT, NB, 1, XG, XQ, BL>, dim3(grid), (pl.NW + 2) * 32, L.total, stream, pr, plw, fo);
 }

@@ -305,7 +305,8 @@ int bitcos_gemv_blend_bf16(const bitcos_weights *W, const uint16_t *x_bf16, int 
  * their sizes, so small matrices run side by side instead of one after the other and the fixed
  * cost of a launch is paid once.  Every job has its own outputs and its own workspace (sized and
  * zero filled as for bitcos_gemv; two jobs must not share one).  Results are identical to
- * n_jobs calls of bitcos_gemv. */
+ * n_jobs calls of bitcos_gemv: bit for bit for K <= 2560 at one token and K <= 5120 from two on (longer
+ * rows may be cut between thread blocks at other places, which can change the last bits of their sums). */
 typedef struct bitcos_gemv_job {
     const bitcos_weights *W;   /* host struct of device pointers */
     const int8_t *x;           /* device int8 [batch][K] */

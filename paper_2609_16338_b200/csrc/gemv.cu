@@ -259,7 +259,7 @@ int gemv_common(int fmt, const uint32_t *payload, const uint32_t *signs, const u
     const int bad = check_common(fmt, payload, signs, tile_off, scales, M, K, x, x_scale, batch, y, acc_debug, workspace,
                                  workspace_bytes);
     if (bad) return bad;
-    const Plan pl = make_plan(M, K, decoder_warps(batch));
+    const Plan pl = one_tile_plan(fmt, M, K, nb_bucket(batch, K));
     Problem pr{};
     fill_problem(pr, payload, signs, tile_off, scales, M, K, x, x_scale, batch, y, acc_debug, workspace);
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
@@ -554,7 +554,6 @@ int gemv_multi_common(const bitcos_gemv_job *jobs, int n_jobs, int batch, void *
             const bitcos_weights *w = prev[i];
             if (!w) return BITCOS_ERR_NULL;
             if (w->M < 1 || w->K < kGroup || w->K % kGroup) return BITCOS_ERR_SHAPE;
-            pm.pl[i] = make_plan(w->M, w->K, decoder_warps(batch));
             pm.pr[i].M = w->M;
             pm.pr[i].K = w->K;
             kprev = w->K > kprev ? w->K : kprev;
@@ -609,7 +608,6 @@ int gemv_multi_common(const bitcos_gemv_job *jobs, int n_jobs, int batch, void *
         if (bad) return bad;
         for (int i = 0; i < j; ++i)
             if (jobs[i].workspace == jb.workspace) return BITCOS_ERR_SHAPE;      // jobs run concurrently
-        ma.pl[j] = make_plan(jb.W->M, jb.W->K, decoder_warps(batch));
         fill_problem(ma.pr[j], jb.W->bitmap, jb.W->signs, jb.W->tile_off, jb.W->scales, jb.W->M, jb.W->K, jb.x,
                      jb.x_scale, batch, jb.y, nullptr, jb.workspace);
     }
@@ -667,7 +665,7 @@ int bitcos_gemv_phased(const bitcos_gemv_job *jobs, const int *job_phase, int n_
         if (bad) return bad;
         for (int i = 0; i < j; ++i)
             if (jobs[i].workspace == jb.workspace) return BITCOS_ERR_SHAPE;
-        pa.pl[j] = make_plan(jb.W->M, jb.W->K, decoder_warps(batch));
+        pa.pl[j] = one_tile_plan(kBitcos, jb.W->M, jb.W->K, batch);
         fill_problem(pa.pr[j], jb.W->bitmap, jb.W->signs, jb.W->tile_off, jb.W->scales, jb.W->M, jb.W->K, jb.x,
                      jb.x_scale, batch, jb.y, nullptr, jb.workspace);
     }
@@ -701,7 +699,6 @@ int bitcos_gemv_multi_plan(const int64_t *M, const int64_t *K, int n_jobs, int b
     int64_t kmax = 0;
     for (int j = 0; j < n_jobs; ++j) {
         if (M[j] < 1 || K[j] < kGroup || K[j] % kGroup) return BITCOS_ERR_SHAPE;
-        ma.pl[j] = make_plan(M[j], K[j], decoder_warps(batch));
         ma.pr[j].M = M[j];
         ma.pr[j].K = K[j];
         ma.pr[j].G = static_cast<int>(K[j] / kGroup);
@@ -764,7 +761,7 @@ int bitcos_gemv_blend_bf16(const bitcos_weights *W, const uint16_t *x_bf16, int 
     const int bad = check_common(kBitcos, W->bitmap, W->signs, W->tile_off, W->scales, W->M, W->K, x,
                                  reinterpret_cast<const float *>(x), batch, y, nullptr, workspace, workspace_bytes);
     if (bad) return bad;
-    const Plan pl = make_plan(W->M, W->K, decoder_warps(8));
+    const Plan pl = one_tile_plan(kBitcos, W->M, W->K, batch <= 4 ? 4 : 8);
     Problem pr{};
     fill_problem(pr, W->bitmap, W->signs, W->tile_off, W->scales, W->M, W->K, x, nullptr, batch, y, nullptr, workspace);
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
@@ -780,7 +777,7 @@ int bitcos_gemv_bf16(const bitcos_weights *W, const uint16_t *x_bf16, int batch,
     const int bad = check_common(kBitcos, W->bitmap, W->signs, W->tile_off, W->scales, W->M, W->K, x,
                                  reinterpret_cast<const float *>(x), batch, y, acc_debug, workspace, workspace_bytes);
     if (bad) return bad;
-    const Plan pl = make_plan(W->M, W->K, decoder_warps(batch));
+    const Plan pl = one_tile_plan(kBitcos, W->M, W->K, nb_bucket(batch, W->K));
     Problem pr{};
     fill_problem(pr, W->bitmap, W->signs, W->tile_off, W->scales, W->M, W->K, x, nullptr, batch, y, acc_debug, workspace);
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);

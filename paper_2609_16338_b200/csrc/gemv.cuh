@@ -79,7 +79,8 @@ struct Plan {
     int CS;          // column blocks per row
     int RBC;         // row blocks per item (1 unless CS == 1)
     int NW;          // decoder warps per thread block = ceil(CG * RBC / tpw)
-    int tpw;         // tiles of an item per decoder warp: 1, or 2 on large matrices
+    int tpw;         // tiles of an item per decoder warp: 1, or 2 or 3 on large matrices
+    int sub, wsub, wrow;   // make_run_plan: tiles and warps of a column block of the one-tile plan, warps of a row
     int64_t items;   // ceil(RB / RBC) * CS
     int cyclic;      // 1: blocks take whole row-block chunks round robin; 0: contiguous balanced ranges
     int stages;      // depth of the shared-memory ring (2 .. kMaxStages), set at launch
@@ -256,17 +257,51 @@ inline Plan make_plan(int64_t M, int64_t K, int max_warps_per_block, int tpw = 1
 }
 
 // Several tiles per warp (BITCOS, two tokens and more): a warp takes tpw neighbouring groups of one row block and adds
-// their sums in registers, so with whole rows per item a row block takes ceil(G / tpw) warps.
-inline Plan make_run_plan(int64_t M, int64_t K, int max_warps, int tpw) {
+// their sums in registers.
+// The bits of a product must not depend on how many tiles its launch gives a warp (a launch of several products has
+// more tiles than each of them), so both plans add in one order: runs of tpw groups inside a column block of the one-tile
+// plan, the runs of a column block, the column blocks one after the other.  A wide item is therefore as many whole column
+// blocks of the one-tile plan (sub groups, wsub warps each) as its warps hold.  At three tiles per warp the one-tile plan's
+// column blocks are made a little uneven where that takes a warp less a row and lets an item hold two rows (20 groups: 11 and
+// 9, seven warps, for 10 and 10, eight); and rows of more than 40 groups are cut by their own width instead, because fourteen
+// warps hold only two such column blocks (200 groups would be eight items instead of five): their last bits may
+// differ from the one-tile plan's.  own_order: a product that no launch of several takes (the 16-bit variant).
+__host__ __device__ constexpr bool one_order(int G, int tpw) { return tpw == 2 || G <= 40; }
+inline int row_warps(int G, int cg, int tpw) { return G / cg * ((cg + tpw - 1) / tpw) + (G % cg + tpw - 1) / tpw; }
+
+// The one-tile plan of a product that other launches run with tpw tiles per warp.
+inline Plan make_one_tile_plan(int64_t M, int64_t K, int max_warps, int tpw) {
+    Plan p = make_plan(M, K, max_warps);
+    const int G = static_cast<int>(K / kGroup), whole = (G + tpw - 1) / tpw;
+    if (tpw != 3 || !one_order(G, tpw) || p.CS == 1) return p;
+    int cg = p.CG;
+    while (cg < max_warps && (row_warps(G, cg, tpw) > max_warps || max_warps / row_warps(G, cg, tpw) < max_warps / whole)) ++cg;
+    p.CG = p.NW = cg;
+    return p;
+}
+
+inline Plan make_run_plan(int64_t M, int64_t K, int max_warps, int tpw, bool own_order) {
+    const int G = static_cast<int>(K / kGroup);
+    const int64_t RB = padded_rows(M) / kRows;
     Plan p = make_plan(M, K, max_warps, tpw);
-    if (p.CS == 1) {
-        const int wr = (p.CG + tpw - 1) / tpw;
-        const int64_t RB = padded_rows(M) / kRows;
-        p.RBC = max_warps / wr;
-        if (p.RBC > RB) p.RBC = static_cast<int>(RB);
-        p.NW = p.RBC * wr;
-        p.items = (RB + p.RBC - 1) / p.RBC;
+    if (own_order || !one_order(G, tpw)) {
+        p.sub = p.CG;
+        p.wsub = p.wrow = (p.CG + tpw - 1) / tpw;
+    } else {
+        p.sub = make_one_tile_plan(M, K, max_warps, tpw).CG;
+        p.wsub = (p.sub + tpw - 1) / tpw;
+        p.wrow = row_warps(G, p.sub, tpw);
     }
+    if (p.CS == 1) {
+        p.RBC = static_cast<int>(std::min<int64_t>(max_warps / p.wrow, RB));
+        p.NW = p.RBC * p.wrow;
+    } else if (p.sub < p.CG) {
+        const int subs = (G + p.sub - 1) / p.sub, fit = max_warps / p.wsub, items = (subs + fit - 1) / fit, n = (subs + items - 1) / items;
+        p.CG = n * p.sub;
+        p.CS = (G + p.CG - 1) / p.CG;
+        p.NW = p.wrow = n * p.wsub;
+    }
+    p.items = (RB + p.RBC - 1) / p.RBC * p.CS;
     return p;
 }
 
@@ -325,6 +360,11 @@ __host__ __device__ constexpr bool fragment_order(int fmt, int nb) { return fmt 
 // Tiles per warp in large launches (wants_two_tiles): two, or three with the fourteen decoder warps of more than eight tokens, which two
 // tiles each would leave four of idle where rows have 20 or 40 groups (25600x5120 at sixteen tokens 27.1 -> 24.7 us).
 __host__ __device__ constexpr int wide_tiles(int fmt, int nb) { return fragment_order(fmt, nb) && nb > 8 ? 3 : 2; }
+
+// The plan with one tile per warp.
+inline Plan one_tile_plan(int fmt, int64_t M, int64_t K, int nb_template) {
+    return make_one_tile_plan(M, K, decoder_warps(nb_template), wide_tiles(fmt, nb_template));
+}
 
 // scr: the tensor-core path passes its rows through transposition buffers
 __host__ __device__ inline SmemLayout smem_layout(int fmt, const Plan &pl, int G, int nbmax, int64_t K, bool scr) {
@@ -1112,11 +1152,12 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
         ItemIter it;
         int kk = 0;             // items consumed so far, over all segments
         int es = 0;             // stage of the item the epilogue looks at next
-        // The sums of n <= 20 partial sums, in an order that depends on n alone.  This one warp serves every row block of
-        // the launch at the few issue slots the decoders leave it (one in six clocks or so), and with short rows they come
-        // fast (six tiles a row block at K = 768): what counts there is its instructions, with long rows its latency at the
-        // end of a launch.  Clocks per tile and multiprocessor at eight tokens against twenty guarded loads a sum and a
-        // scale fetched per output: K = 768 300 -> 182, K = 2048 180 -> 148, K = 2560 163 -> 145.
+        // The sums of n tiles, in an order that depends on n alone: neighbours first (with sixteen tokens neighbouring threes),
+        // which is what a warp with several tiles has added up already (kPairs; see make_run_plan).  This one warp serves
+        // every row block of the launch at the few issue slots the decoders leave it (one in six clocks or so), and with short
+        // rows they come fast (six tiles a row block at K = 768): what counts there is its instructions, with long rows its latency at
+        // the end of a launch.  Clocks per tile and multiprocessor at eight tokens against twenty guarded loads a sum and
+        // a scale fetched per output: K = 768 300 -> 182, K = 2048 180 -> 148, K = 2560 163 -> 145.
         // Up to two tokens (spaced NB * 32 floats apart): a tree of pairs, all loads before the first addition.
         auto tree = [&](auto size, const float *base, int n) {
             constexpr int N = decltype(size)::value;
@@ -1130,6 +1171,7 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
             return v[0];
         };
         auto sum_groups20 = [&](const float *base, int n) {
+            if (kPairs) return tree(std::integral_constant<int, 10>{}, base, n);
             if (n <= 8) return tree(std::integral_constant<int, 8>{}, base, n);
             return tree(std::integral_constant<int, kMaxWarps>{}, base, n);
         };
@@ -1139,42 +1181,101 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
             if (TPW == 2 && !kPairs && n > kMaxWarps) t += sum_groups20(base + kMaxWarps * NB * kRows, n - kMaxWarps);
             return t;
         };
-        // Tensor-core layout: four tokens at a time, spaced one warp's rows apart; more than eight in two batches of ten,
+        // Tensor-core layout: four tokens at a time, spaced one warp's rows apart; more than eight tiles in two batches of ten,
         // all loads of a batch before its first addition (three smaller batches cost the sixteen-token layer 3 %).
         constexpr int RF = NB;
         auto add4 = [](float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); };
-        auto sum_groups4 = [&](const float *base, int n) {
-            auto at = [&](int j) { return *reinterpret_cast<const float4 *>(base + j * kRows * RF); };
-            float4 tot = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (n > 8) {
+        const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
+        auto in_tens = [&](const float *base, int n) {
+            float4 tot = none;
 #pragma unroll
-                for (int j0 = 0; j0 < kMaxWarps; j0 += 10) {
-                    float4 v[10];
+            for (int j0 = 0; j0 < kMaxWarps; j0 += 10) {
+                float4 v[10];
 #pragma unroll
-                    for (int j = 0; j < 10; ++j) v[j] = (j0 + j < n) ? at(j0 + j) : make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int j = 0; j < 10; ++j) v[j] = (j0 + j < n) ? *reinterpret_cast<const float4 *>(base + (j0 + j) * kRows * RF) : none;
 #pragma unroll
-                    for (int w2 = 1; w2 < 10; w2 *= 2)
+                for (int w2 = 1; w2 < 10; w2 *= 2)
 #pragma unroll
-                        for (int j = 0; j + w2 < 10; j += 2 * w2) v[j] = add4(v[j], v[j + w2]);
-                    tot = add4(tot, v[0]);
-                }
-                return tot;
+                    for (int j = 0; j + w2 < 10; j += 2 * w2) v[j] = add4(v[j], v[j + w2]);
+                tot = add4(tot, v[0]);
             }
+            return tot;
+        };
+        auto sum_tiles4 = [&](const float *base, int n) {
+            if (n > 8) return in_tens(base, n);
+            auto at = [&](int j) { return *reinterpret_cast<const float4 *>(base + j * kRows * RF); };
+            float4 tot = none;
 #pragma unroll 1
             for (; n >= 4; n -= 4, base += 4 * kRows * RF) {
                 const float4 a = at(0), b = at(1), c = at(2), d = at(3);
                 tot = add4(tot, add4(add4(a, b), add4(c, d)));
             }
             if (n >= 1) {
-                const float4 a = at(0);
+                float4 a = at(0);
                 if (n >= 2) {
                     const float4 b = at(1);
-                    if (n == 3) tot = add4(tot, at(2));
-                    tot = add4(tot, b);
+                    if (!kFrag && n == 3) tot = add4(tot, at(2));
+                    if (kFrag) a = add4(a, b);
+                    else tot = add4(tot, b);
+                    if (kFrag && n == 3) a = add4(a, at(2));
                 }
                 tot = add4(tot, a);
             }
             return tot;
+        };
+        // the same from the sums of neighbouring tiles (n of them: nine tiles and more are five and more)
+        auto sum_pairs4 = [&](const float *base, int n) {
+            auto at = [&](int j) { return *reinterpret_cast<const float4 *>(base + j * kRows * RF); };
+            if (n > 4) {
+                float4 v[10];
+#pragma unroll
+                for (int j = 0; j < 10; ++j) v[j] = (j < 5 || j < n) ? at(j) : none;
+                return add4(add4(add4(add4(v[0], v[1]), add4(v[2], v[3])), v[4]), add4(add4(add4(v[5], v[6]), add4(v[7], v[8])), v[9]));
+            }
+            float4 tot = none;
+#pragma unroll 1
+            for (; n >= 2; n -= 2, base += 2 * kRows * RF) tot = add4(tot, add4(at(0), at(1)));
+            if (n) tot = add4(tot, at(0));
+            return tot;
+        };
+        // Sixteen tokens: by threes, the at most five threes by pairs; from n single tiles ..
+        auto sum_threes4 = [&](const float *base, int n) {
+            // (without branches, so that the loads of all tokens are under way together)
+            auto up_to = [&](auto size) {
+                constexpr int N = decltype(size)::value;
+                float4 v[N], t[(N + 2) / 3];
+#pragma unroll
+                for (int i = 0; i < N; ++i) v[i] = i < n ? *reinterpret_cast<const float4 *>(base + i * kRows * RF) : none;
+#pragma unroll
+                for (int i = 0; i < N; ++i) t[i / 3] = i % 3 ? add4(t[i / 3], v[i]) : v[i];
+                if constexpr (N <= 3) return t[0];
+                else if constexpr (N <= 6) return add4(t[0], t[1]);
+                else return add4(add4(add4(t[0], t[1]), add4(t[2], t[3])), t[4]);
+            };
+            if (n <= 3) return up_to(std::integral_constant<int, 3>{});
+            if (n <= 6) return up_to(std::integral_constant<int, 6>{});
+            return up_to(std::integral_constant<int, kWarps16>{});
+        };
+        // .. or from n sums of three (more than five only where rows are cut by their own width)
+        auto sum_of_threes4 = [&](const float *base, int n) {
+            auto at = [&](int j) { return *reinterpret_cast<const float4 *>(base + j * kRows * RF); };
+            if (n > 5) return in_tens(base, n);
+            if (n > 3) {
+                const float4 a = at(0), b = at(1), c = at(2), d = at(3);
+                float4 e = none;
+                if (n > 4) e = at(4);
+                return add4(add4(add4(a, b), add4(c, d)), e);
+            }
+            float4 a = at(0);
+            if (n >= 2) a = add4(a, at(1));
+            if (n == 3) a = add4(a, at(2));
+            return a;
+        };
+        auto sum_groups4 = [&](const float *base, int n) {
+            if constexpr (kFrag && NB > 8 && kPairs) return sum_of_threes4(base, n);
+            else if constexpr (kFrag && NB > 8) return sum_threes4(base, n);
+            else if constexpr (kPairs && !kBlend) return sum_pairs4(base, n);      // (the 16-bit variant has an order of its own)
+            else return sum_tiles4(base, n);
         };
         // one row block's outputs: row m of every token, one M apart
         auto store_rows = [&](int64_t m, const float (&t)[NB]) {
@@ -1186,7 +1287,7 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
             for (int b = 0; b < NB; ++b, out += step)
                 if (b < nb) *out = xscale(b) * t[b];
         };
-        // sums over warps j0 .. j0 + n - 1 of a slot, for this lane's row and every token
+        // the sums of what warps j0 .. j0 + n - 1 left, for this lane's row and every token
         auto sums = [&](const float *rs, int j0, int n, float (&tot)[NB]) {
             if (NB >= kMmaMinBatch) {
 #pragma unroll
@@ -1202,6 +1303,22 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
 #pragma unroll
                 for (int b = 0; b < NB; ++b)
                     tot[b] = (b < pr.nb(pb)) ? sum_groups(rs + (j0 * NB + b) * kRows + lane, n) : 0.f;
+            }
+        };
+        // The same over n tiles of a row that begin at warp j0.  Several tiles per warp in fragment order (kSubs): one column block
+        // of the one-tile plan after the other (two of them, sixteen tokens' up to three), added to tot (fresh: instead of it).
+        constexpr bool kSubs = kPairs && !kBlend;
+        auto row_sums = [&](const float *rs, int j0, int n, float (&tot)[NB], bool fresh) {
+            if constexpr (kSubs) {
+#pragma unroll 1
+                for (; n > 0; n -= pl.sub, j0 += pl.wsub, fresh = false) {
+                    float t[NB];
+                    sums(rs, j0, ((n < pl.sub ? n : pl.sub) + TPW - 1) / TPW, t);
+#pragma unroll
+                    for (int b = 0; b < NB; ++b) tot[b] = fresh ? t[b] : tot[b] + t[b];
+                }
+            } else {
+                sums(rs, j0, kPairs ? (n + TPW - 1) / TPW : n, tot);
             }
         };
         do {
@@ -1240,11 +1357,11 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
                 // whole row blocks: one output per row.  The sums are formed first, the slot is
                 // handed back, and only then are the outputs stored, so that the release of the
                 // slot never waits for a global store.
-                const int nrb = r.nt / pb.G, parts = kPairs ? (pb.G + TPW - 1) / TPW : pb.G;
+                const int nrb = r.nt / pb.G, parts = kPairs ? pl.wrow : pb.G;
                 for (int i = 0; i < nrb; ++i) {
                     const int64_t m = static_cast<int64_t>(r.rb0 + i) * kRows + lane;
                     float t_b[NB];
-                    sums(rs, i * parts, parts, t_b);
+                    row_sums(rs, i * parts, pb.G, t_b, true);
                     if (i == nrb - 1) {
                         __syncwarp();
                         if (lane == 0) mbar_arrive(bar0 + 8u * (kBarRedEmpty + slot));
@@ -1255,10 +1372,14 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
             }
             // one column block of row block rb0: add it to the running sum
             const bool starts = (r.cs == 0) || (k == 0);
-            float t_b[NB];
-            sums(rs, 0, kPairs ? (r.nt + TPW - 1) / TPW : r.nt, t_b);
+            if constexpr (kSubs) {
+                row_sums(rs, 0, r.nt, run, starts);
+            } else {
+                float t_b[NB];
+                row_sums(rs, 0, r.nt, t_b, true);
 #pragma unroll
-            for (int b = 0; b < NB; ++b) run[b] = starts ? t_b[b] : run[b] + t_b[b];
+                for (int b = 0; b < NB; ++b) run[b] = starts ? t_b[b] : run[b] + t_b[b];
+            }
             __syncwarp();
             if (lane == 0) mbar_arrive(bar0 + 8u * (kBarRedEmpty + slot));
             const bool ends = (r.cs == pl.CS - 1) || (k == wk.count - 1);
@@ -1318,11 +1439,22 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
         const uint32_t lane4 = static_cast<uint32_t>(lane) * 4u;
         // CS == 1: tile t of an item always is row block t / G of the chunk, group t % G
         // (a phased launch works these out again for every job)
-        int rbl = 0, g_first = 0;
+        // several tiles: run number warp - wrow rbl of the row, the runs of a column block of the one-tile plan after those
+        // of the one before it; the run has n_run tiles, fewer at the end of the column block or of the row
+        int rbl = 0, g_first = 0, n_run = 1;
         auto place = [&]() {
-            const int wr = (pb.G + TPW - 1) / TPW;       // warps per row block when items are whole rows
+            const int wr = kBlend ? (pb.G + TPW - 1) / TPW : kPairs ? pl.wrow : pb.G;      // warps per row block when items are whole rows
             rbl = pl.CS == 1 ? warp / wr : 0;
-            g_first = (warp - rbl * wr) * TPW;
+            g_first = warp - rbl * wr;
+            if (kBlend) {
+                g_first *= TPW;
+            } else if (kPairs) {
+                const int cb = g_first / pl.wsub;
+                g_first = cb * pl.sub + (g_first - cb * pl.wsub) * TPW;
+                int g_end = (cb + 1) * pl.sub;
+                if (pl.CS == 1 && g_end > pb.G) g_end = pb.G;
+                n_run = g_end - g_first < TPW ? g_end - g_first : TPW;
+            }
         };
         place();
         int tile0 = rbl * pb.G + g_first;
@@ -1451,7 +1583,7 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
 #pragma unroll 1
             for (int ti = 0; ti < TPW; ++ti) {
                 const int tile = tile0 + ti;
-                if (tile >= nt || (TPW > 1 && pl.CS == 1 && g_first + ti >= pb.G)) break;
+                if (tile >= nt || (kPairs && (kBlend ? pl.CS == 1 && g_first + ti >= pb.G : ti >= n_run))) break;
                 // group: the item's first (0 when items are whole rows) + the tile's place in its row block
                 const int grp = static_cast<int>(d.y) + g_first + ti;
                 const uint8_t *xs = kXQ ? reinterpret_cast<const uint8_t *>(q_scr)
@@ -1551,8 +1683,10 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
                                 v = (t4 & 2) ? hi : lo;
                             }
                             float y = sc * static_cast<float>(v);
-                            if (kXQ) y *= q_scale[r];
-                            else if (kXG && !kBlend) y *= xg[h][r];
+                            // (a group scale makes the product inexact: rounded before it is added, as it is where a tile's
+                            // sum is all that a warp leaves; bf16 scale times sum is exact, the 16-bit variant has one plan)
+                            if (kXQ) y = kPairs ? __fmul_rn(y, q_scale[r]) : y * q_scale[r];
+                            else if (kXG && !kBlend) y = kPairs ? __fmul_rn(y, xg[h][r]) : y * xg[h][r];
                             ysum[h][j][r] += y;
                             if constexpr (Segs::kDebug) if (pb.acc_debug) {
                                 const int b = 8 * h + n0 + r;
@@ -2551,8 +2685,8 @@ inline bool wants_two_tiles(int fmt, int64_t items, int64_t tiles, int nb_templa
 }
 inline int64_t tile_count(int64_t M, int64_t K) { return padded_rows(M) / kRows * (K / kGroup); }
 // The plan of such a product.
-inline Plan two_tile_plan(int fmt, int64_t M, int64_t K, int nb_template) {
-    return fragment_order(fmt, nb_template) ? make_run_plan(M, K, decoder_warps(nb_template), wide_tiles(fmt, nb_template))
+inline Plan two_tile_plan(int fmt, int64_t M, int64_t K, int nb_template, bool own_order = false) {
+    return fragment_order(fmt, nb_template) ? make_run_plan(M, K, decoder_warps(nb_template), wide_tiles(fmt, nb_template), own_order)
                                             : make_plan(M, K, decoder_warps(nb_template), 2);
 }
 
@@ -2575,7 +2709,7 @@ int launch(const Problem &pr, const Plan &pl_in, cudaStream_t stream, const uint
     if (rc) return rc;
     // (with and without the accumulator dump: the same plan, so the same order of the sums)
     const bool two = kTwo && wants_two_tiles(FMT, pl_in.items, tile_count(pr.M, pr.K), NB, sms);
-    const Plan pl = two ? two_tile_plan(FMT, pr.M, pr.K, NB) : pl_in;
+    const Plan pl = two ? two_tile_plan(FMT, pr.M, pr.K, NB, BL) : pl_in;
     int grid = 1;
     Plan plw = pl;
     choose_walk(plw, small_launch_cap(pl.items, sms), &grid);
@@ -2633,7 +2767,10 @@ inline void fill_first_copies(FirstCopies &c, const Problem &pr, const Plan &pl,
 // item counts).  Returns the total number of blocks.
 inline int plan_multi(MultiArgs &ma, int nb_template, int sms, bool *two_out, int *grids) {
     int64_t total_items = 0;
-    for (int j = 0; j < ma.n; ++j) total_items += ma.pl[j].items;
+    for (int j = 0; j < ma.n; ++j) {
+        ma.pl[j] = one_tile_plan(kBitcos, ma.pr[j].M, ma.pr[j].K, nb_template);
+        total_items += ma.pl[j].items;
+    }
     // enough items altogether: every problem with two tiles per decoder warp
     int64_t tiles = 0;
     for (int j = 0; j < ma.n; ++j) tiles += tile_count(ma.pr[j].M, ma.pr[j].K);

@@ -5,7 +5,6 @@ Scales spread over many powers of two, so that no sum of a few of them is exact 
 import numpy as np
 import pytest
 
-
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
@@ -66,3 +65,40 @@ def test_the_accumulator_dump_changes_nothing(bc, fmt, batches, M, K):
             y2, acc2 = bc.bitcos_gemv_group_scales(W, x, xg, acc_debug=True, workspace=ws)
             assert torch.equal(acc, acc2) and torch.equal(y, y2), B
     assert bc.workspace_status(ws) == 0
+
+
+# Two to eight products that are launched with one tile per warp each and with several together, and one product above the
+# line beside one below it: whole rows in an item, one and two column blocks of even and odd width, at the end
+# of a row a run that is not full.
+SETS = [[(8192, 2560)] * 2, [(4096, 384)] * 7 + [(9472 * 32, 128)], [(8190, 2432)] * 2, [(4096, 1792)] * 6, [(4096, 1664)] * 6,
+        [(4096, 5120)] * 2, [(4100, 4992)] * 2, [(4600, 4736)] * 2, [(6144, 3456)] * 2, [(6144, 3200)] * 2, [(8192, 5120), (1024, 5120), (1024, 2688)]]
+
+
+@pytest.mark.parametrize("shapes", SETS, ids=lambda s: "+".join("%dx%d" % mk for mk in s[:2]))
+def test_several_products_in_a_launch_have_the_bits_of_each_alone(bc, shapes):
+    Ws = [bc.bitcos_pack_device(*matrix(i, M, K)) for i, (M, K) in enumerate(shapes)]
+    wss = [bc.make_workspace(M, K) for M, K in shapes]
+    ys = {B: [torch.empty((B, M), device="cuda") for M, _ in shapes] for B in (1, 2, 3, 8, 16)}
+    for B in ys:
+        if B == 1 and max(K for _, K in shapes) > 2560:
+            continue              # (one token: rows of more than 20 groups are cut by the launch's own plan)
+        acts = {K: activations(K + B, B, K) for _, K in shapes}
+        token = {K: xg[:, 0].contiguous() for K, (_, xg) in acts.items()}
+        jobs = [(W, acts[W.K][0], token[W.K], y, ws) for W, y, ws in zip(Ws, ys[B], wss)]
+        bc.bitcos_gemv_multi(jobs)
+        for W, x, xs, y, ws in jobs:
+            assert torch.equal(y, bc.bitcos_gemv(W, x, xs, workspace=ws)[0]), (B, W.M, W.K)
+        if B <= 2 and max(K for _, K in shapes) <= 2560:
+            phased = [torch.empty_like(y) for y in ys[B]]
+            bc.bitcos_gemv_phased([j[:3] + (y, j[4]) for j, y in zip(jobs, phased)], [0] * len(jobs), bc.make_phased_sync())
+            assert all(torch.equal(a, b) for a, b in zip(phased, ys[B])), B
+        jobs = [(W, acts[W.K][0], acts[W.K][1], y, ws) for W, y, ws in zip(Ws, ys[B], wss)]
+        bc.bitcos_gemv_multi_group_scales(jobs)
+        for W, x, xg, y, ws in jobs:
+            assert torch.equal(y, bc.bitcos_gemv_group_scales(W, x, xg, workspace=ws)[0]), (B, W.M, W.K, "group scales")
+        if B <= 2:
+            bf16 = {K: torch.randn((B, K), generator=torch.Generator(device="cuda").manual_seed(K), device="cuda").to(torch.bfloat16) for K in acts}
+            bc.bitcos_gemv_multi_bf16([(W, bf16[W.K], None, y, ws) for W, y, ws in zip(Ws, ys[B], wss)])
+            for W, y, ws in zip(Ws, ys[B], wss):
+                assert torch.equal(y, bc.bitcos_gemv_bf16(W, bf16[W.K], workspace=ws)[0]), (B, W.M, W.K, "bf16")
+    assert not any(bc.workspace_status(ws) for ws in wss)

@@ -286,7 +286,8 @@ int bitcos_gemv_bf16(const bitcos_weights *W, const uint16_t *x_bf16, int batch,
                      void *workspace, size_t workspace_bytes, void *cuda_stream);
 
 /* The 16-bit variant of Sections II-B / II-D: no activation quantisation; the bf16 activations are
- * multiplied with the weights as bf16 +1 / 0 / -1 and each group's sum with its bf16 scale,
+ * multiplied with the weights as bf16 +2^-8 / 0 / -2^-8 and each group's sum with its bf16 scale (the outputs
+ * with 2^8: no group's sum leaves the range of fp32 unless the output does),
  *     y[b][m] = sum over k of (W[m][k] * s[m][k / 128]) * x[b][k],
  * on the tensor cores (mma.m16n8k16, bf16 operands, fp32 accumulation over each group of 128; the
  * groups are then added in fp32 in the fixed order of the other products).  Every product is exact

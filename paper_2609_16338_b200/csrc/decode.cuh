@@ -85,7 +85,9 @@ constexpr LutBig make_bitcos_lut() {
 }
 
 // BITCOS as bf16 (the 16-bit variant): byte address = ((s << 4) | m) * 256 + lane * 8; an entry is the four weights as
-// bf16 +1 / 0 / -1, two to a word.
+// bf16 +2^-8 / 0 / -2^-8, two to a word: a group's sum of 128 finite activations then cannot leave fp32's range before its scale is
+// applied (the outputs are multiplied by kBf16WeightInverse, which is exact).
+constexpr float kBf16WeightInverse = 256.f;
 constexpr LutBig make_bitcos_bf16_lut() {
     const Lut256 base = make_nibble_lut();
     LutBig t{};
@@ -94,7 +96,7 @@ constexpr LutBig make_bitcos_bf16_lut() {
         uint32_t w = 0;
         for (int i = 0; i < 2; ++i) {
             const uint32_t b = (e >> (8 * i)) & 0xFFu;
-            w |= (b == 0 ? 0u : b == 1 ? 0x3F80u : 0xBF80u) << (16 * i);
+            w |= (b == 0 ? 0u : b == 1 ? 0x3B80u : 0xBB80u) << (16 * i);
         }
         t.v[idx] = w;
     }
@@ -272,10 +274,10 @@ struct FragmentRows {
             if (k < 3) pos[i] = __dp4a(e[2 * i + 1], e[2 * i + 1], pos[i]);
         }
     }
-    // The same as bf16 +-1 for mma.m16n8k16, nibble j = 0 .. 7 of the four rows: e[2 i] = weights 0 and 1, e[2 i + 1] =
+    // The same as bf16 +-2^-8 for mma.m16n8k16, nibble j = 0 .. 7 of the four rows: e[2 i] = weights 0 and 1, e[2 i + 1] =
     // weights 2 and 3 (two words from an 8-byte entry of the bf16 table; B holds the presence words moved down by four, so
     // that odd nibbles use the same table: open() is followed by shift_presence()).  A non-zero bf16 weight's
-    // high byte is 63 or 191, both -1 modulo 32, so 31 times its high byte counts 1 in the five bits that a rotation uses.
+    // high byte is 59 or 187, both 27 modulo 32, so 19 times its high byte counts 1 in the five bits that a rotation uses.
     __device__ __forceinline__ void shift_presence() {
 #pragma unroll
         for (int i = 0; i < 4; ++i) B[i] = P[i] >> 4;
@@ -288,7 +290,7 @@ struct FragmentRows {
             const uint2 v = lds64(lut, bit_select(t, R, 0xF000u));
             e[2 * i] = v.x;
             e[2 * i + 1] = v.y;
-            if (j < 7) pos[i] = static_cast<int>(dp4a_uu(v.y, 0x1F001F00u, dp4a_uu(v.x, 0x1F001F00u, static_cast<uint32_t>(pos[i]))));
+            if (j < 7) pos[i] = static_cast<int>(dp4a_uu(v.y, 0x13001300u, dp4a_uu(v.x, 0x13001300u, static_cast<uint32_t>(pos[i]))));
         }
     }
 };

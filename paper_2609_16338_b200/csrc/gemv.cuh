@@ -776,7 +776,7 @@ struct Share {
 };
 
 // If this block's arrival was the last one: add the shares in slot order and write the outputs.
-template <int NB, bool XG>
+template <int NB, bool XG, bool BL>
 __device__ __forceinline__ void finish_share(const Problem &pr, const Plan &pl, const int (&xr)[NB], const Share &sh,
                                              int lane) {
     const unsigned int old = __shfl_sync(0xFFFFFFFFu, sh.old, 0);
@@ -789,7 +789,7 @@ __device__ __forceinline__ void finish_share(const Problem &pr, const Plan &pl, 
             float tot = 0.f;
             for (int j = 0; j < sh.sharers; ++j)
                 tot += __ldcg(pr.partial + ((static_cast<int64_t>(sh.rb) * pl.CS + j) * pr.nb + b) * kRows + lane);
-            if (m < pr.M) pr.y[(pr.out_row0 + b) * pr.M + m] = XG ? tot : __ldg(pr.x_scale + xr[b]) * tot;
+            if (m < pr.M) pr.y[(pr.out_row0 + b) * pr.M + m] = BL ? kBf16WeightInverse * tot : XG ? tot : __ldg(pr.x_scale + xr[b]) * tot;
         }
     }
     if (lane == 0) pr.counters[sh.rb] = 0u;    // leave the counter ready for the next call
@@ -1146,7 +1146,7 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
         // per-token activation scales, fetched once per segment (sixteen: a cached load per output block)
         constexpr bool kHoldScales = !kXG && NB <= 8;
         float xsc[kHoldScales ? NB : 1] = {};
-        auto xscale = [&](int b) { return kXG ? 1.f : kHoldScales ? xsc[kHoldScales ? b : 0] : __ldg(pb.x_scale + xr[b]); };
+        auto xscale = [&](int b) { return kBlend ? kBf16WeightInverse : kXG ? 1.f : kHoldScales ? xsc[kHoldScales ? b : 0] : __ldg(pb.x_scale + xr[b]); };
         Share pend[2];
         int n_pend = 0;
         ItemIter it;
@@ -1409,7 +1409,7 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
                 pend[n_pend++] = sh;      // at most two per block: its first and its last row block
             }
         }
-        for (int i = 0; i < n_pend; ++i) finish_share<NB, kXG>(pb, pl, xr, pend[i], lane);
+        for (int i = 0; i < n_pend; ++i) finish_share<NB, kXG, kBlend>(pb, pl, xr, pend[i], lane);
         if constexpr (Segs::kHetero) src.signal_done(lane);      // this block's outputs of the phase are written
         if (lane == 0) BITCOS_TLP(src, 5);
         have = next_segment();
@@ -1630,7 +1630,7 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
                 }
                 if (kXQ && grp != q_g) quantize_group(grp);
                 if (NB < kMmaMinBatch) load_x(grp, xs);
-                // int32 sums, or fp32 ones of the 16-bit variant: weights +-1 against the activations as they are, the scale
+                // int32 sums, or fp32 ones of the 16-bit variant: weights +-2^-8 against the activations as they are, the scale
                 // applied to the group's sum (every product is exact).  Its table holds bf16 words, so that a lookup is two
                 // fragment registers: 18944 -> 56832 x 5120 176 clocks per tile and multiprocessor at one token, 213 at four and
                 // eight; 8192x5120 at four tokens 13.8 -> 11.3 us against rebuilding +-s from int8 weights and a pass

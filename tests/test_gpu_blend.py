@@ -81,6 +81,23 @@ def test_blend_product_exact_cases(bc):
         assert np.array_equal(y1.cpu().numpy().astype(np.float64), ref1), k
 
 
+@pytest.mark.parametrize("size,scale", [(1e38, 0.002), (3.3e38, 2.0 ** -11), (1e-37, 0.75), (1.0, 2.0 ** 100), (1e-30, 2.0 ** 126)])
+def test_blend_product_at_the_ends_of_the_range(bc, size, scale):
+    """Finite activations whose sum over a group leaves fp32's range although the output does not, and the smallest
+    ones; large scales.  (The smallest: what an output may lose to fp32's smallest step, 2^-149 times 2^8, is allowed for.)"""
+    M, K = 64, 1280
+    W = datagen.trits(4250, M, K, 0.42)
+    W[:8] = np.abs(W[:8])                          # (rows whose sums do not cancel)
+    for B in (1, 8):
+        x = datagen.bf16_bits_to_f32(datagen.f32_to_bf16_bits((size * (0.5 + 0.5 * np.abs(np.sin(np.arange(B * K)))).astype(np.float32)).reshape(B, K)))
+        S = datagen.f32_to_bf16_bits(np.full((M, K // 128), scale, np.float32))
+        y_ref, mag = oracle.gemv_dense_blend(W, S, x)
+        assert np.isfinite(x).all() and (np.abs(y_ref) < 3.4e38).all()
+        y = bc.bitcos_gemv_blend_bf16(bc.bitcos_pack(W, S).to_device(), dev_bf16(datagen.f32_to_bf16_bits(x).reshape(B, K)))
+        err = np.abs(y.cpu().numpy().astype(np.float64) - y_ref)
+        assert (err <= REL * mag + 2.0 ** -140).all(), (size, scale, B, err.max())
+
+
 def test_blend_product_rejects_large_batches(bc):
     W, S = datagen.trits(4200, 64, 256, 0.4), datagen.scales(4200, 64, 256)
     with pytest.raises(bc.BitcosError) as e:

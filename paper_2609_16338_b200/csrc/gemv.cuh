@@ -2762,6 +2762,20 @@ inline void fill_first_copies(FirstCopies &c, const Problem &pr, const Plan &pl,
     c.bar = L.bar;
 }
 
+// Multiprocessors shared between n jobs in proportion to their items: cap[j] of at most sms altogether, at least one each.  (The
+// blocks that the smallest jobs are rounded up to come from the largest: no launch is wider than the machine, and of a
+// phased launch every block is resident.)
+inline void share_multiprocessors(const int64_t *items, int n, int sms, int64_t *cap) {
+    int64_t total = 0, sum = 0;
+    for (int j = 0; j < n; ++j) total += items[j];
+    for (int j = 0; j < n; ++j) {
+        cap[j] = items[j];
+        if (total > sms) cap[j] = std::max<int64_t>(1, items[j] * sms / total);
+        sum += cap[j];
+    }
+    for (; sum > std::max(sms, n); --sum) --*std::max_element(cap, cap + n);
+}
+
 // Grids of a multi launch: whether it runs two tiles per decoder warp, and each job's plan, walk
 // and number of thread blocks (the multiprocessors shared between the jobs in proportion to their
 // item counts).  Returns the total number of blocks.
@@ -2784,14 +2798,9 @@ inline int plan_multi(MultiArgs &ma, int nb_template, int sms, bool *two_out, in
     }
     *two_out = two;
     sms = small_launch_cap(total_items, sms);
-    int64_t cap[kMaxJobs], sum = 0;
-    for (int j = 0; j < ma.n; ++j) {
-        cap[j] = ma.pl[j].items;
-        if (total_items > sms) cap[j] = std::max<int64_t>(1, ma.pl[j].items * sms / total_items);
-        sum += cap[j];
-    }
-    // (the blocks that the smallest jobs were rounded up to come from the largest: no launch is wider than the machine)
-    for (; sum > std::max(sms, ma.n); --sum) --*std::max_element(cap, cap + ma.n);
+    int64_t items[kMaxJobs], cap[kMaxJobs];
+    for (int j = 0; j < ma.n; ++j) items[j] = ma.pl[j].items;
+    share_multiprocessors(items, ma.n, sms, cap);
     int next = 0;
     for (int j = 0; j < ma.n; ++j) {
         choose_walk(ma.pl[j], static_cast<int>(cap[j]), &grids[j]);
@@ -3059,19 +3068,15 @@ int launch_phased(PhasedArgs &pa, int n_jobs, const int *job_phase, cudaStream_t
     int grid = 1;
     for (int p = 0; p < pa.n_phases; ++p) {
         // the multiprocessors are shared between the phase's jobs in proportion to their item counts
-        int64_t total_items = 0;
+        int64_t items[kMaxJobs], cap[kMaxJobs];
+        int n = 0, next = 0;
         for (int j = 0; j < n_jobs; ++j)
-            if (job_phase[j] == p) total_items += pa.pl[j].items;
-        int next = 0;
-        for (int j = 0; j < n_jobs; ++j) {
+            if (job_phase[j] == p) items[n++] = pa.pl[j].items;
+        share_multiprocessors(items, n, sms, cap);
+        for (int j = 0, i = 0; j < n_jobs; ++j) {
             if (job_phase[j] != p) continue;
-            int64_t cap = pa.pl[j].items;
-            if (total_items > sms) {
-                cap = pa.pl[j].items * sms / total_items;
-                if (cap < 1) cap = 1;
-            }
             int blocks = 1;
-            choose_walk(pa.pl[j], static_cast<int>(cap), &blocks);
+            choose_walk(pa.pl[j], static_cast<int>(cap[i++]), &blocks);
             if (next + blocks > kMaxGrid) return BITCOS_ERR_SHAPE;
             pa.pl[j].NW = layout.NW;
             pa.pl[j].stages = layout.stages;

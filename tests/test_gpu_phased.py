@@ -65,6 +65,24 @@ def test_decoder_layer_in_one_launch(bc, B):
         assert torch.equal(j[3], y0)
 
 
+def test_a_large_job_beside_six_of_one_block(bc):
+    """Every job of a phase gets a block, and together they are no more than the multiprocessors: a block that was not
+    resident would hold up the phase that follows until the bounded waits run out."""
+    shapes = [(32, 128)] * 6 + [(19200, 2560), (2560, 2560)]
+    jobs, _ = make_jobs(bc, shapes, 1, 4050)
+    for rep in range(2):
+        for j in jobs:
+            j[3].fill_(float("nan"))
+        bc.bitcos_gemv_phased(jobs, [0] * 7 + [1], bc.make_phased_sync())
+        torch.cuda.synchronize()
+        assert not any(bc.workspace_status(j[4]) for j in jobs)
+    phased = [j[3].clone() for j in jobs]
+    bc.bitcos_gemv_multi(jobs[:7])
+    bc.bitcos_gemv_multi(jobs[7:])
+    torch.cuda.synchronize()
+    assert all(torch.equal(j[3], y0) for j, y0 in zip(jobs, phased))
+
+
 def test_odd_shapes_and_phase_layouts(bc):
     """Ragged row counts, rows cut into column blocks, a phase with one tiny job, two phases only,
     a single phase, and all four phases with one job each."""

@@ -380,7 +380,10 @@ def _stream() -> int:
     if _raw_stream is None:
         import torch
         torch.cuda.init()
-        _raw_stream = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+        try:
+            _raw_stream = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+        except AttributeError:              # (names that torch does not promise)
+            _raw_stream = (lambda device: torch.cuda.current_stream(device).cuda_stream), torch.cuda.current_device
     stream, device = _raw_stream
     return stream(device())
 

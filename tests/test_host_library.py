@@ -150,6 +150,20 @@ def test_error_codes():
                        None, C.c_void_p(16), 8, None) == 6
 
 
+def test_stream_handle_without_torchs_private_names(monkeypatch):
+    """The binding takes the current stream's handle from names that torch does not promise; where they are
+    missing, from the public ones."""
+    torch = pytest.importorskip("torch")
+    from types import SimpleNamespace
+    from paper_2609_16338_b200 import binding
+    monkeypatch.setattr(binding, "_raw_stream", None)
+    monkeypatch.setattr(torch.cuda, "init", lambda: None)
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 3)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda device: SimpleNamespace(cuda_stream=1000 + device))
+    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)
+    assert binding._stream() == 1003
+
+
 def test_group_pairs_helper():
     order, ge, gb, xr, mx = bc.group_pairs([5, 2, 5, 7, 2, 5], [0, 0, 1, 1, 2, 2])
     assert list(ge) == [2, 5, 7] and list(gb) == [0, 2, 5, 6] and mx == 3

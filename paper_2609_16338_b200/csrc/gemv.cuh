@@ -1773,8 +1773,8 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
     }
     if (warp == 0 && lane == 0) BITCOS_TL(3, clock64());
     bool tl_first = true;
-    constexpr int RS = red_slots(NB);
     constexpr bool kMma = NB >= kMmaMinBatch;          // contraction on the tensor cores
+    static_assert(kFrag || !kXG || NB == 1, "group scales and 16-bit activations: one token here, from two on in fragment order");
     constexpr int NH = NB > 8 ? 2 : 1;                 // 8-token halves of the batch
     constexpr int NV = kMma ? NH * 8 : NB;             // partial sums a lane hands to the epilogue warp
     const uint32_t lane4 = static_cast<uint32_t>(lane) * 4u;
@@ -1795,17 +1795,9 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
         }
     };
     uint32_t bf[NH][8];
-    float xgq[NH][2];           // group scales of the two tokens whose accumulators this lane holds
     auto load_bf = [&](int g) {
 #pragma unroll
         for (int h = 0; h < NH; ++h) {
-            if (kXG && !kXQ) {
-#pragma unroll
-                for (int r = 0; r < 2; ++r) {
-                    const int b = 8 * h + 2 * (lane & 3) + r;
-                    xgq[h][r] = (b < pr.nb(pb)) ? __ldg(pb.x_scale + static_cast<int64_t>(b) * pb.G + g) : 0.f;
-                }
-            }
             int4 u0 = make_int4(0, 0, 0, 0), u1 = make_int4(0, 0, 0, 0);
             if (xfrag[h]) {
                 const int4 *px = reinterpret_cast<const int4 *>(xfrag[h] + static_cast<int64_t>(g) * kGroup);
@@ -1840,11 +1832,11 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
     float *rd_lane0 = red + static_cast<uint32_t>(warp * NB) * kRows + lane;
     int kk = 0;                 // items decoded so far, over all segments
     bool x_ready = false;
-    // 16-bit activations: the group this warp has quantised last, its scales, and its buffer
-    // ([token][128] int8 inside the activation area)
+    // 16-bit activations (one token): the group this warp has quantised last, its scale, and its buffer
+    // (128 int8 inside the activation area)
     int q_g = -1;
-    float q_scale[NB < kMmaMinBatch ? NB : 1] = {};
-    uint32_t *q_scr = reinterpret_cast<uint32_t *>(smem + L.x) + static_cast<uint32_t>(warp) * (NB * kRows);
+    float q_scale = 0.f;
+    uint32_t *q_scr = reinterpret_cast<uint32_t *>(smem + L.x) + static_cast<uint32_t>(warp) * kRows;
     bool more_segments = false;
     do {
     if (!(kLate && kMma)) {
@@ -1889,15 +1881,10 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
         // early, so that the decode hides the latency (not before the dependency is resolved)
         if (kMma && pl.CS != 1 && busy && (!kLate || x_ready)) load_bf(g);
         // 16-bit activations of a group this warp has not quantised yet: fetched ahead of the decode too
-        uint2 qv[NB < kMmaMinBatch ? NB : 1];
+        uint2 qv;
         bool q_have = false;
         auto fetch_group = [&]() {
-#pragma unroll
-            for (int b = 0; b < NB; ++b)
-                if (NB == 1 || b < pr.nb(pb))
-                    qv[NB < kMmaMinBatch ? b : 0] =
-                        __ldg(reinterpret_cast<const uint2 *>(reinterpret_cast<const uint16_t *>(pb.x) + static_cast<int64_t>(b) * pb.K +
-                                                              static_cast<int64_t>(g) * kGroup) + lane);
+            qv = __ldg(reinterpret_cast<const uint2 *>(reinterpret_cast<const uint16_t *>(pb.x) + static_cast<int64_t>(g) * kGroup) + lane);
             q_have = true;
         };
         if (kXQ && busy && x_ready && g != q_g) fetch_group();
@@ -1980,7 +1967,6 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
 #pragma unroll
                         for (int r = 0; r < 4; ++r) {
                             ysum[(h * 2 + mh) * 4 + r] = scq[2 * mh + (r >> 1)] * static_cast<float>(acc[h][mh][r]);
-                            if (kXG) ysum[(h * 2 + mh) * 4 + r] *= xgq[h][r & 1];
                             if (Segs::kDebug && pb.acc_debug) {
                                 const int b = 8 * h + 2 * (lane & 3) + (r & 1);
                                 const int64_t m = (static_cast<int64_t>(d.z) + my_rbl) * kRows + 16 * mh + (lane >> 2) + 8 * (r >> 1);
@@ -2008,44 +1994,28 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
             }
             if (kXQ && g != q_g) {
                 // 16-bit activations: this warp quantises the group its tile multiplies (four values
-                // per lane, largest magnitude by shuffles) into its own 128 bytes per token
+                // per lane, largest magnitude by shuffles) into its own 128 bytes
                 if (!q_have) fetch_group();        // (first tile: the dependency has only just been resolved)
                 __syncwarp();                     // the previous tile's contraction has read the buffer
+                float a = fmaxf(fmaxf(fabsf(bf16_lo(qv.x)), fabsf(bf16_hi(qv.x))), fmaxf(fabsf(bf16_lo(qv.y)), fabsf(bf16_hi(qv.y))));
 #pragma unroll
-                for (int b = 0; b < NB; ++b) {
-                    if (NB == 1 || b < pr.nb(pb)) {
-                        const uint2 v = qv[NB < kMmaMinBatch ? b : 0];
-                        float a = fmaxf(fmaxf(fabsf(bf16_lo(v.x)), fabsf(bf16_hi(v.x))),
-                                        fmaxf(fabsf(bf16_lo(v.y)), fabsf(bf16_hi(v.y))));
-#pragma unroll
-                        for (int dd = 16; dd; dd >>= 1) a = fmaxf(a, __shfl_xor_sync(0xFFFFFFFFu, a, dd));
-                        a = fmaxf(a, kAmaxFloor);
-                        const float inv = __fdiv_rn(127.0f, a);
-                        q_scale[NB < kMmaMinBatch ? b : 0] = __fdiv_rn(a, 127.0f);
-                        q_scr[b * kRows + lane] = quant_pair(v.x, inv) | (quant_pair(v.y, inv) << 16);
-                    }
-                }
+                for (int dd = 16; dd; dd >>= 1) a = fmaxf(a, __shfl_xor_sync(0xFFFFFFFFu, a, dd));
+                a = fmaxf(a, kAmaxFloor);
+                const float inv = __fdiv_rn(127.0f, a);
+                q_scale = __fdiv_rn(a, 127.0f);
+                q_scr[lane] = quant_pair(qv.x, inv) | (quant_pair(qv.y, inv) << 16);
                 __syncwarp();
                 q_g = g;
             }
-            float xgs[NB < kMmaMinBatch ? NB : 1];
-            if (kXQ) {
-#pragma unroll
-                for (int b = 0; b < NB; ++b) xgs[NB < kMmaMinBatch ? b : 0] = q_scale[NB < kMmaMinBatch ? b : 0];
-            } else if (kXG && !kMma) {
-                // (after the dependency wait: the scales come from the kernel before this one)
-#pragma unroll
-                for (int b = 0; b < NB; ++b)
-                    if (NB == 1 || b < pr.nb(pb))
-                        xgs[NB < kMmaMinBatch ? b : 0] = __ldg(pb.x_scale + static_cast<int64_t>(b) * pb.G + g);
-            }
+            // (after the dependency wait: the scales come from the kernel before this one)
+            const float xgs = kXQ ? q_scale : kXG ? __ldg(pb.x_scale + g) : 1.f;
 #pragma unroll
             for (int b = 0; b < NB; ++b) {
                 if (kMma) break;
                 if (NB == 1 || b < pr.nb(pb)) {       // a call has at least one token
                     const int a = contract<FMT>(w, reinterpret_cast<const int4 *>(xs + static_cast<uint32_t>(b) * (kXQ ? static_cast<uint32_t>(kGroup) : static_cast<uint32_t>(x_stride(pb.K)))), lane);
                     ysum[b] = sc * static_cast<float>(a);
-                    if (kXG) ysum[b] *= xgs[NB < kMmaMinBatch ? b : 0];
+                    if (kXG) ysum[b] *= xgs;
                     if (Segs::kDebug && pb.acc_debug) {
                         const int64_t m = (static_cast<int64_t>(d.z) + my_rbl) * kRows + lane;
                         if (m < pb.M) pb.acc_debug[((pr.out_row0(pb) + b) * pb.M + m) * pb.G + g] = a;

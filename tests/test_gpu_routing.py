@@ -1,4 +1,4 @@
-"""Routed products: the device's grouping of the pairs, and the grouped kernels' token parts and tile pairs.
+"""Routed products: the device's grouping of the pairs, and the grouped kernels' token parts.
 
 bitcos_group_pairs_device against the host's stable grouping: one pair, warps and blocks of pairs with remainders, the
 largest list, every expert the same, expert ids out of range (dropped; the rest of the lists filled)."""
@@ -49,9 +49,9 @@ def dev(a):
 @pytest.mark.parametrize("M,K,experts,most", [(768, 2048, 28, 16), (2048, 640, 32, 16), (2000, 768, 28, 8), (96, 640, 40, 16), (1000, 4096, 12, 13),
                                               (640, 1280, 30, 2), (64, 128, 8, 16)])
 def test_groups_of_every_size(bc, M, K, experts, most):
-    """Groups of 1 .. most tokens, both sides of the line from which a warp takes two tiles (64 tiles per multiprocessor),
-    odd numbers of groups of 128; more than eight tokens of a group run as two parts.  One group too many tokens, one
-    expert that does not exist, an empty group: skipped, the two malformed ones with status 2."""
+    """Groups of 1 .. most tokens, rows in one piece (one flat list of items; more than eight tokens of a group run as two
+    parts) and rows cut into column blocks (K = 4096), odd numbers of groups of 128.  One group with too many tokens, one
+    that names no expert, an empty group: skipped, the two malformed ones with status 2."""
     Ws = [datagen.trits(60 + e % 5, M, K, 0.33) for e in range(experts)]
     Ss = [datagen.scales(60 + e, M, K) for e in range(experts)]
     E = bc.DeviceExperts([bc.bitcos_pack(Ws[e], Ss[e]).to_device() for e in range(experts)])
@@ -70,15 +70,14 @@ def test_groups_of_every_size(bc, M, K, experts, most):
     # group 3 takes all of group 4's pairs and more (too many), group 6 names no expert
     bad_begin, bad_expert = begin.copy(), group_expert.copy()
     bucket = next(b for b in (1, 2, 4, 8, 16) if b >= most)
-    if begin[6] - begin[3] > bucket:
-        bad_begin[4:6] = begin[6]
+    assert begin[6] - begin[3] > bucket
+    bad_begin[4:6] = begin[6]
     bad_expert[6] = experts
     ws = bc.make_workspace(M, K, copies=experts)
     y2 = torch.full_like(y, 7.0)
     bc.bitcos_gemv_grouped(E, dev(bad_expert), dev(bad_begin), dev(rows), most, dev(x), dev(xs), y=y2, workspace=ws)
     want = y.clone()
     want[begin[6]:begin[7]] = 7.0
-    if begin[6] - begin[3] > bucket:
-        want[begin[3]:begin[6]] = 7.0
+    want[begin[3]:begin[6]] = 7.0
     assert torch.equal(y2, want)
     assert bc.workspace_status(ws) == 2

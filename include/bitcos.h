@@ -238,11 +238,11 @@ int bitcos_decode_probe_variant(int variant, const uint32_t *bitmap, const uint3
  * entry offset + running population count locate each row's sign window, a 256-entry
  * (presence nibble, sign nibble) table as in Eq. 4 rebuilds four weights at a time as int8,
  * dp4a accumulates int32 per group, the bf16 group scale and the per-token scale are applied
- * in fp32).  The paper measures one token; for batch >= 3 the same int32 group accumulators come
- * from int8 tensor-core instructions (mma.m16n8k32) fed with the decoded rows, so that the weights
- * are decoded once per call whatever the batch.  The accumulators are exact for every batch; y is
- * deterministic for a given batch size and device (fixed summation order), and the summation
- * order over groups may differ between batch sizes.
+ * in fp32).  The paper measures one token; for batch >= 2 the same int32 group accumulators come
+ * from int8 tensor-core instructions (mma.m16n8k32), for whose operand order the tiles are decoded, so
+ * that the weights are decoded once per call whatever the batch.  The accumulators are exact for every
+ * batch; y is deterministic for a given batch size and device (fixed summation order, the same with and
+ * without the accumulator dump), and the summation order over groups may differ between batch sizes.
  *   W            host struct holding device pointers
  *   x            device int8 [batch][K], row major
  *   x_scale      device float [batch]
@@ -456,7 +456,7 @@ typedef struct bitcos_gemv_host_job {
 } bitcos_gemv_host_job;
 int bitcos_gemv_multi_host(const bitcos_gemv_host_job *jobs, int n_jobs, int batch, void *cuda_stream);
 
-/* A whole sequence of phases from host buffers with ONE copy in, ONE copy out and ONE wait: the
+/* A whole sequence of phases from host buffers with one block in, one block out and ONE wait: the
  * host-buffer form for callers that run several dependent products per step (a decoder layer's
  * q | k | v, o, gate | up, down) and keep activations and results on the host.  The caller lays every
  * job's x and x_scale out inside one device block `in_device` (and the same bytes, at the same
@@ -464,7 +464,8 @@ int bitcos_gemv_multi_host(const bitcos_gemv_host_job *jobs, int n_jobs, int bat
  * `out_device`; jobs[] holds the DEVICE addresses, as for bitcos_gemv_multi.  The call copies
  * in_host -> in_device (in_bytes), runs one launch per phase (job_phase as for bitcos_gemv_phased;
  * each launch is told its neighbours as by bitcos_gemv_multi_chained), copies out_device ->
- * out_host (out_bytes) and waits for the stream, so out_host is valid on return.  Pinned host
+ * out_host (out_bytes) and waits for the stream, so out_host is valid on return and holds out_device as the
+ * last phase left it (a replay, below, copies outputs that no later phase writes while the later phases run).  Pinned host
  * blocks keep the two copies asynchronous until the wait.
  * Replay: the second call with the same arguments (every pointer, size and descriptor field
  * compared by value) records the step as a CUDA graph on a stream of the library's own; that call and
@@ -495,7 +496,8 @@ int bit2_gemv(const uint32_t *words, const uint16_t *scales_tiled, int64_t M, in
  * The caller lists the P (token, expert) pairs grouped by expert: group i covers pairs
  * group_begin[i] .. group_begin[i+1]-1 (at most max_group_size <= 16 per group), all using expert
  * group_expert[i]; pair p reads activation row pair_xrow[p] of x[n_xrows][K] and writes y[p][M].
- * Each listed expert's packed bytes are read once.  No activation function, routing weight
+ * Each listed expert's packed bytes are read once, those of a group of more than 8 pairs (BITCOS, K <= 2560)
+ * twice, the second time from L2: such a group runs as two.  No activation function, routing weight
  * or sum over experts is applied (the paper runs its mixture-of-experts checkpoints end to end only,
  * Table I; this is the per-expert product such a layer needs).
  *   experts       device array of bitcos_weights (device pointers inside), n_experts entries

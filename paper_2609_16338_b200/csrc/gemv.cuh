@@ -358,7 +358,10 @@ __host__ __device__ constexpr int64_t x_stride(int64_t K) { return K + 16; }
 __host__ __device__ constexpr bool fragment_order(int fmt, int nb) { return fmt == kBitcos && nb >= 2; }
 
 // Tiles per warp in large launches (wants_two_tiles): two, or three with the fourteen decoder warps of more than eight tokens, which two
-// tiles each would leave four of idle where rows have 20 or 40 groups (25600x5120 at sixteen tokens 27.1 -> 24.7 us).
+// tiles each would leave four of idle where rows have 20 or 40 groups (25600x5120 at sixteen tokens 27.1 -> 24.7 us).  At
+// other lengths three tiles fill fewer warps (28 or 56 groups: 10 of 14, 22 or 43: 8); against one tile per warp they
+// are faster at all of them (32000 tiles at sixteen tokens, rows of 14, 22, 28, 43 and 56 groups: 35.3 -> 27.4, 35.8 -> 29.2, 33.2 -> 26.7,
+// 42.5 -> 32.9, 30.6 -> 26.9 us), two tiles per warp have not been measured there.
 __host__ __device__ constexpr int wide_tiles(int fmt, int nb) { return fragment_order(fmt, nb) && nb > 8 ? 3 : 2; }
 
 // The plan with one tile per warp.

@@ -24,6 +24,7 @@ import json
 import os
 import subprocess
 import sys
+import tempfile
 import threading
 import time
 
@@ -627,7 +628,10 @@ def run_cuda(args):
         line["moe"] = moe_detail(bc, torch, stream)
     if args.all_configs:
         line["device_pack"] = pack_detail(bc, torch)
-    print(json.dumps(line))
+    if args.tables:
+        with open(args.tables, "w") as f:
+            json.dump(line, f, indent=1)
+    print(json.dumps(short_line(line, args.tables)))
     ranks.close()
 
 
@@ -658,6 +662,26 @@ def quantised_layer_steps(bc, torch, layer, groups, replicas, ys, wss):
             bc.bitcos_gemv_multi_bf16(mj)
 
     return step_q, step_b
+
+
+def short_line(line, tables):
+    """What is printed: one line short enough for a log that keeps only the end of a run's output.  How each figure was
+    taken in words, the spreads and the tables of all configurations are in the file `tables`."""
+    def five(v):
+        return float("%.6g" % v) if isinstance(v, float) else v
+
+    def some(name, *keys):
+        return {k: five(line[name][k]) for k in keys}
+
+    out = {k: five(v) for k, v in line.items() if not isinstance(v, (dict, list))}
+    out["config"] = some("config", "workload", "batch", "algorithmic_bytes_per_step", "replicas")
+    out["config"]["l2"] = "rotated copies larger than L2"
+    out["roofline"] = some("roofline", "bound", "achieved", "peak", "unit", "frac", "traffic")
+    out["cpu_baseline"] = some("cpu_baseline", "value", "unit", "cores", "kind")
+    out["e2e"] = some("e2e", "value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "steps")
+    out["clocks"] = line["clocks"]
+    out["tables"] = tables
+    return out
 
 
 def two_term_roofline(bc, z, peak_gbs, sm_mhz, sms=148):
@@ -1109,6 +1133,8 @@ def moe_detail(bc, torch, stream, E=128, top_k=8, z=0.3288):
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
+    ap.add_argument("--tables", default=os.path.join(tempfile.gettempdir(), "bitcos_bench_tables.json"),
+                    help="file for the tables of all configurations and the full line (empty: none)")
     ap.add_argument("--steps", type=int, default=None)
     ap.add_argument("--warmup", type=int, default=3)
     ap.add_argument("--impl", default="cuda", choices=["cuda", "reference"])

@@ -472,7 +472,7 @@ def bitcos_gemv_bf16(W: DeviceBitcos, x_bf16, y=None, acc_debug=None, workspace=
 
 
 def bitcos_gemv_blend_bf16(W: DeviceBitcos, x_bf16, y=None, workspace=None):
-    """The 16-bit variant: weights rebuilt as +-s times unquantised bfloat16 activations [batch, K], batch 1..8."""
+    """The 16-bit variant: weights times unquantised bfloat16 activations [batch, K], the bf16 scales applied per group; batch 1..8."""
     _check_bf16(x_bf16)
     batch = x_bf16.size(0)
     if workspace is None:

@@ -69,15 +69,15 @@ struct LutBig {
     uint32_t v[kLutBytes / 4];
 };
 
-// BITCOS: byte address = key * 256 + sub * 128 + lane * 4;
+// BITCOS: byte address = sub * 32768 + key * 128 + lane * 4;
 //   sub 0 ("even" nibbles): key = (s << 4) | m;  sub 1 ("odd" nibbles): key = (m << 4) | s,
-// so that a presence BYTE placed in address bits 8..15 needs only its other nibble replaced
+// so that a presence BYTE placed in address bits 7..14 needs only its other nibble replaced
 // by the four sign bits.
 constexpr LutBig make_bitcos_lut() {
     const Lut256 base = make_nibble_lut();
     LutBig t{};
     for (int idx = 0; idx < kLutBytes / 4; ++idx) {
-        const int key = idx >> 6, sub = (idx >> 5) & 1;
+        const int key = (idx >> 5) & 255, sub = idx >> 13;
         const int src = sub ? (((key & 15) << 4) | (key >> 4)) : key;
         t.v[idx] = base.v[src];
     }
@@ -203,6 +203,43 @@ __device__ __forceinline__ void bitcos_decode_row(const uint4 bm, const uint32_t
     }
 }
 
+// ---------------------------------------------------------------------------------------------
+// Decoder A as the products run it at one token: a row's 32 int8x4 words as above, with 32 instructions less and with sixteen
+// more of them off the integer pipe.  An unsigned dp4a with 0x80 at byte k puts presence byte k of a word on address bits 7 .. 14 and adds
+// lane * 4, where a byte permutation took that pipe; a word's sign window stays where it is and is
+// rotated by a running position, to which dp4a(e, e, pos) adds a nibble's population count, where the window was
+// moved up for the key and down by the count.  Clocks per tile and multiprocessor at one token (18944 -> 56832 x 5120, 4096 ->
+// 18944 x 12288): 105.7 -> 102.1, 113.5 -> 108.5; the running position alone 104.1, 110.4, the dp4a key alone 104.4, 113.2.
+// ---------------------------------------------------------------------------------------------
+__device__ __forceinline__ uint32_t presence_key(uint32_t word, int k, uint32_t lane4) { return dp4a_uu(word, 0x80u << (8 * k), lane4); }
+constexpr uint32_t kOddTable = kLutBytes / 2;
+
+__device__ __forceinline__ void bitcos_decode_row_keyed(const uint4 bm, const uint32_t *sp, uint32_t sh, const uint8_t *lut, uint32_t lane4,
+                                                        int (&w)[32]) {
+    uint32_t A[4], B[4];
+    sign_windows(bm, sp, sh, A);
+    const uint32_t P[4] = {bm.x, bm.y, bm.z, bm.w};
+    int pos[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        B[j] = __funnelshift_r(A[j], A[j], 4);
+        pos[j] = 21;                                  // a right rotation by 21 puts bit 0 on bit 11 (of B: bit 4 on bit 7)
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t R = presence_key(P[j], k, lane4);
+            int e = static_cast<int>(lds32(lut, bit_select(__funnelshift_r(A[j], A[j], pos[j]), R, 0x7800u)));
+            w[8 * j + 2 * k] = e;
+            pos[j] = __dp4a(e, e, pos[j]);
+            e = static_cast<int>(lds32(lut + kOddTable, bit_select(__funnelshift_r(B[j], B[j], pos[j]), R, 0x0780u)));
+            w[8 * j + 2 * k + 1] = e;
+            if (k < 3) pos[j] = __dp4a(e, e, pos[j]);
+        }
+    }
+}
+
 // Inclusive scan over the lanes of a warp (the shuffle's own in-range predicate guards each addition).
 __device__ __forceinline__ uint32_t warp_scan_add(uint32_t v) {
 #pragma unroll
@@ -234,7 +271,7 @@ __device__ __forceinline__ uint32_t dp2a_lo(uint32_t a, uint32_t b, uint32_t c) 
 // scans of the population counts, two to a register (a tile has at most 4096 non-zeros).
 // Every word keeps its sign window fixed and a running position: dp4a(e, e, pos) adds a nibble's
 // population count in the instruction that computes it, and one rotate brings the next four sign bits to
-// bits 12..15 (even nibbles; from a copy turned by four, to bits 8..11 for odd ones).
+// bits 11..14 (even nibbles; from a copy turned by four, to bits 7..10 for odd ones).
 // ---------------------------------------------------------------------------------------------
 struct FragmentRows {
     uint32_t P[4], A[4], B[4];
@@ -257,20 +294,19 @@ struct FragmentRows {
             const uint32_t o = (at[i] >> 3) & ~3u;
             A[i] = __funnelshift_r(lds32(sg, o), lds32(sg, o + 4u), at[i]);
             B[i] = __funnelshift_r(A[i], A[i], 4);
-            pos[i] = 20;                              // a right rotation by 20 puts bit 0 on bit 12
+            pos[i] = 21;                              // a right rotation by 21 puts bit 0 on bit 11
         }
     }
     // fragment registers of byte k (nibbles 2 k and 2 k + 1) of the four rows: e[2 i], e[2 i + 1]
     __device__ __forceinline__ void step(int k, const uint8_t *lut, uint32_t lane4, int (&e)[8]) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            // address bits 0..6 = lane * 4, bits 8..15 = presence byte k (bits 16.. are 0)
-            const uint32_t R = __byte_perm(P[i], lane4, 0x6504 | (k << 4));
+            const uint32_t R = presence_key(P[i], k, lane4);
             uint32_t t = __funnelshift_r(A[i], A[i], pos[i]);
-            e[2 * i] = static_cast<int>(lds32(lut, bit_select(t, R, 0xF000u)));
+            e[2 * i] = static_cast<int>(lds32(lut, bit_select(t, R, 0x7800u)));
             pos[i] = __dp4a(e[2 * i], e[2 * i], pos[i]);
             t = __funnelshift_r(B[i], B[i], pos[i]);
-            e[2 * i + 1] = static_cast<int>(lds32(lut + 128, bit_select(t, R, 0x0F00u)));
+            e[2 * i + 1] = static_cast<int>(lds32(lut + kOddTable, bit_select(t, R, 0x0780u)));
             if (k < 3) pos[i] = __dp4a(e[2 * i + 1], e[2 * i + 1], pos[i]);
         }
     }
@@ -280,7 +316,10 @@ struct FragmentRows {
     // high byte is 59 or 187, both 27 modulo 32, so 19 times its high byte counts 1 in the five bits that a rotation uses.
     __device__ __forceinline__ void shift_presence() {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) B[i] = P[i] >> 4;
+        for (int i = 0; i < 4; ++i) {
+            B[i] = P[i] >> 4;
+            pos[i] = 20;                              // its keys lie one bit higher
+        }
     }
     __device__ __forceinline__ void step_bf16(int j, const uint8_t *lut, uint32_t lane8, uint32_t (&e)[8]) {
 #pragma unroll

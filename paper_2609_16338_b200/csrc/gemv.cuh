@@ -1912,7 +1912,7 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
                 const uint32_t toff = *reinterpret_cast<const uint32_t *>(stage + off_toff + ((d.x >> 8) << 2));
                 const uint32_t cursor = toff + static_cast<uint32_t>(incl - c) - d.w;
                 const uint32_t *sp = reinterpret_cast<const uint32_t *>(stage + off_sign + ((cursor >> 5) << 2));
-                bitcos_decode_row(bm, sp, cursor & 31u, lut, lane4, w);
+                bitcos_decode_row_keyed(bm, sp, cursor & 31u, lut, lane4, w);
             } else if (FMT == kTrit5) {
                 const int WPR = (26 * pb.G + 3) / 4;
                 // words of the stage: row block my_rbl of the chunk, counted from the chunk's first word

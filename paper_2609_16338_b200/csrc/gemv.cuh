@@ -476,6 +476,19 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
     return mbar_wait_slow(bar, parity);
 }
 
+// Four additions, packed in two instructions where the registers allow it (with sixteen tokens the pairs cost copies: 32B-model layer
+// 103.7 -> 105.8 us).
+template <bool PACKED>
+__device__ __forceinline__ float4 add_quads(float4 a, float4 b) {
+    if (!PACKED) return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
+    float4 c;
+    asm("{\n\t.reg .b64 x, y;\n\tmov.b64 x, {%4, %5};\n\tmov.b64 y, {%8, %9};\n\tadd.rn.f32x2 x, x, y;\n\tmov.b64 {%0, %1}, x;\n\t"
+        "mov.b64 x, {%6, %7};\n\tmov.b64 y, {%10, %11};\n\tadd.rn.f32x2 x, x, y;\n\tmov.b64 {%2, %3}, x;\n\t}"
+        : "=f"(c.x), "=f"(c.y), "=f"(c.z), "=f"(c.w)
+        : "f"(a.x), "f"(a.y), "f"(a.z), "f"(a.w), "f"(b.x), "f"(b.y), "f"(b.z), "f"(b.w));
+    return c;
+}
+
 // Four 8x8 matrices of 16-bit elements from shared memory, one row address per lane: as int8 data
 // this is exactly the A operand (16 rows x 32 bytes) of mma.m16n8k32.
 __device__ __forceinline__ void ldmatrix_x4(uint32_t (&a)[4], uint32_t addr) {
@@ -849,7 +862,9 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
                                              bool first_sent = false) {
     // first_sent: the caller has already initialised the barriers of stage 0 and of the lookup table
     // and issued the table's copy and the copies of this block's first item (send_first_copies)
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // (through a shuffle, so that what depends on it is in uniform registers; not with sixteen tokens, 170.5 -> 174 clocks per tile)
+    const int warp = NB > 8 ? static_cast<int>(threadIdx.x >> 5) : __shfl_sync(0xFFFFFFFFu, static_cast<int>(threadIdx.x >> 5), 0);
+    const int lane = threadIdx.x & 31;
     const int prod_warp = static_cast<int>(blockDim.x >> 5) - 1;      // the producer: always the block's last warp
     if (static_cast<int>(threadIdx.x) == prod_warp * 32) BITCOS_TL(16, clock64());
     // The problem and the plan of the segment a warp role is working on.  The plain and the grouped
@@ -1187,22 +1202,34 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
         // Tensor-core layout: four tokens at a time, spaced one warp's rows apart; more than eight tiles in two batches of ten,
         // all loads of a batch before its first addition (three smaller batches cost the sixteen-token layer 3 %).
         constexpr int RF = NB;
-        auto add4 = [](float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); };
+        auto add4 = [](float4 a, float4 b) { return add_quads<(NB <= 8)>(a, b); };
         const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
+        // (A guarded load takes four instructions.  A batch that is full, or as long as the second one of rows of 16 or 18 groups, has none:
+        // with packed additions and the warp's number in uniform registers MoE pass of 128 experts 57.6 -> 56.2 us, 18944 -> 56832 x 5120
+        // at four | eight tokens 121 | 127 -> 117 | 126 clocks per tile.)
+        auto batch = [&](auto size, const float *base, int n) {
+            constexpr int N = decltype(size)::value;         // tiles, 0: n of them
+            float4 v[10];
+#pragma unroll
+            for (int j = 0; j < 10; ++j) v[j] = (N ? j < N : j < n) ? *reinterpret_cast<const float4 *>(base + j * kRows * RF) : none;
+#pragma unroll
+            for (int w2 = 1; w2 < 10; w2 *= 2)
+#pragma unroll
+                for (int j = 0; j + w2 < 10; j += 2 * w2)
+                    if (!N || j + w2 < N) v[j] = add4(v[j], v[j + w2]);
+            return v[0];
+        };
         auto in_tens = [&](const float *base, int n) {
-            float4 tot = none;
-#pragma unroll
-            for (int j0 = 0; j0 < kMaxWarps; j0 += 10) {
-                float4 v[10];
-#pragma unroll
-                for (int j = 0; j < 10; ++j) v[j] = (j0 + j < n) ? *reinterpret_cast<const float4 *>(base + (j0 + j) * kRows * RF) : none;
-#pragma unroll
-                for (int w2 = 1; w2 < 10; w2 *= 2)
-#pragma unroll
-                    for (int j = 0; j + w2 < 10; j += 2 * w2) v[j] = add4(v[j], v[j + w2]);
-                tot = add4(tot, v[0]);
-            }
-            return tot;
+            if constexpr (NB > 8) return add4(batch(std::integral_constant<int, 0>{}, base, n), batch(std::integral_constant<int, 0>{}, base + 10 * kRows * RF, n - 10));
+            if (n < 10) return batch(std::integral_constant<int, 0>{}, base, n);
+            const float4 tot = batch(std::integral_constant<int, 10>{}, base, 10);
+            base += 10 * kRows * RF;
+            n -= 10;
+            if (n == 0) return tot;
+            if (n == 10) return add4(tot, batch(std::integral_constant<int, 10>{}, base, n));
+            if (n == 6) return add4(tot, batch(std::integral_constant<int, 6>{}, base, n));
+            if (n == 8) return add4(tot, batch(std::integral_constant<int, 8>{}, base, n));
+            return add4(tot, batch(std::integral_constant<int, 0>{}, base, n));
         };
         auto sum_tiles4 = [&](const float *base, int n) {
             if (n > 8) return in_tens(base, n);
@@ -1231,8 +1258,13 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
             auto at = [&](int j) { return *reinterpret_cast<const float4 *>(base + j * kRows * RF); };
             if (n > 4) {
                 float4 v[10];
+                if (n == 10) {
 #pragma unroll
-                for (int j = 0; j < 10; ++j) v[j] = (j < 5 || j < n) ? at(j) : none;
+                    for (int j = 0; j < 10; ++j) v[j] = at(j);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 10; ++j) v[j] = (j < 5 || j < n) ? at(j) : none;
+                }
                 return add4(add4(add4(add4(v[0], v[1]), add4(v[2], v[3])), v[4]), add4(add4(add4(v[5], v[6]), add4(v[7], v[8])), v[9]));
             }
             float4 tot = none;

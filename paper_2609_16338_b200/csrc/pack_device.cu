@@ -1,18 +1,23 @@
 // Device-side BITCOS packer: dense int8 trits and row-major bf16 scales in device memory -> the
 // four packed buffers of the layout in bitcos.h (Section II-A of the paper: presence bitmap,
 // compacted sign vector in the same order; entry offsets per tile), byte for byte what the host
-// packer writes.  Three kernels: bitmap + scales + per-tile counts (and the sign vector zeroed); an exclusive
-// scan of the counts (the entry offsets); the sign vector.  One warp per 32 x 128 tile.
+// packer writes.  One warp per 32 x 128 tile.
 //
-// Bound by memory: the trits (a byte each) are read twice, the second time from L2 where they fit there.
-// Eight lanes take a row's 128 bytes, 16 weights a lane, four rows a load: whole lines, where one lane per row
-// (the products' order) touched 32 rows a load at half a sector each.  Those 16-weight chunks in the order (load, lane)
-// are the tile's weights in order, so the masks go out as 16-bit stores of 64 bytes a warp, and the sign bits
-// of a chunk lie where a scan of the chunk counts puts them.
+// Bound by memory: a byte a weight read, an eighth of one written twice.  Eight lanes take a row's 128 bytes, 16 weights a lane, four rows
+// a load: whole lines, where one lane per row (the products' order) touched 32 rows a load at half a sector each.  Those
+// 16-weight chunks in the order (load, lane) are the tile's weights in order, and the sign bits of a chunk lie where a
+// scan of the chunk counts puts them.
 //
-// 8192x5120 (42 MB of trits), a whole call through the binding: 156 -> 89 us.  The kernels take 35 of them (13 + 6 + 19
-// before they overlapped, from L2 at the second reading), the rest is one wait for the stream and the caller's
-// allocations; two waits, two fills, the offsets copied out and a copy of the sign vector by the copy engine went.
+// Where a tile's sign bits go is known only when everything before it has been counted.  From kOnceMin tiles up to kOnceTiles per
+// multiprocessor one kernel does all of it (pack_once_kernel): a block keeps the compacted sign bits of its tiles in shared memory
+// until every block has counted, so that the trits are read and looked at once.  Smaller matrices (a cooperative launch costs the
+// caller about 8 us more than an ordinary one), larger ones and calls that find no state to share take three kernels:
+// bitmap + scales + per-tile counts (and the sign vector zeroed); an exclusive scan of the counts (the entry offsets); the sign
+// vector, from a second reading, mostly from L2.
+//
+// A whole call through the binding, three kernels -> one, us: 2560 tiles 59 -> 61, 5120 67 -> 67, 10240 (8192x5120) 86 -> 76, 20480 117 -> 91,
+// 32000 (25600x5120) 154 -> 107.  Of the 76 about 40 are allocations and calls in Python, 33 the kernel, 8 of which the trits would pass in
+// at the memory's rate; a tile is about 1140 warp instructions, which bounds it (1.4 ns a tile), behind them the blocks' meeting.
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -36,6 +41,7 @@ constexpr int kPackWarps = 8;       // tiles per thread block
 constexpr int kFlagTrit = 0;        // a weight outside {-1, 0, +1}
 constexpr int kFlagScale = 1;       // a scale that is negative, NaN or Inf
 constexpr int kFlagOverflow = 2;    // more than 2^32 - 1 non-zero weights
+constexpr int kFlagWait = 3;        // (one-pass kernel) the blocks did not meet in time
 constexpr int kNnzLo = 4;           // 64-bit count of non-zero weights (two words, 8-byte aligned)
 
 inline int check_cuda(cudaError_t e) {
@@ -47,21 +53,21 @@ inline int check_cuda(cudaError_t e) {
 inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 inline int64_t padded_rows(int64_t M) { return (M + kRows - 1) / kRows * kRows; }
 
-// 16 consecutive weights (a 16-byte load) -> presence and negative masks of 16 bits; `bad` collects what is not in
-// {-1, 0, +1} (any bit of it).  A trit's bit 0 says present, its bit 7 negative; a negative one must be 0xFF, any
-// other 0 or 1.  The multiplications gather one bit per byte (distinct bits, no carries).
-__device__ __forceinline__ void masks16(const uint4 &v, uint32_t &pres, uint32_t &neg, uint32_t &bad) {
+// 16 consecutive weights (a 16-byte load) -> presence and negative masks of 16 bits.  A trit's bit 0 says present, its bit 7 negative, and
+// a dp4a with the powers of two gathers four of them.  `squares` sums the squares: they are the number of non-zero weights
+// unless one is not in {-1, 0, +1} (an even one adds 4 or more to the squares and nothing to the count, an odd one 9 or more and one).
+__device__ __forceinline__ void masks16(const uint4 &v, uint32_t &pres, uint32_t &neg, int &squares) {
     const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-    uint32_t p = 0u, n = 0u;
+    uint32_t p[2], n[2];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const uint32_t top = w[i] & 0x80808080u, all = (top >> 7) * 0xFFu;
-        bad |= (w[i] ^ all) & (0xFEFEFEFEu | all);
-        p = (p >> 4) | (((w[i] & 0x01010101u) * 0x10204080u) & 0xF0000000u);
-        n = (n >> 4) | ((top * 0x00204081u) & 0xF0000000u);
+    for (int i = 0; i < 2; ++i) {
+        p[i] = __dp4a(w[2 * i + 1] & 0x01010101u, 0x80402010u, __dp4a(w[2 * i] & 0x01010101u, 0x08040201u, 0u));
+        n[i] = __dp4a(w[2 * i + 1] & 0x80808080u, 0x80402010u, __dp4a(w[2 * i] & 0x80808080u, 0x08040201u, 0u));      // (times 128)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) squares = __dp4a(static_cast<int>(w[2 * i + j]), static_cast<int>(w[2 * i + j]), squares);
     }
-    pres = p >> 16;
-    neg = n >> 16;
+    pres = p[0] + (p[1] << 8);
+    neg = (n[0] + (n[1] << 8)) >> 7;
 }
 
 // Chunk i of this lane in the tile (row block rb, group g): weights 16 (lane % 8) .. + 15 of row 4 i + lane / 8; rows
@@ -70,6 +76,27 @@ __device__ __forceinline__ uint4 load_chunk(const int8_t *__restrict__ trits, in
     const int64_t m = rb * kRows + 4 * i + (lane >> 3);
     if (m >= M) return make_uint4(0u, 0u, 0u, 0u);
     return __ldg(reinterpret_cast<const uint4 *>(trits + m * K + static_cast<int64_t>(g) * kGroup) + (lane & 7));
+}
+
+// The bits of both halves of `src` at the set positions of the halves of `mask`, packed towards bit 0 of each half (the inverse
+// of the deposit of Fig. 4): parallel-suffix compress, in round i every selected bit moves right by 2^i if the number of
+// unselected positions below it has bit i set.
+__device__ __forceinline__ uint32_t extract_halves(uint32_t src, uint32_t mask) {
+    uint32_t x = src & mask, m = mask;
+    uint32_t mk = (~m << 1) & 0xFFFEFFFEu;       // the unselected positions, moved up by one: what lies below each bit
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        uint32_t mp = mk ^ ((mk << 1) & 0xFFFEFFFEu);      // prefix parity of mk, half by half
+        mp ^= (mp << 2) & 0xFFFCFFFCu;
+        mp ^= (mp << 4) & 0xFFF0FFF0u;
+        mp ^= (mp << 8) & 0xFF00FF00u;
+        const uint32_t mv = mp & m;              // bits to move in this round (they stay in their half: 2^i positions below are unselected)
+        m = (m ^ mv) | (mv >> (1 << i));
+        const uint32_t t = x & mv;
+        x = (x ^ t) | (t >> (1 << i));
+        mk &= ~mp;
+    }
+    return x;
 }
 
 // Kernel 1: bitmap, scales in tile order, number of non-zero weights per tile (into tile_off, with two bits above it for
@@ -84,7 +111,7 @@ __global__ void __launch_bounds__(kPackWarps * 32) pack_bitmap_kernel(const int8
                                                                       uint4 *__restrict__ signs, int64_t sign_quads) {
     const int lane = threadIdx.x & 31;
     const int G = static_cast<int>(K / kGroup);
-    uint32_t bad = 0u;
+    int squares = 0;
     const int64_t t = static_cast<int64_t>(blockIdx.x) * kPackWarps + (threadIdx.x >> 5);
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (t < n_tiles) {
@@ -100,13 +127,14 @@ __global__ void __launch_bounds__(kPackWarps * 32) pack_bitmap_kernel(const int8
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             uint32_t pres, neg;
-            masks16(v[i], pres, neg, bad);
+            masks16(v[i], pres, neg, squares);
             bitmap[t * 256 + 32 * i + lane] = static_cast<uint16_t>(pres);
             c += __popc(pres);
         }
         scales_tiled[t * kRows + lane] = s;
+        const bool bad = static_cast<uint32_t>(squares) != c;
         c = __reduce_add_sync(0xFFFFFFFFu, c);
-        if (__any_sync(0xFFFFFFFFu, bad != 0u)) c |= kBadTrit;
+        if (__any_sync(0xFFFFFFFFu, bad)) c |= kBadTrit;
         if (__any_sync(0xFFFFFFFFu, (s & 0x8000u) || (s & 0x7F80u) == 0x7F80u)) c |= kBadScale;
         if (lane == 0) tile_off[t] = c;
     }
@@ -206,29 +234,6 @@ __global__ void __launch_bounds__(kScanThreads) scan_counts_kernel(uint32_t *__r
     __threadfence_system();
 }
 
-// The bits of `src` at the set positions of `mask`, packed towards bit 0 (the inverse of the
-// deposit of Fig. 4).
-__device__ __forceinline__ uint32_t extract_bits(uint32_t src, uint32_t mask) {
-    // parallel-suffix compress: in round i every selected bit moves right by 2^i if the number of
-    // unselected positions below it has bit i set (five rounds for 32 bits)
-    uint32_t x = src & mask, m = mask;
-    uint32_t mk = ~m << 1;                       // the unselected positions, moved up by one: what lies below each bit
-#pragma unroll
-    for (int i = 0; i < 5; ++i) {
-        uint32_t mp = mk ^ (mk << 1);            // prefix parity of mk
-        mp ^= mp << 2;
-        mp ^= mp << 4;
-        mp ^= mp << 8;
-        mp ^= mp << 16;
-        const uint32_t mv = mp & m;              // bits to move in this round
-        m = (m ^ mv) | (mv >> (1 << i));
-        const uint32_t t = x & mv;
-        x = (x ^ t) | (t >> (1 << i));
-        mk &= ~mp;
-    }
-    return x;
-}
-
 // Kernel 3: the sign vector.  Tile t owns the bits tile_off[t] .. tile_off[t + 1] - 1; its chunks' sign bits are gathered in
 // shared memory, aligned to the vector's words, and go out as whole words, the first and the last (which the tile may
 // share with its neighbours) by an atomic OR.  Two chunks are compacted at a time, in the halves of one word.  Nothing
@@ -254,10 +259,11 @@ __global__ void __launch_bounds__(kPackWarps * 32) pack_signs_kernel(const int8_
         uint32_t both[4], cnt[4], at0[4], at1[4], at = 0u;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            uint32_t p0, n0, p1, n1, bad = 0u;
-            masks16(v[2 * i], p0, n0, bad);
-            masks16(v[2 * i + 1], p1, n1, bad);
-            both[i] = extract_bits(n0 | (n1 << 16), p0 | (p1 << 16));
+            uint32_t p0, n0, p1, n1;
+            int unused = 0;                          // (kernel 1 has looked at the values)
+            masks16(v[2 * i], p0, n0, unused);
+            masks16(v[2 * i + 1], p1, n1, unused);
+            both[i] = extract_halves(n0 | (n1 << 16), p0 | (p1 << 16));
             cnt[i] = __popc(p0) | (__popc(p1) << 16);
             uint32_t upto = cnt[i];                  // (at most 512 per load: both scans in one register)
 #pragma unroll
@@ -287,8 +293,8 @@ __global__ void __launch_bounds__(kPackWarps * 32) pack_signs_kernel(const int8_
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const uint32_t c0 = cnt[i] & 0xFFFFu;    // (at most 16)
-            put(sh0 + at0[i], both[i] & ((1u << c0) - 1u), c0);
-            put(sh0 + at1[i], both[i] >> c0, cnt[i] >> 16);
+            put(sh0 + at0[i], both[i] & 0xFFFFu, c0);
+            put(sh0 + at1[i], both[i] >> 16, cnt[i] >> 16);
         }
         __syncwarp();
         uint32_t *out = signs + (first >> 5);
@@ -303,17 +309,208 @@ __global__ void __launch_bounds__(kPackWarps * 32) pack_signs_kernel(const int8_
     }
 }
 
+// All of it in one pass: every block has a contiguous range of the tiles (its sign bits are contiguous too).  It counts and
+// compacts them, the sign bits into 512 bytes of shared memory a tile, publishes its total, waits until every block has, and writes
+// its offsets and sign words.  One block per multiprocessor at most and a cooperative launch, so all blocks are
+// resident; the wait is bounded.
+constexpr int kOnceThreads = 1024;
+constexpr int kOnceTiles = 440;                  // per block: 516 bytes each
+constexpr int kOnceMin = 6144;                   // tiles: from here on one pass is faster (see above)
+constexpr int kOnceBlocks = 256;
+constexpr int kReportSlots = 64;
+struct OnceState {                               // one per report slot and device, all zero between calls
+    unsigned int arrived, left;
+    unsigned int total[kOnceBlocks];             // a block's non-zeros, with the two bits above kCountMask for what is wrong with its tiles
+};
+__device__ OnceState g_once_state[kReportSlots];
+
+__global__ void __launch_bounds__(kOnceThreads, 1) pack_once_kernel(const int8_t *__restrict__ trits, const uint16_t *__restrict__ scales, int64_t M,
+                                                                   int64_t K, uint32_t *__restrict__ bitmap, uint16_t *__restrict__ scales_tiled,
+                                                                   uint32_t *__restrict__ tile_off, uint32_t *__restrict__ off_host, int n_tiles,
+                                                                   int n_words, uint32_t *__restrict__ signs, int64_t sign_quads,
+                                                                   unsigned long long max_nnz, int slot, volatile unsigned int *report) {
+    extern __shared__ __align__(16) uint32_t shared[];
+    __shared__ uint32_t s_bad, s_warp[kOnceThreads / 32];
+    __shared__ unsigned int s_ok;
+    OnceState &st = g_once_state[slot];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nb = static_cast<int>(gridDim.x), b = static_cast<int>(blockIdx.x);
+    const int G = static_cast<int>(K / kGroup);
+    const int q = n_tiles / nb, rem = n_tiles - q * nb, t_lo = b * q + (b < rem ? b : rem), mine = q + (b < rem ? 1 : 0), most = q + (rem ? 1 : 0);
+    uint32_t *words = shared, *count = shared + most * 128;      // [tile][128], [tile]
+    if (threadIdx.x == 0) {
+        s_bad = 0u;
+        s_ok = 1u;
+    }
+    __syncthreads();
+    // zeros over this block's share of the sign vector
+    for (int64_t i = static_cast<int64_t>(b) * kOnceThreads + threadIdx.x; i < sign_quads; i += static_cast<int64_t>(nb) * kOnceThreads)
+        reinterpret_cast<uint4 *>(signs)[i] = make_uint4(0u, 0u, 0u, 0u);
+    // ---- counts, bitmap, scales; sign bits into shared memory
+    uint4 v[8];
+    uint16_t s_v = 0;
+    auto fetch = [&](int lt, uint4 (&o)[8], uint16_t &sc) {
+        const int t = t_lo + lt, rb = t / G, g = t - rb * G;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) o[i] = load_chunk(trits, M, K, rb, g, i, lane);
+        const int64_t m = static_cast<int64_t>(rb) * kRows + lane;
+        sc = m < M ? __ldg(scales + m * G + g) : static_cast<uint16_t>(0);
+    };
+    for (int lt = warp; lt < mine; lt += kOnceThreads / 32) {
+        fetch(lt, v, s_v);
+        const int64_t t = t_lo + lt;
+        uint32_t *buf = words + lt * 128;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) buf[32 * i + lane] = 0u;
+        uint32_t both[4], cnt[4], at0[4], at1[4], at = 0u, c = 0u;
+        int squares = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            uint32_t p0, n0, p1, n1;
+            masks16(v[2 * i], p0, n0, squares);
+            masks16(v[2 * i + 1], p1, n1, squares);
+            // presence words: even lanes store those of load 2 i, odd lanes those of load 2 i + 1
+            const uint32_t give = (lane & 1) ? p0 : p1, got = __shfl_xor_sync(0xFFFFFFFFu, give, 1);
+            const uint32_t word = (lane & 1) ? got | (p1 << 16) : p0 | (got << 16);
+            bitmap[t * 128 + 32 * i + 16 * (lane & 1) + (lane >> 1)] = word;
+            both[i] = extract_halves(n0 | (n1 << 16), p0 | (p1 << 16));
+            cnt[i] = __popc(p0) | (__popc(p1) << 16);
+            c += cnt[i];
+            uint32_t upto = cnt[i];                  // (at most 512 per load: both scans in one register)
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, upto, d);
+                if (lane >= d) upto += o;
+            }
+            const uint32_t total = __shfl_sync(0xFFFFFFFFu, upto, 31), before = upto - cnt[i];
+            at0[i] = at + (before & 0xFFFFu);
+            at1[i] = at + (total & 0xFFFFu) + (before >> 16);
+            at += (total & 0xFFFFu) + (total >> 16);
+        }
+        scales_tiled[t * kRows + lane] = s_v;
+        uint32_t flags = 0u;
+        if (__any_sync(0xFFFFFFFFu, static_cast<uint32_t>(squares) != (c & 0xFFFFu) + (c >> 16))) flags |= kBadTrit;
+        if (__any_sync(0xFFFFFFFFu, (s_v & 0x8000u) || (s_v & 0x7F80u) == 0x7F80u)) flags |= kBadScale;
+        if (lane == 0) {
+            count[lt] = at;
+            if (flags) atomicOr(&s_bad, flags);
+        }
+        __syncwarp();                                // (the zeros, before the bits)
+        auto put = [&](uint32_t pos, uint32_t bits) {
+            const uint32_t lo = bits << (pos & 31u), hi = __funnelshift_l(bits, 0u, pos);
+            if (lo) atomicOr(buf + (pos >> 5), lo);
+            if (hi) atomicOr(buf + (pos >> 5) + 1, hi);
+        };
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            put(at0[i], both[i] & 0xFFFFu);
+            put(at1[i], both[i] >> 16);
+        }
+    }
+    __syncthreads();
+    // ---- this block's total, and every tile's place behind the block's first sign bit (a tile per thread)
+    const uint32_t c = threadIdx.x < static_cast<unsigned>(mine) ? count[threadIdx.x] : 0u;
+    uint32_t upto = c;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, upto, d);
+        if (lane >= d) upto += o;
+    }
+    if (lane == 31) s_warp[warp] = upto;
+    __syncthreads();
+    uint32_t before = 0u, total = 0u;
+    for (int w = 0; w < kOnceThreads / 32; ++w) {
+        if (w < warp) before += s_warp[w];
+        total += s_warp[w];
+    }
+    const uint32_t place = before + upto - c;
+    if (threadIdx.x == 0) {
+        st.total[b] = total | s_bad;
+        __threadfence();
+        atomicAdd(&st.arrived, 1u);
+        unsigned long long t0 = 0;
+        for (uint32_t i = 0;; ++i) {
+            unsigned int n;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(n) : "l"(&st.arrived) : "memory");
+            if (n >= static_cast<unsigned>(nb)) break;
+            if ((i & 15u) == 15u) {
+                unsigned long long now;
+                asm volatile("mov.u64 %0, %globaltimer;" : "=l"(now));
+                if (!t0) t0 = now;
+                else if (now - t0 > 500ull * 1000 * 1000) {
+                    s_ok = 0u;
+                    break;
+                }
+            }
+        }
+    }
+    __syncthreads();
+    if (!s_ok) {
+        if (threadIdx.x == 0) report[kFlagWait] = 1u;
+        return;
+    }
+    // ---- the blocks before this one, and what is wrong anywhere
+    uint32_t base = 0u, all = 0u, wrong = 0u;
+    for (int j = lane; j < nb; j += 32) {            // (every warp for itself)
+        const uint32_t x = __ldcg(st.total + j);
+        wrong |= x & ~kCountMask;
+        all += x & kCountMask;
+        if (j < b) base += x & kCountMask;
+    }
+    base = __reduce_add_sync(0xFFFFFFFFu, base);
+    all = __reduce_add_sync(0xFFFFFFFFu, all);
+    wrong = __reduce_or_sync(0xFFFFFFFFu, wrong);
+    if (threadIdx.x < static_cast<unsigned>(mine)) {
+        count[threadIdx.x] = place;
+        tile_off[t_lo + threadIdx.x] = base + place;
+        if (off_host) off_host[t_lo + threadIdx.x] = base + place;
+    }
+    if (b == nb - 1) {
+        for (int i = n_tiles + static_cast<int>(threadIdx.x); i < n_words; i += kOnceThreads) {
+            tile_off[i] = i == n_tiles ? all : 0u;
+            if (off_host) off_host[i] = i == n_tiles ? all : 0u;
+        }
+        if (threadIdx.x == 0) {
+            report[kFlagTrit] = (wrong & kBadTrit) ? 1u : 0u;
+            report[kFlagScale] = (wrong & kBadScale) ? 1u : 0u;
+            report[kFlagOverflow] = 0u;
+            report[kNnzLo] = all;
+            report[kNnzLo + 1] = 0u;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(&st.left, 1u) == static_cast<unsigned>(nb - 1)) st.arrived = st.left = 0u;      // (every block has read the totals)
+    // ---- the sign words; the first and the last of a tile may hold bits of its neighbours
+    if (!wrong && all <= max_nnz) {
+        for (int lt = warp; lt < mine; lt += kOnceThreads / 32) {
+            const uint32_t *buf = words + lt * 128;
+            const uint32_t from = count[lt], bits = (lt + 1 < mine ? count[lt + 1] : total) - from;
+            const uint32_t first = base + from, sh = first & 31u, full = (sh + bits) >> 5;
+            uint32_t *out = signs + (first >> 5);
+            for (uint32_t i = lane; i < (sh + bits + 31u) >> 5; i += 32) {
+                const uint32_t w = __funnelshift_l(i ? buf[i - 1] : 0u, i < 128u ? buf[i] : 0u, sh);
+                if ((i == 0 && sh) || i >= full) {
+                    if (w) atomicOr(out + i, w);
+                } else {
+                    out[i] = w;
+                }
+            }
+        }
+    }
+}
+
 // Non-zero count and validity only (to size the sign vector before packing).
 __global__ void __launch_bounds__(256) count_nnz_kernel(const int8_t *__restrict__ trits, int64_t n16,
                                                         unsigned int *__restrict__ flags) {
     unsigned long long c = 0ull;
-    uint32_t bad = 0u;
+    bool bad = false;
     const uint4 *src = reinterpret_cast<const uint4 *>(trits);
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n16;
          i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
         const uint4 v = __ldg(src + i);
         uint32_t pres, neg;
-        masks16(v, pres, neg, bad);
+        int squares = 0;
+        masks16(v, pres, neg, squares);
+        bad = bad || squares != __popc(pres);
         c += __popc(pres);
     }
 #pragma unroll
@@ -334,7 +531,6 @@ int grid_for(int64_t units, int per_block) {
 // The host's end of scan_counts_kernel's report: 64-byte slots of one pinned page, mapped into every device, taken for the
 // time of a call (a copy of 32 bytes to pageable memory costs about 10 us more than this).  A caller that finds no
 // free slot gets none and reads the scratch words by a copy.
-constexpr int kReportSlots = 64;
 struct ReportSlot {
     static std::atomic<uint64_t> &taken() {
         static std::atomic<uint64_t> t{0};
@@ -370,6 +566,50 @@ struct ReportSlot {
     ReportSlot &operator=(const ReportSlot &) = delete;
     unsigned int *host() const { return slot < 0 ? nullptr : page() + slot * 16; }
 };
+
+// The one-pass kernel's launch: BITCOS_OK, an error, or kNotOnce if it does not take this matrix here.
+constexpr int kNotOnce = 1;
+template <typename... KArgs, typename... Args>
+int launch_once(void (*kernel)(KArgs...), int64_t n_tiles, cudaStream_t stream, Args... args) {
+    constexpr int kMaxDev = 32;
+    static std::atomic<int> blocks_of[kMaxDev];      // multiprocessors, once the kernel is set up there; -1: it cannot run
+    int dev = 0;
+    int rc = check_cuda(cudaGetDevice(&dev));
+    if (rc) return rc;
+    if (dev >= kMaxDev) return kNotOnce;
+    int sms = blocks_of[dev].load();
+    if (sms == 0) {
+        int coop = 0;
+        rc = check_cuda(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        if (!rc) rc = check_cuda(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
+        if (rc) return rc;
+        if (!coop || cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kOnceTiles * 516) != cudaSuccess) {
+            cudaGetLastError();
+            sms = -1;
+        }
+        blocks_of[dev].store(sms);
+    }
+    if (sms < 0) return kNotOnce;
+    if (sms > kOnceBlocks) sms = kOnceBlocks;
+    const int64_t grid = sms, most = (n_tiles + grid - 1) / grid;
+    if (most > kOnceTiles) return kNotOnce;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(static_cast<unsigned>(grid));
+    cfg.blockDim = dim3(kOnceThreads);
+    cfg.dynamicSmemBytes = static_cast<size_t>(most) * 516;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
+    if (e == cudaErrorCooperativeLaunchTooLarge) {
+        cudaGetLastError();
+        return kNotOnce;
+    }
+    return check_cuda(e);
+}
 
 // A launch that may start while the kernel before it is still running (what depends on it waits in the kernel).
 template <typename... KArgs, typename... Args>
@@ -444,11 +684,25 @@ int bitcos_pack_device(const int8_t *trits, const uint16_t *scales_bf16, int64_t
         rc = check_cuda(cudaHostGetDevicePointer(reinterpret_cast<void **>(&report_dev), report.host(), 0));
         if (rc) return rc;
     }
+    bool once = false;
+    if (report.host() && n_tiles >= kOnceMin && n_tiles <= static_cast<int64_t>(kOnceTiles) * kOnceBlocks) {
+        report.host()[kFlagWait] = 0u;
+        rc = launch_once(pack_once_kernel, n_tiles, stream, trits, scales_bf16, M, K, bitmap, scales_tiled, tile_off, off_mapped, static_cast<int>(n_tiles),
+                         static_cast<int>(off_bytes / 4), signs, static_cast<int64_t>(sign_capacity_bytes / 16), max_nnz, report.slot,
+                         static_cast<volatile unsigned int *>(report_dev));
+        once = rc != kNotOnce;
+        if (once && rc) return rc;
+    }
     auto enqueue = [&]() -> int {
+        int e = BITCOS_OK;
+        if (once) {
+            if (tile_off_host && !off_mapped) e = check_cuda(cudaMemcpyAsync(tile_off_host, tile_off, off_bytes, cudaMemcpyDeviceToHost, stream));
+            return e;
+        }
         pack_bitmap_kernel<<<static_cast<unsigned>(grid), kPackWarps * 32, 0, stream>>>(
             trits, scales_bf16, M, K, reinterpret_cast<uint16_t *>(bitmap), scales_tiled, tile_off, n_tiles, reinterpret_cast<uint4 *>(signs),
             static_cast<int64_t>(sign_capacity_bytes / 16));
-        int e = check_cuda(cudaGetLastError());
+        e = check_cuda(cudaGetLastError());
         if (!e)
             e = launch_behind(scan_counts_kernel, 1, kScanThreads, stream, tile_off, off_mapped, n_tiles, static_cast<int64_t>(off_bytes / 4),
                               flags, static_cast<volatile unsigned int *>(report_dev));
@@ -472,6 +726,13 @@ int bitcos_pack_device(const int8_t *trits, const uint16_t *scales_bf16, int64_t
         rc = read_flags(scratch, stream, h);         // (waits for the stream)
     }
     if (rc) return rc;
+    if (once && h[kFlagWait]) {
+        // (not all blocks were resident together: leave the state as a call finds it)
+        static const OnceState zero{};
+        cudaMemcpyToSymbolAsync(g_once_state, &zero, sizeof zero, sizeof zero * static_cast<size_t>(report.slot), cudaMemcpyHostToDevice, stream);
+        cudaStreamSynchronize(stream);
+        return check_cuda(cudaErrorLaunchTimeout);
+    }
     if (h[kFlagTrit]) return BITCOS_ERR_TRIT;
     if (h[kFlagScale]) return BITCOS_ERR_SCALE;
     if (h[kFlagOverflow]) return BITCOS_ERR_OVERFLOW;

@@ -156,3 +156,45 @@ def test_device_pack_with_offsets_to_memory_that_is_pinned_in_part(bc):
             assert torch.equal(off, want.tile_off) and torch.equal(bitmap, want.bitmap), pinned
         if pinned:
             assert int(rt.cudaHostUnregister(host.ctypes.data)) == 0
+
+
+@pytest.mark.parametrize("M,K", [(32 * 6143, 128), (32 * 6144, 128), (32 * 6145 - 7, 128), (32 * 1537, 512), (4097, 6144), (32 * 65121, 128)])
+def test_device_pack_in_one_pass_and_in_three_kernels(bc, M, K):
+    """Matrices on both sides of the lines between the packer's two ways (6144 tiles, 440 tiles per multiprocessor), whole, against
+    their upper and lower parts: the same bitmap and scales, offsets that go on where the upper part ends, the same sign bits."""
+    gen = torch.Generator(device="cuda").manual_seed(M + K)
+    t = torch.randint(-1, 2, (M, K), generator=gen, device="cuda", dtype=torch.int8)
+    top = M // 64 * 32
+    # a multiple of 32 non-zeros above the cut, so that the sign words of the parts can be laid end to end
+    extra = int((t[:top] != 0).sum()) % 32
+    t.view(-1)[(t.view(-1)[:top * K] != 0).nonzero()[:extra, 0]] = 0
+    sc = (0.01 + torch.rand((M, K // 128), generator=gen, device="cuda")).to(torch.bfloat16)
+    whole, parts = bc.bitcos_pack_device(t, sc), [bc.bitcos_pack_device(a.contiguous(), b.contiguous()) for a, b in ((t[:top], sc[:top]), (t[top:], sc[top:]))]
+    assert whole.nnz == parts[0].nnz + parts[1].nnz == int((t != 0).sum()) and parts[0].nnz % 32 == 0
+    assert torch.equal(whole.bitmap, torch.cat([p.bitmap for p in parts])) and torch.equal(whole.scales, torch.cat([p.scales for p in parts]))
+    first, words = parts[0].tile_off_host.size - 1, parts[0].nnz // 32
+    off = np.concatenate([parts[0].tile_off_host[:-1], parts[1].tile_off_host + np.uint32(parts[0].nnz)])
+    assert np.array_equal(whole.tile_off_host, off) and np.array_equal(u32(whole.tile_off)[:off.size], off) and first == top // 32 * (K // 128)
+    last = (whole.nnz + 31) // 32
+    assert torch.equal(whole.signs[:last], torch.cat([parts[0].signs[:words], parts[1].signs[:last - words]])) and not whole.signs[last:].any()
+
+
+def test_device_pack_in_one_pass_reports_what_is_wrong(bc):
+    """A bad trit or scale in the last block of a large matrix, and the next call, which finds the shared state as it should be."""
+    M, K = 8192, 5120
+    gen = torch.Generator(device="cuda").manual_seed(9)
+    t = torch.randint(-1, 2, (M, K), generator=gen, device="cuda", dtype=torch.int8)
+    sc = torch.full((M, K // 128), 0.5, device="cuda").to(torch.bfloat16)
+    want = bc.bitcos_pack_device(t, sc)
+    for value in (2, -2, 127, -128):
+        bad = t.clone()
+        bad[M - 1, K - 1] = value
+        with pytest.raises(bc.BitcosError):
+            bc.bitcos_pack_device(bad, sc)
+    for value in (-1.0, float("inf"), float("nan")):
+        bad = sc.clone()
+        bad[M - 1, 0] = value
+        with pytest.raises(bc.BitcosError):
+            bc.bitcos_pack_device(t, bad)
+    again = bc.bitcos_pack_device(t, sc)
+    assert torch.equal(again.signs, want.signs) and torch.equal(again.tile_off, want.tile_off)

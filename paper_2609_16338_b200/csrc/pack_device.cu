@@ -15,9 +15,10 @@
 // bitmap + scales + per-tile counts (and the sign vector zeroed); an exclusive scan of the counts (the entry offsets); the sign
 // vector, from a second reading, mostly from L2.
 //
-// A whole call through the binding, three kernels -> one, us: 2560 tiles 59 -> 61, 5120 67 -> 67, 10240 (8192x5120) 86 -> 76, 20480 117 -> 91,
-// 32000 (25600x5120) 154 -> 107.  Of the 76 about 40 are allocations and calls in Python, 33 the kernel, 8 of which the trits would pass in
-// at the memory's rate; a tile is about 1140 warp instructions, which bounds it (1.4 ns a tile), behind them the blocks' meeting.
+// A whole call through the binding, three kernels -> one, us: 2560 tiles 59 -> 61, 5120 67 -> 66, 10240 (8192x5120) 86 -> 75, 20480 117 -> 88,
+// 32000 (25600x5120) 153 -> 103.  Of the 75 about 40 are allocations and calls in Python; the trits would pass in 6.4 at the memory's
+// rate.  A tile is about 1100 warp instructions (a quarter of them the compress), 0.19 us a tile and multiprocessor, which bounds the
+// kernel; behind the tiles come the blocks' meeting and the sign words.
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -309,6 +310,14 @@ __global__ void __launch_bounds__(kPackWarps * 32) pack_signs_kernel(const int8_
     }
 }
 
+// Inclusive scan over the lanes of a warp (the shuffle's own in-range predicate guards each addition).
+__device__ __forceinline__ uint32_t scan_add(uint32_t v) {
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1)
+        asm volatile("{\n\t.reg .b32 o;\n\t.reg .pred p;\n\tshfl.sync.up.b32 o|p, %0, %1, 0, 0xFFFFFFFF;\n\t@p add.u32 %0, %0, o;\n\t}" : "+r"(v) : "r"(d));
+    return v;
+}
+
 // All of it in one pass: every block has a contiguous range of the tiles (its sign bits are contiguous too).  It counts and
 // compacts them, the sign bits into 512 bytes of shared memory a tile, publishes its total, waits until every block has, and writes
 // its offsets and sign words.  One block per multiprocessor at most and a cooperative launch, so all blocks are
@@ -350,10 +359,16 @@ __global__ void __launch_bounds__(kOnceThreads, 1) pack_once_kernel(const int8_t
     uint16_t s_v = 0;
     auto fetch = [&](int lt, uint4 (&o)[8], uint16_t &sc) {
         const int t = t_lo + lt, rb = t / G, g = t - rb * G;
+        const int64_t m = static_cast<int64_t>(rb) * kRows, row = m + (lane >> 3);
+        const int8_t *from = trits + row * K + g * kGroup + 16 * (lane & 7);
+        if (m + kRows <= M) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) o[i] = load_chunk(trits, M, K, rb, g, i, lane);
-        const int64_t m = static_cast<int64_t>(rb) * kRows + lane;
-        sc = m < M ? __ldg(scales + m * G + g) : static_cast<uint16_t>(0);
+            for (int i = 0; i < 8; ++i, from += 4 * K) o[i] = __ldg(reinterpret_cast<const uint4 *>(from));
+        } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i, from += 4 * K) o[i] = row + 4 * i < M ? __ldg(reinterpret_cast<const uint4 *>(from)) : make_uint4(0u, 0u, 0u, 0u);
+        }
+        sc = m + lane < M ? __ldg(scales + (m + lane) * G + g) : static_cast<uint16_t>(0);
     };
     for (int lt = warp; lt < mine; lt += kOnceThreads / 32) {
         fetch(lt, v, s_v);
@@ -375,12 +390,7 @@ __global__ void __launch_bounds__(kOnceThreads, 1) pack_once_kernel(const int8_t
             both[i] = extract_halves(n0 | (n1 << 16), p0 | (p1 << 16));
             cnt[i] = __popc(p0) | (__popc(p1) << 16);
             c += cnt[i];
-            uint32_t upto = cnt[i];                  // (at most 512 per load: both scans in one register)
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, upto, d);
-                if (lane >= d) upto += o;
-            }
+            const uint32_t upto = scan_add(cnt[i]);  // (at most 512 per load: both scans in one register)
             const uint32_t total = __shfl_sync(0xFFFFFFFFu, upto, 31), before = upto - cnt[i];
             at0[i] = at + (before & 0xFFFFu);
             at1[i] = at + (total & 0xFFFFu) + (before >> 16);
@@ -395,10 +405,14 @@ __global__ void __launch_bounds__(kOnceThreads, 1) pack_once_kernel(const int8_t
             if (flags) atomicOr(&s_bad, flags);
         }
         __syncwarp();                                // (the zeros, before the bits)
+        const uint32_t buf_at = static_cast<uint32_t>(__cvta_generic_to_shared(buf));
         auto put = [&](uint32_t pos, uint32_t bits) {
+            // (without branches: few chunks have no negative weight, and one in four reaches into the next word)
             const uint32_t lo = bits << (pos & 31u), hi = __funnelshift_l(bits, 0u, pos);
-            if (lo) atomicOr(buf + (pos >> 5), lo);
-            if (hi) atomicOr(buf + (pos >> 5) + 1, hi);
+            asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\tred.shared.or.b32 [%0], %1;\n\t@p red.shared.or.b32 [%0 + 4], %2;\n\t}" ::"r"(
+                             buf_at + ((pos >> 3) & ~3u)),
+                         "r"(lo), "r"(hi)
+                         : "memory");
         };
 #pragma unroll
         for (int i = 0; i < 4; ++i) {

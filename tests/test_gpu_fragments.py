@@ -85,3 +85,21 @@ def test_16_bit_variant(bc, groups, blocks):
         err = np.abs(y.cpu().numpy().astype(np.float64) - y_ref)
         assert (err <= 2e-5 * mag).all(), (groups, B)
     assert bc.workspace_status(ws) == 0
+
+
+@pytest.mark.parametrize("groups", [9, 10, 11, 13, 15, 16, 17, 18, 19, 20, 36, 38])
+def test_partial_sums_in_full_and_guarded_batches(bc, groups):
+    """The epilogue adds a row block's sums ten at a time, a batch of ten, eight or six without guards; rows of every such number of
+    tiles (36 and 38: two column blocks of 18 and 19), all three formats, four to sixteen tokens."""
+    M, K = 32 * 7 - 3, 128 * groups
+    W, S = datagen.trits(700 + groups, M, K, 0.42), datagen.scales(700 + groups, M, K)
+    ws, tiled = bc.make_workspace(M, K), bc.scales_tile(S, M, K)
+    calls = ((bc.bitcos_gemv, bc.bitcos_pack(W, S).to_device()), (bc.trit5_gemv, bc.plain_to_device(bc.trit5_pack(W), tiled, M, K)),
+             (bc.bit2_gemv, bc.plain_to_device(bc.bit2_pack(W), tiled, M, K)))
+    for B in (4, 7, 16):
+        x, xs = datagen.activations(700 + groups + B, B, K)
+        _, y_ref, mag = oracle.gemv_dense(W, S, x, xs)
+        for call, Wd in calls:
+            y, _ = call(Wd, dev(x), dev(xs), workspace=ws)
+            check(y, y_ref, mag, (call.__name__, groups, B))
+    assert bc.workspace_status(ws) == 0

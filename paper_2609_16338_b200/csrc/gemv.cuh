@@ -476,8 +476,8 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
     return mbar_wait_slow(bar, parity);
 }
 
-// Four additions, packed in two instructions where the registers allow it (with sixteen tokens the pairs cost copies: 32B-model layer
-// 103.7 -> 105.8 us).
+// Four additions, packed in two instructions where that pays (with sixteen tokens the pairs and the unguarded batches below cost the
+// 32B-model layer 103.5 -> 106 us, in the 16-bit variant 8192x5120 at four tokens 11.30 -> 11.40).
 template <bool PACKED>
 __device__ __forceinline__ float4 add_quads(float4 a, float4 b) {
     if (!PACKED) return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
@@ -862,8 +862,9 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
                                              bool first_sent = false) {
     // first_sent: the caller has already initialised the barriers of stage 0 and of the lookup table
     // and issued the table's copy and the copies of this block's first item (send_first_copies)
-    // (through a shuffle, so that what depends on it is in uniform registers; not with sixteen tokens, 170.5 -> 174 clocks per tile)
-    const int warp = NB > 8 ? static_cast<int>(threadIdx.x >> 5) : __shfl_sync(0xFFFFFFFFu, static_cast<int>(threadIdx.x >> 5), 0);
+    // (through a shuffle, so that what depends on it is in uniform registers; not with sixteen tokens, 170.5 -> 174 clocks per tile;
+    // the 16-bit variant gains nothing)
+    const int warp = NB > 8 || Segs::kBlend ? static_cast<int>(threadIdx.x >> 5) : __shfl_sync(0xFFFFFFFFu, static_cast<int>(threadIdx.x >> 5), 0);
     const int lane = threadIdx.x & 31;
     const int prod_warp = static_cast<int>(blockDim.x >> 5) - 1;      // the producer: always the block's last warp
     if (static_cast<int>(threadIdx.x) == prod_warp * 32) BITCOS_TL(16, clock64());
@@ -1202,7 +1203,7 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
         // Tensor-core layout: four tokens at a time, spaced one warp's rows apart; more than eight tiles in two batches of ten,
         // all loads of a batch before its first addition (three smaller batches cost the sixteen-token layer 3 %).
         constexpr int RF = NB;
-        auto add4 = [](float4 a, float4 b) { return add_quads<(NB <= 8)>(a, b); };
+        auto add4 = [](float4 a, float4 b) { return add_quads<(NB <= 8 && !kBlend)>(a, b); };
         const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
         // (A guarded load takes four instructions.  A batch that is full, or as long as the second one of rows of 16 or 18 groups, has none:
         // with packed additions and the warp's number in uniform registers MoE pass of 128 experts 57.6 -> 56.2 us, 18944 -> 56832 x 5120
@@ -1220,7 +1221,7 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
             return v[0];
         };
         auto in_tens = [&](const float *base, int n) {
-            if constexpr (NB > 8) return add4(batch(std::integral_constant<int, 0>{}, base, n), batch(std::integral_constant<int, 0>{}, base + 10 * kRows * RF, n - 10));
+            if constexpr (NB > 8 || kBlend) return add4(batch(std::integral_constant<int, 0>{}, base, n), batch(std::integral_constant<int, 0>{}, base + 10 * kRows * RF, n - 10));
             if (n < 10) return batch(std::integral_constant<int, 0>{}, base, n);
             const float4 tot = batch(std::integral_constant<int, 10>{}, base, 10);
             base += 10 * kRows * RF;

@@ -26,8 +26,8 @@
 // so that lookups never conflict.  Entries are the four weights as int8 (w = p - 2n, Eq. 2)
 // ready for dp4a or the tensor cores.  A lane's position in the sign vector is the tile's entry offset
 // plus a warp prefix sum over the rows' population counts; the four 32-bit presence words of
-// a lane's row are decoded as four independent chains, each shifting its own sign window by
-// the number of sign bits a nibble consumed.
+// a lane's row are decoded as four independent chains, each rotating its own sign window by
+// a running position that advances by the sign bits a nibble consumed.
 #ifndef BITCOS_GEMV_CUH
 #define BITCOS_GEMV_CUH
 

@@ -207,6 +207,10 @@ int bitcos_workspace_status(const void *workspace, void *cuda_stream, int *statu
  * cycles (device, uint64 [blocks]) receives each block's elapsed SM clock cycles; cycles per 32
  * weights per multiprocessor = cycles / (iters * warps_per_block * 128). */
 int bitcos_decode_probe(int format, int warps_per_block, int iters, int blocks, uint64_t *cycles, void *cuda_stream);
+/* The same with the tile's sums: sums = NULL or device int32 [warps_per_block][32], the group accumulators of every
+ * warp's rows (row r in lane r) in the last of block 0's passes. */
+int bitcos_decode_probe_sums(int format, int warps_per_block, int iters, int blocks, uint64_t *cycles, int32_t *sums,
+                             void *cuda_stream);
 
 /* The same measurement for each of the library's BITCOS decoders, on real packed tiles, with the
  * accumulators handed back so that every decoder can be checked (Section II-D notes that the unpack

@@ -24,7 +24,7 @@ EXPORTED_SYMBOLS = [
     "bitcos_unpack", "bitcos_scales_tile", "bitcos_scales_untile", "trit5_pack_sizes", "trit5_pack",
     "trit5_unpack", "bit2_pack_sizes", "bit2_pack", "bit2_unpack", "bitcos_gemv_workspace_bytes",
     "bitcos_workspace_init", "bitcos_workspace_status", "bitcos_gemv", "trit5_gemv", "bit2_gemv", "bitcos_gemv_grouped",
-    "bitcos_gemv_host_staging_bytes", "bitcos_gemv_host", "bitcos_gemv_static", "bitcos_decode_probe", "bitcos_gemv_multi",
+    "bitcos_gemv_host_staging_bytes", "bitcos_gemv_host", "bitcos_gemv_static", "bitcos_decode_probe", "bitcos_decode_probe_sums", "bitcos_gemv_multi",
     "bitcos_gemv_multi_host", "bitcos_quantize_activations", "bitcos_gemv_group_scales",
     "bitcos_choose_format", "bitcos_count_nnz_device", "bitcos_pack_device", "bitcos_gemv_bf16", "bitcos_gemv_multi_bf16",
     "bitcos_gemv_multi_group_scales", "bitcos_gemv_blend_bf16", "bitcos_decode_probe_variant", "bitcos_gemv_phased", "bitcos_gemv_phases_host", "trit5_gemv_grouped", "bit2_gemv_grouped", "bitcos_gemv_static_status", "bitcos_wait_probe", "bitcos_group_pairs_device", "bitcos_gemv_grouped_lists", "bitcos_gemv_multi_chained", "bitcos_gemv_multi_plan",
@@ -100,6 +100,7 @@ def load_library():
     L.bitcos_gemv_host.argtypes = [C.POINTER(_Weights), vp, vp, C.c_int, vp, vp, sz, vp, sz, vp]
     L.bitcos_gemv_static.argtypes = [C.POINTER(_Weights), vp, vp, C.c_int, vp, vp]
     L.bitcos_decode_probe.argtypes = [C.c_int, C.c_int, C.c_int, C.c_int, vp, vp]
+    L.bitcos_decode_probe_sums.argtypes = [C.c_int, C.c_int, C.c_int, C.c_int, vp, vp, vp]
     L.bitcos_decode_probe_variant.argtypes = [C.c_int, vp, vp, sz, vp, C.c_int, vp, C.c_int, C.c_int, vp, vp, vp]
     L.bitcos_gemv_multi.argtypes = [C.POINTER(_Job), C.c_int, C.c_int, vp]
     pi = C.POINTER(C.c_int)
@@ -769,15 +770,18 @@ def bitcos_gemv_multi_bf16(jobs):
     return [j[3] for j in mj.keep]
 
 
-def bitcos_decode_probe(fmt: int, warps_per_block: int, iters: int, blocks: int):
-    """Cycles per 32 weights per multiprocessor of the on-chip decode (the roofline's gamma)."""
+def bitcos_decode_probe(fmt: int, warps_per_block: int, iters: int, blocks: int, want_sums: bool = False):
+    """Cycles per 32 weights per multiprocessor of the on-chip decode (the roofline's gamma), and the int32
+    accumulators [warps_per_block, 32] of the last pass if asked for."""
     import torch
     cyc = torch.zeros(blocks, dtype=torch.int64, device="cuda")
-    _check(load_library().bitcos_decode_probe(fmt, warps_per_block, iters, blocks, cyc.data_ptr(), _stream()),
-           "bitcos_decode_probe")
+    sums = torch.zeros((warps_per_block, TILE_ROWS), dtype=torch.int32, device="cuda") if want_sums else None
+    _check(load_library().bitcos_decode_probe_sums(fmt, warps_per_block, iters, blocks, cyc.data_ptr(),
+                                                   sums.data_ptr() if sums is not None else None, _stream()), "bitcos_decode_probe_sums")
     torch.cuda.synchronize()
     c = cyc.cpu().numpy().astype(np.float64)
-    return float(np.median(c)) / (iters * warps_per_block * 128.0)
+    gamma = float(np.median(c)) / (iters * warps_per_block * 128.0)
+    return (gamma, sums) if want_sums else gamma
 
 
 PROBE_VARIANTS = ("shifted window", "running position", "byte table", "no table", "lane = bit", "split row 1+3",

@@ -71,3 +71,39 @@ def test_every_decoder_matches_the_oracle(bc, variant):
             gamma, acc = bc.bitcos_decode_probe_variant(variant, Wd, first, n, x, 3, 2, want_acc=True)
             assert gamma > 0
             assert np.array_equal(acc.cpu().numpy(), ref[first:first + n]), (bc.PROBE_VARIANTS[variant], case, first, n)
+
+
+def synthetic_tile(fmt, odd):
+    """Weights [32, 128] and activations [128] of the tile that bitcos_decode_probe makes on the chip: words hashed from
+    their numbers, read by the packed layouts' own rules; odd = an odd pass."""
+    def hashed(v):
+        v = np.asarray(v, dtype=np.uint32)
+        for shift, factor in ((16, 0x7FEB352D), (15, 0x846CA68B), (16, 1)):
+            v = (v ^ (v >> np.uint32(shift))) * np.uint32(factor)
+        return v
+    i = np.arange(1792 // 4, dtype=np.uint32)
+    h = [hashed(i * np.uint32(4) + np.uint32(n)) for n in (1, 2, 3, 4)]
+    words = h[0] | (h[1] & h[2] & h[3])
+    x = hashed(1000 + np.arange(32, dtype=np.uint32)).view(np.int8).astype(np.int64)
+    if fmt == 0:                                     # signs from byte 1024 on; odd passes begin one sign bit later
+        bits = np.unpackbits(words[:128].view(np.uint8), bitorder="little").reshape(32, 128).astype(np.int64)
+        signs = np.unpackbits(words[256:].view(np.uint8), bitorder="little").astype(np.int64)
+        rank = (np.cumsum(bits.ravel()) - 1).reshape(32, 128)
+        return bits * (1 - 2 * signs[np.minimum(rank + odd, signs.size - 1)]), x
+    if fmt == 1:                                     # word q of row r at 32 q + r; odd groups begin at byte 2
+        words = sum(((v & 0xFF) % 243) << np.uint32(8 * n) for n, v in enumerate(h))
+        row = np.ascontiguousarray(words[:224].reshape(7, 32).T).view(np.uint8)[:, 2 * odd:2 * odd + 26].astype(np.int64)
+        return np.stack([row // 3 ** n % 3 - 1 for n in range(5)], axis=2).reshape(32, 130)[:, :128], x
+    words = (words & np.uint32(0x55555555)).reshape(-1, 4)        # 16-byte chunk c of row r at 32 c + r; odd passes one chunk later
+    row = np.concatenate([words[odd:odd + 32], words[32 + odd:64 + odd]], axis=1)
+    code = np.stack([(row >> np.uint32(8 * (n % 4) + 2 * (n // 4))) & 3 for n in range(16)], axis=2).reshape(32, 128)
+    return code.astype(np.int64) - 1, x
+
+
+@pytest.mark.parametrize("fmt", range(3))
+@pytest.mark.parametrize("warps,iters", [(20, 4), (7, 3), (22, 1)])
+def test_the_probe_of_the_products_decoders_decodes(bc, fmt, warps, iters):
+    """bitcos_decode_probe times the decoders that the products run on the tables that the products use: its sums are the tile's."""
+    gamma, sums = bc.bitcos_decode_probe(fmt, warps, iters, 2, want_sums=True)
+    W, x = synthetic_tile(fmt, (iters - 1) & 1)
+    assert gamma > 0 and np.array_equal(sums.cpu().numpy(), np.tile(W @ x, (warps, 1)))

@@ -8,17 +8,17 @@
 // 16-weight chunks in the order (load, lane) are the tile's weights in order, and the sign bits of a chunk lie where a
 // scan of the chunk counts puts them.
 //
-// Where a tile's sign bits go is known only when everything before it has been counted.  From kOnceMin tiles up to kOnceTiles per
-// multiprocessor one kernel does all of it (pack_once_kernel): a block keeps the compacted sign bits of its tiles in shared memory
-// until every block has counted, so that the trits are read and looked at once.  Smaller matrices (a cooperative launch costs the
-// caller about 8 us more than an ordinary one), larger ones and calls that find no state to share take three kernels:
-// bitmap + scales + per-tile counts (and the sign vector zeroed); an exclusive scan of the counts (the entry offsets); the sign
-// vector, from a second reading, mostly from L2.
+// Where a tile's sign bits go is known only when everything before it has been counted.  One kernel does all of it (pack_once_kernel): a
+// block keeps the compacted sign bits of its tiles in shared memory until the tiles before have been counted, so that the
+// trits are read and looked at once.  Matrices with more tiles than its ranges hold and calls that find no state to share
+// take three kernels: bitmap + scales + per-tile counts (and the sign vector zeroed); an exclusive scan of the counts (the entry
+// offsets); the sign vector, from a second reading, mostly from L2.
 //
-// A whole call through the binding, three kernels -> one, us: 2560 tiles 59 -> 61, 5120 67 -> 66, 10240 (8192x5120) 86 -> 75, 20480 117 -> 88,
-// 32000 (25600x5120) 153 -> 103.  Of the 75 about 40 are allocations and calls in Python; the trits would pass in 6.4 at the memory's
-// rate.  A tile is about 1100 warp instructions (a quarter of them the compress), 0.19 us a tile and multiprocessor, which bounds the
-// kernel; behind the tiles come the blocks' meeting and the sign words.
+// A whole call through the binding, three kernels -> one, us: 32 tiles 78 -> 72, 400 79 -> 77, 1600 82 -> 81, 2560 83 -> 84, 4096 86 -> 84, 6144
+// 76 -> 75, 10240 (8192x5120) 88 -> 81, 20480 118 -> 98, 32000 (25600x5120) 154 -> 116, 64000 243 -> 176 (as a cooperative launch of one block of 1024
+// threads per multiprocessor the last four took 82, 100, 115 and 188).  About 40 of them are allocations and calls in Python; the
+// trits of 8192x5120 would pass in 6.4 at the memory's rate.  A tile is about 1100 warp instructions (a quarter of them the
+// compress), 0.19 us a tile and multiprocessor, which bounds the kernel; behind the tiles come the look-back and the sign words.
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -42,7 +42,7 @@ constexpr int kPackWarps = 8;       // tiles per thread block
 constexpr int kFlagTrit = 0;        // a weight outside {-1, 0, +1}
 constexpr int kFlagScale = 1;       // a scale that is negative, NaN or Inf
 constexpr int kFlagOverflow = 2;    // more than 2^32 - 1 non-zero weights
-constexpr int kFlagWait = 3;        // (one-pass kernel) the blocks did not meet in time
+constexpr int kFlagWait = 3;        // (one-pass kernel) a wait for the tiles before ran out
 constexpr int kNnzLo = 4;           // 64-bit count of non-zero weights (two words, 8-byte aligned)
 
 inline int check_cuda(cudaError_t e) {
@@ -318,42 +318,99 @@ __device__ __forceinline__ uint32_t scan_add(uint32_t v) {
     return v;
 }
 
-// All of it in one pass: every block has a contiguous range of the tiles (its sign bits are contiguous too).  It counts and
-// compacts them, the sign bits into 512 bytes of shared memory a tile, publishes its total, waits until every block has, and writes
-// its offsets and sign words.  One block per multiprocessor at most and a cooperative launch, so all blocks are
-// resident; the wait is bounded.
-constexpr int kOnceThreads = 1024;
-constexpr int kOnceTiles = 440;                  // per block: 516 bytes each
-constexpr int kOnceMin = 6144;                   // tiles: from here on one pass is faster (see above)
-constexpr int kOnceBlocks = 256;
+// All of it in one pass: a block takes the next range of the tiles (its sign bits are contiguous too).  It counts and
+// compacts them, the sign bits into 512 bytes of shared memory a tile, publishes its total, adds up those of the ranges before its
+// own, and writes its offsets and sign words.  The sum is a decoupled look-back (Merrill and Garland, "Single-pass Parallel Prefix Scan
+// with Decoupled Look-back", 2016): a word per range, first its own total, then the total up to and with it.
+// A range is taken by a ticket, and a block waits for lower tickets only: those blocks are running and wait for none above
+// them, so the kernel ends whatever else is on the chip, as few of its blocks as may find room at a time (a cooperative launch
+// of one block per multiprocessor waited for all of the chip to be free).  The waits are bounded all the same.
+constexpr int kOnceThreads = 256;
+constexpr int kOnceTiles = 88;                   // per range at most: 516 bytes each, together within the 48 KB that need no attribute
+constexpr int kOnceStep = 8;                     // tiles per range at least: one per warp
+constexpr int kOnceBlocks = 4;                   // resident per multiprocessor (64 registers a thread)
+constexpr int kOnceRanges = 2048;
+constexpr unsigned long long kOnceLimitNs = 500ull * 1000 * 1000;
 constexpr int kReportSlots = 64;
-struct OnceState {                               // one per report slot and device, all zero between calls
-    unsigned int arrived, left;
-    unsigned int total[kOnceBlocks];             // a block's non-zeros, with the two bits above kCountMask for what is wrong with its tiles
+// A range's word: its count, what is wrong with it, how far the count reaches, and the number of the call (words of
+// earlier calls are thereby void: nothing has to be cleared between calls, whatever became of them).
+constexpr int kWordBad = 32, kWordState = 34, kWordTag = 36;
+constexpr unsigned int kStateOwn = 1u, kStateUpTo = 2u, kStateGaveUp = 3u;
+constexpr unsigned long long kOnceTags = 1ull << (64 - kWordTag);
+struct OnceState {                               // one per report slot and device
+    unsigned int ticket;                         // 0 between calls: every block takes one, and the last one wraps
+    unsigned long long range[kOnceRanges];
 };
 __device__ OnceState g_once_state[kReportSlots];
 
-__global__ void __launch_bounds__(kOnceThreads, 1) pack_once_kernel(const int8_t *__restrict__ trits, const uint16_t *__restrict__ scales, int64_t M,
+__device__ __forceinline__ unsigned long long range_word(uint32_t count, uint32_t bad, unsigned int state, unsigned long long tag) {
+    return count | static_cast<unsigned long long>(bad >> 30) << kWordBad | static_cast<unsigned long long>(state) << kWordState | tag << kWordTag;
+}
+__device__ __forceinline__ void publish(unsigned long long *at, unsigned long long word) {
+    __threadfence();
+    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(at), "l"(word) : "memory");
+}
+
+// Total and faults of the ranges before range r (one warp); false if a wait ran out here or there.
+__device__ __forceinline__ bool look_back(const OnceState &st, int r, unsigned long long tag, int lane, unsigned long long limit_ns, uint32_t &base,
+                                          uint32_t &bad) {
+    base = bad = 0u;
+    for (int nearest = r - 1;; nearest -= 32) {
+        const int j = nearest - lane;
+        unsigned long long word, t0 = 0;
+        uint32_t use;                                // the lanes up to and with the first whose total reaches back to the beginning
+        bool to_the_start;
+        for (uint32_t i = 0;; ++i) {
+            word = range_word(0u, 0u, kStateUpTo, tag);      // (in front of the first range)
+            if (j >= 0) asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(word) : "l"(st.range + j) : "memory");
+            const unsigned int state = (word >> kWordTag) == tag ? static_cast<unsigned int>(word >> kWordState) & 3u : 0u;
+            const uint32_t ready = __ballot_sync(0xFFFFFFFFu, state != 0u), up_to = __ballot_sync(0xFFFFFFFFu, state == kStateUpTo);
+            if (__any_sync(0xFFFFFFFFu, state == kStateGaveUp)) return false;
+            to_the_start = up_to != 0u;
+            use = 2u * (up_to & (0u - up_to)) - 1u;  // (all lanes if there is none, or only the last)
+            if ((ready & use) == use) break;
+            if ((i & 15u) == 15u) {
+                unsigned long long now;
+                asm volatile("mov.u64 %0, %globaltimer;" : "=l"(now));
+                if (!t0) t0 = now;
+                if (__any_sync(0xFFFFFFFFu, now - t0 > limit_ns)) return false;
+            }
+        }
+        const bool mine = (use >> lane) & 1u;
+        base += __reduce_add_sync(0xFFFFFFFFu, mine ? static_cast<uint32_t>(word) : 0u);
+        bad |= __reduce_or_sync(0xFFFFFFFFu, mine ? (static_cast<uint32_t>(word >> kWordBad) & 3u) << 30 : 0u);
+        if (to_the_start) return true;
+    }
+}
+
+__global__ void __launch_bounds__(kOnceThreads, kOnceBlocks) pack_once_kernel(const int8_t *__restrict__ trits, const uint16_t *__restrict__ scales, int64_t M,
                                                                    int64_t K, uint32_t *__restrict__ bitmap, uint16_t *__restrict__ scales_tiled,
                                                                    uint32_t *__restrict__ tile_off, uint32_t *__restrict__ off_host, int n_tiles,
-                                                                   int n_words, uint32_t *__restrict__ signs, int64_t sign_quads,
-                                                                   unsigned long long max_nnz, int slot, volatile unsigned int *report) {
+                                                                   int per_range, int n_words, uint32_t *__restrict__ signs, int64_t sign_quads,
+                                                                   unsigned long long max_nnz, int slot, unsigned long long tag,
+                                                                   unsigned long long limit_ns, volatile unsigned int *report) {
     extern __shared__ __align__(16) uint32_t shared[];
-    __shared__ uint32_t s_bad, s_warp[kOnceThreads / 32];
-    __shared__ unsigned int s_ok;
+    __shared__ uint32_t s_bad, s_base, s_warp[kOnceThreads / 32];
+    __shared__ int s_range, s_ok;
     OnceState &st = g_once_state[slot];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nb = static_cast<int>(gridDim.x), b = static_cast<int>(blockIdx.x);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_ranges = static_cast<int>(gridDim.x);
     const int G = static_cast<int>(K / kGroup);
-    const int q = n_tiles / nb, rem = n_tiles - q * nb, t_lo = b * q + (b < rem ? b : rem), mine = q + (b < rem ? 1 : 0), most = q + (rem ? 1 : 0);
-    uint32_t *words = shared, *count = shared + most * 128;      // [tile][128], [tile]
+    uint32_t *words = shared, *count = shared + per_range * 128;      // [tile][128], [tile]
     if (threadIdx.x == 0) {
         s_bad = 0u;
-        s_ok = 1u;
+        s_range = static_cast<int>(atomicInc(&st.ticket, static_cast<unsigned int>(n_ranges - 1)));
     }
     __syncthreads();
-    // zeros over this block's share of the sign vector
-    for (int64_t i = static_cast<int64_t>(b) * kOnceThreads + threadIdx.x; i < sign_quads; i += static_cast<int64_t>(nb) * kOnceThreads)
-        reinterpret_cast<uint4 *>(signs)[i] = make_uint4(0u, 0u, 0u, 0u);
+    const int r = s_range, t_lo = r * per_range, mine = n_tiles - t_lo < per_range ? n_tiles - t_lo : per_range;
+    // Zeros over the sign vector: the words that would be this range's if every weight were there, and a share of what lies behind all of
+    // those.  Sign bits never lie further back, so a range's zeros are written over by itself and later ranges only, which
+    // have waited for its word.
+    uint4 *const zeros = reinterpret_cast<uint4 *>(signs);
+    const uint4 none = make_uint4(0u, 0u, 0u, 0u);
+    const int64_t z_lo = static_cast<int64_t>(t_lo) * 32, z_hi = z_lo + mine * 32 < sign_quads ? z_lo + mine * 32 : sign_quads;
+    for (int64_t i = z_lo + threadIdx.x; i < z_hi; i += kOnceThreads) zeros[i] = none;
+    for (int64_t i = static_cast<int64_t>(n_tiles) * 32 + r * kOnceThreads + threadIdx.x; i < sign_quads; i += static_cast<int64_t>(n_ranges) * kOnceThreads)
+        zeros[i] = none;
     // ---- counts, bitmap, scales; sign bits into shared memory
     uint4 v[8];
     uint16_t s_v = 0;
@@ -421,92 +478,68 @@ __global__ void __launch_bounds__(kOnceThreads, 1) pack_once_kernel(const int8_t
         }
     }
     __syncthreads();
-    // ---- this block's total, and every tile's place behind the block's first sign bit (a tile per thread)
+    // ---- this range's total, and every tile's place behind the range's first sign bit (a tile per thread)
     const uint32_t c = threadIdx.x < static_cast<unsigned>(mine) ? count[threadIdx.x] : 0u;
-    uint32_t upto = c;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, upto, d);
-        if (lane >= d) upto += o;
-    }
+    const uint32_t upto = scan_add(c);
     if (lane == 31) s_warp[warp] = upto;
     __syncthreads();
     uint32_t before = 0u, total = 0u;
+#pragma unroll
     for (int w = 0; w < kOnceThreads / 32; ++w) {
         if (w < warp) before += s_warp[w];
         total += s_warp[w];
     }
     const uint32_t place = before + upto - c;
-    if (threadIdx.x == 0) {
-        st.total[b] = total | s_bad;
-        __threadfence();
-        atomicAdd(&st.arrived, 1u);
-        unsigned long long t0 = 0;
-        for (uint32_t i = 0;; ++i) {
-            unsigned int n;
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(n) : "l"(&st.arrived) : "memory");
-            if (n >= static_cast<unsigned>(nb)) break;
-            if ((i & 15u) == 15u) {
-                unsigned long long now;
-                asm volatile("mov.u64 %0, %globaltimer;" : "=l"(now));
-                if (!t0) t0 = now;
-                else if (now - t0 > 500ull * 1000 * 1000) {
-                    s_ok = 0u;
-                    break;
-                }
+    if (warp == 0) {
+        uint32_t base = 0u, bad = 0u;
+        if (r && lane == 0) publish(st.range + r, range_word(total, s_bad, kStateOwn, tag));
+        const bool ok = look_back(st, r, tag, lane, limit_ns, base, bad);
+        __syncwarp();                                // (what the lanes have acquired, before lane 0 passes it on)
+        if (lane == 0) {
+            bad |= s_bad;
+            publish(st.range + r, range_word(base + total, bad, ok ? kStateUpTo : kStateGaveUp, tag));
+            s_base = base;
+            s_ok = ok;
+            if (!ok) {
+                report[kFlagWait] = 1u;
+            } else if (r == n_ranges - 1) {
+                report[kFlagTrit] = (bad & kBadTrit) ? 1u : 0u;
+                report[kFlagScale] = (bad & kBadScale) ? 1u : 0u;
+                report[kFlagOverflow] = 0u;          // (kOnceTiles x kOnceRanges tiles hold fewer than 2^32 weights)
+                report[kNnzLo] = base + total;
+                report[kNnzLo + 1] = 0u;
             }
         }
     }
     __syncthreads();
-    if (!s_ok) {
-        if (threadIdx.x == 0) report[kFlagWait] = 1u;
-        return;
-    }
-    // ---- the blocks before this one, and what is wrong anywhere
-    uint32_t base = 0u, all = 0u, wrong = 0u;
-    for (int j = lane; j < nb; j += 32) {            // (every warp for itself)
-        const uint32_t x = __ldcg(st.total + j);
-        wrong |= x & ~kCountMask;
-        all += x & kCountMask;
-        if (j < b) base += x & kCountMask;
-    }
-    base = __reduce_add_sync(0xFFFFFFFFu, base);
-    all = __reduce_add_sync(0xFFFFFFFFu, all);
-    wrong = __reduce_or_sync(0xFFFFFFFFu, wrong);
+    if (!s_ok) return;
+    const uint32_t base = s_base;
     if (threadIdx.x < static_cast<unsigned>(mine)) {
         count[threadIdx.x] = place;
         tile_off[t_lo + threadIdx.x] = base + place;
         if (off_host) off_host[t_lo + threadIdx.x] = base + place;
     }
-    if (b == nb - 1) {
+    if (r == n_ranges - 1) {
         for (int i = n_tiles + static_cast<int>(threadIdx.x); i < n_words; i += kOnceThreads) {
-            tile_off[i] = i == n_tiles ? all : 0u;
-            if (off_host) off_host[i] = i == n_tiles ? all : 0u;
-        }
-        if (threadIdx.x == 0) {
-            report[kFlagTrit] = (wrong & kBadTrit) ? 1u : 0u;
-            report[kFlagScale] = (wrong & kBadScale) ? 1u : 0u;
-            report[kFlagOverflow] = 0u;
-            report[kNnzLo] = all;
-            report[kNnzLo + 1] = 0u;
+            tile_off[i] = i == n_tiles ? base + total : 0u;
+            if (off_host) off_host[i] = i == n_tiles ? base + total : 0u;
         }
     }
     __syncthreads();
-    if (threadIdx.x == 0 && atomicAdd(&st.left, 1u) == static_cast<unsigned>(nb - 1)) st.arrived = st.left = 0u;      // (every block has read the totals)
-    // ---- the sign words; the first and the last of a tile may hold bits of its neighbours
-    if (!wrong && all <= max_nnz) {
-        for (int lt = warp; lt < mine; lt += kOnceThreads / 32) {
-            const uint32_t *buf = words + lt * 128;
-            const uint32_t from = count[lt], bits = (lt + 1 < mine ? count[lt + 1] : total) - from;
-            const uint32_t first = base + from, sh = first & 31u, full = (sh + bits) >> 5;
-            uint32_t *out = signs + (first >> 5);
-            for (uint32_t i = lane; i < (sh + bits + 31u) >> 5; i += 32) {
-                const uint32_t w = __funnelshift_l(i ? buf[i - 1] : 0u, i < 128u ? buf[i] : 0u, sh);
-                if ((i == 0 && sh) || i >= full) {
-                    if (w) atomicOr(out + i, w);
-                } else {
-                    out[i] = w;
-                }
+    // ---- the sign words; the first and the last of a tile may hold bits of its neighbours.  A vector that is too small gets those
+    // that fit (the host reports it).
+    for (int lt = warp; lt < mine; lt += kOnceThreads / 32) {
+        const uint32_t *buf = words + lt * 128;
+        const uint32_t from = count[lt], bits = (lt + 1 < mine ? count[lt + 1] : total) - from;
+        const uint32_t first = base + from, sh = first & 31u, full = (sh + bits) >> 5;
+        if (static_cast<unsigned long long>(first) + bits > max_nnz) break;
+        uint32_t *out = signs + (first >> 5);
+        for (uint32_t i = lane; i < (sh + bits + 31u) >> 5; i += 32) {
+            const uint32_t w = __funnelshift_l(i ? buf[i - 1] : 0u, i < 128u ? buf[i] : 0u, sh);
+            if ((i == 0 && sh) || i >= full) {
+                if (w) atomicOr(out + i, w);
+            } else {
+                out[i] = w;
             }
         }
     }
@@ -542,6 +575,19 @@ int grid_for(int64_t units, int per_block) {
     return static_cast<int>(want < 1 ? 1 : (want < cap ? want : cap));
 }
 
+// As few ranges as the chip holds blocks: all start together and look back once, at their ends (ranges of 8 | 16 | 32 tiles took
+// 144 | 144 | 130 us where 55 take 116, 25600x5120, and 96 | 89 | 85 where 18 take 81, 8192x5120).
+int tiles_per_range(int64_t n_tiles) {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) sms = 128;
+    const int64_t at_once = static_cast<int64_t>(sms) * kOnceBlocks;
+    const int64_t rounds = (n_tiles + at_once * kOnceTiles - 1) / (at_once * kOnceTiles);
+    int64_t per_range = (n_tiles + at_once * rounds - 1) / (at_once * rounds);
+    if (per_range < kOnceStep) per_range = kOnceStep;
+    while (per_range * kOnceRanges < n_tiles) ++per_range;
+    return static_cast<int>(per_range);
+}
+
 // The host's end of scan_counts_kernel's report: 64-byte slots of one pinned page, mapped into every device, taken for the
 // time of a call (a copy of 32 bytes to pageable memory costs about 10 us more than this).  A caller that finds no
 // free slot gets none and reads the scratch words by a copy.
@@ -560,6 +606,11 @@ struct ReportSlot {
             return static_cast<unsigned int *>(v);
         }();
         return p;
+    }
+    // numbers for the calls that use a slot's device state (by its holder only)
+    static unsigned long long next_tag(int slot) {
+        static unsigned long long used[kReportSlots];
+        return ++used[slot];
     }
     int slot = -1;
     ReportSlot() {
@@ -580,50 +631,6 @@ struct ReportSlot {
     ReportSlot &operator=(const ReportSlot &) = delete;
     unsigned int *host() const { return slot < 0 ? nullptr : page() + slot * 16; }
 };
-
-// The one-pass kernel's launch: BITCOS_OK, an error, or kNotOnce if it does not take this matrix here.
-constexpr int kNotOnce = 1;
-template <typename... KArgs, typename... Args>
-int launch_once(void (*kernel)(KArgs...), int64_t n_tiles, cudaStream_t stream, Args... args) {
-    constexpr int kMaxDev = 32;
-    static std::atomic<int> blocks_of[kMaxDev];      // multiprocessors, once the kernel is set up there; -1: it cannot run
-    int dev = 0;
-    int rc = check_cuda(cudaGetDevice(&dev));
-    if (rc) return rc;
-    if (dev >= kMaxDev) return kNotOnce;
-    int sms = blocks_of[dev].load();
-    if (sms == 0) {
-        int coop = 0;
-        rc = check_cuda(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        if (!rc) rc = check_cuda(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
-        if (rc) return rc;
-        if (!coop || cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kOnceTiles * 516) != cudaSuccess) {
-            cudaGetLastError();
-            sms = -1;
-        }
-        blocks_of[dev].store(sms);
-    }
-    if (sms < 0) return kNotOnce;
-    if (sms > kOnceBlocks) sms = kOnceBlocks;
-    const int64_t grid = sms, most = (n_tiles + grid - 1) / grid;
-    if (most > kOnceTiles) return kNotOnce;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(static_cast<unsigned>(grid));
-    cfg.blockDim = dim3(kOnceThreads);
-    cfg.dynamicSmemBytes = static_cast<size_t>(most) * 516;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
-    if (e == cudaErrorCooperativeLaunchTooLarge) {
-        cudaGetLastError();
-        return kNotOnce;
-    }
-    return check_cuda(e);
-}
 
 // A launch that may start while the kernel before it is still running (what depends on it waits in the kernel).
 template <typename... KArgs, typename... Args>
@@ -698,19 +705,23 @@ int bitcos_pack_device(const int8_t *trits, const uint16_t *scales_bf16, int64_t
         rc = check_cuda(cudaHostGetDevicePointer(reinterpret_cast<void **>(&report_dev), report.host(), 0));
         if (rc) return rc;
     }
-    bool once = false;
-    if (report.host() && n_tiles >= kOnceMin && n_tiles <= static_cast<int64_t>(kOnceTiles) * kOnceBlocks) {
-        report.host()[kFlagWait] = 0u;
-        rc = launch_once(pack_once_kernel, n_tiles, stream, trits, scales_bf16, M, K, bitmap, scales_tiled, tile_off, off_mapped, static_cast<int>(n_tiles),
-                         static_cast<int>(off_bytes / 4), signs, static_cast<int64_t>(sign_capacity_bytes / 16), max_nnz, report.slot,
-                         static_cast<volatile unsigned int *>(report_dev));
-        once = rc != kNotOnce;
-        if (once && rc) return rc;
+    bool once = report.host() && n_tiles <= static_cast<int64_t>(kOnceTiles) * kOnceRanges;
+    unsigned long long tag = 0;
+    if (once) {
+        tag = ReportSlot::next_tag(report.slot);
+        once = tag < kOnceTags;
     }
     auto enqueue = [&]() -> int {
         int e = BITCOS_OK;
         if (once) {
-            if (tile_off_host && !off_mapped) e = check_cuda(cudaMemcpyAsync(tile_off_host, tile_off, off_bytes, cudaMemcpyDeviceToHost, stream));
+            const int per_range = tiles_per_range(n_tiles);
+            report.host()[kFlagWait] = 0u;
+            pack_once_kernel<<<static_cast<unsigned>((n_tiles + per_range - 1) / per_range), kOnceThreads, static_cast<size_t>(per_range) * 516, stream>>>(
+                trits, scales_bf16, M, K, bitmap, scales_tiled, tile_off, off_mapped, static_cast<int>(n_tiles), per_range,
+                static_cast<int>(off_bytes / 4), signs, static_cast<int64_t>(sign_capacity_bytes / 16), max_nnz, report.slot, tag, kOnceLimitNs,
+                static_cast<volatile unsigned int *>(report_dev));
+            e = check_cuda(cudaGetLastError());
+            if (!e && tile_off_host && !off_mapped) e = check_cuda(cudaMemcpyAsync(tile_off_host, tile_off, off_bytes, cudaMemcpyDeviceToHost, stream));
             return e;
         }
         pack_bitmap_kernel<<<static_cast<unsigned>(grid), kPackWarps * 32, 0, stream>>>(
@@ -740,13 +751,7 @@ int bitcos_pack_device(const int8_t *trits, const uint16_t *scales_bf16, int64_t
         rc = read_flags(scratch, stream, h);         // (waits for the stream)
     }
     if (rc) return rc;
-    if (once && h[kFlagWait]) {
-        // (not all blocks were resident together: leave the state as a call finds it)
-        static const OnceState zero{};
-        cudaMemcpyToSymbolAsync(g_once_state, &zero, sizeof zero, sizeof zero * static_cast<size_t>(report.slot), cudaMemcpyHostToDevice, stream);
-        cudaStreamSynchronize(stream);
-        return check_cuda(cudaErrorLaunchTimeout);
-    }
+    if (once && h[kFlagWait]) return check_cuda(cudaErrorLaunchTimeout);      // (a block in front of another one stood still)
     if (h[kFlagTrit]) return BITCOS_ERR_TRIT;
     if (h[kFlagScale]) return BITCOS_ERR_SCALE;
     if (h[kFlagOverflow]) return BITCOS_ERR_OVERFLOW;

@@ -198,3 +198,22 @@ def test_device_pack_in_one_pass_reports_what_is_wrong(bc):
             bc.bitcos_pack_device(t, bad)
     again = bc.bitcos_pack_device(t, sc)
     assert torch.equal(again.signs, want.signs) and torch.equal(again.tile_off, want.tile_off)
+
+
+def test_device_pack_needs_no_free_chip(bc):
+    """Kernels that stay on a few multiprocessors neither hold a pack up nor keep it from starting: it returns while they run."""
+    M, K = 8192, 5120
+    gen = torch.Generator(device="cuda").manual_seed(11)
+    t = torch.randint(-1, 2, (M, K), generator=gen, device="cuda", dtype=torch.int8)
+    sc = torch.full((M, K // 128), 0.5, device="cuda").to(torch.bfloat16)
+    want = [bc.bitcos_pack_device(t, sc) for _ in range(2)][1]       # (and every buffer is in torch's cache)
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in range(4)]
+    for s in streams:
+        with torch.cuda.stream(s):
+            torch.cuda._sleep(400_000_000)                           # one thread each, about 0.2 s
+    got = bc.bitcos_pack_device(t, sc)
+    running = [not s.query() for s in streams]
+    torch.cuda.synchronize()
+    assert all(running)
+    assert torch.equal(got.signs, want.signs) and torch.equal(got.tile_off, want.tile_off) and torch.equal(got.bitmap, want.bitmap)

@@ -493,7 +493,7 @@ __global__ void __launch_bounds__(kOnceThreads, kOnceBlocks) pack_once_kernel(co
     if (warp == 0) {
         uint32_t base = 0u, bad = 0u;
         if (r && lane == 0) publish(st.range + r, range_word(total, s_bad, kStateOwn, tag));
-        const bool ok = look_back(st, r, tag, lane, limit_ns, base, bad);
+        const bool ok = (limit_ns || !r) && look_back(st, r, tag, lane, limit_ns, base, bad);
         __syncwarp();                                // (what the lanes have acquired, before lane 0 passes it on)
         if (lane == 0) {
             bad |= s_bad;
@@ -679,6 +679,13 @@ int bitcos_count_nnz_device(const int8_t *trits, int64_t M, int64_t K, uint64_t 
 int bitcos_pack_device(const int8_t *trits, const uint16_t *scales_bf16, int64_t M, int64_t K, uint32_t *bitmap,
                        uint32_t *signs, size_t sign_capacity_bytes, uint32_t *tile_off, uint16_t *scales_tiled,
                        uint32_t *tile_off_host, uint64_t *nnz_out, void *scratch, void *cuda_stream) {
+    return bitcos_pack_device_limited(trits, scales_bf16, M, K, bitmap, signs, sign_capacity_bytes, tile_off, scales_tiled, tile_off_host, nnz_out,
+                                      scratch, kOnceLimitNs, nullptr, cuda_stream);
+}
+
+int bitcos_pack_device_limited(const int8_t *trits, const uint16_t *scales_bf16, int64_t M, int64_t K, uint32_t *bitmap, uint32_t *signs,
+                               size_t sign_capacity_bytes, uint32_t *tile_off, uint16_t *scales_tiled, uint32_t *tile_off_host, uint64_t *nnz_out,
+                               void *scratch, uint64_t limit_ns, int *kernels, void *cuda_stream) {
     if (!trits || !scales_bf16 || !bitmap || !signs || !tile_off || !scales_tiled || !scratch) return BITCOS_ERR_NULL;
     if (M < 1 || K < kGroup || K % kGroup != 0) return BITCOS_ERR_SHAPE;
     if (!aligned16(trits) || !aligned16(scales_bf16) || !aligned16(bitmap) || !aligned16(signs) || !aligned16(tile_off) ||
@@ -718,7 +725,7 @@ int bitcos_pack_device(const int8_t *trits, const uint16_t *scales_bf16, int64_t
             report.host()[kFlagWait] = 0u;
             pack_once_kernel<<<static_cast<unsigned>((n_tiles + per_range - 1) / per_range), kOnceThreads, static_cast<size_t>(per_range) * 516, stream>>>(
                 trits, scales_bf16, M, K, bitmap, scales_tiled, tile_off, off_mapped, static_cast<int>(n_tiles), per_range,
-                static_cast<int>(off_bytes / 4), signs, static_cast<int64_t>(sign_capacity_bytes / 16), max_nnz, report.slot, tag, kOnceLimitNs,
+                static_cast<int>(off_bytes / 4), signs, static_cast<int64_t>(sign_capacity_bytes / 16), max_nnz, report.slot, tag, limit_ns,
                 static_cast<volatile unsigned int *>(report_dev));
             e = check_cuda(cudaGetLastError());
             if (!e && tile_off_host && !off_mapped) e = check_cuda(cudaMemcpyAsync(tile_off_host, tile_off, off_bytes, cudaMemcpyDeviceToHost, stream));
@@ -738,20 +745,27 @@ int bitcos_pack_device(const int8_t *trits, const uint16_t *scales_bf16, int64_t
             e = check_cuda(cudaMemcpyAsync(tile_off_host, tile_off, off_bytes, cudaMemcpyDeviceToHost, stream));
         return e;
     };
-    rc = enqueue();
-    if (rc) {
-        cudaStreamSynchronize(stream);               // what was enqueued writes the report's slot and the caller's buffers
-        return rc;
-    }
     unsigned int h[8];
-    if (report.host()) {
-        rc = check_cuda(cudaStreamSynchronize(stream));
-        for (int i = 0; i < 8; ++i) h[i] = static_cast<const volatile unsigned int *>(report.host())[i];
-    } else {
-        rc = read_flags(scratch, stream, h);         // (waits for the stream)
+    for (int launched = 0;;) {
+        rc = enqueue();
+        if (rc) {
+            cudaStreamSynchronize(stream);           // what was enqueued writes the report's slot and the caller's buffers
+            return rc;
+        }
+        launched += once ? 1 : 3;
+        if (kernels) *kernels = launched;
+        if (report.host()) {
+            rc = check_cuda(cudaStreamSynchronize(stream));
+            for (int i = 0; i < 8; ++i) h[i] = static_cast<const volatile unsigned int *>(report.host())[i];
+        } else {
+            rc = read_flags(scratch, stream, h);     // (waits for the stream)
+        }
+        if (rc) return rc;
+        if (!once || !h[kFlagWait]) break;
+        // A block in front of another one stood still for longer than the limit.  The three kernels wait for nothing of the kind,
+        // and write every output anew.
+        once = false;
     }
-    if (rc) return rc;
-    if (once && h[kFlagWait]) return check_cuda(cudaErrorLaunchTimeout);      // (a block in front of another one stood still)
     if (h[kFlagTrit]) return BITCOS_ERR_TRIT;
     if (h[kFlagScale]) return BITCOS_ERR_SCALE;
     if (h[kFlagOverflow]) return BITCOS_ERR_OVERFLOW;

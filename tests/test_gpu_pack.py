@@ -217,3 +217,65 @@ def test_device_pack_needs_no_free_chip(bc):
     torch.cuda.synchronize()
     assert all(running)
     assert torch.equal(got.signs, want.signs) and torch.equal(got.tile_off, want.tile_off) and torch.equal(got.bitmap, want.bitmap)
+
+
+class CPack:
+    """The C call with buffers of its own, so that a test sees all of them whatever the call returns."""
+
+    def __init__(self, bc, t, sc, sign_bytes=None, stream=None):
+        import ctypes as C
+        self.bc, self.L, self.t, self.sc, (M, K) = bc, bc.load_library(), t, sc, t.shape
+        n = [C.c_size_t(0) for _ in range(4)]
+        assert self.L.bitcos_pack_sizes(M, K, int((t != 0).sum()), *[C.byref(v) for v in n]) == 0
+        self.need = n[1].value
+        self.sign_bytes = self.need if sign_bytes is None else sign_bytes(self.need)
+        self.bitmap, self.off = (torch.full((v.value // 4,), -1, dtype=torch.int32, device="cuda") for v in (n[0], n[2]))
+        self.signs = torch.full((self.sign_bytes // 4 + 16,), -1, dtype=torch.int32, device="cuda")
+        self.scales = torch.full((n[3].value // 2,), -1, dtype=torch.int16, device="cuda")
+        self.scratch = torch.empty(256, dtype=torch.uint8, device="cuda")
+        self.off_host = torch.full((n[2].value // 4,), -1, dtype=torch.int32, pin_memory=True)
+        self.stream = stream or torch.cuda.current_stream()
+        torch.cuda.synchronize()
+
+    def run(self, limit_ns=500_000_000):
+        import ctypes as C
+        nnz, kernels, (M, K) = C.c_uint64(0), C.c_int(0), self.t.shape
+        rc = self.L.bitcos_pack_device_limited(
+            self.t.data_ptr(), self.sc.data_ptr(), M, K, self.bitmap.data_ptr(), self.signs.data_ptr(), self.sign_bytes, self.off.data_ptr(),
+            self.scales.data_ptr(), self.off_host.data_ptr(), C.byref(nnz), self.scratch.data_ptr(), limit_ns, C.byref(kernels),
+            self.stream.cuda_stream)
+        return rc, kernels.value, nnz.value
+
+    def equals(self, W):
+        """All of this call's buffers against a packed matrix; nothing behind the sign vector was touched."""
+        n, full = W.signs.numel(), self.sign_bytes // 16 * 4
+        return (torch.equal(self.bitmap, W.bitmap) and torch.equal(self.off, W.tile_off) and torch.equal(self.scales, W.scales)
+                and torch.equal(self.signs[:n], W.signs) and not self.signs[n:full].any() and bool((self.signs[full:] == -1).all())
+                and np.array_equal(self.off_host.numpy()[:W.tile_off_host.size].view(np.uint32), W.tile_off_host))
+
+
+def trits_and_scales(seed, M, K):
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    t = torch.randint(-1, 2, (M, K), generator=gen, device="cuda", dtype=torch.int8)
+    return t, (0.01 + torch.rand((M, K // 128), generator=gen, device="cuda")).to(torch.bfloat16)
+
+
+@pytest.mark.parametrize("M,K", [(32, 1024), (32, 1152), (300, 1280), (2560, 2560), (4097, 6144), (32 * 4737, 128), (25600, 5120)])
+def test_device_pack_goes_on_when_its_wait_runs_out(bc, M, K):
+    """With no time to wait every block but the first gives up; the call then packs in three kernels, and the same state serves the
+    calls after it.  (Up to eight tiles are one block's, which waits for nobody.)"""
+    t, sc = trits_and_scales(31 + M + K, M, K)
+    W = bc.bitcos_pack_device(t, sc)
+    gives_up = (M + 31) // 32 * (K // 128) > 8
+    for limit, want in ((500_000_000, 1), (0, 4 if gives_up else 1), (0, 4 if gives_up else 1), (500_000_000, 1)):
+        call = CPack(bc, t, sc)
+        assert call.run(limit) == (0, want, W.nnz) and call.equals(W), limit
+    if not gives_up:
+        return
+    bad = t.clone()
+    bad[M - 1, K - 1] = 3
+    assert CPack(bc, bad, sc).run(0)[:2] == (4, 4)
+    bad = sc.clone()
+    bad[M - 1, 0] = -1.0
+    assert CPack(bc, t, bad).run(0)[:2] == (5, 4)
+    assert CPack(bc, t, sc, lambda need: need - 16).run(0)[:2] == (6, 4)

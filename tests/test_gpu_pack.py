@@ -158,10 +158,11 @@ def test_device_pack_with_offsets_to_memory_that_is_pinned_in_part(bc):
             assert int(rt.cudaHostUnregister(host.ctypes.data)) == 0
 
 
-@pytest.mark.parametrize("M,K", [(32 * 6143, 128), (32 * 6144, 128), (32 * 6145 - 7, 128), (32 * 1537, 512), (4097, 6144), (32 * 65121, 128)])
+@pytest.mark.parametrize("M,K", [(32 * 6143, 128), (32 * 6144, 128), (32 * 6145 - 7, 128), (32 * 1537, 512), (4097, 6144), (32 * 65121, 128),
+                                 (32 * 180224, 128), (32 * 180225, 128)])
 def test_device_pack_in_one_pass_and_in_three_kernels(bc, M, K):
-    """Matrices on both sides of the lines between the packer's two ways (6144 tiles, 440 tiles per multiprocessor), whole, against
-    their upper and lower parts: the same bitmap and scales, offsets that go on where the upper part ends, the same sign bits."""
+    """Matrices of many sizes and on both sides of the line between the packer's two ways (180224 tiles), whole, against their
+    upper and lower parts: the same bitmap and scales, offsets that go on where the upper part ends, the same sign bits."""
     gen = torch.Generator(device="cuda").manual_seed(M + K)
     t = torch.randint(-1, 2, (M, K), generator=gen, device="cuda", dtype=torch.int8)
     top = M // 64 * 32
@@ -177,6 +178,9 @@ def test_device_pack_in_one_pass_and_in_three_kernels(bc, M, K):
     assert np.array_equal(whole.tile_off_host, off) and np.array_equal(u32(whole.tile_off)[:off.size], off) and first == top // 32 * (K // 128)
     last = (whole.nnz + 31) // 32
     assert torch.equal(whole.signs[:last], torch.cat([parts[0].signs[:words], parts[1].signs[:last - words]])) and not whole.signs[last:].any()
+    del parts, off
+    call = CPack(bc, t, sc)
+    assert call.run() == (0, 1 if (M + 31) // 32 * (K // 128) <= 180224 else 3, whole.nnz) and call.equals(whole)
 
 
 def test_device_pack_in_one_pass_reports_what_is_wrong(bc):
@@ -279,3 +283,64 @@ def test_device_pack_goes_on_when_its_wait_runs_out(bc, M, K):
     bad[M - 1, 0] = -1.0
     assert CPack(bc, t, bad).run(0)[:2] == (5, 4)
     assert CPack(bc, t, sc, lambda need: need - 16).run(0)[:2] == (6, 4)
+
+
+@pytest.mark.parametrize("M,K", [(96, 640), (2560, 2560), (8192, 5120)])
+def test_device_pack_and_the_size_of_the_sign_vector(bc, M, K):
+    """One bit short, exactly as large as needed, and larger: the error, and zeros up to the end of what was given."""
+    t, sc = trits_and_scales(47 + M, M, K)
+    W = bc.bitcos_pack_device(t, sc)
+    for more, rc in ((-16, 6), (0, 0), (16, 0), (32 * 1024 + 48, 0), (2 * M * K // 8, 0)):
+        call = CPack(bc, t, sc, lambda need: need + more)
+        assert call.run()[:2] == (rc, 1), more
+        if rc == 0:
+            assert call.equals(W), more
+        assert bool((call.signs[call.sign_bytes // 4:] == -1).all()), more
+
+
+def test_device_pack_from_several_threads(bc):
+    """Four host threads pack matrices of different sizes on streams of their own, over and over: every call has state of its own."""
+    import threading
+    jobs = [(trits_and_scales(61 + i, M, K), torch.cuda.Stream()) for i, (M, K) in enumerate(((8192, 5120), (2555, 6912), (25600, 5120), (96, 1280)))]
+    want = [bc.bitcos_pack_device(t, sc) for (t, sc), _ in jobs]
+    right = []
+
+    def work(i):
+        (t, sc), stream = jobs[i]
+        with torch.cuda.stream(stream):
+            for n in range(12):
+                call = CPack(bc, t, sc, stream=stream)
+                if call.run(0 if n % 4 == 3 else 500_000_000)[0] == 0 and call.equals(want[i]):
+                    right.append((i, n))
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(len(jobs))]
+    for th in threads:
+        th.start()
+    for th in threads:
+        th.join()
+    assert sorted(right) == [(i, n) for i in range(len(jobs)) for n in range(12)]
+
+
+def test_device_pack_when_all_states_are_taken(bc):
+    """Seventy calls at a time, held up behind a kernel that waits: 64 find a state, the others pack in three kernels."""
+    import threading
+    t, sc = trits_and_scales(71, 640, 2560)
+    want = bc.bitcos_pack_device(t, sc)
+    n = 70
+    calls = [CPack(bc, t, sc, stream=torch.cuda.Stream()) for _ in range(n)]
+    ready, got = threading.Barrier(n), [None] * n
+
+    def work(i):
+        with torch.cuda.stream(calls[i].stream):
+            torch.cuda._sleep(800_000_000)
+        ready.wait()
+        got[i] = calls[i].run()
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(n)]
+    for th in threads:
+        th.start()
+    for th in threads:
+        th.join()
+    torch.cuda.synchronize()
+    assert sorted(k for _, k, _ in got) == [1] * 64 + [3] * (n - 64)
+    assert all(rc == 0 and nnz == want.nnz for rc, _, nnz in got) and all(c.equals(want) for c in calls)

@@ -1205,32 +1205,24 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
         constexpr int RF = NB;
         auto add4 = [](float4 a, float4 b) { return add_quads<(NB <= 8 && !kBlend)>(a, b); };
         const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
-        // (A guarded load takes four instructions.  A batch that is full, or as long as the second one of rows of 16 or 18 groups, has none:
-        // with packed additions and the warp's number in uniform registers MoE pass of 128 experts 57.6 -> 56.2 us, 18944 -> 56832 x 5120
-        // at four | eight tokens 121 | 127 -> 117 | 126 clocks per tile.)
-        auto batch = [&](auto size, const float *base, int n) {
-            constexpr int N = decltype(size)::value;         // tiles, 0: n of them
+        auto batch = [&](const float *base, int n) {
             float4 v[10];
 #pragma unroll
-            for (int j = 0; j < 10; ++j) v[j] = (N ? j < N : j < n) ? *reinterpret_cast<const float4 *>(base + j * kRows * RF) : none;
+            for (int j = 0; j < 10; ++j) v[j] = j < n ? *reinterpret_cast<const float4 *>(base + j * kRows * RF) : none;
 #pragma unroll
             for (int w2 = 1; w2 < 10; w2 *= 2)
 #pragma unroll
-                for (int j = 0; j + w2 < 10; j += 2 * w2)
-                    if (!N || j + w2 < N) v[j] = add4(v[j], v[j + w2]);
+                for (int j = 0; j + w2 < 10; j += 2 * w2) v[j] = add4(v[j], v[j + w2]);
             return v[0];
         };
+        // The second batch is left out of rows of nine or ten tiles (128 experts of 768 x 1152 | 1280 at eight tokens 11.0 | 11.7 -> 10.3 | 11.0 us;
+        // with sixteen tokens and in the 16-bit variant there is no such test).  A form without guards for full batches and for second ones of six
+        // or eight tiles gained nothing at those lengths and cost every other one: 4736 rows of 12 | 17 | 19 groups at eight
+        // tokens 4.9 | 5.3 | 5.3 -> 5.1 | 5.5 | 5.5 us, without it 4.8 | 5.2 | 5.2; 16 | 18 groups 5.3 | 5.3 -> 5.2 | 5.2 with and without.
         auto in_tens = [&](const float *base, int n) {
-            if constexpr (NB > 8 || kBlend) return add4(batch(std::integral_constant<int, 0>{}, base, n), batch(std::integral_constant<int, 0>{}, base + 10 * kRows * RF, n - 10));
-            if (n < 10) return batch(std::integral_constant<int, 0>{}, base, n);
-            const float4 tot = batch(std::integral_constant<int, 10>{}, base, 10);
-            base += 10 * kRows * RF;
-            n -= 10;
-            if (n == 0) return tot;
-            if (n == 10) return add4(tot, batch(std::integral_constant<int, 10>{}, base, n));
-            if (n == 6) return add4(tot, batch(std::integral_constant<int, 6>{}, base, n));
-            if (n == 8) return add4(tot, batch(std::integral_constant<int, 8>{}, base, n));
-            return add4(tot, batch(std::integral_constant<int, 0>{}, base, n));
+            const float4 tot = batch(base, n);
+            if (NB <= 8 && !kBlend && n <= 10) return tot;
+            return add4(tot, batch(base + 10 * kRows * RF, n - 10));
         };
         auto sum_tiles4 = [&](const float *base, int n) {
             if (n > 8) return in_tens(base, n);
@@ -1255,11 +1247,13 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
             return tot;
         };
         // the same from the sums of neighbouring tiles (n of them: nine tiles and more are five and more)
+        // (Ten of them without guards: at four tokens large launches of rows of 14 | 19 | 20 groups 11.23 | 10.88 | 10.96 -> 11.10 | 10.84 | 10.90 us; at
+        // eight the second form costs all lengths, 12 | 17 | 20 groups 12.8 | 11.4 | 11.5 -> 13.9 | 12.0 | 11.7.)
         auto sum_pairs4 = [&](const float *base, int n) {
             auto at = [&](int j) { return *reinterpret_cast<const float4 *>(base + j * kRows * RF); };
             if (n > 4) {
                 float4 v[10];
-                if (n == 10) {
+                if (NB < 8 && n == 10) {
 #pragma unroll
                     for (int j = 0; j < 10; ++j) v[j] = at(j);
                 } else {

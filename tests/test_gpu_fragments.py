@@ -89,7 +89,7 @@ def test_16_bit_variant(bc, groups, blocks):
 
 @pytest.mark.parametrize("groups", [9, 10, 11, 13, 15, 16, 17, 18, 19, 20, 36, 38])
 def test_partial_sums_in_full_and_guarded_batches(bc, groups):
-    """The epilogue adds a row block's sums ten at a time, a batch of ten, eight or six without guards; rows of every such number of
+    """The epilogue adds a row block's sums ten at a time, with a second batch for more than ten; rows of such numbers of
     tiles (36 and 38: two column blocks of 18 and 19), all three formats, four to sixteen tokens."""
     M, K = 32 * 7 - 3, 128 * groups
     W, S = datagen.trits(700 + groups, M, K, 0.42), datagen.scales(700 + groups, M, K)

@@ -1203,26 +1203,38 @@ __device__ __forceinline__ void run_segments(const Segs &segs, const Plan &pl_in
         // Tensor-core layout: four tokens at a time, spaced one warp's rows apart; more than eight tiles in two batches of ten,
         // all loads of a batch before its first addition (three smaller batches cost the sixteen-token layer 3 %).
         constexpr int RF = NB;
-        auto add4 = [](float4 a, float4 b) { return add_quads<(NB <= 8 && !kBlend)>(a, b); };
+        // (2-bit rows at eight tokens: packed additions and the short form of in_tens cost 25600 x 5120 20.9 -> 21.7 us, 12288 x 4096 9.5 -> 9.9, and give
+        // rows of nine groups 6.2 -> 5.7)
+        constexpr bool kShortSums = NB <= 8 && !kBlend && !(FMT == kBit2 && NB == 8);
+        auto add4 = [](float4 a, float4 b) { return add_quads<kShortSums>(a, b); };
         const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
-        auto batch = [&](const float *base, int n) {
+        auto batch = [&](auto full, const float *base, int n) {
             float4 v[10];
 #pragma unroll
-            for (int j = 0; j < 10; ++j) v[j] = j < n ? *reinterpret_cast<const float4 *>(base + j * kRows * RF) : none;
+            for (int j = 0; j < 10; ++j) v[j] = decltype(full)::value || j < n ? *reinterpret_cast<const float4 *>(base + j * kRows * RF) : none;
 #pragma unroll
             for (int w2 = 1; w2 < 10; w2 *= 2)
 #pragma unroll
                 for (int j = 0; j + w2 < 10; j += 2 * w2) v[j] = add4(v[j], v[j + w2]);
             return v[0];
         };
-        // The second batch is left out of rows of nine or ten tiles (128 experts of 768 x 1152 | 1280 at eight tokens 11.0 | 11.7 -> 10.3 | 11.0 us;
-        // with sixteen tokens and in the 16-bit variant there is no such test).  A form without guards for full batches and for second ones of six
-        // or eight tiles gained nothing at those lengths and cost every other one: 4736 rows of 12 | 17 | 19 groups at eight
-        // tokens 4.9 | 5.3 | 5.3 -> 5.1 | 5.5 | 5.5 us, without it 4.8 | 5.2 | 5.2; 16 | 18 groups 5.3 | 5.3 -> 5.2 | 5.2 with and without.
+        // The second batch is left out of rows of nine or ten tiles (96 experts of 768 x 1152 | 1280 at eight tokens 11.0 | 11.7 -> 10.3 | 11.0 us).
+        // Forms of a batch without guards grow this warp's code, which costs every length: with forms for full batches and for second ones
+        // of six or eight, 4736 rows of 12 | 17 | 19 groups at eight tokens went from 4.9 | 5.3 | 5.3 to 5.1 | 5.5 | 5.5 us, without them 4.8 |
+        // 5.2 | 5.2; 16 | 18 groups 5.3 | 5.3 -> 5.2 | 5.2 with and without.  Full batches alone pay at five-trit rows and eight tokens
+        // (25600 x 5120 26.1 -> 24.7, 16384 x 5120 17.3 -> 16.9, 18944 x 1536 8.0 -> 8.2).
         auto in_tens = [&](const float *base, int n) {
-            const float4 tot = batch(base, n);
-            if (NB <= 8 && !kBlend && n <= 10) return tot;
-            return add4(tot, batch(base + 10 * kRows * RF, n - 10));
+            const float *second = base + 10 * kRows * RF;
+            if constexpr (FMT == kTrit5 && NB == 8) {
+                if (n >= 10) {
+                    const float4 tot = batch(std::true_type{}, base, 10);
+                    if (n == 10) return tot;
+                    return add4(tot, n == 20 ? batch(std::true_type{}, second, 10) : batch(std::false_type{}, second, n - 10));
+                }
+            }
+            const float4 tot = batch(std::false_type{}, base, n);
+            if (kShortSums && n <= 10) return tot;
+            return add4(tot, batch(std::false_type{}, second, n - 10));
         };
         auto sum_tiles4 = [&](const float *base, int n) {
             if (n > 8) return in_tens(base, n);

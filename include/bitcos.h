@@ -235,15 +235,17 @@ int bitcos_decode_probe_sums(int format, int warps_per_block, int iters, int blo
  *   variant 0  shifted window: (presence nibble, sign nibble) table of Eq. 4, the window of a word
  *              shifted by each nibble's population count; decode into registers, then contract
  *   variant 1  running position: the same table, windows never shifted, a running bit position per
- *              word updated by the dp4a that counts; contraction fused (what the products run)
+ *              word updated by the dp4a that counts; contraction fused
  *   variant 2  byte table: eight weights per step from a 3^8-entry table behind a 256-entry index
  *   variant 3  no table: the deposit of Fig. 4 with shifts and masks, contraction on bit planes
  *   variant 4  lane = bit: one presence word per warp step, sign slot = population count of the
  *              lower bits, products added across the warp
  *   variant 5, 6, 7  split row: the first 1, 2, 3 presence words of a row as variant 1, the others as
  *              variant 3 (loads the shared-memory pipe and the integer ALU at the same time)
+ *   variant 8  keyed row: running positions, the key of a presence byte by dp4a, decode into registers,
+ *              then contract (what the products run at one token, on their table)
  * ERR_CAPACITY if the item does not fit into shared memory with the variant's tables. */
-#define BITCOS_PROBE_VARIANTS 8
+#define BITCOS_PROBE_VARIANTS 9
 int bitcos_decode_probe_variant(int variant, const uint32_t *bitmap, const uint32_t *signs, size_t sign_bytes,
                                 const uint32_t *tile_off, int n_tiles, const int8_t *x, int iters, int blocks,
                                 uint64_t *cycles, int32_t *acc_out, void *cuda_stream);

@@ -786,7 +786,7 @@ def bitcos_decode_probe(fmt: int, warps_per_block: int, iters: int, blocks: int,
 
 
 PROBE_VARIANTS = ("shifted window", "running position", "byte table", "no table", "lane = bit", "split row 1+3",
-                  "split row 2+2", "split row 3+1")
+                  "split row 2+2", "split row 3+1", "keyed row")
 
 
 def bitcos_decode_probe_variant(variant: int, W: DeviceBitcos, first_tile: int, n_tiles: int, x, iters: int, blocks: int,

@@ -5,7 +5,7 @@
 // The GPU has no bit-deposit instruction (Fig. 4), so the scatter of the compacted signs onto the
 // present positions is done in software.  Several structurally different ways of doing it live
 // here, so that their on-chip cost (the gamma of the paper's two-term roofline, Eq. 6) can be
-// measured side by side; the GEMV kernels use the cheapest one.
+// measured side by side; the products run bitcos_decode_row_keyed at one token and FragmentRows from two on.
 #ifndef BITCOS_DECODE_CUH
 #define BITCOS_DECODE_CUH
 
@@ -174,11 +174,12 @@ __device__ __forceinline__ void sign_windows(const uint4 bm, const uint32_t *sp,
 }
 
 // ---------------------------------------------------------------------------------------------
-// Decoder A ("shifted window"): the 256-entry (presence nibble, sign nibble) table of Eq. 4; every
-// word keeps its sign window in a register and shifts it by the number of sign bits a nibble
+// Decoder A ("shifted window"; in the decode-rate probe only, as are decoders B to F): the 256-entry (presence nibble,
+// sign nibble) table of Eq. 4; every word keeps its sign window in a register and shifts it by the number of sign bits a nibble
 // consumed (dp4a(e, e) of the looked-up entry).  Produces the row's 32 int8x4 words; the
 // contraction follows as a separate step.  Five instructions per nibble besides the contraction:
-// shift-left, bit-select, table load, dp4a popcount, shift-right.
+// shift-left, bit-select, table load, dp4a popcount, shift-right.  The tables of A, B and F are laid out by
+// key * 256 + sub * 128 + lane * 4, a presence byte in address bits 8..15 (probe.cu makes them).
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ void bitcos_decode_row(const uint4 bm, const uint32_t *sp, uint32_t sh, const uint8_t *lut,
                                                   uint32_t lane4, int (&w)[32]) {
@@ -223,7 +224,7 @@ __device__ __forceinline__ void bitcos_decode_row_keyed(const uint4 bm, const ui
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         B[j] = __funnelshift_r(A[j], A[j], 4);
-        pos[j] = 21;                                  // a right rotation by 21 puts bit 0 on bit 11 (of B: bit 4 on bit 7)
+        pos[j] = 21;                                  // a right rotation by 21 puts bit 0 on bit 11 (B's bit 28, the same sign, on bit 7)
     }
 #pragma unroll
     for (int k = 0; k < 4; ++k) {

@@ -68,9 +68,9 @@ probe_variant_kernel(const uint32_t *__restrict__ bitmap, const uint32_t *__rest
 
     // ---- set-up (untimed): tables, the item's packed bytes, activations in both orders
     if (VAR <= 1 || VAR >= 5) {
-        // byte address = key * 256 + sub * 128 + lane * 4 (see make_bitcos_lut)
+        // byte address = key * 256 + sub * 128 + lane * 4; the products' decoder (8): as in make_bitcos_lut
         for (int idx = threadIdx.x; idx < kLutBytes / 4; idx += blockDim.x) {
-            const int key = idx >> 6, sub = (idx >> 5) & 1;
+            const int key = VAR == 8 ? (idx >> 5) & 255 : idx >> 6, sub = VAR == 8 ? idx >> 13 : (idx >> 5) & 1;
             reinterpret_cast<uint32_t *>(lut)[idx] = g_probe_nibble_lut.v[sub ? (((key & 15) << 4) | (key >> 4)) : key];
         }
     }
@@ -117,9 +117,10 @@ probe_variant_kernel(const uint32_t *__restrict__ bitmap, const uint32_t *__rest
             const uint32_t cursor = toff + static_cast<uint32_t>(incl - c);
             const uint32_t *sp = s_signs + (cursor >> 5) + at;
             const uint8_t *xg = s_x + warp * 128 + at, *xpg = s_xp + warp * 128 + at;
-            if (VAR == 0) {
+            if (VAR == 0 || VAR == 8) {
                 int w[32];
-                bitcos_decode_row(bm, sp, cursor & 31u, lut, lane4, w);
+                if (VAR == 0) bitcos_decode_row(bm, sp, cursor & 31u, lut, lane4, w);
+                else bitcos_decode_row_keyed(bm, sp, cursor & 31u, lut, lane4, w);
                 asm volatile("" ::: "memory");
                 a = row_contract(w, reinterpret_cast<const int4 *>(xg));
             } else if (VAR == 1) {
@@ -193,6 +194,7 @@ extern "C" int bitcos_decode_probe_variant(int variant, const uint32_t *bitmap, 
         case 4: return launch_probe<4>(bitmap, signs, tile_off, sw, x, n_tiles, iters, blocks, out, acc_out, stream);
         case 5: return launch_probe<5>(bitmap, signs, tile_off, sw, x, n_tiles, iters, blocks, out, acc_out, stream);
         case 6: return launch_probe<6>(bitmap, signs, tile_off, sw, x, n_tiles, iters, blocks, out, acc_out, stream);
-        default: return launch_probe<7>(bitmap, signs, tile_off, sw, x, n_tiles, iters, blocks, out, acc_out, stream);
+        case 7: return launch_probe<7>(bitmap, signs, tile_off, sw, x, n_tiles, iters, blocks, out, acc_out, stream);
+        default: return launch_probe<8>(bitmap, signs, tile_off, sw, x, n_tiles, iters, blocks, out, acc_out, stream);
     }
 }

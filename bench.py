@@ -895,7 +895,7 @@ def quant_detail(bc, torch, stream):
 
 def pack_detail(bc, torch):
     """Device-side packing (set-up path): int8 trits + bf16 scales in device memory -> the BITCOS
-    buffers.  Wall time of the whole call (three kernels, two stream waits, the sign vector cut to size), against
+    buffers.  Wall time of the whole call (one kernel, one stream wait, the sign vector cut to size), against
     the bytes it has to move once: the trits in, the packed buffers out."""
     import time
     import datagen

@@ -494,8 +494,8 @@ __device__ __forceinline__ int bitcos_row_dot_bytes(const uint4 bm, const uint32
 
 // ---------------------------------------------------------------------------------------------
 // Decoder D ("no table"): the deposit of Fig. 4 carried out with shifts and masks on whole 32-bit
-// words (five rounds that move the sign bits up by 16, 8, 4, 2 and 1 places under masks derived
-// from the presence word by a parallel-prefix count of its zeros), then the contraction on bit
+// words (the expand of Warren, "Hacker's Delight", 2nd ed., section 7-5: five rounds that move the sign bits up by 16, 8, 4, 2 and
+// 1 places under masks derived from the presence word by a parallel-prefix count of its zeros), then the contraction on bit
 // planes: a presence (or negative) word masked with 0x01010101 << i holds bits 8 b + i as bytes of
 // value 2^i, which an unsigned-by-signed dp4a multiplies with the four activations of those
 // positions; acc = sum(p * x) - 2 sum(n * x), Eq. 2.  No shared-memory table at all.

@@ -476,7 +476,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
     return mbar_wait_slow(bar, parity);
 }
 
-// Four additions, packed in two instructions where that pays (with sixteen tokens the pairs and the unguarded batches below cost the
+// Four additions, packed in two instructions where that pays (with sixteen tokens pairs, and batches without guards, cost the
 // 32B-model layer 103.5 -> 106 us, in the 16-bit variant 8192x5120 at four tokens 11.30 -> 11.40).
 template <bool PACKED>
 __device__ __forceinline__ float4 add_quads(float4 a, float4 b) {

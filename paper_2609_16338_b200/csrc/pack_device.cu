@@ -80,7 +80,8 @@ __device__ __forceinline__ uint4 load_chunk(const int8_t *__restrict__ trits, in
 }
 
 // The bits of both halves of `src` at the set positions of the halves of `mask`, packed towards bit 0 of each half (the inverse
-// of the deposit of Fig. 4): parallel-suffix compress, in round i every selected bit moves right by 2^i if the number of
+// of the deposit of Fig. 4): the parallel-suffix compress of Warren, "Hacker's Delight", 2nd ed., section 7-4, its shifts kept inside the
+// halves; in round i every selected bit moves right by 2^i if the number of
 // unselected positions below it has bit i set.
 __device__ __forceinline__ uint32_t extract_halves(uint32_t src, uint32_t mask) {
     uint32_t x = src & mask, m = mask;

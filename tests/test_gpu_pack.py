@@ -328,17 +328,22 @@ def test_device_pack_when_all_states_are_taken(bc):
     want = bc.bitcos_pack_device(t, sc)
     n = 70
     calls = [CPack(bc, t, sc, stream=torch.cuda.Stream()) for _ in range(n)]
-    ready, got = threading.Barrier(n), [None] * n
+    ready, got = threading.Barrier(n + 1), [None] * n
 
     def work(i):
-        with torch.cuda.stream(calls[i].stream):
-            torch.cuda._sleep(800_000_000)
         ready.wait()
         got[i] = calls[i].run()
 
     threads = [threading.Thread(target=work, args=(i,)) for i in range(n)]
     for th in threads:
         th.start()
+    holder = torch.cuda.Stream()
+    with torch.cuda.stream(holder):
+        torch.cuda._sleep(1_500_000_000)                             # one thread, about 0.8 s
+    for c in calls:
+        if c.stream.cuda_stream != holder.cuda_stream:
+            c.stream.wait_stream(holder)
+    ready.wait()
     for th in threads:
         th.join()
     torch.cuda.synchronize()

@@ -149,9 +149,9 @@ int bitcos_count_nnz_device(const int8_t *trits, int64_t M, int64_t K, uint64_t 
  * tile_off size receiving a copy (for bitcos_weights.tile_off_host).  nnz_out (optional, host).
  * ERR_TRIT / ERR_SCALE / ERR_OVERFLOW as for bitcos_pack; ERR_CAPACITY if the sign vector does
  * not fit (outputs are then incomplete).
- * One kernel packs matrices of up to 180224 tiles, in any number of blocks that find room beside whatever else runs on
+ * One kernel packs matrices of 6144 to 180224 tiles, in any number of blocks that find room beside whatever else runs on
  * the device: a block waits only for blocks that started before it, half a second at most.  If that runs out, and for
- * larger matrices, three kernels do the work, which wait for nothing.  Calls from several threads and on several streams
+ * other sizes, three kernels do the work, which wait for nothing.  Calls from several threads and on several streams
  * may overlap (a scratch each). */
 int bitcos_pack_device(const int8_t *trits, const uint16_t *scales_bf16, int64_t M, int64_t K, uint32_t *bitmap,
                        uint32_t *signs, size_t sign_capacity_bytes, uint32_t *tile_off, uint16_t *scales_tiled,

@@ -8,17 +8,18 @@
 // 16-weight chunks in the order (load, lane) are the tile's weights in order, and the sign bits of a chunk lie where a
 // scan of the chunk counts puts them.
 //
-// Where a tile's sign bits go is known only when everything before it has been counted.  One kernel does all of it (pack_once_kernel): a
-// block keeps the compacted sign bits of its tiles in shared memory until the tiles before have been counted, so that the
-// trits are read and looked at once.  Matrices with more tiles than its ranges hold and calls that find no state to share
-// take three kernels: bitmap + scales + per-tile counts (and the sign vector zeroed); an exclusive scan of the counts (the entry
-// offsets); the sign vector, from a second reading, mostly from L2.
+// Where a tile's sign bits go is known only when everything before it has been counted.  From kOnceMin tiles on one kernel does all of it
+// (pack_once_kernel): a block keeps the compacted sign bits of its tiles in shared memory until the tiles before have been
+// counted, so that the trits are read and looked at once.  Smaller matrices, those with more tiles than its ranges hold and calls that
+// find no state to share take three kernels: bitmap + scales + per-tile counts (and the sign vector zeroed); an exclusive scan of
+// the counts (the entry offsets); the sign vector, from a second reading, mostly from L2.
 //
-// A whole call through the binding, three kernels -> one, us: 32 tiles 78 -> 72, 400 79 -> 77, 1600 82 -> 81, 2560 83 -> 84, 4096 86 -> 84, 6144
-// 76 -> 75, 10240 (8192x5120) 88 -> 81, 20480 118 -> 98, 32000 (25600x5120) 154 -> 116, 64000 243 -> 176 (as a cooperative launch of one block of 1024
-// threads per multiprocessor the last four took 82, 100, 115 and 188).  About 40 of them are allocations and calls in Python; the
-// trits of 8192x5120 would pass in 6.4 at the memory's rate.  A tile is about 1100 warp instructions (a quarter of them the
-// compress), 0.19 us a tile and multiprocessor, which bounds the kernel; behind the tiles come the look-back and the sign words.
+// A C call, three kernels -> one, medians of calls in turn, us: 64 tiles 21.2 -> 19.2, 256 21.7 -> 21.8, 1024 22.4 -> 23.9, 2560 32.6 -> 34.0, 4096 28.9 ->
+// 31.0, 6144 33.6 -> 33.5, 8192 38.9 -> 34.9, 10240 (8192x5120) 43.4 -> 38.1, 20480 70.6 -> 53.8, 32000 (25600x5120) 104.7 -> 69.0.  With few tiles the
+// look-back's trips to L2 are a larger part than a second reading.  Through the binding 8192x5120 takes 77 (as a cooperative launch of
+// one block of 1024 threads per multiprocessor 81), about 40 of them allocations and calls in Python; the trits would pass in 6.4 at
+// the memory's rate.  A tile is about 1100 warp instructions (a quarter of them the compress), 0.19 us a tile and multiprocessor, which bounds the
+// kernel; behind the tiles come the look-back and the sign words.
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -328,7 +329,7 @@ __device__ __forceinline__ uint32_t scan_add(uint32_t v) {
 // of one block per multiprocessor waited for all of the chip to be free).  The waits are bounded all the same.
 constexpr int kOnceThreads = 256;
 constexpr int kOnceTiles = 88;                   // per range at most: 516 bytes each, together within the 48 KB that need no attribute
-constexpr int kOnceStep = 8;                     // tiles per range at least: one per warp
+constexpr int kOnceMin = 6144;                   // tiles: from here on one kernel is faster (see above)
 constexpr int kOnceBlocks = 4;                   // resident per multiprocessor (64 registers a thread)
 constexpr int kOnceRanges = 2048;
 constexpr unsigned long long kOnceLimitNs = 500ull * 1000 * 1000;
@@ -584,7 +585,6 @@ int tiles_per_range(int64_t n_tiles) {
     const int64_t at_once = static_cast<int64_t>(sms) * kOnceBlocks;
     const int64_t rounds = (n_tiles + at_once * kOnceTiles - 1) / (at_once * kOnceTiles);
     int64_t per_range = (n_tiles + at_once * rounds - 1) / (at_once * rounds);
-    if (per_range < kOnceStep) per_range = kOnceStep;
     while (per_range * kOnceRanges < n_tiles) ++per_range;
     return static_cast<int>(per_range);
 }
@@ -713,7 +713,7 @@ int bitcos_pack_device_limited(const int8_t *trits, const uint16_t *scales_bf16,
         rc = check_cuda(cudaHostGetDevicePointer(reinterpret_cast<void **>(&report_dev), report.host(), 0));
         if (rc) return rc;
     }
-    bool once = report.host() && n_tiles <= static_cast<int64_t>(kOnceTiles) * kOnceRanges;
+    bool once = report.host() && n_tiles >= kOnceMin && n_tiles <= static_cast<int64_t>(kOnceTiles) * kOnceRanges;
     unsigned long long tag = 0;
     if (once) {
         tag = ReportSlot::next_tag(report.slot);

@@ -161,7 +161,7 @@ def test_device_pack_with_offsets_to_memory_that_is_pinned_in_part(bc):
 @pytest.mark.parametrize("M,K", [(32 * 6143, 128), (32 * 6144, 128), (32 * 6145 - 7, 128), (32 * 1537, 512), (4097, 6144), (32 * 65121, 128),
                                  (32 * 180224, 128), (32 * 180225, 128)])
 def test_device_pack_in_one_pass_and_in_three_kernels(bc, M, K):
-    """Matrices of many sizes and on both sides of the line between the packer's two ways (180224 tiles), whole, against their
+    """Matrices on both sides of the lines between the packer's two ways (6144 and 180224 tiles), whole, against their
     upper and lower parts: the same bitmap and scales, offsets that go on where the upper part ends, the same sign bits."""
     gen = torch.Generator(device="cuda").manual_seed(M + K)
     t = torch.randint(-1, 2, (M, K), generator=gen, device="cuda", dtype=torch.int8)
@@ -180,7 +180,7 @@ def test_device_pack_in_one_pass_and_in_three_kernels(bc, M, K):
     assert torch.equal(whole.signs[:last], torch.cat([parts[0].signs[:words], parts[1].signs[:last - words]])) and not whole.signs[last:].any()
     del parts, off
     call = CPack(bc, t, sc)
-    assert call.run() == (0, 1 if (M + 31) // 32 * (K // 128) <= 180224 else 3, whole.nnz) and call.equals(whole)
+    assert call.run() == (0, kernels(M, K), whole.nnz) and call.equals(whole)
 
 
 def test_device_pack_in_one_pass_reports_what_is_wrong(bc):
@@ -243,12 +243,12 @@ class CPack:
 
     def run(self, limit_ns=500_000_000):
         import ctypes as C
-        nnz, kernels, (M, K) = C.c_uint64(0), C.c_int(0), self.t.shape
+        nnz, launched, (M, K) = C.c_uint64(0), C.c_int(0), self.t.shape
         rc = self.L.bitcos_pack_device_limited(
             self.t.data_ptr(), self.sc.data_ptr(), M, K, self.bitmap.data_ptr(), self.signs.data_ptr(), self.sign_bytes, self.off.data_ptr(),
-            self.scales.data_ptr(), self.off_host.data_ptr(), C.byref(nnz), self.scratch.data_ptr(), limit_ns, C.byref(kernels),
+            self.scales.data_ptr(), self.off_host.data_ptr(), C.byref(nnz), self.scratch.data_ptr(), limit_ns, C.byref(launched),
             self.stream.cuda_stream)
-        return rc, kernels.value, nnz.value
+        return rc, launched.value, nnz.value
 
     def equals(self, W):
         """All of this call's buffers against a packed matrix; nothing behind the sign vector was touched."""
@@ -258,31 +258,35 @@ class CPack:
                 and np.array_equal(self.off_host.numpy()[:W.tile_off_host.size].view(np.uint32), W.tile_off_host))
 
 
+def kernels(M, K):
+    """How many kernels pack a matrix if no wait runs out."""
+    return 1 if 6144 <= (M + 31) // 32 * (K // 128) <= 180224 else 3
+
+
 def trits_and_scales(seed, M, K):
     gen = torch.Generator(device="cuda").manual_seed(seed)
     t = torch.randint(-1, 2, (M, K), generator=gen, device="cuda", dtype=torch.int8)
     return t, (0.01 + torch.rand((M, K // 128), generator=gen, device="cuda")).to(torch.bfloat16)
 
 
-@pytest.mark.parametrize("M,K", [(32, 1024), (32, 1152), (300, 1280), (2560, 2560), (4097, 6144), (32 * 4737, 128), (25600, 5120)])
+@pytest.mark.parametrize("M,K", [(300, 1280), (32 * 6143, 128), (32 * 6144, 128), (4097, 6144), (32 * 6513, 128), (25600, 5120)])
 def test_device_pack_goes_on_when_its_wait_runs_out(bc, M, K):
     """With no time to wait every block but the first gives up; the call then packs in three kernels, and the same state serves the
-    calls after it.  (Up to eight tiles are one block's, which waits for nobody.)"""
+    calls after it."""
     t, sc = trits_and_scales(31 + M + K, M, K)
     W = bc.bitcos_pack_device(t, sc)
-    gives_up = (M + 31) // 32 * (K // 128) > 8
-    for limit, want in ((500_000_000, 1), (0, 4 if gives_up else 1), (0, 4 if gives_up else 1), (500_000_000, 1)):
+    in_time = kernels(M, K)
+    given_up = 4 if in_time == 1 else 3
+    for limit, want in ((500_000_000, in_time), (0, given_up), (0, given_up), (500_000_000, in_time)):
         call = CPack(bc, t, sc)
         assert call.run(limit) == (0, want, W.nnz) and call.equals(W), limit
-    if not gives_up:
-        return
     bad = t.clone()
     bad[M - 1, K - 1] = 3
-    assert CPack(bc, bad, sc).run(0)[:2] == (4, 4)
+    assert CPack(bc, bad, sc).run(0)[:2] == (4, given_up)
     bad = sc.clone()
     bad[M - 1, 0] = -1.0
-    assert CPack(bc, t, bad).run(0)[:2] == (5, 4)
-    assert CPack(bc, t, sc, lambda need: need - 16).run(0)[:2] == (6, 4)
+    assert CPack(bc, t, bad).run(0)[:2] == (5, given_up)
+    assert CPack(bc, t, sc, lambda need: need - 16).run(0)[:2] == (6, given_up)
 
 
 @pytest.mark.parametrize("M,K", [(96, 640), (2560, 2560), (8192, 5120)])
@@ -292,7 +296,7 @@ def test_device_pack_and_the_size_of_the_sign_vector(bc, M, K):
     W = bc.bitcos_pack_device(t, sc)
     for more, rc in ((-16, 6), (0, 0), (16, 0), (32 * 1024 + 48, 0), (2 * M * K // 8, 0)):
         call = CPack(bc, t, sc, lambda need: need + more)
-        assert call.run()[:2] == (rc, 1), more
+        assert call.run()[:2] == (rc, kernels(M, K)), more
         if rc == 0:
             assert call.equals(W), more
         assert bool((call.signs[call.sign_bytes // 4:] == -1).all()), more
@@ -324,7 +328,7 @@ def test_device_pack_from_several_threads(bc):
 def test_device_pack_when_all_states_are_taken(bc):
     """Seventy calls at a time, held up behind a kernel that waits: 64 find a state, the others pack in three kernels."""
     import threading
-    t, sc = trits_and_scales(71, 640, 2560)
+    t, sc = trits_and_scales(71, 6144, 4096)
     want = bc.bitcos_pack_device(t, sc)
     n = 70
     calls = [CPack(bc, t, sc, stream=torch.cuda.Stream()) for _ in range(n)]

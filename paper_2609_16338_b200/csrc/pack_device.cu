@@ -15,7 +15,7 @@
 // the counts (the entry offsets); the sign vector, from a second reading, mostly from L2.
 //
 // A C call, three kernels -> one, medians of calls in turn, us: 64 tiles 21.2 -> 19.2, 256 21.7 -> 21.8, 1024 22.4 -> 23.9, 2560 32.6 -> 34.0, 4096 28.9 ->
-// 31.0, 6144 33.6 -> 33.5, 8192 38.9 -> 34.9, 10240 (8192x5120) 43.4 -> 38.1, 20480 70.6 -> 53.8, 32000 (25600x5120) 104.7 -> 69.0.  With few tiles the
+// 31.0, 6144 33.6 -> 33.5, 8192 38.9 -> 34.9, 10240 (8192x5120) 43.4 -> 38.1, 20480 70.6 -> 51.3, 32000 (25600x5120) 104.7 -> 65.6.  With few tiles the
 // look-back's trips to L2 are a larger part than a second reading.  Through the binding 8192x5120 takes 77 (as a cooperative launch of
 // one block of 1024 threads per multiprocessor 81), about 40 of them allocations and calls in Python; the trits would pass in 6.4 at
 // the memory's rate.  A tile is about 1100 warp instructions (a quarter of them the compress), 0.19 us a tile and multiprocessor, which bounds the
@@ -404,15 +404,6 @@ __global__ void __launch_bounds__(kOnceThreads, kOnceBlocks) pack_once_kernel(co
     }
     __syncthreads();
     const int r = s_range, t_lo = r * per_range, mine = n_tiles - t_lo < per_range ? n_tiles - t_lo : per_range;
-    // Zeros over the sign vector: the words that would be this range's if every weight were there, and a share of what lies behind all of
-    // those.  Sign bits never lie further back, so a range's zeros are written over by itself and later ranges only, which
-    // have waited for its word.
-    uint4 *const zeros = reinterpret_cast<uint4 *>(signs);
-    const uint4 none = make_uint4(0u, 0u, 0u, 0u);
-    const int64_t z_lo = static_cast<int64_t>(t_lo) * 32, z_hi = z_lo + mine * 32 < sign_quads ? z_lo + mine * 32 : sign_quads;
-    for (int64_t i = z_lo + threadIdx.x; i < z_hi; i += kOnceThreads) zeros[i] = none;
-    for (int64_t i = static_cast<int64_t>(n_tiles) * 32 + r * kOnceThreads + threadIdx.x; i < sign_quads; i += static_cast<int64_t>(n_ranges) * kOnceThreads)
-        zeros[i] = none;
     // ---- counts, bitmap, scales; sign bits into shared memory
     uint4 v[8];
     uint16_t s_v = 0;
@@ -479,6 +470,16 @@ __global__ void __launch_bounds__(kOnceThreads, kOnceBlocks) pack_once_kernel(co
             put(at1[i], both[i] >> 16);
         }
     }
+    // Zeros over the sign vector: the words that would be this range's if every weight were there, and a share of what lies behind all of
+    // those.  Sign bits never lie further back, so a range's zeros are written over by itself and later ranges only, which
+    // have waited for its word.  (Behind the reading of the tiles: in front of it 16384x5120 | 25600x5120 took 53.3 | 68.7 us a call, here
+    // 51.3 | 65.6.)
+    uint4 *const zeros = reinterpret_cast<uint4 *>(signs);
+    const uint4 none = make_uint4(0u, 0u, 0u, 0u);
+    const int64_t z_lo = static_cast<int64_t>(t_lo) * 32, z_hi = z_lo + mine * 32 < sign_quads ? z_lo + mine * 32 : sign_quads;
+    for (int64_t i = z_lo + threadIdx.x; i < z_hi; i += kOnceThreads) zeros[i] = none;
+    for (int64_t i = static_cast<int64_t>(n_tiles) * 32 + r * kOnceThreads + threadIdx.x; i < sign_quads; i += static_cast<int64_t>(n_ranges) * kOnceThreads)
+        zeros[i] = none;
     __syncthreads();
     // ---- this range's total, and every tile's place behind the range's first sign bit (a tile per thread)
     const uint32_t c = threadIdx.x < static_cast<unsigned>(mine) ? count[threadIdx.x] : 0u;
